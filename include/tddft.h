@@ -68,8 +68,11 @@ typedef enum { TDDFT_F64 = 0, TDDFT_F32 = 1 } tddft_dtype;
 typedef enum { TDDFT_PRECOND_DIAG = 0, TDDFT_PRECOND_RID = 1 } tddft_precond;
 
 /* Arithmetic of the solve.
- * PLAIN: every step in FP64 (factors, products, subspace algebra).
- * MIXED: exact products with FP32 factors and FP32 accumulation, or, when
+ * PLAIN: every step in FP64 (factors, products, subspace algebra); the exchange
+ *        products run on the tensor cores as exact integer slices of the FP64
+ *        operands (56 bits per row, error below that of FP64 arithmetic).
+ * MIXED: exact products with FP32 factors (exchange: exact integer slices, 32
+ *        bits per row; Coulomb: FP32 accumulation), or, when
  *        `tensor_cores` is set, on the tcgen05 tensor cores with every operand
  *        (factors, trial vectors, the first contraction's results) scaled by
  *        a power of two and split into FP16 hi + lo parts (22 significand
@@ -415,8 +418,8 @@ tddft_status tddft_pool_usage(int device, unsigned long long* used_current,
  * totals; 0 stops.  tddft_profile_read returns, for that contraction, the
  * number of launches, their summed device time (ms) and the algorithmic
  * flops (2*M*N*K per launch) since the last reset: which = 0 for the
- * tcgen05 kernel (tensor_cores on), 1 for the SIMT kernel (tensor cores
- * off).  Other values:
+ * tcgen05 kernel (tensor_cores on), 1 for the contraction of products without
+ * tensor_cores (the sliced FP64 / FP32 kernel and the sum of its K splits).  Other values:
  * TDDFT_ERR_ARG.                                                          */
 tddft_status tddft_profile(tddft_ctx* ctx, int enable);
 tddft_status tddft_profile_read(const tddft_ctx* ctx, int which, long long* launches,

@@ -12,10 +12,14 @@
 //   K2: Q[n][i][P][j] = sum_b L_ov[P][i][b] X[n][j][b]
 //       K2[(n,i)][a] = sum_(P,j) Q[(n,i)][(P,j)] L_ov[P][j][a]
 // P is processed in chunks so the intermediates stay within a bounded
-// workspace; the second contractions of K1 and K2 (most of the flops) run on the
-// tcgen05 tensor cores when asked (MIXED precision).
+// workspace; the contractions of K1 and K2 (most of the flops) run on the tcgen05
+// tensor cores: as FP16 hi + lo operands when asked (MIXED with tensor_cores,
+// tc_gemm.cuh), else as exact slices of the FP64 or FP32 operands
+// (slice_gemm.cuh).  Only BF16 ris rows against FP32 vectors without
+// tensor_cores run on the FP32 units.
 #include "ctx.cuh"
 #include "skinny.cuh"
+#include "slice_gemm.cuh"
 #include "tc_gemm.cuh"
 #include "vecops.cuh"
 
@@ -90,11 +94,14 @@ KernelProfile::~KernelProfile() {
 }
 
 namespace {
-// Exchange intermediates of one P-chunk: SIMT contractions keep them within
-// 512 MB; the tensor-core path takes 4 GB, so that a contraction launch covers
+// Exchange intermediates of one P-chunk: SIMT contractions (BF16 ris rows) keep
+// them within 512 MB; the tensor-core path takes 4 GB, so that a contraction launch covers
 // many auxiliary rows (longer K loops per CTA, fewer launches and pipeline fills).
 constexpr size_t kChunkBytes = 512ull << 20;
 constexpr size_t kChunkBytesTC = 4ull << 30;
+// The sliced contractions (slice_gemm.cuh) keep Z and Q, their slices and the
+// factors' slices of a chunk: 1 GB in all.
+constexpr size_t kChunkBytesSliced = 1ull << 30;
 // k-blocks one CTA accumulates in FP32 before its split-K partial is summed
 // (fixed order) with the others: the rounding of an FP32 run grows with its
 // length, and runs over a whole P-chunk of the exchange contraction (~1e4 MMA
@@ -121,6 +128,106 @@ void check_tc_error(Ctx& c) {
   if (h != 0) {
     TD_CUDA(cudaMemsetAsync(c.tc_err.p, 0, 4, c.s));
     throw Error(TDDFT_ERR_CUDA, "tensor-core kernel wait timed out (code " + std::to_string(h) + ")");
+  }
+}
+
+// K1 (and K2) of an FP64 or FP32 factor set, every contraction on the tensor cores
+// by exact slicing (slice_gemm.cuh): no FP64 or FP32 vector arithmetic beyond
+// the cuts.  Xw: trial vectors in the factors' type.
+static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw, int m, bool need_k2, void* K1,
+                            void* K2, cudaStream_t s) {
+  const int no = d.no, nv = d.nv, ov = d.ov;
+  const DType t = f.dt;
+  const size_t es = dtype_size(t), sb = 2 * (size_t)slice_count(t);
+  const size_t nop = tc_pad(no), nvp = tc_pad(nv);
+  const size_t per_row = (size_t)m * no * (nv * es + nvp * sb) + (no * nop + nv * nvp) * sb +
+                         (need_k2 ? (size_t)m * no * (no * es + nop * sb) + (no * nvp + nv * nop) * sb : 0);
+  const int pc = chunk_rows(f.nK, (long long)per_row, 1, kChunkBytesSliced);
+  struct Cut {
+    SliceOperand o;
+    DevBuf parts, exps;
+    void alloc(cudaStream_t st) {
+      parts = DevBuf(slice_bytes(o), st);
+      exps = DevBuf((size_t)o.rows * 4, st);
+    }
+    void cut(cudaStream_t st) { slice_cut(o, parts.p, exps.as<int>(), st); }
+    int* e() const { return exps.as<int>(); }
+  };
+  auto operand = [&](const void* p, int rows, int np, int K) {
+    Cut c;
+    c.o.p = p;
+    c.o.t = t;
+    c.o.rows = rows;
+    c.o.np = np;
+    c.o.K = K;
+    return c;
+  };
+  // X^T per vector: rows (n, a), k = j; X: rows (n, j), k = b
+  Cut xt = operand(Xw, m * nv, 1, no), xs = operand(Xw, m * no, 1, nv);
+  xt.o.R = nv; xt.o.rs1 = ov; xt.o.rs0 = 1; xt.o.ks = nv;
+  xt.alloc(s);
+  xt.cut(s);
+  if (need_k2) {
+    xs.o.rs0 = nv;
+    xs.alloc(s);
+    xs.cut(s);
+  }
+  DevBuf Zb((size_t)m * no * pc * nv * es, s), Qb;
+  if (need_k2) Qb = DevBuf((size_t)m * no * pc * no * es, s);
+  // chunk operands, allocated for the first (largest) chunk
+  Cut oo = operand(nullptr, pc * no, 1, no), vv = operand(nullptr, nv, pc, nv), z = operand(Zb.p, m * no, pc, nv);
+  Cut ov_ = operand(nullptr, pc * no, 1, nv), vo = operand(nullptr, nv, pc, no), q = operand(Qb.p, m * no, pc, no);
+  oo.o.rs0 = no; oo.o.p_outer = true;
+  vv.o.rs0 = nv; vv.o.ps = (long long)nv * nv; vv.o.p_outer = true;
+  z.o.ps = nv;
+  ov_.o.rs0 = nv; ov_.o.p_outer = true;
+  vo.o.rs0 = 1; vo.o.ks = nv; vo.o.ps = ov; vo.o.p_outer = true;
+  q.o.ps = no;
+  oo.alloc(s);
+  vv.alloc(s);
+  z.alloc(s);
+  if (need_k2) {
+    ov_.alloc(s);
+    vo.alloc(s);
+    q.alloc(s);
+  }
+  for (int p0 = 0; p0 < f.nK; p0 += pc) {
+    const int pn = (f.nK - p0 < pc) ? f.nK - p0 : pc;
+    const double beta = p0 > 0 ? 1.0 : 0.0;
+    // Z[n][i][P][a] = sum_j Koo[P][i][j] X[n][j][a]
+    oo.o.p = (const char*)f.Koo + (size_t)p0 * no * no * es;
+    oo.o.rows = pn * no;
+    oo.cut(s);
+    slice_gemm_scatter(xt.o, xt.parts.p, xt.e(), oo.o, oo.parts.p, oo.e(), Zb.p,
+                       SliceScatter{nv, no, (long long)no * pn * nv, (long long)pn * nv, nv}, d.tc_err, s);
+    z.o.rs0 = (long long)pn * nv;
+    z.o.np = pn;
+    z.cut(s);
+    vv.o.p = (const char*)f.Kvv + (size_t)p0 * nv * nv * es;
+    vv.o.np = pn;
+    vv.cut(s);
+    const bool timed = d.prof_simt && d.prof_simt->on;
+    if (timed) d.prof_simt->begin(s);
+    slice_gemm(z.o, z.parts.p, z.e(), vv.o, vv.parts.p, vv.e(), K1, beta, d.tc_err, s);
+    if (timed)
+      d.prof_simt->end(s, 2.0 * m * no * (double)nv * (double)pn * nv,
+                       (double)es * ((double)m * no * pn * nv + (double)pn * nv * nv +
+                                     (double)m * no * nv * (p0 > 0 ? 2.0 : 1.0)));
+    if (need_k2) {
+      // Q[n][i][P][j] = sum_b Kov[P][i][b] X[n][j][b]
+      ov_.o.p = (const char*)f.Kov + (size_t)p0 * ov * es;
+      ov_.o.rows = pn * no;
+      ov_.cut(s);
+      slice_gemm_scatter(xs.o, xs.parts.p, xs.e(), ov_.o, ov_.parts.p, ov_.e(), Qb.p,
+                         SliceScatter{no, no, (long long)no * pn * no, (long long)pn * no, no}, d.tc_err, s);
+      q.o.rs0 = (long long)pn * no;
+      q.o.np = pn;
+      q.cut(s);
+      vo.o.p = ov_.o.p;
+      vo.o.np = pn;
+      vo.cut(s);
+      slice_gemm(q.o, q.parts.p, q.e(), vo.o, vo.parts.p, vo.e(), K2, beta, d.tc_err, s);
+    }
   }
 }
 
@@ -305,7 +412,10 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
                       d.tc_err, s, nullptr, 0.0, 0.0, f16 ? kExchangeKb : 0);
         }
       }
+    } else if (f.dt != DType::BF16) {
+      exchange_sliced(d, f, Xw, m, need_k2, K1b.p, K2b.p, s);
     } else {
+      // ris rows (BF16) against FP32 trial vectors on the FP32 units
       DevBuf Zb((size_t)m * no * pc * nv * ew, s);
       DevBuf Qb;
       if (need_k2) Qb = DevBuf((size_t)m * no * pc * no * ew, s);
@@ -324,8 +434,6 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
         gemm(z, s);
         const int Mz = m * no;
         const long long Kz = (long long)pn * nv;
-        const bool timed = d.prof_simt && d.prof_simt->on && f.dt != DType::BF16;
-        if (timed) d.prof_simt->begin(s);
         GemmDesc k;
         k.acc64 = f64;
         k.M = Mz; k.N = nv; k.K = (int)Kz;
@@ -334,10 +442,6 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
         k.C = K1b.p; k.tc = tw; k.scm = nv; k.scn = 1;
         k.beta = (p0 > 0) ? 1.0 : 0.0;
         gemm_splitk(k, auto_splits(k.M, k.N, k.K), s);
-        if (timed)
-          d.prof_simt->end(s, 2.0 * Mz * (double)nv * (double)Kz,
-                           (double)ew * Mz * (double)Kz + (double)es * Kz * nv +
-                               (double)ew * Mz * nv * (p0 > 0 ? 2.0 : 1.0));
         if (need_k2) {
           // Q[n][i][P][j] = sum_b Kov[P][i][b] X[n][j][b]
           GemmDesc q;

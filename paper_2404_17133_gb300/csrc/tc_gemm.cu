@@ -708,6 +708,25 @@ CUtensorMap make_map(const void* base, const cuuint64_t dims[3], const cuuint64_
 
 }  // namespace
 
+CUtensorMap tc_map_f16_4d(const void* base, const uint64_t dims[4], const uint64_t strides[3], const uint32_t box[4],
+                          int swizzle_bytes) {
+  TD_REQUIRE((reinterpret_cast<uintptr_t>(base) & 15) == 0, TDDFT_ERR_ARG, "TMA base not 16-byte aligned");
+  TD_REQUIRE(strides[0] % 16 == 0 && strides[1] % 16 == 0 && strides[2] % 16 == 0, TDDFT_ERR_ARG,
+             "TMA strides not 16-byte multiples");
+  CUtensorMap m;
+  cuuint64_t d[4], st[3];
+  cuuint32_t b[4];
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  for (int i = 0; i < 4; ++i) { d[i] = dims[i]; b[i] = box[i]; }
+  for (int i = 0; i < 3; ++i) st[i] = strides[i];
+  CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(base), d, st, b, es,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  TD_REQUIRE(r == CUDA_SUCCESS, TDDFT_ERR_CUDA, "cuTensorMapEncodeTiled failed");
+  return m;
+}
+
 int tc_pad(int nv) { return (nv + 7) & ~7; }
 int tc_pad16(int n) { return (n + 15) & ~15; }
 
@@ -759,7 +778,7 @@ int sm_count() {
 // (units per CTA + a fixed per-CTA cost of `overhead` units), so a last,
 // nearly empty wave costs as much as a full one.  Tries the splits that fill
 // one to four waves and keeps the cheapest (the fewest splits on ties).
-int wave_splits(int tiles, int total, int overhead, int sms = 0) {
+int wave_splits(int tiles, int total, int overhead, int sms) {
   if (sms <= 0) sms = sm_count();
   int best = 1;
   long long best_cost = -1;

@@ -1,5 +1,8 @@
 // tcgen05 tensor-core contractions of the exchange terms (FP16 or BF16 hi+lo splits, FP8 ris).
 #pragma once
+#include <cstdint>
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace tddft {
@@ -14,6 +17,15 @@ enum class TcElt : int { BF16 = 0, F16 = 1 };
 int tc_pad(int nv);
 // Row pitch (elements) of the padded FP8 operands: n rounded up to 16.
 int tc_pad16(int n);
+
+// SMs of the current device (queried once).
+int sm_count();
+// K splits of `tiles` output tiles over `total` units so that whole waves of one
+// CTA per SM (or of `sms` slots) are filled; `overhead`: a CTA's fixed cost in units.
+int wave_splits(int tiles, int total, int overhead, int sms = 0);
+// 4-D tiled TMA map over FP16 elements (strides in bytes; 64- or 128-byte swizzle).
+CUtensorMap tc_map_f16_4d(const void* base, const uint64_t dims[4], const uint64_t strides[3], const uint32_t box[4],
+                          int swizzle_bytes);
 
 // Factor rows src [rows][n1][n2] (F64, F32 or BF16) -> hi (+ lo unless NULL)
 // [rows][n2][tc_pad(n1)] of element type et, transposed in the last two
