@@ -171,16 +171,9 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 }
 
 
-// CL = 2: the CTAs run in clusters of two along the M tiles; both need the same
-// B tile, so each loads half of its rows and multicasts them to both (halving
-// each SM's B traffic), and a stage is refilled only after both CTAs' MMAs
-// have read it (their commits arrive on both CTAs' `empty` barriers).
-// CX = 2 (with CL = 2): clusters of 2 x 2, the two CTAs of each N pair also
-// share their A tile the same way.  Cluster rank r = x + CX y: the CTAs that
-// share r's A tile are those of its row y, those that share its B tile those
-// of its column x; r's stage is written by both, so r's `empty` barrier counts
-// the commits of all of them (CL + CX - 1).
-template <int MODE, int ET, int CL = 1, int RB = 128, int CX = 1>
+// One CTA per output tile: problems with a single M tile (k1_pair_kernel takes
+// the others).
+template <int MODE, int ET, int RB = 128>
 __global__ void __launch_bounds__(THREADS, 1)
 k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ CUtensorMap mA_lo,
              const __grid_constant__ CUtensorMap mB_hi, const __grid_constant__ CUtensorMap mB_lo,
@@ -191,7 +184,6 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
   constexpr int B_OFF = a_split(MODE) ? 2 * AB : AB;                // first B tile in a stage
   constexpr int BKE = Elem<ET>::BKE * RB / 128;                     // K elements per k-block
   constexpr int KSTEPS = RB / 32;                                   // 32-byte K steps per k-block
-  constexpr int CN = CL * CX;                                       // CTAs per cluster
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -206,15 +198,8 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
   const int k_end = min(p.total, k_begin + p.per_split);
   const int nk = max(0, k_end - k_begin);
 
-  const uint32_t crank = CN > 1 ? cluster_rank() : 0u;
-  const uint32_t cx = crank % CX, cy = crank / CX;
-  uint16_t mask_a = 0, mask_b = 0;   // CTAs receiving this CTA's A / B rows
-#pragma unroll
-  for (int x = 0; x < CX; ++x) mask_a |= (uint16_t)(1u << (x + CX * cy));
-#pragma unroll
-  for (int y = 0; y < CL; ++y) mask_b |= (uint16_t)(1u << (cx + CX * y));
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], CL + CX - 1); }
+    for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -224,7 +209,6 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   __syncthreads();
-  if constexpr (CN > 1) cluster_sync_all();   // every barrier of the cluster initialised
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
@@ -239,42 +223,20 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
       const int P = kb / p.nab, a0 = (kb - P * p.nab) * BKE;
       unsigned char* st = smem + s * STAGE_BYTES;
       mbar_expect_tx(&full[s], STAGE_BYTES);
-      if constexpr (CX > 1) {
-        // this CTA's share of the A rows, to every CTA of its row
-        constexpr int HA = AB / CX;
-        const int mh = m0 + (int)cx * (BM / CX);
-        tma_load_3d_mc(st + cx * HA, &mA_hi, &full[s], a0, P, mh, mask_a);
-        if (a_split(MODE)) tma_load_3d_mc(st + AB + cx * HA, &mA_lo, &full[s], a0, P, mh, mask_a);
-      } else {
-        tma_load_3d(st, &mA_hi, &full[s], a0, P, m0);
-        if (a_split(MODE)) tma_load_3d(st + AB, &mA_lo, &full[s], a0, P, m0);
-      }
-      if constexpr (CL > 1) {
-        // this CTA's share of the B rows, to every CTA of its column
-        constexpr int HB = BB / CL;
-        const int nh = n0 + (int)cy * (BN / CL);
-        tma_load_3d_mc(st + B_OFF + cy * HB, &mB_hi, &full[s], a0, nh, P, mask_b);
-        if (b_split(MODE)) tma_load_3d_mc(st + B_OFF + BB + cy * HB, &mB_lo, &full[s], a0, nh, P, mask_b);
-      } else {
-        tma_load_3d(st + B_OFF, &mB_hi, &full[s], a0, n0, P);
-        if (b_split(MODE)) tma_load_3d(st + B_OFF + BB, &mB_lo, &full[s], a0, n0, P);
-      }
+      tma_load_3d(st, &mA_hi, &full[s], a0, P, m0);
+      if (a_split(MODE)) tma_load_3d(st + AB, &mA_lo, &full[s], a0, P, m0);
+      tma_load_3d(st + B_OFF, &mB_hi, &full[s], a0, n0, P);
+      if (b_split(MODE)) tma_load_3d(st + B_OFF + BB, &mB_lo, &full[s], a0, n0, P);
     }
     // let the copies already issued land before the CTA can exit
     for (int i = max(0, nk - STAGES); i < nk; ++i) {
       if (!mbar_wait(&full[i % STAGES], (uint32_t)(i / STAGES) & 1u)) { atomicOr(p.err, 2); break; }
     }
-    if constexpr (CN > 1) {
-      // and the peers' last commits arrive on this CTA's `empty` barriers
-      for (int i = nk; i < nk + STAGES; ++i) {
-        if (!mbar_wait(&empty[i % STAGES], ((uint32_t)(i / STAGES) & 1u) ^ 1u)) { atomicOr(p.err, 2); break; }
-      }
-    }
   } else if (warp == 1 && lane == 0) {
     // ---- MMA issuer.  The MMA spans only the tile's columns below N
     // (rounded up to 16) and, in the last k-block of each P, only the 32-byte
     // K steps below Kin: the skipped products are of TMA's zero fill.
-    const int nb_cta = max(16, min(BN, (p.N - n0 + 15) & ~15));   // >= 16: a padding tile of a cluster
+    const int nb_cta = min(BN, (p.N - n0 + 15) & ~15);
     const uint32_t idesc = idesc_of<ET>(nb_cta);
     bool ok = true;
     for (int i = 0; i < nk; ++i) {
@@ -295,8 +257,7 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
           if (a_split(MODE)) mma_op<ET>(tmem, sdesc_rb<RB>(st + AB) + off, bh + off, 1u, idesc);
         }
       }
-      if constexpr (CN > 1) mma_commit_mc(&empty[s], (uint16_t)(mask_a | mask_b));
-      else mma_commit(&empty[s]);
+      mma_commit(&empty[s]);
     }
     (void)ok;
     mma_commit(done);   // fires when every MMA issued above has completed
@@ -349,9 +310,251 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
   if (warp == 1) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
   }
-  if constexpr (CN > 1) cluster_sync_all();   // no CTA leaves while another may still signal it
 }
 
+// Row pairs of CTAs on one 256-row tile (cta_group::2): the pair's tcgen05.mma
+// takes 128 A rows and half of the B rows from each CTA's shared memory, so
+// every SM reads and stores only half of B.  That is what bounds the single-CTA
+// form: per 16-element K step of the hi + lo products it reads 36 KB of operands
+// and receives 24 KB by TMA in the 384 cycles of its MMAs, against 128 bytes per
+// cycle of shared memory; here 24 KB (20 KB with A_hi held in the operand
+// collector for its two products) and 16 KB.
+// CX = 2: clusters of two pairs along N, which also share their A rows (each CTA
+// loads half of its rows and multicasts them to the CTA of the other pair that
+// needs the same ones).
+// Cluster rank = h + 2 y: h the row half, y the pair; the pair's leader is h = 0.
+// All four (two) CTAs' loads of a pair's stage signal the leader's `full`
+// barrier, the leader's commit frees the stage in every CTA that writes it.
+// N is cut into tiles of whole 32-column units, as equal as they can be: tiles
+// of 256 columns and a remainder would leave a cluster's lighter pair waiting.
+template <int MODE, int RB> struct PCfg {
+  static constexpr int AB = BM * RB, HB = (BN / 2) * RB;   // one part of A, of half of B
+  static constexpr int STAGE_BYTES = n_parts_a(MODE) * AB + n_parts_b(MODE) * HB;
+  static constexpr int STAGES = 196608 / STAGE_BYTES;
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+};
+
+struct PairParams {
+  int M, N, Kin, nab, total, per_split;
+  int nt, nt0, mp;   // N tiles (padded to whole clusters; real ones), M tile pairs
+  int nq, nr;        // 32-column units per N tile; the first nr tiles have one more
+  int b_rows;        // rows of half of the widest B tile (the TMA box)
+  float* part;
+  int* err;
+};
+
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
+// Load into this CTA (or, with a mask, into the same offset of its CTAs), signalling
+// the mbarrier `bar` (a shared::cluster address) of the pair's leader.
+__device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
+                                                 int c2) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair_mc(void* dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
+                                                    int c2, uint16_t mask) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster"
+      ".cta_group::2 [%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "h"(mask)
+      : "memory");
+}
+
+// Pair MMA; KEEP: 0 plain, 1 the A operand stays in the collector, 2 its last use.
+template <int ET, int KEEP>
+__device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t accum, uint32_t idesc) {
+#define TD_MMA2(kind, coll)                                                                       \
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"                                     \
+               " tcgen05.mma.cta_group::2." kind coll " [%0], %1, %2, %3, p;\n}\n" ::"r"(d),      \
+               "l"(a), "l"(b), "r"(idesc), "r"(accum))
+  if constexpr (ET == ET_E4M3) {
+    TD_MMA2("kind::f8f6f4", "");
+  } else if constexpr (KEEP == 1) {
+    TD_MMA2("kind::f16", ".collector::a::fill");
+  } else if constexpr (KEEP == 2) {
+    TD_MMA2("kind::f16", ".collector::a::lastuse");
+  } else {
+    TD_MMA2("kind::f16", "");
+  }
+#undef TD_MMA2
+}
+
+__device__ __forceinline__ void commit_pair(uint64_t* bar, uint16_t mask) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"(mask)
+      : "memory");
+}
+
+template <int MODE, int ET, int CX, int RB>
+__global__ void __launch_bounds__(THREADS, 1)
+k1_pair_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ CUtensorMap mA_lo,
+               const __grid_constant__ CUtensorMap mB_hi, const __grid_constant__ CUtensorMap mB_lo,
+               const PairParams p) {
+  using C = PCfg<MODE, RB>;
+  constexpr int STAGES = C::STAGES;
+  constexpr int B_OFF = n_parts_a(MODE) * C::AB;
+  constexpr int BKE = Elem<ET>::BKE * RB / 128;   // K elements per k-block
+  constexpr int KSTEPS = RB / 32;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * C::STAGE_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* done = empty + STAGES;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const int h = (int)(rank & 1u), y = (int)(rank >> 1);
+  // N pairs fastest: the clusters that run together share their A rows through L2
+  const int cid = blockIdx.x / (2 * CX), ntc = p.nt / CX;
+  const int t = (cid % ntc) * CX + y;
+  const int m0 = ((cid / ntc) % p.mp) * 2 * BM + h * BM;
+  const int z = cid / (ntc * p.mp);
+  const int n0 = 32 * (min(t, p.nt0) * p.nq + min(t, p.nr));
+  const int width = t < p.nt0 ? 32 * (p.nq + (t < p.nr ? 1 : 0)) : 32;   // a padding tile is all zero fill
+  const int k_begin = z * p.per_split;
+  const int nk = max(0, min(p.total, k_begin + p.per_split) - k_begin);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], CX); }
+    mbar_init(done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)), "r"(BN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+  }
+  __syncthreads();
+  cluster_sync_all();   // every barrier of the cluster initialised
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0 && lane == 0) {
+    // ---- TMA producer (both CTAs of the pair)
+    const uint32_t lead_full = mapa(smem_u32(full), rank & ~1u);
+    const uint32_t bytes = 2u * (n_parts_a(MODE) * C::AB + n_parts_b(MODE) * (uint32_t)p.b_rows * RB);
+    const uint16_t mask_a = (uint16_t)((1u << h) | (1u << (h + 2)));   // CX = 2: the CTAs of this row half
+    const int nh = n0 + h * (width / 2);
+    for (int i = 0; i < nk; ++i) {
+      const int s = i % STAGES;
+      if (!mbar_wait(&empty[s], ((uint32_t)(i / STAGES) & 1u) ^ 1u)) { atomicOr(p.err, 1); break; }
+      const int kb = k_begin + i;
+      const int P = kb / p.nab, a0 = (kb - P * p.nab) * BKE;
+      unsigned char* st = smem + s * C::STAGE_BYTES;
+      const uint32_t bar = lead_full + (uint32_t)(s * 8);
+      if (h == 0) mbar_expect_tx(&full[s], bytes);
+      if constexpr (CX > 1) {
+        constexpr int HA = C::AB / 2;
+        const int mh = m0 + y * (BM / 2);
+        tma_load_3d_pair_mc(st + y * HA, &mA_hi, bar, a0, P, mh, mask_a);
+        if (a_split(MODE)) tma_load_3d_pair_mc(st + C::AB + y * HA, &mA_lo, bar, a0, P, mh, mask_a);
+      } else {
+        tma_load_3d_pair(st, &mA_hi, bar, a0, P, m0);
+        if (a_split(MODE)) tma_load_3d_pair(st + C::AB, &mA_lo, bar, a0, P, m0);
+      }
+      tma_load_3d_pair(st + B_OFF, &mB_hi, bar, a0, nh, P);
+      if (b_split(MODE)) tma_load_3d_pair(st + B_OFF + C::HB, &mB_lo, bar, a0, nh, P);
+    }
+    // let the copies already issued (they signal the leader) land, and the last
+    // commits arrive on this CTA's `empty` barriers, before a CTA can exit
+    if (h == 0)
+      for (int i = max(0, nk - STAGES); i < nk; ++i)
+        if (!mbar_wait(&full[i % STAGES], (uint32_t)(i / STAGES) & 1u)) { atomicOr(p.err, 2); break; }
+    for (int i = nk; i < nk + STAGES; ++i)
+      if (!mbar_wait(&empty[i % STAGES], ((uint32_t)(i / STAGES) & 1u) ^ 1u)) { atomicOr(p.err, 2); break; }
+  } else if (warp == 1 && lane == 0 && h == 0) {
+    // ---- MMA issuer (the leader): M = 256, N = width; the last k-block of a P
+    // issues only the 32-byte K steps below Kin
+    const uint32_t idesc =
+        (1u << 4) | Elem<ET>::TYPE_BITS | ((uint32_t)(width >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
+    const uint16_t mask_all = (uint16_t)((1u << (2 * CX)) - 1);
+    for (int i = 0; i < nk; ++i) {
+      const int s = i % STAGES;
+      if (!mbar_wait(&full[s], (uint32_t)(i / STAGES) & 1u)) { atomicOr(p.err, 4); break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      unsigned char* st = smem + s * C::STAGE_BYTES;
+      const uint64_t ah = sdesc_rb<RB>(st), bh = sdesc_rb<RB>(st + B_OFF);
+      const int rem = p.Kin - ((k_begin + i) % p.nab) * BKE;
+      const int nks = rem >= BKE ? KSTEPS : (rem * KSTEPS + BKE - 1) / BKE;
+#pragma unroll
+      for (int kk = 0; kk < KSTEPS; ++kk) {
+        if (kk < nks) {
+          const uint64_t off = (uint64_t)(kk * 32) >> 4;
+          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
+          if (b_split(MODE)) {
+            mma_pair<ET, 1>(tmem, ah + off, bh + off, acc, idesc);
+            mma_pair<ET, 2>(tmem, ah + off, sdesc_rb<RB>(st + B_OFF + C::HB) + off, 1u, idesc);
+          } else {
+            mma_pair<ET, 0>(tmem, ah + off, bh + off, acc, idesc);
+          }
+          if (a_split(MODE)) mma_pair<ET, 0>(tmem, sdesc_rb<RB>(st + C::AB) + off, bh + off, 1u, idesc);
+        }
+      }
+      commit_pair(&empty[s], mask_all);
+    }
+    commit_pair(done, (uint16_t)(3u << (2 * y)));   // fires when every MMA issued above has completed
+  } else if (warp >= 2) {
+    // ---- epilogue: this CTA's 128 rows, TMEM -> registers -> FP32 partial tile
+    const int q = warp & 3;
+    const int row = m0 + q * 32 + lane;
+    bool have = mbar_wait(done, 0);
+    if (!have) atomicOr(p.err, 8);
+    have = __all_sync(0xffffffffu, have);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    float* out = p.part + (size_t)z * p.M * p.N;
+#pragma unroll 1
+    for (int c = 0; c < width; c += 16) {
+      uint32_t v[16];
+      if (nk > 0 && have) {
+        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c;
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15},"
+            " [%16];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+              "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+            : "r"(taddr));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = 0u;
+      }
+      if (row < p.M) {
+        const int col0 = n0 + c;
+        float* o = out + (size_t)row * p.N + col0;
+        if ((p.N & 3) == 0 && col0 + 16 <= p.N) {
+#pragma unroll
+          for (int j = 0; j < 16; j += 4)
+            *reinterpret_cast<float4*>(o + j) = make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]),
+                                                            __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]));
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (col0 + j < p.N) o[j] = __uint_as_float(v[j]);
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_sync_all();   // no CTA frees its half or leaves while the other may still use it
+  if (warp == 1) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
+  }
+}
 
 // ---------------------------------------------------------------------------
 // Stage-1 contractions of the exchange terms, batched over P:
@@ -810,21 +1013,19 @@ bool cluster_quads_enabled() {
 
 // CTAs of the paired contraction that can be resident at once: two per
 // co-resident cluster (an SM left over in a GPC takes no pair).
-int pair_slots(int et) {
-  static int cached[2] = {0, 0};
-  int& c = cached[et == ET_F16 ? 1 : 0];
+int pair_slots() {
+  static int c = 0;
   if (c == 0) {
-    const void* k = et == ET_F16 ? (const void*)k1_tc_kernel<BOTH, ET_F16, 2, 64>
-                                 : (const void*)k1_tc_kernel<BOTH, ET_BF16, 2, 64>;
-    const int smem = Cfg<BOTH, 64>::SMEM_BYTES;
+    const void* k = (const void*)k1_pair_kernel<BOTH, ET_F16, 1, 64>;
+    const int smem = PCfg<BOTH, 64>::SMEM_BYTES;
     ensure_smem(k, smem);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1;
-    at[0].val.clusterDim.y = 2;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(1, 2, 1);
+    cfg.gridDim = dim3(2, 1, 1);
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.attrs = at;
@@ -838,6 +1039,113 @@ int pair_slots(int et) {
   }
   return c;
 }
+
+// Operands of one contraction; the pointers are FP16 / BF16 parts or e4m3 bytes.
+struct Contraction {
+  const void *Ahi, *Alo;
+  int M, pn, Kin;
+  const void *Bhi, *Blo;
+  int N, ldk, es;      // row pitch (elements), element bytes
+  int total, per, splits, nab;
+  float* part;
+  int* err;
+  cudaStream_t s;
+  KernelProfile* prof;
+  double prof_flops, prof_bytes;
+};
+
+template <int MODE, int ET, int RB>
+void launch_pair(const Contraction& c) {
+  constexpr int BKE = Elem<ET>::BKE * RB / 128;
+  const int mt = (c.M + BM - 1) / BM, nt0 = (c.N + BN - 1) / BN;
+  const int cx = nt0 > 1 && cluster_quads_enabled() ? 2 : 1;
+  const int units = (c.N + 31) / 32;
+  PairParams p;
+  p.M = c.M;
+  p.N = c.N;
+  p.Kin = c.Kin;
+  p.nab = c.nab;
+  p.total = c.total;
+  p.per_split = c.per;
+  p.nt0 = nt0;
+  p.nt = (nt0 + cx - 1) / cx * cx;
+  p.mp = (mt + 1) / 2;
+  p.nq = units / nt0;
+  p.nr = units % nt0;
+  p.b_rows = 16 * (p.nq + (p.nr ? 1 : 0));
+  p.part = c.part;
+  p.err = c.err;
+  const cuuint64_t dA[3] = {(cuuint64_t)c.Kin, (cuuint64_t)c.pn, (cuuint64_t)c.M};
+  const cuuint64_t sA[2] = {(cuuint64_t)c.ldk * c.es, (cuuint64_t)c.pn * c.ldk * c.es};
+  const cuuint32_t bA[3] = {(cuuint32_t)BKE, 1, (cuuint32_t)(BM / cx)};
+  const cuuint64_t dB[3] = {(cuuint64_t)c.Kin, (cuuint64_t)c.N, (cuuint64_t)c.pn};
+  const cuuint64_t sB[2] = {(cuuint64_t)c.ldk * c.es, (cuuint64_t)c.N * c.ldk * c.es};
+  const cuuint32_t bB[3] = {(cuuint32_t)BKE, (cuuint32_t)p.b_rows, 1};
+  const CUtensorMap mAh = make_map(c.Ahi, dA, sA, bA, ET, RB), mBh = make_map(c.Bhi, dB, sB, bB, ET, RB);
+  const CUtensorMap mAl = c.Alo ? make_map(c.Alo, dA, sA, bA, ET, RB) : mAh;
+  const CUtensorMap mBl = c.Blo ? make_map(c.Blo, dB, sB, bB, ET, RB) : mBh;
+  auto go = [&](auto kernel) {
+    constexpr int smem = PCfg<MODE, RB>::SMEM_BYTES;
+    ensure_smem((const void*)kernel, smem);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2 * cx;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(2 * p.mp * p.nt * c.splits), 1, 1);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = c.s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (c.prof) c.prof->begin(c.s);
+    TD_CUDA(cudaLaunchKernelEx(&cfg, kernel, mAh, mAl, mBh, mBl, p));
+    if (c.prof) c.prof->end(c.s, c.prof_flops, c.prof_bytes);
+  };
+  if (cx > 1) go(k1_pair_kernel<MODE, ET, 2, RB>);
+  else go(k1_pair_kernel<MODE, ET, 1, RB>);
+}
+
+template <int MODE, int ET, int RB>
+void launch_single(const Contraction& c) {
+  constexpr int BKE = Elem<ET>::BKE * RB / 128;
+  const cuuint64_t dA[3] = {(cuuint64_t)c.Kin, (cuuint64_t)c.pn, (cuuint64_t)c.M};
+  const cuuint64_t sA[2] = {(cuuint64_t)c.ldk * c.es, (cuuint64_t)c.pn * c.ldk * c.es};
+  const cuuint32_t bA[3] = {(cuuint32_t)BKE, 1, BM};
+  const cuuint64_t dB[3] = {(cuuint64_t)c.Kin, (cuuint64_t)c.N, (cuuint64_t)c.pn};
+  const cuuint64_t sB[2] = {(cuuint64_t)c.ldk * c.es, (cuuint64_t)c.N * c.ldk * c.es};
+  const cuuint32_t bB[3] = {(cuuint32_t)BKE, BN, 1};
+  const CUtensorMap mAh = make_map(c.Ahi, dA, sA, bA, ET, RB), mBh = make_map(c.Bhi, dB, sB, bB, ET, RB);
+  const CUtensorMap mAl = c.Alo ? make_map(c.Alo, dA, sA, bA, ET, RB) : mAh;
+  const CUtensorMap mBl = c.Blo ? make_map(c.Blo, dB, sB, bB, ET, RB) : mBh;
+  const Params p{c.M, c.N, c.Kin, c.nab, c.total, c.per, c.part, c.err};
+  const dim3 grid((c.N + BN - 1) / BN, (c.M + BM - 1) / BM, c.splits);
+  constexpr int smem = Cfg<MODE, RB>::SMEM_BYTES;
+  ensure_smem((const void*)k1_tc_kernel<MODE, ET, RB>, smem);
+  if (c.prof) c.prof->begin(c.s);
+  k1_tc_kernel<MODE, ET, RB><<<grid, THREADS, smem, c.s>>>(mAh, mAl, mBh, mBl, p);
+  if (c.prof) c.prof->end(c.s, c.prof_flops, c.prof_bytes);
+}
+
+// Pairs of CTAs where there are two M tiles or more, one CTA per tile below;
+// both form the same sums, bit for bit (TDDFT_TC_CLUSTER=0 keeps single CTAs).
+template <int MODE, int ET, int RB>
+void launch_contraction(const Contraction& c) {
+  if (c.M > BM && cluster_pairs_enabled()) launch_pair<MODE, ET, RB>(c);
+  else launch_single<MODE, ET, RB>(c);
+  count_launch();
+  TD_LAUNCH_CHECK();
+}
+
+void sum_splits(const Contraction& c, float* out, bool accumulate, const float* scale) {
+  const long long MN = (long long)c.M * c.N;
+  long long g = (MN + 255) / 256;
+  if (g > 152 * 16) g = 152 * 16;
+  k_sum_splits<<<(unsigned)g, 256, 0, c.s>>>(c.part, c.splits, MN, out, accumulate ? 1 : 0, scale);
+  count_launch();
+  TD_LAUNCH_CHECK();
+}
 }  // namespace
 
 void tc_contract(const void* Ahi, const void* Alo, int M, int pn, int Kin, const void* Bhi, const void* Blo,
@@ -845,92 +1153,30 @@ void tc_contract(const void* Ahi, const void* Alo, int M, int pn, int Kin, const
                  KernelProfile* prof, double prof_flops, double prof_bytes, int max_kb) {
   if (M <= 0 || pn <= 0 || N <= 0) return;
   TD_REQUIRE(Alo != nullptr || Blo == nullptr, TDDFT_ERR_ARG, "tc_contract: B split without A split");
-  const int et = elem_of(elt);
   const int mode = Alo ? (Blo ? BOTH : ASPLIT) : SINGLE;
-  // the split-B products run on 64-byte K rows (a four-deep ring), the others on 128-byte rows
+  TD_REQUIRE(mode == (elt == TcElt::F16 ? BOTH : ASPLIT), TDDFT_ERR_ARG,
+             "tc_contract: FP16 operands come as hi + lo on both sides, BF16 ones with a plain B");
+  // the split-B products run on 64-byte K rows (a deeper ring), the others on 128-byte rows
   const int rb = mode == BOTH ? 64 : 128;
   const int bke = BK * rb / 128;
-  const int ldk = tc_pad(Kin);
   const int nab = (Kin + bke - 1) / bke;
   const int total = pn * nab;
   if (max_kb > 0) max_kb = max_kb * (BK / bke);   // max_kb counts 64-element k-blocks
-  const int mt0 = (M + BM - 1) / BM, nt0 = (N + BN - 1) / BN;
-  // split-B products in pairs of M tiles that share each B tile through a
-  // cluster multicast (TDDFT_TC_CLUSTER=0 turns this off; the results are the
-  // same bits either way: every CTA issues the same MMAs on the same data)
-  const bool pair = mode == BOTH && mt0 > 1 && cluster_pairs_enabled();
-  const int mt = pair ? (mt0 + 1) & ~1 : mt0;
-  // and, with two or more N tiles, in 2 x 2 clusters whose N pairs also share each A tile
-  const int cx = pair && nt0 > 1 && cluster_quads_enabled() ? 2 : 1;
-  const int nt = cx > 1 ? (nt0 + 1) & ~1 : nt0;
+  const int mt = (M + BM - 1) / BM, nt = (N + BN - 1) / BN;
   // a CTA's fixed cost (barriers, TMEM, pipeline fill, 128 KB epilogue) is about
   // four 64-element k-blocks of MMA work.  The split count depends on the
   // problem only (its own tiles, the pairs' residency), not on the cluster
   // shape of the launch: every shape then forms the same sums, bit for bit.
-  const bool pairable = mode == BOTH && mt0 > 1;
-  int splits = wave_splits(mt0 * nt0, total, 4 * (BK / bke), pairable ? pair_slots(et) : 0);
+  int splits = wave_splits(mt * nt, total, 4 * (BK / bke), mode == BOTH && mt > 1 ? pair_slots() : 0);
   if (max_kb > 0) splits = std::max(splits, (total + max_kb - 1) / max_kb);   // bounded accumulation runs
   const int per = (total + splits - 1) / splits;
   splits = (total + per - 1) / per;
-
-  const cuuint64_t dA[3] = {(cuuint64_t)Kin, (cuuint64_t)pn, (cuuint64_t)M};
-  const cuuint64_t sA[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)pn * ldk * 2};
-  const cuuint32_t bA[3] = {(cuuint32_t)bke, 1, (cuuint32_t)(BM / cx)};   // a quad's N pair loads half an A tile each
-  const cuuint64_t dB[3] = {(cuuint64_t)Kin, (cuuint64_t)N, (cuuint64_t)pn};
-  const cuuint64_t sB[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)N * ldk * 2};
-  const cuuint32_t bB[3] = {(cuuint32_t)bke, (cuuint32_t)(pair ? BN / 2 : BN), 1};   // a pair loads half a B tile each
-  CUtensorMap mAh = make_map(Ahi, dA, sA, bA, et, rb), mBh = make_map(Bhi, dB, sB, bB, et, rb);
-  CUtensorMap mAl = Alo ? make_map(Alo, dA, sA, bA, et, rb) : mAh;
-  CUtensorMap mBl = Blo ? make_map(Blo, dB, sB, bB, et, rb) : mBh;
-
   DevBuf part((size_t)splits * M * N * 4, s);
-  Params p{M, N, Kin, nab, total, per, part.as<float>(), err};
-  dim3 grid(nt, mt, splits);
-  auto launch = [&](auto kernel, int smem) {
-    ensure_smem((const void*)kernel, smem);
-    if (prof) prof->begin(s);
-    kernel<<<grid, THREADS, smem, s>>>(mAh, mAl, mBh, mBl, p);
-    if (prof) prof->end(s, prof_flops, prof_bytes);
-  };
-  auto launch_pair = [&](auto kernel, int smem) {
-    ensure_smem((const void*)kernel, smem);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cx;
-    at[0].val.clusterDim.y = 2;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (prof) prof->begin(s);
-    TD_CUDA(cudaLaunchKernelEx(&cfg, kernel, mAh, mAl, mBh, mBl, p));
-    if (prof) prof->end(s, prof_flops, prof_bytes);
-  };
-  if (et == ET_F16) {
-    if (pair && cx > 1) launch_pair(k1_tc_kernel<BOTH, ET_F16, 2, 64, 2>, Cfg<BOTH, 64>::SMEM_BYTES);
-    else if (pair) launch_pair(k1_tc_kernel<BOTH, ET_F16, 2, 64>, Cfg<BOTH, 64>::SMEM_BYTES);
-    else if (mode == BOTH) launch(k1_tc_kernel<BOTH, ET_F16, 1, 64>, Cfg<BOTH, 64>::SMEM_BYTES);
-    else if (mode == ASPLIT) launch(k1_tc_kernel<ASPLIT, ET_F16>, Cfg<ASPLIT>::SMEM_BYTES);
-    else launch(k1_tc_kernel<SINGLE, ET_F16>, Cfg<SINGLE>::SMEM_BYTES);
-  } else {
-    if (pair && cx > 1) launch_pair(k1_tc_kernel<BOTH, ET_BF16, 2, 64, 2>, Cfg<BOTH, 64>::SMEM_BYTES);
-    else if (pair) launch_pair(k1_tc_kernel<BOTH, ET_BF16, 2, 64>, Cfg<BOTH, 64>::SMEM_BYTES);
-    else if (mode == BOTH) launch(k1_tc_kernel<BOTH, ET_BF16, 1, 64>, Cfg<BOTH, 64>::SMEM_BYTES);
-    else if (mode == ASPLIT) launch(k1_tc_kernel<ASPLIT, ET_BF16>, Cfg<ASPLIT>::SMEM_BYTES);
-    else launch(k1_tc_kernel<SINGLE, ET_BF16>, Cfg<SINGLE>::SMEM_BYTES);
-  }
-  count_launch();
-  TD_LAUNCH_CHECK();
-  const long long MN = (long long)M * N;
-  long long g = (MN + 255) / 256;
-  if (g > 152 * 16) g = 152 * 16;
-  k_sum_splits<<<(unsigned)g, 256, 0, s>>>(part.as<float>(), splits, MN, out, accumulate ? 1 : 0, scale);
-  count_launch();
-  TD_LAUNCH_CHECK();
+  const Contraction c{Ahi, Alo, M, pn, Kin, Bhi, Blo, N, tc_pad(Kin), 2, total, per, splits, nab,
+                      part.as<float>(), err, s, prof, prof_flops, prof_bytes};
+  if (mode == BOTH) launch_contraction<BOTH, ET_F16, 64>(c);
+  else launch_contraction<ASPLIT, ET_BF16, 128>(c);
+  sum_splits(c, out, accumulate, scale);
 }
 
 void tc_contract8(const unsigned char* Ahi, const unsigned char* Alo, int M, int pn, int Kin,
@@ -939,34 +1185,17 @@ void tc_contract8(const unsigned char* Ahi, const unsigned char* Alo, int M, int
   if (M <= 0 || pn <= 0 || N <= 0) return;
   TD_REQUIRE(Ahi && Alo && B && scale, TDDFT_ERR_ARG, "tc_contract8: operands missing");
   constexpr int BKE = Elem<ET_E4M3>::BKE;
-  const int ldk = tc_pad16(Kin);
   const int nab = (Kin + BKE - 1) / BKE;
   const int total = pn * nab;
   const int mt = (M + BM - 1) / BM, nt = (N + BN - 1) / BN;
   int splits = wave_splits(mt * nt, total, 4);
   const int per = (total + splits - 1) / splits;
   splits = (total + per - 1) / per;
-  const cuuint64_t dA[3] = {(cuuint64_t)Kin, (cuuint64_t)pn, (cuuint64_t)M};
-  const cuuint64_t sA[2] = {(cuuint64_t)ldk, (cuuint64_t)pn * ldk};
-  const cuuint32_t bA[3] = {(cuuint32_t)BKE, 1, BM};
-  const cuuint64_t dB[3] = {(cuuint64_t)Kin, (cuuint64_t)N, (cuuint64_t)pn};
-  const cuuint64_t sB[2] = {(cuuint64_t)ldk, (cuuint64_t)N * ldk};
-  const cuuint32_t bB[3] = {(cuuint32_t)BKE, BN, 1};
-  CUtensorMap mAh = make_map(Ahi, dA, sA, bA, ET_E4M3), mAl = make_map(Alo, dA, sA, bA, ET_E4M3);
-  CUtensorMap mB = make_map(B, dB, sB, bB, ET_E4M3);
   DevBuf part((size_t)splits * M * N * 4, s);
-  Params p{M, N, Kin, nab, total, per, part.as<float>(), err};
-  dim3 grid(nt, mt, splits);
-  ensure_smem((const void*)k1_tc_kernel<ASPLIT, ET_E4M3>, Cfg<ASPLIT>::SMEM_BYTES);
-  k1_tc_kernel<ASPLIT, ET_E4M3><<<grid, THREADS, Cfg<ASPLIT>::SMEM_BYTES, s>>>(mAh, mAl, mB, mB, p);
-  count_launch();
-  TD_LAUNCH_CHECK();
-  const long long MN = (long long)M * N;
-  long long g = (MN + 255) / 256;
-  if (g > 152 * 16) g = 152 * 16;
-  k_sum_splits<<<(unsigned)g, 256, 0, s>>>(part.as<float>(), splits, MN, out, accumulate ? 1 : 0, scale);
-  count_launch();
-  TD_LAUNCH_CHECK();
+  const Contraction c{Ahi, Alo, M, pn, Kin, B, nullptr, N, tc_pad16(Kin), 1, total, per, splits, nab,
+                      part.as<float>(), err, s, nullptr, 0.0, 0.0};
+  launch_contraction<ASPLIT, ET_E4M3, 128>(c);
+  sum_splits(c, out, accumulate, scale);
 }
 
 namespace {
