@@ -271,7 +271,7 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       DevBuf th((size_t)m * nJp * 2, s), tl((size_t)m * nJp * 2, s);
       tc_transpose_split(t.p, DType::F32, 1, f.nJ, m, th.p, tl.p, TcElt::F16, sct.as<float>(), s);
       tc_inv_prod(sct.as<float>(), f.tc_scale + 4, fac.as<float>(), s);      // 1 / (s_t s_ov)
-      tc_contract(th.p, tl.p, m, 1, f.nJ, f.JovT_hi, f.JovT_lo, ov, Jb.as<float>(), false, TcElt::F16,
+      tc_contract(th.p, tl.p, nJp, m, 1, f.nJ, f.JovT_hi, f.JovT_lo, ov, Jb.as<float>(), false, TcElt::F16,
                   fac.as<float>(), d.tc_err, s, nullptr, 0.0, 0.0, kCoulombKb);
     } else {
       DevBuf t((size_t)f.nJ * m * ew, s);
@@ -302,7 +302,8 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
     if (need_k2) K2b = DevBuf(mov * ew, s);
     const bool use_tc = tensor_cores && !f64 && f.Kvv_hi && f.Kvo_hi && f.Koo_hi && f.Kovp_hi;
     TD_REQUIRE(!tensor_cores || f64 || use_tc, TDDFT_ERR_ARG, "tensor-core factor copies missing");
-    const int pc = chunk_rows(f.nK, (long long)m * ov * (long long)ew, m, use_tc ? kChunkBytesTC : kChunkBytes);
+    const int pc = use_tc ? chunk_rows(f.nK, (long long)m * no * tc_zpad(nv, 2) * 4, m, kChunkBytesTC)
+                          : chunk_rows(f.nK, (long long)m * ov * (long long)ew, m, kChunkBytes);
     const size_t es = dtype_size(f.dt);
     // 16-bit tensor-core operand pointer at element offset o
     auto at16 = [](const void* b, size_t o) { return static_cast<const void*>(static_cast<const uint16_t*>(b) + o); };
@@ -315,6 +316,7 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       // sums are multiplied back by 1/g (tc_fp8_scales).
       TD_REQUIRE(f.Kvv8 && f.Kvo8 && f.s_vv, TDDFT_ERR_ARG, "FP8 ris copies missing");
       const int nvp = tc_pad(nv), nop = tc_pad(no), nv16 = tc_pad16(nv), no16 = tc_pad16(no);
+      const int nvz = tc_zpad(nv, 1), noz = tc_zpad(no, 1);
       const DType xt = x32 ? DType::F32 : DType::F64;
       DevBuf sc((size_t)(2 + 2 * f.nK) * 4, s), kap(16, s);
       tc_fp8_scales(X, xt, m, no, nv, f.s_vv, f.rho_oo, f.s_vo, f.rho_ov, f.nK, sc.as<float>(), kap.as<unsigned>(), s);
@@ -329,25 +331,23 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
         Xs_lo = DevBuf((size_t)m * no * nvp * 2, s);
         tc_pad_split(X, xt, (long long)m * no, nv, Xs_hi.p, Xs_lo.p, TcElt::BF16, nullptr, s);
       }
-      DevBuf Zhi((size_t)m * no * pc * nv16, s), Zlo((size_t)m * no * pc * nv16, s), Qhi, Qlo;
+      DevBuf Zhi((size_t)m * no * pc * nvz, s), Zlo((size_t)m * no * pc * nvz, s), Qhi, Qlo;
       if (need_k2) {
-        Qhi = DevBuf((size_t)m * no * pc * no16, s);
-        Qlo = DevBuf((size_t)m * no * pc * no16, s);
+        Qhi = DevBuf((size_t)m * no * pc * noz, s);
+        Qlo = DevBuf((size_t)m * no * pc * noz, s);
       }
       const int Mz = m * no;
       for (int p0 = 0; p0 < f.nK; p0 += pc) {
         const int pn = (f.nK - p0 < pc) ? f.nK - p0 : pc;
-        tc_stage1_fp8(Xt_hi.as<__nv_bfloat16>(), Xt_lo.as<__nv_bfloat16>(), m * nv, no,
-                      static_cast<const __nv_bfloat16*>(f.Koo_hi) + (size_t)p0 * no * nop, no, pn, nv, mu1 + p0,
-                      Zhi.as<unsigned char>(),
-                      Zlo.as<unsigned char>(), d.tc_err, s);
+        tc_stage1_fp8(Xt_hi.as<__nv_bfloat16>(), Xt_lo.as<__nv_bfloat16>(), m, nv, no,
+                      static_cast<const __nv_bfloat16*>(f.Koo_hi) + (size_t)p0 * no * nop, no, pn, mu1 + p0,
+                      Zhi.as<unsigned char>(), Zlo.as<unsigned char>(), d.tc_err, s);
         tc_contract8(Zhi.as<unsigned char>(), Zlo.as<unsigned char>(), Mz, pn, nv,
                      f.Kvv8 + (size_t)p0 * nv * nv16, nv, K1b.as<float>(), p0 > 0, inv1, d.tc_err, s);
         if (need_k2) {
-          tc_stage1_fp8(Xs_hi.as<__nv_bfloat16>(), Xs_lo.as<__nv_bfloat16>(), m * no, nv,
-                        static_cast<const __nv_bfloat16*>(f.Kovp_hi) + (size_t)p0 * no * nvp, no, pn, no, mu2 + p0,
-                        Qhi.as<unsigned char>(),
-                        Qlo.as<unsigned char>(), d.tc_err, s);
+          tc_stage1_fp8(Xs_hi.as<__nv_bfloat16>(), Xs_lo.as<__nv_bfloat16>(), m, no, nv,
+                        static_cast<const __nv_bfloat16*>(f.Kovp_hi) + (size_t)p0 * no * nvp, no, pn, mu2 + p0,
+                        Qhi.as<unsigned char>(), Qlo.as<unsigned char>(), d.tc_err, s);
           tc_contract8(Qhi.as<unsigned char>(), Qlo.as<unsigned char>(), Mz, pn, no,
                        f.Kvo8 + (size_t)p0 * nv * no16, nv, K2b.as<float>(), p0 > 0, inv2, d.tc_err, s);
         }
@@ -383,19 +383,19 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
         Xs_lo = DevBuf((size_t)m * no * nvp * 2, s);
         tc_pad_split(X, xt, (long long)m * no, nv, Xs_hi.p, Xs_lo.p, et, sx, s);
       }
-      DevBuf Zhi((size_t)m * no * pc * nvp * 2, s), Zlo((size_t)m * no * pc * nvp * 2, s), Qhi, Qlo;
+      const int nvz = tc_zpad(nv, 2), noz = tc_zpad(no, 2);
+      DevBuf Zhi((size_t)m * no * pc * nvz * 2, s), Zlo((size_t)m * no * pc * nvz * 2, s), Qhi, Qlo;
       if (need_k2) {
-        Qhi = DevBuf((size_t)m * no * pc * nop * 2, s);
-        Qlo = DevBuf((size_t)m * no * pc * nop * 2, s);
+        Qhi = DevBuf((size_t)m * no * pc * noz * 2, s);
+        Qlo = DevBuf((size_t)m * no * pc * noz * 2, s);
       }
       const int Mz = m * no;
       for (int p0 = 0; p0 < f.nK; p0 += pc) {
         const int pn = (f.nK - p0 < pc) ? f.nK - p0 : pc;
-        tc_stage1(Xt_hi.p, Xt_lo.p, m * nv, no, at16(f.Koo_hi, (size_t)p0 * no * nop),
-                  f16 ? at16(f.Koo_lo, (size_t)p0 * no * nop) : nullptr, no, pn, nv, et, mz, Zhi.p, Zlo.p,
-                  d.tc_err, s);
+        tc_stage1(Xt_hi.p, Xt_lo.p, m, nv, no, at16(f.Koo_hi, (size_t)p0 * no * nop),
+                  f16 ? at16(f.Koo_lo, (size_t)p0 * no * nop) : nullptr, no, pn, et, mz, Zhi.p, Zlo.p, d.tc_err, s);
         const bool timed = d.prof && d.prof->on && f16;
-        tc_contract(Zhi.p, Zlo.p, Mz, pn, nv, at16(f.Kvv_hi, (size_t)p0 * nv * nvp),
+        tc_contract(Zhi.p, Zlo.p, nvz, Mz, pn, nv, at16(f.Kvv_hi, (size_t)p0 * nv * nvp),
                     f16 ? at16(f.Kvv_lo, (size_t)p0 * nv * nvp) : nullptr, nv, K1b.as<float>(), p0 > 0, et, f1,
                     d.tc_err, s, timed ? d.prof : nullptr, 2.0 * Mz * (double)nv * (double)pn * nv,
                     // Z hi+lo [Mz][pn*nv], L_vv chunk [pn*nv][nv] (hi+lo for FP16), K1 FP32
@@ -404,10 +404,9 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
                         4.0 * Mz * (double)nv * (p0 > 0 ? 2.0 : 1.0),
                     f16 ? kExchangeKb : 0);
         if (need_k2) {
-          tc_stage1(Xs_hi.p, Xs_lo.p, m * no, nv, at16(f.Kovp_hi, (size_t)p0 * no * nvp),
-                    f16 ? at16(f.Kovp_lo, (size_t)p0 * no * nvp) : nullptr, no, pn, no, et, mq, Qhi.p, Qlo.p,
-                    d.tc_err, s);
-          tc_contract(Qhi.p, Qlo.p, Mz, pn, no, at16(f.Kvo_hi, (size_t)p0 * nv * nop),
+          tc_stage1(Xs_hi.p, Xs_lo.p, m, no, nv, at16(f.Kovp_hi, (size_t)p0 * no * nvp),
+                    f16 ? at16(f.Kovp_lo, (size_t)p0 * no * nvp) : nullptr, no, pn, et, mq, Qhi.p, Qlo.p, d.tc_err, s);
+          tc_contract(Qhi.p, Qlo.p, noz, Mz, pn, no, at16(f.Kvo_hi, (size_t)p0 * nv * nop),
                       f16 ? at16(f.Kvo_lo, (size_t)p0 * nv * nop) : nullptr, nv, K2b.as<float>(), p0 > 0, et, f2,
                       d.tc_err, s, nullptr, 0.0, 0.0, f16 ? kExchangeKb : 0);
         }

@@ -1,8 +1,8 @@
 // tcgen05 tensor-core contraction over the auxiliary index,
-//   C[m][n] (+)= sum_P sum_k A[m][P][k] B[P][n][k],
+//   C[m][n] (+)= sum_P sum_k A[P][m][k] B[P][n][k],
 // used for the exchange terms of the response products (Eq. hessian):
-//   K1[(n,i)][b] = sum_P sum_a Z[(n,i)][P][a] L^P_ab      ((ij|ab) term, k = a)
-//   K2[(n,i)][a] = sum_P sum_j Q[(n,i)][P][j] L^P_ja      ((ib|ja) term, k = j)
+//   K1[(n,i)][b] = sum_P sum_a Z[P][(n,i)][a] L^P_ab      ((ij|ab) term, k = a)
+//   K2[(n,i)][a] = sum_P sum_j Q[P][(n,i)][j] L^P_ja      ((ib|ja) term, k = j)
 // K1's contraction is the dominant cost of every product (about 70-90% of flops).
 //
 // Exact operator: every operand is scaled by a power of two s (so that
@@ -16,7 +16,7 @@
 // vectors as BF16 hi + lo.
 //
 // Layout / mapping (all K-major, so both operands stream along k):
-//   A viewed as a 3-D tensor (k: Kin, P: pn, row: M), row pitch pn*ldk
+//   A viewed as a 3-D tensor (k: Kin, P: pn, row: M), rows of ldk, M rows per P
 //   B viewed as a 3-D tensor (k: Kin, n: N, P: pn), rows of ldk; for K1 the
 //          rows of the symmetric L^P are its columns, for K2 B is L^P_ov
 //          stored transposed ([P][a][j])
@@ -63,13 +63,12 @@ template <int ET> struct Elem {
   static constexpr uint32_t TYPE_BITS = ET == ET_BF16 ? ((1u << 7) | (1u << 10)) : 0u;
 };
 constexpr int elem_of(TcElt e) { return e == TcElt::F16 ? ET_F16 : ET_BF16; }
-// Operand split modes: SINGLE = one product; BOTH = A and B as hi + lo
-// (hi*hi + hi*lo + lo*hi); ASPLIT = A as hi + lo, B a plain operand
-// (hi*B + lo*B: exact with respect to B, e.g. FP32 vectors against BF16 ris factors).
-enum SplitMode : int { SINGLE = 0, BOTH = 1, ASPLIT = 2 };
-__host__ __device__ constexpr bool a_split(int m) { return m != SINGLE; }
+// Operand split modes: BOTH = A and B as hi + lo (hi*hi + hi*lo + lo*hi); ASPLIT =
+// A as hi + lo, B a plain operand (hi*B + lo*B: exact with respect to B, e.g.
+// FP32 vectors against BF16 ris factors).
+enum SplitMode : int { BOTH = 1, ASPLIT = 2 };
 __host__ __device__ constexpr bool b_split(int m) { return m == BOTH; }
-__host__ __device__ constexpr int n_parts_a(int m) { return a_split(m) ? 2 : 1; }
+__host__ __device__ constexpr int n_parts_a(int) { return 2; }
 __host__ __device__ constexpr int n_parts_b(int m) { return b_split(m) ? 2 : 1; }
 
 // Ring of the contraction kernel for rows of RB bytes along K (128: one
@@ -78,12 +77,10 @@ __host__ __device__ constexpr int n_parts_b(int m) { return b_split(m) ? 2 : 1; 
 // tiles fill 96 KB per 128-byte stage, use it for a four-deep ring).
 template <int MODE, int RB = 128> struct Cfg {
   static constexpr int STAGE_BYTES = (n_parts_a(MODE) * A_BYTES + n_parts_b(MODE) * B_BYTES) * RB / 128;
-  static constexpr int STAGES = (MODE == SINGLE ? 4 : (MODE == ASPLIT ? 3 : 2)) * 128 / RB;   // ~192 KB ring
+  static constexpr int STAGES = (MODE == ASPLIT ? 3 : 2) * 128 / RB;   // ~192 KB ring
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
 };
 constexpr int THREADS = 192;
-constexpr int S1_EPI_WARPS = 16;                   // stage-1 epilogue warps (4 per TMEM lane quadrant)
-constexpr int S1_THREADS = 64 + 32 * S1_EPI_WARPS;   // producer, MMA and the epilogue warps
 
 struct Params {
   int M, N;          // output rows / columns
@@ -139,27 +136,6 @@ __device__ __forceinline__ uint64_t sdesc_rb(const void* p) {
          (4ull << 61);
 }
 
-// TMA load into the same shared-memory offset of every CTA in `mask` of the
-// cluster, signalling each one's mbarrier at the same offset.
-__device__ __forceinline__ void tma_load_3d_mc(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1,
-                                               int c2, uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster"
-      " [%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "h"(mask)
-      : "memory");
-}
-
-// Arrive on the mbarrier at this offset in every CTA of `mask` when the MMAs
-// issued so far have completed.
-__device__ __forceinline__ void mma_commit_mc(uint64_t* bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "h"(mask)
-      : "memory");
-}
-
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -181,7 +157,7 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
   constexpr int STAGES = Cfg<MODE, RB>::STAGES;
   constexpr int STAGE_BYTES = Cfg<MODE, RB>::STAGE_BYTES;
   constexpr int AB = A_BYTES * RB / 128, BB = B_BYTES * RB / 128;   // one part tile
-  constexpr int B_OFF = a_split(MODE) ? 2 * AB : AB;                // first B tile in a stage
+  constexpr int B_OFF = 2 * AB;                                     // first B tile in a stage
   constexpr int BKE = Elem<ET>::BKE * RB / 128;                     // K elements per k-block
   constexpr int KSTEPS = RB / 32;                                   // 32-byte K steps per k-block
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -224,7 +200,7 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
       unsigned char* st = smem + s * STAGE_BYTES;
       mbar_expect_tx(&full[s], STAGE_BYTES);
       tma_load_3d(st, &mA_hi, &full[s], a0, P, m0);
-      if (a_split(MODE)) tma_load_3d(st + AB, &mA_lo, &full[s], a0, P, m0);
+      tma_load_3d(st + AB, &mA_lo, &full[s], a0, P, m0);
       tma_load_3d(st + B_OFF, &mB_hi, &full[s], a0, n0, P);
       if (b_split(MODE)) tma_load_3d(st + B_OFF + BB, &mB_lo, &full[s], a0, n0, P);
     }
@@ -254,7 +230,7 @@ k1_tc_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ 
           const uint64_t off = (uint64_t)(kk * 32) >> 4;   // 32 bytes along K per MMA
           mma_op<ET>(tmem, ah + off, bh + off, (i > 0 || kk > 0) ? 1u : 0u, idesc);
           if (b_split(MODE)) mma_op<ET>(tmem, ah + off, sdesc_rb<RB>(st + B_OFF + BB) + off, 1u, idesc);
-          if (a_split(MODE)) mma_op<ET>(tmem, sdesc_rb<RB>(st + AB) + off, bh + off, 1u, idesc);
+          mma_op<ET>(tmem, sdesc_rb<RB>(st + AB) + off, bh + off, 1u, idesc);
         }
       }
       mma_commit(&empty[s]);
@@ -459,10 +435,10 @@ k1_pair_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant_
         constexpr int HA = C::AB / 2;
         const int mh = m0 + y * (BM / 2);
         tma_load_3d_pair_mc(st + y * HA, &mA_hi, bar, a0, P, mh, mask_a);
-        if (a_split(MODE)) tma_load_3d_pair_mc(st + C::AB + y * HA, &mA_lo, bar, a0, P, mh, mask_a);
+        tma_load_3d_pair_mc(st + C::AB + y * HA, &mA_lo, bar, a0, P, mh, mask_a);
       } else {
         tma_load_3d_pair(st, &mA_hi, bar, a0, P, m0);
-        if (a_split(MODE)) tma_load_3d_pair(st + C::AB, &mA_lo, bar, a0, P, m0);
+        tma_load_3d_pair(st + C::AB, &mA_lo, bar, a0, P, m0);
       }
       tma_load_3d_pair(st + B_OFF, &mB_hi, bar, a0, nh, P);
       if (b_split(MODE)) tma_load_3d_pair(st + B_OFF + C::HB, &mB_lo, bar, a0, nh, P);
@@ -499,7 +475,7 @@ k1_pair_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant_
           } else {
             mma_pair<ET, 0>(tmem, ah + off, bh + off, acc, idesc);
           }
-          if (a_split(MODE)) mma_pair<ET, 0>(tmem, sdesc_rb<RB>(st + C::AB) + off, bh + off, 1u, idesc);
+          mma_pair<ET, 0>(tmem, sdesc_rb<RB>(st + C::AB) + off, bh + off, 1u, idesc);
         }
       }
       commit_pair(&empty[s], mask_all);
@@ -557,23 +533,49 @@ k1_pair_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------
-// Stage-1 contractions of the exchange terms, batched over P:
-//   C_P[r][c] = sum_(k<K) A[r][k] B_P[c][k]   (r < M, c < N <= 256)
-// written as BF16 hi (+ lo) into the stage-2 operand layout
-//   out[(g*N + c)][P][ri] with r = g*R + ri, row pitch pn*ldo (ldo = pad8(R)):
-//   K1: A = X^T per trial vector ([(n,a)][j]), B_P = L^P_oo ([i][j]) -> Z[(n,i)][P][a]
-//   K2: A = X ([(n,j)][b]),            B_P = L^P_ov ([i][b]) -> Q[(n,i)][P][j]
-// Persistent over P: the CTA owns one M-tile and the P range blockIdx.y*ppc ...;
-// k-blocks of A and B_P stream through a TMA/mbarrier ring; the TMEM
-// accumulator is double-buffered so the epilogue of one P overlaps the MMAs of
-// the next (tmem_full / tmem_empty barriers).
+// Stage-1 contractions of the exchange terms, for every P and trial vector n:
+//   C_P[n][i][r] = sum_(k<K) L_P[i][k] X[n][r][k]
+// written as hi + lo parts into the stage-2 operand layout
+//   out[P][(n, i)][r], row pitch ldo (128-byte rows, tc_zpad):
+//   K1: L = L_oo ([i][j]), X = X^T per trial vector ([a][j])  -> Z[P][(n,i)][a]
+//   K2: L = L_ov ([i][b]), X = X ([j][b])                     -> Q[P][(n,i)][j]
+// One product over all rows (P, i) and columns (n, r): the columns run along the
+// contiguous index of the output, so a thread (one TMEM lane = one row) converts
+// 16 consecutive results at once, and each warp passes its piece through shared
+// memory and writes 64-byte runs, the two halves of a line right after one
+// another.  (With the roles swapped and rows of [(n,i)][P][r] it stored single
+// 2-byte elements, 27 instructions per result.)  What bounds it: the stores of Z
+// and the conversions share the load/store unit (n_vir 400: 0.45 ms without the
+// stores, 0.93 with them); n_vir 1350: the MMAs' share of that, 0.68 of 1.05 ms.
+// Straight 32-byte stores per row (46 L1 cycles an instruction) and bulk copies of
+// 128 bytes (12 cycles each) were slower.
+// Measured, 20 vectors of 60 x 400, 2000 rows: Z 1002 -> 931 us, Q 627 -> 278;
+// 13 vectors of 24 x 144, 840 rows: Z 84 -> 43; 40 vectors of 150 x 1350, 127
+// rows: Z 1340 -> 1050; FP8 ris, 20 vectors of 150 x 1350, 150 rows: 865 -> 472.
+// Tiles of 256 rows x up to 256 columns by CTA pairs (cta_group::2, as in
+// k1_pair_kernel), clusters of two persistent over the tiles; the TMEM
+// accumulator is double-buffered so the stores of one tile overlap the MMAs of
+// the next.  A tile's columns are gn whole trial vectors of wr columns each
+// (R <= 128) or a part of one in whole 64-column units, so that 16-byte stores
+// never cross vectors and a part begins on a 128-byte line.
+// Rows of the output are padded to 128 bytes: with rows of pad8(R) elements the
+// 64- to 512-byte runs of the stores straddled lines and sectors, which the L2
+// completes from DRAM (1.5 to 3.5 TB/s written in a pattern of 2704-byte rows
+// against 6.2 TB/s with 2816-byte ones, 7.1 TB/s for one long run).
+constexpr int S1_EPI_WARPS = 16;                     // four per TMEM lane quadrant
+constexpr int S1_THREADS = 64 + 32 * S1_EPI_WARPS;   // producer, MMA and the epilogue warps
+constexpr int S1_RB = 64;                            // bytes of K per shared-memory row
+
 struct S1Params {
-  int M, N, R, ldo, pn, ppc, nkb;
-  int K;               // k extent (the last k-block issues only the MMAs it needs)
-  int nb;              // MMA N (multiple of 16, >= N)
-  int acc_cols;        // TMEM columns per accumulator buffer
-  int stages, stage_bytes, a_bytes, b_bytes;
-  int a_res_bytes;     // RES: the resident A tile (every k-block, every part)
+  int rows, no, pn;    // pn * no rows (P, i)
+  int R, m, ldo;       // columns (n, r): r < R, n < m
+  int K, nkb;
+  int gn, wr;          // gn > 1: trial vectors per tile and their column pitch
+  int nt0, nq, nr;     // gn == 1: tiles per trial vector, col_unit-column units per tile (+1 for the first nr)
+  int mt, ntile;       // row tiles, column tiles
+  int mseg, units;     // row tiles of one unit of work, units (column tile fastest)
+  int col_unit;        // columns of a unit (64, or 32 where one tile holds the vector)
+  int b_rows;          // rows of half of the widest B tile
   void* out_hi;        // BF16 / FP16 parts (2-byte elements) or e4m3 bytes
   void* out_lo;
   // FP16 output: the accumulator times *mul before its split; FP8 output:
@@ -583,235 +585,367 @@ struct S1Params {
   int* err;
 };
 
-__device__ __forceinline__ unsigned char to_e4m3(float x) {
-  return (unsigned char)__nv_cvt_float_to_fp8(x, __NV_SATFINITE, __NV_E4M3);
+__device__ __forceinline__ uint32_t pack_e4m3x4(const float* x) {
+  const uint32_t a = __nv_cvt_float2_to_fp8x2(make_float2(x[0], x[1]), __NV_SATFINITE, __NV_E4M3);
+  const uint32_t b = __nv_cvt_float2_to_fp8x2(make_float2(x[2], x[3]), __NV_SATFINITE, __NV_E4M3);
+  return a | (b << 16);
 }
 __device__ __forceinline__ float from_e4m3(unsigned char q) {
   return __half2float(__half(__nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)q, __NV_E4M3)));
 }
 
-// RES: the CTA's A tile (all k-blocks) is loaded once and stays in shared
-// memory while the CTA walks its P range; the ring streams B_P only.
-// CL = 2: the CTAs run in clusters of two along the M tiles; both need the same
-// B_P tiles, so each loads half of the rows and multicasts them to both, and
-// a stage is refilled only when both CTAs' MMAs have read it.
-template <int MODE, int IN, int OUT, bool RES = false, int CL = 1>
+// Two FP32 operations at once.
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mul.rn.f32x2 z, x, y;\n"
+      " mov.b64 {%0, %1}, z;\n}\n" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n sub.rn.f32x2 z, x, y;\n"
+      " mov.b64 {%0, %1}, z;\n}\n" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+
+// hi and lo parts of the 16 accumulator values v times f (BF16: no factor), packed
+// in 32-bit words
+template <int OUT>
+__device__ __forceinline__ void split16(const uint32_t (&v)[16], float f, uint32_t* hi, uint32_t* lo) {
+  if constexpr (OUT == ET_E4M3) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float x[4], r[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) x[t] = __uint_as_float(v[4 * j + t]) * f;
+      hi[j] = pack_e4m3x4(x);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) r[t] = x[t] - from_e4m3((unsigned char)(hi[j] >> (8 * t)));
+      lo[j] = pack_e4m3x4(r);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float2 x = make_float2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+      if constexpr (OUT == ET_F16) {
+        x = mul2(x, make_float2(f, f));
+        const __half2 h = __float22half2_rn(x);
+        const __half2 l = __float22half2_rn(sub2(x, __half22float2(h)));
+        hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+        lo[j] = *reinterpret_cast<const uint32_t*>(&l);
+      } else {
+        const __nv_bfloat162 h = __float22bfloat162_rn(x);
+        const __nv_bfloat162 l = __float22bfloat162_rn(sub2(x, __bfloat1622float2(h)));
+        hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+        lo[j] = *reinterpret_cast<const uint32_t*>(&l);
+      }
+    }
+  }
+}
+
+// LSPLIT: the L operand (A) comes as hi + lo too (three products), else plain
+// (two); X (B) is always hi + lo.  RES (K <= 160): the column tile's X rows stay
+// in shared memory for the row tiles of a unit and the ring streams L only, half
+// the bytes per MMA.
+constexpr int S1_RES_KB = 5;
+template <bool LSPLIT, bool RES> struct S1Cfg {
+  static constexpr int AB = BM * S1_RB, HB = (BN / 2) * S1_RB;
+  static constexpr int STAGE_BYTES = (LSPLIT ? 2 : 1) * AB + (RES ? 0 : 2 * HB);
+  static constexpr int RES_BYTES = RES ? S1_RES_KB * 2 * HB : 0;
+  static constexpr int STAGES = (RES ? 98304 : 163840) / STAGE_BYTES;
+  // epilogue staging per warp: 32 rows of 64 bytes, 16-byte segments XORed with
+  // bits 1-2 of the row (no bank conflicts by rows or by segments)
+  static constexpr int EPI_BYTES = 32 * 64;
+  static constexpr int EPI_OFF = RES_BYTES + STAGES * STAGE_BYTES;
+  static constexpr int SMEM_BYTES = EPI_OFF + S1_EPI_WARPS * EPI_BYTES + 1024 + 512;
+};
+
+template <bool LSPLIT, bool RES, int IN, int OUT>
 __global__ void __launch_bounds__(S1_THREADS, 1)
-k_stage1_tc(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ CUtensorMap mA_lo,
-            const __grid_constant__ CUtensorMap mB_hi, const __grid_constant__ CUtensorMap mB_lo,
-            S1Params p) {
+k_stage1_pair(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ CUtensorMap mA_lo,
+              const __grid_constant__ CUtensorMap mB_hi, const __grid_constant__ CUtensorMap mB_lo,
+              const S1Params p) {
+  using C = S1Cfg<LSPLIT, RES>;
+  constexpr int STAGES = C::STAGES;
+  constexpr int B_OFF = (LSPLIT ? 2 : 1) * C::AB;   // !RES: first B tile in a stage
+  constexpr int BKE = S1_RB / 2;                  // K elements per k-block
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned char* ares = smem;                                   // RES: resident A
-  unsigned char* ring = smem + (RES ? p.a_res_bytes : 0);
-  uint64_t* full = reinterpret_cast<uint64_t*>(ring + p.stages * p.stage_bytes);
-  uint64_t* empty = full + p.stages;
-  uint64_t* tfull = empty + p.stages;      // [2]
-  uint64_t* tempty = tfull + 2;            // [2]
-  uint64_t* afull = tempty + 2;            // RES: the resident A tile has landed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(afull + 1);
+  unsigned char* bres = smem;                       // RES: the X rows, hi and lo per k-block
+  unsigned char* ring = smem + C::RES_BYTES;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::EPI_OFF + S1_EPI_WARPS * C::EPI_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* tfull = empty + STAGES;      // [2] accumulator complete (both CTAs)
+  uint64_t* tempty = tfull + 2;          // [2] accumulator read by this CTA's warps (the leader's: and the other's)
+  uint64_t* bfull = tempty + 2;          // RES: the unit's X rows have landed (leader) ...
+  uint64_t* bempty = bfull + 1;          // ... and its MMAs have read them
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bempty + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.x * BM;
-  const int P0 = blockIdx.y * p.ppc;
-  const int nP = max(0, min(p.pn, P0 + p.ppc) - P0);
-  const uint32_t idesc = idesc_of<IN>(p.nb);
-  const int a_part = RES ? n_parts_a(MODE) * p.a_bytes : 0;   // resident bytes per k-block
-  const int b_off = RES ? 0 : n_parts_a(MODE) * p.a_bytes;     // first B tile in a stage
-  const uint32_t crank = CL > 1 ? cluster_rank() : 0u;
+  const uint32_t rank = cluster_rank();
+  const int h = (int)(rank & 1u);
+  const int ncl = gridDim.x >> 1, cl = blockIdx.x >> 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < p.stages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], CL); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], S1_EPI_WARPS); }
-    mbar_init(afull, 1);
+    for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], S1_EPI_WARPS / 2 + (h == 0 ? 1 : 0)); }
+    mbar_init(bfull, 1);
+    mbar_init(bempty, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(tmem_slot)), "r"(2 * p.acc_cols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)), "r"(2 * BN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   __syncthreads();
-  if constexpr (CL > 1) cluster_sync_all();   // every barrier of the cluster initialised
+  cluster_sync_all();   // every barrier of the cluster initialised
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-  const int nsteps = nP * p.nkb;
+
+  // column tile ct: first trial vector, first r, columns
+  auto columns = [&](int ct, int& n0, int& r0, int& width) {
+    if (p.gn > 1) {
+      n0 = ct * p.gn;
+      r0 = 0;
+      width = p.gn * p.wr;
+    } else {
+      n0 = ct / p.nt0;
+      const int t = ct - n0 * p.nt0;
+      r0 = p.col_unit * (t * p.nq + min(t, p.nr));
+      width = p.col_unit * (p.nq + (t < p.nr ? 1 : 0));
+    }
+  };
 
   if (warp == 0 && lane == 0) {
-    if constexpr (RES) {
-      if (nsteps > 0) {
-        mbar_expect_tx(afull, p.a_res_bytes);
+    // ---- TMA producer (both CTAs)
+    const uint32_t lead_full = mapa(smem_u32(full), 0u), lead_bfull = mapa(smem_u32(bfull), 0u);
+    const uint32_t bytes_a = 2u * (LSPLIT ? 2u : 1u) * C::AB, bytes_b = 4u * (uint32_t)p.b_rows * S1_RB;
+    int i = 0, w = 0;
+    bool ok = true;
+    for (int u = cl; u < p.units && ok; u += ncl, ++w) {
+      int n0, r0, width;
+      columns(u % p.ntile, n0, r0, width);
+      const int nb = p.gn > 1 ? n0 + h * (p.gn / 2) : n0, rb = p.gn > 1 ? 0 : r0 + h * (width / 2);
+      const int mt0 = (u / p.ntile) * p.mseg, mt1 = min(p.mt, mt0 + p.mseg);
+      if constexpr (RES) {
+        if (!mbar_wait(bempty, ((uint32_t)w & 1u) ^ 1u)) { atomicOr(p.err, 16); ok = false; break; }
+        if (h == 0) mbar_expect_tx(bfull, bytes_b * (uint32_t)p.nkb);
         for (int kb = 0; kb < p.nkb; ++kb) {
-          tma_load_3d(ares + kb * a_part, &mA_hi, afull, kb * BK, m0, 0);
-          if (a_split(MODE)) tma_load_3d(ares + kb * a_part + p.a_bytes, &mA_lo, afull, kb * BK, m0, 0);
+          tma_load_3d_pair(bres + kb * 2 * C::HB, &mB_hi, lead_bfull, kb * BKE, rb, nb);
+          tma_load_3d_pair(bres + kb * 2 * C::HB + C::HB, &mB_lo, lead_bfull, kb * BKE, rb, nb);
+        }
+      }
+      for (int mt = mt0; mt < mt1 && ok; ++mt) {
+        const int m0 = mt * 2 * BM + h * BM;
+        for (int kb = 0; kb < p.nkb; ++kb, ++i) {
+          const int s = i % STAGES;
+          if (!mbar_wait(&empty[s], ((uint32_t)(i / STAGES) & 1u) ^ 1u)) { atomicOr(p.err, 16); ok = false; break; }
+          unsigned char* st = ring + s * C::STAGE_BYTES;
+          const uint32_t bar = lead_full + (uint32_t)(s * 8);
+          if (h == 0) mbar_expect_tx(&full[s], bytes_a + (RES ? 0u : bytes_b));
+          tma_load_3d_pair(st, &mA_hi, bar, kb * BKE, m0, 0);
+          if (LSPLIT) tma_load_3d_pair(st + C::AB, &mA_lo, bar, kb * BKE, m0, 0);
+          if constexpr (!RES) {
+            tma_load_3d_pair(st + B_OFF, &mB_hi, bar, kb * BKE, rb, nb);
+            tma_load_3d_pair(st + B_OFF + C::HB, &mB_lo, bar, kb * BKE, rb, nb);
+          }
         }
       }
     }
-    for (int i = 0; i < nsteps; ++i) {
-      const int s = i % p.stages;
-      if (!mbar_wait(&empty[s], ((uint32_t)(i / p.stages) & 1u) ^ 1u)) { atomicOr(p.err, 16); break; }
-      const int P = P0 + i / p.nkb, k0 = (i % p.nkb) * BK;
-      unsigned char* st = ring + s * p.stage_bytes;
-      mbar_expect_tx(&full[s], p.stage_bytes);
-      if constexpr (!RES) {
-        tma_load_3d(st, &mA_hi, &full[s], k0, m0, 0);
-        if (a_split(MODE)) tma_load_3d(st + p.a_bytes, &mA_lo, &full[s], k0, m0, 0);
-      }
-      if constexpr (CL > 1) {
-        // this CTA's half of the B_P rows, to both CTAs of the pair
-        const int hb = p.b_bytes / 2;
-        const int r0 = (int)crank * (p.nb / 2);
-        tma_load_3d_mc(st + b_off + crank * hb, &mB_hi, &full[s], k0, r0, P, (uint16_t)0x3);
-        if (b_split(MODE))
-          tma_load_3d_mc(st + b_off + p.b_bytes + crank * hb, &mB_lo, &full[s], k0, r0, P, (uint16_t)0x3);
-      } else {
-        tma_load_3d(st + b_off, &mB_hi, &full[s], k0, 0, P);
-        if (b_split(MODE)) tma_load_3d(st + b_off + p.b_bytes, &mB_lo, &full[s], k0, 0, P);
-      }
+    // the copies already issued (they signal the leader) land, and the last commits
+    // arrive on this CTA's `empty` barriers, before a CTA can exit
+    if (h == 0)
+      for (int j = max(0, i - STAGES); j < i; ++j)
+        if (!mbar_wait(&full[j % STAGES], (uint32_t)(j / STAGES) & 1u)) { atomicOr(p.err, 32); break; }
+    for (int j = i; j < i + STAGES; ++j)
+      if (!mbar_wait(&empty[j % STAGES], ((uint32_t)(j / STAGES) & 1u) ^ 1u)) { atomicOr(p.err, 32); break; }
+    if (RES && ok) {
+      if (h == 0 && w > 0 && !mbar_wait(bfull, (uint32_t)(w - 1) & 1u)) atomicOr(p.err, 32);
+      if (!mbar_wait(bempty, ((uint32_t)w & 1u) ^ 1u)) atomicOr(p.err, 32);
     }
-    // let the copies already issued land before the CTA can exit
-    for (int i = max(0, nsteps - p.stages); i < nsteps; ++i)
-      if (!mbar_wait(&full[i % p.stages], (uint32_t)(i / p.stages) & 1u)) { atomicOr(p.err, 32); break; }
-    if constexpr (CL > 1) {
-      // and the peer's last commits arrive on this CTA's `empty` barriers
-      for (int i = nsteps; i < nsteps + p.stages; ++i)
-        if (!mbar_wait(&empty[i % p.stages], ((uint32_t)(i / p.stages) & 1u) ^ 1u)) { atomicOr(p.err, 32); break; }
+  } else if (warp == 1 && lane == 0 && h == 0) {
+    // ---- MMA issuer (the leader)
+    int i = 0, j = 0, w = 0;
+    bool ok = true;
+    for (int u = cl; u < p.units && ok; u += ncl, ++w) {
+      int n0, r0, width;
+      columns(u % p.ntile, n0, r0, width);
+      const int mt0 = (u / p.ntile) * p.mseg, mt1 = min(p.mt, mt0 + p.mseg);
+      const uint32_t idesc =
+          (1u << 4) | Elem<IN>::TYPE_BITS | ((uint32_t)(width >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
+      if (RES && !mbar_wait(bfull, (uint32_t)w & 1u)) { atomicOr(p.err, 128); break; }
+      for (int mt = mt0; mt < mt1 && ok; ++mt, ++j) {
+        const int buf = j & 1;
+        if (!mbar_wait(&tempty[buf], ((uint32_t)(j >> 1) & 1u) ^ 1u)) { atomicOr(p.err, 64); ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t acc = tmem + (uint32_t)(buf * BN);
+        for (int kb = 0; kb < p.nkb; ++kb, ++i) {
+          const int s = i % STAGES;
+          if (!mbar_wait(&full[s], (uint32_t)(i / STAGES) & 1u)) { atomicOr(p.err, 128); ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          unsigned char* st = ring + s * C::STAGE_BYTES;
+          unsigned char* bt = RES ? bres + kb * 2 * C::HB : st + B_OFF;
+          const uint64_t ah = sdesc_rb<S1_RB>(st), bh = sdesc_rb<S1_RB>(bt), bl = sdesc_rb<S1_RB>(bt + C::HB);
+          const int rem = p.K - kb * BKE;   // the zero-filled tail issues no MMA
+#pragma unroll
+          for (int kk = 0; kk < S1_RB / 32; ++kk) {
+            if (kk * 16 < rem) {
+              const uint64_t off = (uint64_t)(kk * 32) >> 4;
+              mma_pair<IN, 1>(acc, ah + off, bh + off, (kb > 0 || kk > 0) ? 1u : 0u, idesc);
+              mma_pair<IN, 2>(acc, ah + off, bl + off, 1u, idesc);
+              if (LSPLIT) mma_pair<IN, 0>(acc, sdesc_rb<S1_RB>(st + C::AB) + off, bh + off, 1u, idesc);
+            }
+          }
+          commit_pair(&empty[s], (uint16_t)3);
+        }
+        commit_pair(&tfull[buf], (uint16_t)3);
+      }
+      if (RES) commit_pair(bempty, (uint16_t)3);
     }
   } else if (warp == 1 && lane == 0) {
+    // ---- the other CTA passes its "accumulator read" on to the leader: a remote
+    // arrival releases at cluster scope, which in an epilogue warp would wait for
+    // all of its global stores
+    const uint32_t lead_tempty = mapa(smem_u32(tempty), 0u);
+    int j = 0;
     bool ok = true;
-    if constexpr (RES) {
-      if (nsteps > 0 && !mbar_wait(afull, 0)) { atomicOr(p.err, 128); ok = false; }
-    }
-    for (int j = 0; j < nP && ok; ++j) {
-      const int buf = j & 1;
-      // wait until the epilogue has drained this accumulator buffer (use j/2 - 1)
-      if (!mbar_wait(&tempty[buf], ((uint32_t)(j >> 1) & 1u) ^ 1u)) { atomicOr(p.err, 64); break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t acc = tmem + (uint32_t)(buf * p.acc_cols);
-      for (int kb = 0; kb < p.nkb; ++kb) {
-        const int i = j * p.nkb + kb;
-        const int s = i % p.stages;
-        if (!mbar_wait(&full[s], (uint32_t)(i / p.stages) & 1u)) { atomicOr(p.err, 128); ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        unsigned char* st = ring + s * p.stage_bytes;
-        unsigned char* at = RES ? ares + kb * a_part : st;
-        const uint64_t ah = sdesc(at), bh = sdesc(st + b_off);
-        const int rem = p.K - kb * BK;
-        const int nks = rem >= BK ? BK / 16 : (rem + 15) / 16;   // the zero-filled tail issues no MMA
-#pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-          if (kk < nks) {
-            const uint64_t off = (uint64_t)(kk * 32) >> 4;
-            mma_op<IN>(acc, ah + off, bh + off, (kb > 0 || kk > 0) ? 1u : 0u, idesc);
-            if (b_split(MODE)) mma_op<IN>(acc, ah + off, sdesc(st + b_off + p.b_bytes) + off, 1u, idesc);
-            if (a_split(MODE)) mma_op<IN>(acc, sdesc(at + p.a_bytes) + off, bh + off, 1u, idesc);
-          }
-        }
-        if constexpr (CL > 1) mma_commit_mc(&empty[s], (uint16_t)0x3);
-        else mma_commit(&empty[s]);
+    for (int u = cl; u < p.units && ok; u += ncl) {
+      const int mt0 = (u / p.ntile) * p.mseg, mt1 = min(p.mt, mt0 + p.mseg);
+      for (int mt = mt0; mt < mt1; ++mt, ++j) {
+        const int buf = j & 1;
+        if (!mbar_wait(&tempty[buf], (uint32_t)(j >> 1) & 1u)) { atomicOr(p.err, 64); ok = false; break; }
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                         lead_tempty + (uint32_t)(buf * 8))
+                     : "memory");
       }
-      mma_commit(&tfull[buf]);
     }
   } else if (warp >= 2) {
-    // epilogue warps: TMEM lane quadrant q = warp & 3; the four warps of a
-    // quadrant take the 16-column chunks part, part + 4, part + 8, ...; each
-    // warp loads its next chunk from TMEM while it stores the current one
-    constexpr int NPART = S1_EPI_WARPS / 4;
-    const int q = warp & 3;
-    const int part = (warp - 2) >> 2;
-    const int r = m0 + q * 32 + lane;
-    const int g = r / p.R, ri = r - (r / p.R) * p.R;
-    const size_t cs = (size_t)p.pn * p.ldo;   // output stride between consecutive columns
+    // ---- epilogue: two groups of eight warps take turns by tile, so that one
+    // converts while the other's stores drain; a warp takes TMEM lane quadrant q and
+    // every second 64-column chunk, in two halves (each as hi, then lo) through
+    // the staging rows
+    const int q = warp & 3, part = ((warp - 2) >> 2) & 1, group = (warp - 2) >> 3;
     const float mul = OUT == ET_F16 ? *p.mul : 1.f;
-    auto tmem_ld = [&](uint32_t (&v)[16], uint32_t taddr) {
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15},"
-          " [%16];"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-            "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-            "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(taddr));
-    };
-    auto tmem_wait = [] { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); };
-    auto store = [&](const uint32_t (&v)[16], int c0, int P) {
-      if (r >= p.M) return;
-      const size_t base = (((size_t)g * p.N + c0) * p.pn + P) * p.ldo + ri;
-      const int nc = min(16, p.N - c0);
-      if constexpr (OUT == ET_E4M3) {
-        const float mu = p.mu[P];
-        unsigned char* oh = static_cast<unsigned char*>(p.out_hi) + base;
-        unsigned char* ol = static_cast<unsigned char*>(p.out_lo) + base;
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-          if (t < nc) {
-            const float x = __uint_as_float(v[t]) * mu;
-            const unsigned char h = to_e4m3(x);
-            oh[t * cs] = h;
-            ol[t * cs] = to_e4m3(x - from_e4m3(h));
-          }
-        }
-      } else if constexpr (OUT == ET_F16) {
-        __half* oh = static_cast<__half*>(p.out_hi) + base;
-        __half* ol = static_cast<__half*>(p.out_lo) + base;
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-          if (t < nc) {
-            const float x = __uint_as_float(v[t]) * mul;
-            const __half h = __float2half_rn(x);
-            oh[t * cs] = h;
-            ol[t * cs] = __float2half_rn(x - __half2float(h));
-          }
-        }
-      } else {
-        __nv_bfloat16* oh = static_cast<__nv_bfloat16*>(p.out_hi) + base;
-        __nv_bfloat16* ol = a_split(MODE) ? static_cast<__nv_bfloat16*>(p.out_lo) + base : nullptr;
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-          if (t < nc) {
-            const float x = __uint_as_float(v[t]);
-            const __nv_bfloat16 h = __float2bfloat16_rn(x);
-            oh[t * cs] = h;
-            if (a_split(MODE)) ol[t * cs] = __float2bfloat16_rn(x - __bfloat162float(h));
-          }
-        }
-      }
-    };
-    for (int j = 0; j < nP; ++j) {
-      const int buf = j & 1;
-      bool ok = mbar_wait(&tfull[buf], (uint32_t)(j >> 1) & 1u);
+    constexpr int OB = OUT == ET_E4M3 ? 1 : 2;    // bytes per element
+    constexpr int NW = 4 * OB;                    // 32-bit words of 16 elements
+    constexpr int CC = 64 / OB;                   // columns of a staged piece
+    constexpr int SEG = 16 / OB;                  // columns of a 16-byte segment
+    unsigned char* st = smem + C::EPI_OFF + (warp - 2) * C::EPI_BYTES;
+    unsigned char* srow = st + lane * 64;
+    const int sx = (lane >> 1) & 3;               // segment swizzle of this lane's staging row
+    // the segment that this lane stores: row (lane >> 2) + 8 it, whose swizzle is (lane >> 3) & 3
+    const unsigned char* srd = st + (lane >> 2) * 64 + (((lane & 3) ^ ((lane >> 3) & 3)) * 16);
+    const int prow = p.m * p.no;                  // output rows per P
+    int j = 0;
+    bool ok = true;
+    for (int u = cl; u < p.units && ok; u += ncl) {
+      int n0, r0, width;
+      columns(u % p.ntile, n0, r0, width);
+      const int mt0 = (u / p.ntile) * p.mseg, mt1 = min(p.mt, mt0 + p.mseg);
+    for (int mt = mt0; mt < mt1; ++mt, ++j) {
+      if ((j & 1) != group) continue;
+      const int row = mt * 2 * BM + h * BM + q * 32 + lane;
+      const int buf = group;
+      ok = mbar_wait(&tfull[buf], (uint32_t)(j >> 1) & 1u);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) { if (lane == 0) atomicOr(p.err, 256); break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int P = P0 + j;
-      const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * p.acc_cols);
-      constexpr int STEP = 16 * NPART;
-      uint32_t va[16], vb[16];
-      int c0 = 16 * part;
-      if (c0 < p.N) tmem_ld(va, tbase + (uint32_t)c0);
-      tmem_wait();
-#pragma unroll 1
-      for (; c0 < p.N; c0 += 2 * STEP) {
-        const int c1 = c0 + STEP;
-        if (c1 < p.N) tmem_ld(vb, tbase + (uint32_t)c1);
-        store(va, c0, P);
-        tmem_wait();
-        if (c1 >= p.N) break;
-        if (c1 + STEP < p.N) tmem_ld(va, tbase + (uint32_t)(c1 + STEP));
-        store(vb, c1, P);
-        tmem_wait();
+      // output row of this lane's (P, i) for trial vector 0; -1 beyond the rows
+      const int P = row / p.no;
+      const int orow = row < p.rows ? P * prow + (row - P * p.no) : -1;
+      const float f = OUT == ET_E4M3 ? (row < p.rows ? p.mu[P] : 0.f) : mul;
+      const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
+      // offsets of the rows that this lane stores (four lanes write a row's 64 bytes,
+      // eight rows at a time)
+      long long roff[4];
+#pragma unroll
+      for (int it = 0; it < 4; ++it) {
+        const int o = __shfl_sync(0xffffffffu, orow, it * 8 + (lane >> 2));
+        roff[it] = o < 0 ? -1 : (long long)o * p.ldo * OB;
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])) : "memory");
+      auto read_done = [&] {   // this warp's reads of the accumulator have completed
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])) : "memory");
+      };
+      // this warp's pieces: chunks part and part + 2 in halves of CC columns
+      constexpr int PC = 64 / CC;               // pieces per chunk
+      const int chunks = (width + 63) / 64;
+      const int mine = ((chunks - part + 1) / 2) * PC;
+      int left = 0;                              // pieces that hold columns
+      for (int e = 0; e < mine; ++e) left += ((part + 2 * (e / PC)) * 64 + (e % PC) * CC < width) ? 1 : 0;
+      if (left == 0) read_done();
+#pragma unroll 1
+      for (int e = 0; e < mine; ++e) {
+        const int c0 = (part + 2 * (e / PC)) * 64 + (e % PC) * CC;
+        if (c0 >= width) continue;
+        uint32_t lo[CC / 16][NW];
+        __syncwarp();
+#pragma unroll
+        for (int g = 0; g < CC / 16; g += 2) {
+          uint32_t v[2][16];
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            if (c0 + 16 * (g + u) < width)
+              asm volatile(
+                  "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15},"
+                  " [%16];"
+                  : "=r"(v[u][0]), "=r"(v[u][1]), "=r"(v[u][2]), "=r"(v[u][3]), "=r"(v[u][4]), "=r"(v[u][5]),
+                    "=r"(v[u][6]), "=r"(v[u][7]), "=r"(v[u][8]), "=r"(v[u][9]), "=r"(v[u][10]), "=r"(v[u][11]),
+                    "=r"(v[u][12]), "=r"(v[u][13]), "=r"(v[u][14]), "=r"(v[u][15])
+                  : "r"(tb + (uint32_t)(c0 + 16 * (g + u))));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            uint32_t hi[NW];
+            split16<OUT>(v[u], f, hi, lo[g + u]);
+#pragma unroll
+            for (int k = 0; k < NW; k += 4)
+              *reinterpret_cast<uint4*>(srow + ((((g + u) * OB + k / 4) ^ sx) * 16)) =
+                  make_uint4(hi[k], hi[k + 1], hi[k + 2], hi[k + 3]);
+          }
+        }
+        if (--left == 0) read_done();
+        // this lane's 16-byte segment: trial vector and r (the row's padding is never read)
+        const int seg = (lane & 3) * SEG, c = c0 + seg;
+        const int nn = p.gn > 1 ? c / p.wr : 0;
+        const int n = n0 + nn, r = r0 + c - nn * p.wr;
+        const bool live = c < width && n < p.m && r < p.ldo;
+        const long long coff = ((long long)n * p.no * p.ldo + r) * OB;
+        auto store_rows = [&](unsigned char* out) {
+          __syncwarp();
+#pragma unroll
+          for (int it = 0; it < 4; ++it)
+            if (live && roff[it] >= 0)
+              *reinterpret_cast<uint4*>(out + roff[it] + coff) = *reinterpret_cast<const uint4*>(srd + it * 512);
+        };
+        store_rows(static_cast<unsigned char*>(p.out_hi));
+        __syncwarp();
+#pragma unroll
+        for (int g = 0; g < CC / 16; ++g)
+#pragma unroll
+          for (int k = 0; k < NW; k += 4)
+            *reinterpret_cast<uint4*>(srow + (((g * OB + k / 4) ^ sx) * 16)) =
+                make_uint4(lo[g][k], lo[g][k + 1], lo[g][k + 2], lo[g][k + 3]);
+        store_rows(static_cast<unsigned char*>(p.out_lo));
+      }
+    }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  cluster_sync_all();   // no CTA frees its half or leaves while the other may still use it
   if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * p.acc_cols));
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN));
   }
-  if constexpr (CL > 1) cluster_sync_all();   // neither CTA leaves while the other may still signal it
+}
+
+__device__ __forceinline__ unsigned char to_e4m3(float x) {
+  return (unsigned char)__nv_cvt_float_to_fp8(x, __NV_SATFINITE, __NV_E4M3);
 }
 
 // Sum the split partials into out (FP32), accumulating when asked.
@@ -932,6 +1066,7 @@ CUtensorMap tc_map_f16_4d(const void* base, const uint64_t dims[4], const uint64
 
 int tc_pad(int nv) { return (nv + 7) & ~7; }
 int tc_pad16(int n) { return (n + 15) & ~15; }
+int tc_zpad(int n, int es) { return (n + 128 / es - 1) & ~(128 / es - 1); }
 
 namespace {
 template <typename E>
@@ -1045,7 +1180,7 @@ struct Contraction {
   const void *Ahi, *Alo;
   int M, pn, Kin;
   const void *Bhi, *Blo;
-  int N, ldk, es;      // row pitch (elements), element bytes
+  int N, lda, ldb, es; // row pitches (elements), element bytes
   int total, per, splits, nab;
   float* part;
   int* err;
@@ -1076,10 +1211,10 @@ void launch_pair(const Contraction& c) {
   p.part = c.part;
   p.err = c.err;
   const cuuint64_t dA[3] = {(cuuint64_t)c.Kin, (cuuint64_t)c.pn, (cuuint64_t)c.M};
-  const cuuint64_t sA[2] = {(cuuint64_t)c.ldk * c.es, (cuuint64_t)c.pn * c.ldk * c.es};
+  const cuuint64_t sA[2] = {(cuuint64_t)c.M * c.lda * c.es, (cuuint64_t)c.lda * c.es};
   const cuuint32_t bA[3] = {(cuuint32_t)BKE, 1, (cuuint32_t)(BM / cx)};
   const cuuint64_t dB[3] = {(cuuint64_t)c.Kin, (cuuint64_t)c.N, (cuuint64_t)c.pn};
-  const cuuint64_t sB[2] = {(cuuint64_t)c.ldk * c.es, (cuuint64_t)c.N * c.ldk * c.es};
+  const cuuint64_t sB[2] = {(cuuint64_t)c.ldb * c.es, (cuuint64_t)c.N * c.ldb * c.es};
   const cuuint32_t bB[3] = {(cuuint32_t)BKE, (cuuint32_t)p.b_rows, 1};
   const CUtensorMap mAh = make_map(c.Ahi, dA, sA, bA, ET, RB), mBh = make_map(c.Bhi, dB, sB, bB, ET, RB);
   const CUtensorMap mAl = c.Alo ? make_map(c.Alo, dA, sA, bA, ET, RB) : mAh;
@@ -1111,10 +1246,10 @@ template <int MODE, int ET, int RB>
 void launch_single(const Contraction& c) {
   constexpr int BKE = Elem<ET>::BKE * RB / 128;
   const cuuint64_t dA[3] = {(cuuint64_t)c.Kin, (cuuint64_t)c.pn, (cuuint64_t)c.M};
-  const cuuint64_t sA[2] = {(cuuint64_t)c.ldk * c.es, (cuuint64_t)c.pn * c.ldk * c.es};
+  const cuuint64_t sA[2] = {(cuuint64_t)c.M * c.lda * c.es, (cuuint64_t)c.lda * c.es};
   const cuuint32_t bA[3] = {(cuuint32_t)BKE, 1, BM};
   const cuuint64_t dB[3] = {(cuuint64_t)c.Kin, (cuuint64_t)c.N, (cuuint64_t)c.pn};
-  const cuuint64_t sB[2] = {(cuuint64_t)c.ldk * c.es, (cuuint64_t)c.N * c.ldk * c.es};
+  const cuuint64_t sB[2] = {(cuuint64_t)c.ldb * c.es, (cuuint64_t)c.N * c.ldb * c.es};
   const cuuint32_t bB[3] = {(cuuint32_t)BKE, BN, 1};
   const CUtensorMap mAh = make_map(c.Ahi, dA, sA, bA, ET, RB), mBh = make_map(c.Bhi, dB, sB, bB, ET, RB);
   const CUtensorMap mAl = c.Alo ? make_map(c.Alo, dA, sA, bA, ET, RB) : mAh;
@@ -1148,13 +1283,12 @@ void sum_splits(const Contraction& c, float* out, bool accumulate, const float* 
 }
 }  // namespace
 
-void tc_contract(const void* Ahi, const void* Alo, int M, int pn, int Kin, const void* Bhi, const void* Blo,
+void tc_contract(const void* Ahi, const void* Alo, int lda, int M, int pn, int Kin, const void* Bhi, const void* Blo,
                  int N, float* out, bool accumulate, TcElt elt, const float* scale, int* err, cudaStream_t s,
                  KernelProfile* prof, double prof_flops, double prof_bytes, int max_kb) {
   if (M <= 0 || pn <= 0 || N <= 0) return;
-  TD_REQUIRE(Alo != nullptr || Blo == nullptr, TDDFT_ERR_ARG, "tc_contract: B split without A split");
-  const int mode = Alo ? (Blo ? BOTH : ASPLIT) : SINGLE;
-  TD_REQUIRE(mode == (elt == TcElt::F16 ? BOTH : ASPLIT), TDDFT_ERR_ARG,
+  const int mode = Blo ? BOTH : ASPLIT;
+  TD_REQUIRE(Alo != nullptr && mode == (elt == TcElt::F16 ? BOTH : ASPLIT), TDDFT_ERR_ARG,
              "tc_contract: FP16 operands come as hi + lo on both sides, BF16 ones with a plain B");
   // the split-B products run on 64-byte K rows (a deeper ring), the others on 128-byte rows
   const int rb = mode == BOTH ? 64 : 128;
@@ -1172,7 +1306,7 @@ void tc_contract(const void* Ahi, const void* Alo, int M, int pn, int Kin, const
   const int per = (total + splits - 1) / splits;
   splits = (total + per - 1) / per;
   DevBuf part((size_t)splits * M * N * 4, s);
-  const Contraction c{Ahi, Alo, M, pn, Kin, Bhi, Blo, N, tc_pad(Kin), 2, total, per, splits, nab,
+  const Contraction c{Ahi, Alo, M, pn, Kin, Bhi, Blo, N, lda, tc_pad(Kin), 2, total, per, splits, nab,
                       part.as<float>(), err, s, prof, prof_flops, prof_bytes};
   if (mode == BOTH) launch_contraction<BOTH, ET_F16, 64>(c);
   else launch_contraction<ASPLIT, ET_BF16, 128>(c);
@@ -1192,99 +1326,69 @@ void tc_contract8(const unsigned char* Ahi, const unsigned char* Alo, int M, int
   const int per = (total + splits - 1) / splits;
   splits = (total + per - 1) / per;
   DevBuf part((size_t)splits * M * N * 4, s);
-  const Contraction c{Ahi, Alo, M, pn, Kin, B, nullptr, N, tc_pad16(Kin), 1, total, per, splits, nab,
+  const Contraction c{Ahi, Alo, M, pn, Kin, B, nullptr, N, tc_zpad(Kin, 1), tc_pad16(Kin), 1, total, per, splits, nab,
                       part.as<float>(), err, s, nullptr, 0.0, 0.0};
   launch_contraction<ASPLIT, ET_E4M3, 128>(c);
   sum_splits(c, out, accumulate, scale);
 }
 
 namespace {
-// CTAs of a paired stage-1 launch that can be resident at once (two per
-// co-resident cluster).
-int s1_pair_slots(bool res, int smem) {
-  static int cached[2] = {0, 0}, cached_smem[2] = {0, 0};
-  int& c = cached[res ? 1 : 0];
-  if (c == 0 || cached_smem[res ? 1 : 0] != smem) {
-    cached_smem[res ? 1 : 0] = smem;
-    const void* k = res ? (const void*)k_stage1_tc<BOTH, ET_F16, ET_F16, true, 2>
-                        : (const void*)k_stage1_tc<BOTH, ET_F16, ET_F16, false, 2>;
-    ensure_smem(k, smem);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(2, 1, 1);
-    cfg.blockDim = dim3(S1_THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess || n <= 0) {
-      (void)cudaGetLastError();
-      n = sm_count() / 2;
-    }
-    c = 2 * n;
-  }
-  return c;
-}
-
-// out_is8: e4m3 outputs with per-P multipliers mu (A as hi + lo, B plain);
+// out_is8: e4m3 outputs with per-P multipliers mu (X as BF16 hi + lo, L plain);
 // otherwise 16-bit outputs of the inputs' element type et, FP16 ones times *mul.
-void stage1_impl(const void* Ahi, const void* Alo, int M, int K, const void* Bhi, const void* Blo, int N, int pn,
-                 int R, int et, bool out_is8, void* out_hi, void* out_lo, const float* mul, const float* mu, int* err,
+void stage1_impl(const void* Xhi, const void* Xlo, int m, int R, int K, const void* Lhi, const void* Llo, int no,
+                 int pn, int et, bool out_is8, void* out_hi, void* out_lo, const float* mul, const float* mu, int* err,
                  cudaStream_t s) {
-  if (M <= 0 || pn <= 0 || N <= 0) return;
-  TD_REQUIRE(N <= 256, TDDFT_ERR_ARG, "tc_stage1: N above 256");
-  TD_REQUIRE((Alo != nullptr || Blo == nullptr) &&
-                 (out_is8 ? (out_lo != nullptr && mu != nullptr) : (Alo != nullptr) == (out_lo != nullptr)),
+  if (m <= 0 || R <= 0 || pn <= 0 || no <= 0) return;
+  TD_REQUIRE(no <= 256, TDDFT_ERR_ARG, "tc_stage1: n_occ above 256");
+  TD_REQUIRE(Xhi && Xlo && Lhi && out_hi && out_lo && (!out_is8 || mu != nullptr) && (et == ET_F16) == (Llo != nullptr),
              TDDFT_ERR_ARG, "tc_stage1: hi/lo operands mismatch");
   TD_REQUIRE((et == ET_F16) == (mul != nullptr) && (!out_is8 || et == ET_BF16), TDDFT_ERR_ARG,
              "tc_stage1: FP16 outputs need a multiplier, FP8 outputs BF16 inputs");
-  const int mode = Alo ? (Blo ? BOTH : ASPLIT) : SINGLE;
   const int ldk = tc_pad(K);
-  const int nb = (N + 15) & ~15;
-  int acc_cols = 32;
-  while (acc_cols < nb) acc_cols *= 2;
-  const int a_bytes = BM * BK * 2, b_bytes = nb * BK * 2;
-  const int nkb = (K + BK - 1) / BK;
-  const int mt0 = (M + BM - 1) / BM;
-  // The FP16 exact operands (hi + lo on both sides): the A tile stays resident
-  // when all its k-blocks fit beside a ring of three B stages, and pairs of M
-  // tiles share each B_P tile through a cluster multicast.
-  constexpr int kSmemBudget = 224 * 1024;
-  const int a_res = nkb * n_parts_a(mode) * a_bytes;
-  const int b_stage = n_parts_b(mode) * b_bytes;
-  const bool res = et == ET_F16 && !out_is8 && a_res + 3 * b_stage + 2048 <= kSmemBudget;
-  const bool pair = et == ET_F16 && !out_is8 && mt0 > 1 && cluster_pairs_enabled();
-  const int mt = pair ? (mt0 + 1) & ~1 : mt0;
-  const int stage_bytes = res ? b_stage : n_parts_a(mode) * a_bytes + b_stage;
-  int stages = ((res ? kSmemBudget - a_res - 2048 : 200 * 1024)) / stage_bytes;
-  if (stages > 6) stages = 6;
-  TD_REQUIRE(stages >= 2, TDDFT_ERR_ARG, "tc_stage1: tile too large");
-  const int smem = (res ? a_res : 0) + stages * stage_bytes + 1024 + 256;
-  int groups = wave_splits(mt, pn, 1, pair ? s1_pair_slots(res, smem) : 0);   // units: P-rows
-  const int ppc = (pn + groups - 1) / groups;
-  groups = (pn + ppc - 1) / ppc;
-
-  const cuuint64_t dA[3] = {(cuuint64_t)K, (cuuint64_t)M, 1};
-  const cuuint64_t sA[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)M * ldk * 2};
-  const cuuint32_t bA[3] = {BK, BM, 1};
-  const cuuint64_t dB[3] = {(cuuint64_t)K, (cuuint64_t)N, (cuuint64_t)pn};
-  const cuuint64_t sB[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)N * ldk * 2};
-  const cuuint32_t bB[3] = {BK, (cuuint32_t)(pair ? nb / 2 : nb), 1};   // a pair loads half a B tile each
-  CUtensorMap mAh = make_map(Ahi, dA, sA, bA, et), mBh = make_map(Bhi, dB, sB, bB, et);
-  CUtensorMap mAl = Alo ? make_map(Alo, dA, sA, bA, et) : mAh;
-  CUtensorMap mBl = Blo ? make_map(Blo, dB, sB, bB, et) : mBh;
-  S1Params p{M, N, R, out_is8 ? tc_pad16(R) : tc_pad(R), pn, ppc, nkb, K, nb, acc_cols, stages,
-             stage_bytes, a_bytes, b_bytes, res ? a_res : 0, out_hi, out_lo, mul, mu, err};
-  dim3 grid(mt, groups, 1);
-  auto launch = [&](auto kernel) {
-    ensure_smem((const void*)kernel, smem);
-    kernel<<<grid, S1_THREADS, smem, s>>>(mAh, mAl, mBh, mBl, p);
-  };
-  auto launch_pair = [&](auto kernel) {
+  S1Params p;
+  p.rows = pn * no;
+  p.no = no;
+  p.pn = pn;
+  p.R = R;
+  p.m = m;
+  p.ldo = tc_zpad(R, out_is8 ? 1 : 2);
+  p.K = K;
+  p.nkb = (K + S1_RB / 2 - 1) / (S1_RB / 2);
+  // several trial vectors per tile while they fit, else equal parts of one
+  p.wr = (R + 15) & ~15;
+  p.gn = 1;
+  while (2 * p.gn * p.wr <= BN && p.gn < m) p.gn *= 2;
+  p.nt0 = (R + BN - 1) / BN;
+  p.col_unit = p.nt0 > 1 ? 64 : 32;
+  const int units = (R + p.col_unit - 1) / p.col_unit;
+  p.nq = units / p.nt0;
+  p.nr = units % p.nt0;
+  p.mt = (p.rows + 2 * BM - 1) / (2 * BM);
+  p.ntile = p.gn > 1 ? (m + p.gn - 1) / p.gn : m * p.nt0;
+  p.b_rows = p.gn > 1 ? p.gn / 2 * p.wr : p.col_unit / 2 * (p.nq + (p.nr ? 1 : 0));
+  p.out_hi = out_hi;
+  p.out_lo = out_lo;
+  p.mul = mul;
+  p.mu = mu;
+  p.err = err;
+  TD_REQUIRE((long long)p.mt * p.ntile < (1ll << 30) && (long long)m * no * pn < (1ll << 31), TDDFT_ERR_ARG, "tc_stage1: problem too large");
+  const cuuint64_t dA[3] = {(cuuint64_t)K, (cuuint64_t)p.rows, 1};
+  const cuuint64_t sA[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)p.rows * ldk * 2};
+  const cuuint32_t bA[3] = {S1_RB / 2, BM, 1};
+  const cuuint64_t dB[3] = {(cuuint64_t)K, (cuuint64_t)R, (cuuint64_t)m};
+  const cuuint64_t sB[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)R * ldk * 2};
+  const cuuint32_t bB[3] = {S1_RB / 2, (cuuint32_t)(p.gn > 1 ? p.wr : p.b_rows), (cuuint32_t)(p.gn > 1 ? p.gn / 2 : 1)};
+  const CUtensorMap mAh = make_map(Lhi, dA, sA, bA, et, S1_RB), mBh = make_map(Xhi, dB, sB, bB, et, S1_RB);
+  const CUtensorMap mAl = Llo ? make_map(Llo, dA, sA, bA, et, S1_RB) : mAh;
+  const CUtensorMap mBl = make_map(Xlo, dB, sB, bB, et, S1_RB);
+  // units of up to 16 row tiles (RES: they share the resident X rows), at least six
+  // per cluster where there are that many tiles
+  const int slots = std::max(1, pair_slots() / 2);
+  p.mseg = std::max(1, std::min(16, (int)((long long)p.mt * p.ntile / (6 * slots))));
+  p.units = p.ntile * ((p.mt + p.mseg - 1) / p.mseg);
+  const int clusters = std::min(p.units, slots);
+  const bool res = p.nkb <= S1_RES_KB;
+  auto go = [&](auto kernel, int smem) {
     ensure_smem((const void*)kernel, smem);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -1292,7 +1396,7 @@ void stage1_impl(const void* Ahi, const void* Alo, int M, int K, const void* Bhi
     at[0].val.clusterDim.x = 2;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
-    cfg.gridDim = grid;
+    cfg.gridDim = dim3((unsigned)(2 * clusters), 1, 1);
     cfg.blockDim = dim3(S1_THREADS);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;
@@ -1300,32 +1404,29 @@ void stage1_impl(const void* Ahi, const void* Alo, int M, int K, const void* Bhi
     cfg.numAttrs = 1;
     TD_CUDA(cudaLaunchKernelEx(&cfg, kernel, mAh, mAl, mBh, mBl, p));
   };
-  if (out_is8) {
-    TD_REQUIRE(mode == ASPLIT, TDDFT_ERR_ARG, "tc_stage1: FP8 output needs hi+lo A and a plain B");
-    launch(k_stage1_tc<ASPLIT, ET_BF16, ET_E4M3>);
-  } else if (et == ET_F16) {
-    TD_REQUIRE(mode == BOTH, TDDFT_ERR_ARG, "tc_stage1: FP16 operands come as hi + lo");
-    if (res && pair) launch_pair(k_stage1_tc<BOTH, ET_F16, ET_F16, true, 2>);
-    else if (res) launch(k_stage1_tc<BOTH, ET_F16, ET_F16, true, 1>);
-    else if (pair) launch_pair(k_stage1_tc<BOTH, ET_F16, ET_F16, false, 2>);
-    else launch(k_stage1_tc<BOTH, ET_F16, ET_F16>);
-  } else if (mode == BOTH) launch(k_stage1_tc<BOTH, ET_BF16, ET_BF16>);
-  else if (mode == ASPLIT) launch(k_stage1_tc<ASPLIT, ET_BF16, ET_BF16>);
-  else launch(k_stage1_tc<SINGLE, ET_BF16, ET_BF16>);
+  if (res) {
+    if (out_is8) go(k_stage1_pair<false, true, ET_BF16, ET_E4M3>, S1Cfg<false, true>::SMEM_BYTES);
+    else if (et == ET_F16) go(k_stage1_pair<true, true, ET_F16, ET_F16>, S1Cfg<true, true>::SMEM_BYTES);
+    else go(k_stage1_pair<false, true, ET_BF16, ET_BF16>, S1Cfg<false, true>::SMEM_BYTES);
+  } else {
+    if (out_is8) go(k_stage1_pair<false, false, ET_BF16, ET_E4M3>, S1Cfg<false, false>::SMEM_BYTES);
+    else if (et == ET_F16) go(k_stage1_pair<true, false, ET_F16, ET_F16>, S1Cfg<true, false>::SMEM_BYTES);
+    else go(k_stage1_pair<false, false, ET_BF16, ET_BF16>, S1Cfg<false, false>::SMEM_BYTES);
+  }
   count_launch();
   TD_LAUNCH_CHECK();
 }
 }  // namespace
 
-void tc_stage1(const void* Ahi, const void* Alo, int M, int K, const void* Bhi, const void* Blo, int N, int pn,
-               int R, TcElt et, const float* mul, void* out_hi, void* out_lo, int* err, cudaStream_t s) {
-  stage1_impl(Ahi, Alo, M, K, Bhi, Blo, N, pn, R, elem_of(et), false, out_hi, out_lo, mul, nullptr, err, s);
+void tc_stage1(const void* Xhi, const void* Xlo, int m, int R, int K, const void* Lhi, const void* Llo, int no, int pn,
+               TcElt et, const float* mul, void* out_hi, void* out_lo, int* err, cudaStream_t s) {
+  stage1_impl(Xhi, Xlo, m, R, K, Lhi, Llo, no, pn, elem_of(et), false, out_hi, out_lo, mul, nullptr, err, s);
 }
 
-void tc_stage1_fp8(const __nv_bfloat16* Ahi, const __nv_bfloat16* Alo, int M, int K, const __nv_bfloat16* B,
-                   int N, int pn, int R, const float* mu, unsigned char* out_hi, unsigned char* out_lo, int* err,
+void tc_stage1_fp8(const __nv_bfloat16* Xhi, const __nv_bfloat16* Xlo, int m, int R, int K, const __nv_bfloat16* L,
+                   int no, int pn, const float* mu, unsigned char* out_hi, unsigned char* out_lo, int* err,
                    cudaStream_t s) {
-  stage1_impl(Ahi, Alo, M, K, B, nullptr, N, pn, R, ET_BF16, true, out_hi, out_lo, nullptr, mu, err, s);
+  stage1_impl(Xhi, Xlo, m, R, K, L, nullptr, no, pn, ET_BF16, true, out_hi, out_lo, nullptr, mu, err, s);
 }
 
 // F64/F32/BF16 rows [rows][n] -> hi (+ lo) [rows][tc_pad(n)] (times *scale when given)

@@ -17,6 +17,8 @@ enum class TcElt : int { BF16 = 0, F16 = 1 };
 int tc_pad(int nv);
 // Row pitch (elements) of the padded FP8 operands: n rounded up to 16.
 int tc_pad16(int n);
+// Row pitch (elements of es bytes) of the stage-1 results: whole 128-byte lines.
+int tc_zpad(int n, int es);
 
 // SMs of the current device (queried once).
 int sm_count();
@@ -39,12 +41,11 @@ void tc_transpose_split(const void* src, DType ts, int rows, int n1, int n2, voi
 void tc_pad_split(const void* src, DType ts, long long rows, int n, void* hi, void* lo, TcElt et,
                   const float* scale, cudaStream_t s);
 
-// C[m][n] (+)= s * sum_(P<pn) sum_(k<Kin) A[m][P][k] B[P][n][k] on the tcgen05
-// tensor cores.  A: [M][pn][tc_pad(Kin)], B: [pn][N][tc_pad(Kin)] of element type
+// C[m][n] (+)= s * sum_(P<pn) sum_(k<Kin) A[P][m][k] B[P][n][k] on the tcgen05
+// tensor cores.  A: [pn][M][lda], B: [pn][N][tc_pad(Kin)] of element type
 // et, C: [M][N] FP32, accumulated into when `accumulate`; s = *scale (a device
-// scalar) or 1 when scale is NULL.  Operand splits: with Alo and Blo the three
-// products hi*hi + hi*lo + lo*hi are formed; with Alo alone the two products
-// Ahi*B + Alo*B; with neither one product (Blo without Alo is not allowed).
+// scalar) or 1 when scale is NULL.  FP16: A and B as hi + lo, three products
+// hi*hi + hi*lo + lo*hi; BF16: A as hi + lo, B plain (Blo NULL), two products.
 // Timeouts of the kernel's internal waits are reported by OR-ing a nonzero
 // code into *err.  With `prof`, CUDA events bracket the contraction kernel
 // alone (not the split reduction) and prof_flops / prof_bytes (the launch's
@@ -53,19 +54,19 @@ void tc_pad_split(const void* src, DType ts, long long rows, int n, void* hi, vo
 // split-K partials, summed in a fixed order), for contractions whose K is long enough that the length of
 // the accumulation run sets the rounding error.
 struct KernelProfile;
-void tc_contract(const void* Ahi, const void* Alo, int M, int pn, int Kin, const void* Bhi, const void* Blo,
+void tc_contract(const void* Ahi, const void* Alo, int lda, int M, int pn, int Kin, const void* Bhi, const void* Blo,
                  int N, float* out, bool accumulate, TcElt et, const float* scale, int* err, cudaStream_t s,
                  KernelProfile* prof = nullptr, double prof_flops = 0.0, double prof_bytes = 0.0, int max_kb = 0);
 
-// Stage-1 exchange contraction on the tensor cores, batched over P:
-//   C_P[r][c] = sum_(k<K) A[r][k] B_P[c][k],  A: [M][tc_pad(K)], B: [pn][N][tc_pad(K)],
-// written as hi (+ lo) parts of element type et to out[(g*N + c)][P][ri]
-// (r = g*R + ri, row pitch pn*tc_pad(R)) -- the A operand layout of
-// tc_contract.  N <= 256.  BF16: with lo operands the hi/lo products are
-// formed, mul NULL.  FP16: A and B as hi + lo, and the parts are those of
-// (*mul) C_P (mul a device scalar).
-void tc_stage1(const void* Ahi, const void* Alo, int M, int K, const void* Bhi, const void* Blo, int N, int pn,
-               int R, TcElt et, const float* mul, void* out_hi, void* out_lo, int* err, cudaStream_t s);
+// Stage-1 exchange contraction on the tensor cores, for every P and trial vector:
+//   C_P[n][i][r] = sum_(k<K) L_P[i][k] X[n][r][k],  X: [m][R][tc_pad(K)] as hi + lo,
+//   L: [pn][no][tc_pad(K)],
+// written as hi + lo parts of element type et to out[P][(n, i)][r] (row pitch
+// tc_zpad(R, 2)) -- the A operand layout of tc_contract.  no <= 256.  BF16: L
+// plain (two products), mul NULL.  FP16: L as hi + lo (three products), and the
+// parts are those of (*mul) C_P (mul a device scalar).
+void tc_stage1(const void* Xhi, const void* Xlo, int m, int R, int K, const void* Lhi, const void* Llo, int no, int pn,
+               TcElt et, const float* mul, void* out_hi, void* out_lo, int* err, cudaStream_t s);
 
 // ---- FP16 scales of the exact operator.  Factor-set scale block (8 floats):
 //   [0] s_oo, [1] s_oo * max ||L^P_oo[i][:]||, [2] s_vv, [4] s_ov,
@@ -103,14 +104,14 @@ void tc_row_norm_max(const __nv_bfloat16* src, int rows, int nr, int nc, float* 
 void tc_fp8_scales(const void* X, DType xt, int m, int no, int nv, const float* s_vv, const float* rho_oo,
                    const float* s_vo, const float* rho_ov, int nK, float* out, unsigned* kappa,
                    cudaStream_t s);
-// Stage 1 with e4m3 hi + lo output: out[(g*N + c)][P][ri] (row pitch
-// pn*tc_pad16(R) bytes) = split of mu[P] * C_P[r][c]; A as BF16 hi + lo, B BF16.
-void tc_stage1_fp8(const __nv_bfloat16* Ahi, const __nv_bfloat16* Alo, int M, int K, const __nv_bfloat16* B,
-                   int N, int pn, int R, const float* mu, unsigned char* out_hi, unsigned char* out_lo, int* err,
+// Stage 1 with e4m3 hi + lo output (row pitch tc_zpad(R, 1) bytes): split of
+// mu[P] * C_P; X as BF16 hi + lo, L BF16.
+void tc_stage1_fp8(const __nv_bfloat16* Xhi, const __nv_bfloat16* Xlo, int m, int R, int K, const __nv_bfloat16* L,
+                   int no, int pn, const float* mu, unsigned char* out_hi, unsigned char* out_lo, int* err,
                    cudaStream_t s);
-// out (+)= (*scale) * sum_P sum_k A[m][P][k] B[P][n][k] on the tensor cores
+// out (+)= (*scale) * sum_P sum_k A[P][m][k] B[P][n][k] on the tensor cores
 // (kind::f8f6f4, e4m3 x e4m3, FP32 accumulation): A as e4m3 hi + lo
-// [M][pn][tc_pad16(Kin)], B e4m3 [pn][N][tc_pad16(Kin)]; scale a device scalar.
+// [pn][M][tc_zpad(Kin, 1)], B e4m3 [pn][N][tc_pad16(Kin)]; scale a device scalar.
 void tc_contract8(const unsigned char* Ahi, const unsigned char* Alo, int M, int pn, int Kin,
                   const unsigned char* B, int N, float* out, bool accumulate, const float* scale, int* err,
                   cudaStream_t s);
