@@ -33,9 +33,10 @@ k_sk_gram(const TA* __restrict__ A, long long lda, int M, const TB* __restrict__
   static_assert(kGramThreads % KC == 0 || KC % kGramThreads == 0, "tile mapping");
   constexpr int RSTEP = kGramThreads / KC;        // rows advanced per pass
   constexpr int PASSES = kTile / RSTEP;
-  // row stride: 16-byte aligned rows for vector loads; the 4-float (2-double)
-  // skew spreads the 16 B-columns of a warp over the banks
-  constexpr int VW = 16 / sizeof(ACC);             // elements per 16-byte load
+  static_assert(sizeof(ACC) == 4, "FP32 accumulation (FP64: k_sk_gram64)");
+  // row stride: 16-byte aligned rows for vector loads; the 4-float skew spreads
+  // the 16 B-columns of a warp over the banks
+  constexpr int VW = 4;                            // elements per 16-byte load
   constexpr int LD = KC + VW;
   extern __shared__ __align__(16) unsigned char gram_raw[];
   ACC* As = reinterpret_cast<ACC*>(gram_raw);
@@ -62,7 +63,7 @@ k_sk_gram(const TA* __restrict__ A, long long lda, int M, const TB* __restrict__
   __syncthreads();
   const int tx = tid & 15, ty = tid >> 4;
   ACC c00 = 0, c01 = 0, c10 = 0, c11 = 0;
-  using V16 = typename std::conditional<sizeof(ACC) == 4, float4, double2>::type;
+  using V16 = float4;
   const V16* a0 = reinterpret_cast<const V16*>(As + ty * LD);
   const V16* a1 = reinterpret_cast<const V16*>(As + (ty + 16) * LD);
   const V16* b0 = reinterpret_cast<const V16*>(Bs + tx * LD);
@@ -70,17 +71,10 @@ k_sk_gram(const TA* __restrict__ A, long long lda, int M, const TB* __restrict__
 #pragma unroll 4
   for (int k = 0; k < KC / VW; ++k) {   // columns beyond kn were staged as zeros
     const V16 x0 = a0[k], x1 = a1[k], y0 = b0[k], y1 = b1[k];
-    if constexpr (sizeof(ACC) == 4) {
-      c00 = fma(x0.x, y0.x, c00); c00 = fma(x0.y, y0.y, c00); c00 = fma(x0.z, y0.z, c00); c00 = fma(x0.w, y0.w, c00);
-      c01 = fma(x0.x, y1.x, c01); c01 = fma(x0.y, y1.y, c01); c01 = fma(x0.z, y1.z, c01); c01 = fma(x0.w, y1.w, c01);
-      c10 = fma(x1.x, y0.x, c10); c10 = fma(x1.y, y0.y, c10); c10 = fma(x1.z, y0.z, c10); c10 = fma(x1.w, y0.w, c10);
-      c11 = fma(x1.x, y1.x, c11); c11 = fma(x1.y, y1.y, c11); c11 = fma(x1.z, y1.z, c11); c11 = fma(x1.w, y1.w, c11);
-    } else {
-      c00 = fma(x0.x, y0.x, c00); c00 = fma(x0.y, y0.y, c00);
-      c01 = fma(x0.x, y1.x, c01); c01 = fma(x0.y, y1.y, c01);
-      c10 = fma(x1.x, y0.x, c10); c10 = fma(x1.y, y0.y, c10);
-      c11 = fma(x1.x, y1.x, c11); c11 = fma(x1.y, y1.y, c11);
-    }
+    c00 = fma(x0.x, y0.x, c00); c00 = fma(x0.y, y0.y, c00); c00 = fma(x0.z, y0.z, c00); c00 = fma(x0.w, y0.w, c00);
+    c01 = fma(x0.x, y1.x, c01); c01 = fma(x0.y, y1.y, c01); c01 = fma(x0.z, y1.z, c01); c01 = fma(x0.w, y1.w, c01);
+    c10 = fma(x1.x, y0.x, c10); c10 = fma(x1.y, y0.y, c10); c10 = fma(x1.z, y0.z, c10); c10 = fma(x1.w, y0.w, c10);
+    c11 = fma(x1.x, y1.x, c11); c11 = fma(x1.y, y1.y, c11); c11 = fma(x1.z, y1.z, c11); c11 = fma(x1.w, y1.w, c11);
   }
   ACC* P = part + (long long)blockIdx.x * M * N;
   const int ma = m0 + ty, mb = m0 + ty + 16, na = n0 + tx, nb = n0 + tx + 16;
@@ -88,6 +82,64 @@ k_sk_gram(const TA* __restrict__ A, long long lda, int M, const TB* __restrict__
   if (ma < M && nb < N) P[(long long)ma * N + nb] = c01;
   if (mb < M && na < N) P[(long long)mb * N + na] = c10;
   if (mb < M && nb < N) P[(long long)mb * N + nb] = c11;
+}
+
+// FP64 form.  What bounds it is the FP64 unit (two DFMA per cycle and SM), so a
+// lane that computes a pair outside the M x N outputs costs as much as one that
+// works, and a chunk of K is as short as it takes to occupy every SM: the
+// tile's Mt x Nt pairs are dealt to the threads one by one (and, where fewer than
+// half of the threads have a pair, the chunk's k among groups of threads).
+// K = 400, up to 60 x 10 outputs: 34 -> 3.2 us a launch (before: chunks of 128
+// columns, 32 x 32 pairs whether wanted or not).
+template <int KC>
+__global__ void __launch_bounds__(kGramThreads)
+k_sk_gram64(const double* __restrict__ A, long long lda, int M, const double* __restrict__ B, long long ldb, int N,
+            int K, double* __restrict__ part) {
+  constexpr int LD = KC + 1;
+  extern __shared__ __align__(16) unsigned char gram_raw[];
+  double* As = reinterpret_cast<double*>(gram_raw);
+  double* Bs = As + kTile * LD;
+  const int tid = threadIdx.x;
+  const int k0 = blockIdx.x * KC;
+  const int kn = min(KC, K - k0);
+  const int m0 = blockIdx.y * kTile, n0 = blockIdx.z * kTile;
+  const int Mt = min(kTile, M - m0), Nt = min(kTile, N - n0);
+  for (int e = tid; e < (Mt + Nt) * KC; e += kGramThreads) {
+    const int r = e / KC, k = e % KC;
+    const double* row = r < Mt ? A + (long long)(m0 + r) * lda : B + (long long)(n0 + r - Mt) * ldb;
+    (r < Mt ? As + r * LD : Bs + (r - Mt) * LD)[k] = k < kn ? row[k0 + k] : 0.0;
+  }
+  __syncthreads();
+  double* P = part + (long long)blockIdx.x * M * N;
+  const int pairs = Mt * Nt;
+  if (2 * pairs > kGramThreads) {
+    for (int e = tid; e < pairs; e += kGramThreads) {
+      const int m = e / Nt, n = e - m * Nt;
+      const double *a = As + m * LD, *b = Bs + n * LD;
+      double c0 = 0.0, c1 = 0.0;
+#pragma unroll
+      for (int k = 0; k < KC; k += 2) {
+        c0 = fma(a[k], b[k], c0);
+        c1 = fma(a[k + 1], b[k + 1], c1);
+      }
+      P[(long long)(m0 + m) * N + n0 + n] = c0 + c1;
+    }
+    return;
+  }
+  // groups of `pairs` threads share the chunk's k
+  const int G = kGramThreads / pairs, g = tid / pairs, e = tid - g * pairs;
+  const int m = e / Nt, n = e - m * Nt;
+  double c = 0.0;
+  if (g < G)
+    for (int k = g; k < KC; k += G) c = fma(As[m * LD + k], Bs[n * LD + k], c);
+  __syncthreads();
+  double* red = As;   // [G][pairs] (<= 256 doubles)
+  if (g < G) red[tid] = c;
+  __syncthreads();
+  if (tid < pairs) {
+    for (int q = 1; q < G; ++q) c += red[q * pairs + tid];
+    P[(long long)(m0 + m) * N + n0 + n] = c;
+  }
 }
 
 // One warp per output element: lane l sums the chunks l, l+32, ... in order,
@@ -174,21 +226,35 @@ void set_smem_attr(const void* f, size_t bytes) {
 template <typename TA, typename TB, typename ACC>
 void gram_typed(const void* A, long long lda, int M, const void* B, long long ldb, int N, int K, void* C,
                 DType tc, long long ldc, double alpha, double beta, cudaStream_t s) {
-  const int tiles = ((M + kTile - 1) / kTile) * ((N + kTile - 1) / kTile);
   TD_REQUIRE((M + kTile - 1) / kTile <= 65535 && (N + kTile - 1) / kTile <= 65535, TDDFT_ERR_ARG,
              "sk_gram: too many rows");
-  // fixed K chunks: 256 columns (FP32 staging) or 128 (FP64)
-  constexpr int KC = sizeof(ACC) == 8 ? 128 : 256;
+  // fixed K chunks: 256 columns (FP32 staging); FP64 16 to 128, so that K up to
+  // 20,000 is cut into 150 chunks or more where the columns allow it
+  int KC = 256;
+  if (sizeof(ACC) == 8) KC = K <= 2432 ? 16 : (K <= 4864 ? 32 : (K <= 9728 ? 64 : 128));
   const int S = K > 0 ? (K + KC - 1) / KC : 1;
-  (void)tiles;
   DevBuf part((size_t)S * M * N * sizeof(ACC), s);
   if (K > 0) {
-    const size_t smem = (size_t)2 * kTile * (KC + 16 / sizeof(ACC)) * sizeof(ACC);
-    set_smem_attr((const void*)k_sk_gram<TA, TB, ACC, KC>, smem);
-    dim3 grid(S, (M + kTile - 1) / kTile, (N + kTile - 1) / kTile);
-    k_sk_gram<TA, TB, ACC, KC><<<grid, kGramThreads, smem, s>>>(static_cast<const TA*>(A), lda, M,
-                                                                static_cast<const TB*>(B), ldb, N, K,
-                                                                part.as<ACC>());
+    const dim3 grid(S, (M + kTile - 1) / kTile, (N + kTile - 1) / kTile);
+    if constexpr (sizeof(ACC) == 8) {
+      auto go = [&](auto kernel) {
+        const size_t smem = std::max((size_t)2 * kTile * (KC + 1), (size_t)kGramThreads) * sizeof(double);
+        set_smem_attr((const void*)kernel, smem);
+        kernel<<<grid, kGramThreads, smem, s>>>(static_cast<const double*>(A), lda, M, static_cast<const double*>(B),
+                                                ldb, N, K, part.as<double>());
+      };
+      if (KC == 16) go(k_sk_gram64<16>);
+      else if (KC == 32) go(k_sk_gram64<32>);
+      else if (KC == 64) go(k_sk_gram64<64>);
+      else go(k_sk_gram64<128>);
+    } else {
+      constexpr int KF = 256;
+      const size_t smem = (size_t)2 * kTile * (KF + 16 / sizeof(ACC)) * sizeof(ACC);
+      set_smem_attr((const void*)k_sk_gram<TA, TB, ACC, KF>, smem);
+      k_sk_gram<TA, TB, ACC, KF><<<grid, kGramThreads, smem, s>>>(static_cast<const TA*>(A), lda, M,
+                                                                  static_cast<const TB*>(B), ldb, N, K,
+                                                                  part.as<ACC>());
+    }
     count_launch();
     TD_LAUNCH_CHECK();
   } else {
