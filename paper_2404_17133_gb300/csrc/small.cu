@@ -4,8 +4,8 @@
 // GB300 executes FP64 at about 1/64 of the FP32 SIMT rate, so the O(n^3) parts
 // run in FP32 and FP64 is kept to O(n^2 k) work:
 //   * eig32: parallel cyclic Jacobi (round-robin pair ordering, n/2 disjoint
-//     rotations per round) in FP32, one CTA, matrix and eigenvectors in shared
-//     memory;
+//     rotations per round) in FP32: the matrix by one CTA in shared memory, the
+//     eigenvectors row by row from the rotations it writes down;
 //   * refine_lowest: for each wanted eigenpair, Newton-type corrections
 //     q <- q - sum_{j != i} v_j (v_j^T r) / (lam_j - lam), r = Hq - lam q, with
 //     the FP32 eigenvectors v_j (one CTA per pair), then Cholesky-QR of the k
@@ -41,6 +41,26 @@ __device__ double block_sum(double v, double* red) {
   }
   __syncthreads();
   return red[32];
+}
+
+// 1 / x and 1 / sqrt(x) for the pivots.  An FP64 division or square root is a
+// dozen dependent FP64 instructions on a unit that issues one per 64 cycles; a
+// FP32 estimate and two Newton steps (error 1e-7 -> 1e-14 -> the last bits)
+// take four (six).  Values that FP32 cannot hold take the division.
+__device__ __forceinline__ float fast_rcp(float x) { return 1.f / x; }
+__device__ __forceinline__ double fast_rcp(double x) {
+  const double ax = fabs(x);
+  if (!(ax > 1e-30 && ax < 1e30)) return 1.0 / x;
+  double y = (double)(1.f / (float)x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+__device__ __forceinline__ double fast_rsqrt(double x) {
+  if (!(x > 1e-30 && x < 1e30)) return 1.0 / sqrt(x);
+  double y = (double)rsqrtf((float)x);
+  const double hx = 0.5 * x;
+  y = fma(y, fma(-hx * y, y, 0.5), y);
+  return fma(y, fma(-hx * y, y, 0.5), y);
 }
 
 template <typename T> __device__ __forceinline__ T big_theta();
@@ -142,31 +162,203 @@ __device__ int diag_rank(const T* A, int ld, int n, int t) {
   return r;
 }
 
-__global__ void __launch_bounds__(1024) k_eig32(const double* __restrict__ H, int ldh, int n,
-                                                float* __restrict__ lam32, float* __restrict__ vec32) {
+// The rotations of one Jacobi run in order: [round][pair] (c, s), and behind
+// them the number of rounds and the rank of each diagonal entry.
+constexpr int kJacSweeps = 16;
+constexpr int kJacHalf = kSmallMax / 2;                       // pairs per round
+constexpr size_t kJacRounds = (size_t)kJacSweeps * (kSmallMax - 1);
+constexpr size_t kJacBytes = kJacRounds * kJacHalf * sizeof(float2) + (1 + kSmallMax) * sizeof(int);
+
+// eig32, part 1: the same cyclic Jacobi as jacobi_cta on the upper triangle of A
+// alone, by one CTA.  A round is bound by shared memory (n = 160, both triangles
+// and Q: 410 KB in 3200 cycles; here 100 KB), so Q is left to k_jacobi_q, which
+// replays the rotations this kernel writes down.  Casida matrices of a 10-state
+// solve (n up to 160): 1612 us before, 853 and 60 now; n up to 60: 470, 298 and 20.
+__global__ void __launch_bounds__(1024) k_jacobi_a(const double* __restrict__ H, int ldh, int n,
+                                                   float* __restrict__ lam32, float2* __restrict__ rot,
+                                                   int* __restrict__ info) {
   extern __shared__ float sm32[];
-  __shared__ int pp[kSmallMax / 2 + 1], qq[kSmallMax / 2 + 1];
-  __shared__ float cc[kSmallMax / 2 + 1], ss[kSmallMax / 2 + 1];
+  __shared__ float2 cs[kJacHalf];
   __shared__ unsigned smax;
   __shared__ double red[33];
-  const int NP = (n + 1) & ~1, ld = NP + 1;
+  const int NP = (n + 1) & ~1, ld = NP + 1, half = NP / 2;
   float* A = sm32;
-  float* Q = sm32 + NP * ld;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   double f2 = 0.0;
-  for (int idx = threadIdx.x; idx < NP * NP; idx += blockDim.x) {
+  for (int idx = tid; idx < NP * NP; idx += blockDim.x) {
     int r = idx / NP, c = idx - r * NP;
     double v = 0.0;
     if (r < n && c < n) v = 0.5 * (H[(long long)r * ldh + c] + H[(long long)c * ldh + r]);
     f2 += v * v;
     A[r * ld + c] = (float)v;
-    Q[r * ld + c] = (r == c) ? 1.f : 0.f;
   }
-  double frob = sqrt(block_sum(f2, red));
-  jacobi_cta<float>(A, Q, n, ld, frob, 16, 2e-7, pp, qq, cc, ss, &smax);
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    int r = diag_rank(A, ld, n, t);
+  const double frob = sqrt(block_sum(f2, red));
+  const float stop = (float)(2e-7 * frob), skip = (float)(2e-10 * frob);
+  int rounds = 0;
+  for (int sweep = 0; sweep < kJacSweeps; ++sweep) {
+    if (tid == 0) smax = 0u;
+    __syncthreads();
+    for (int r = 0; r < NP - 1; ++r, ++rounds) {
+      if (tid < half) {
+        int p, q;
+        if (tid == 0) {
+          p = r;
+          q = NP - 1;
+        } else {
+          p = r + tid;
+          if (p >= NP - 1) p -= NP - 1;
+          q = r - tid;
+          if (q < 0) q += NP - 1;
+        }
+        float c = 1.f, s = 0.f;
+        if (p < n && q < n) {
+          float* e = A + min(p, q) * ld + max(p, q);
+          const float apq = *e, aa = fabsf(apq);
+          if (aa > skip) {
+            atomicMax(&smax, __float_as_uint(aa));
+            const float app = A[p * ld + p], aqq = A[q * ld + q];
+            const float theta = (aqq - app) / (2.f * apq), at = fabsf(theta);
+            const float t = at > big_theta<float>() ? 0.5f / theta
+                                                    : (theta < 0 ? -1.f : 1.f) / (at + sqrtf(theta * theta + 1.f));
+            c = 1.f / sqrtf(t * t + 1.f);
+            s = t * c;
+            // the 2 x 2 block itself (rows [[c, -s], [s, c]], columns its transpose)
+            const float y00 = c * app - s * apq, y01 = c * apq - s * aqq;
+            const float y10 = s * app + c * apq, y11 = s * apq + c * aqq;
+            A[p * ld + p] = c * y00 - s * y01;
+            A[q * ld + q] = s * y10 + c * y11;
+            *e = 0.f;
+          }
+        }
+        cs[tid] = make_float2(c, s);
+        rot[(size_t)rounds * kJacHalf + tid] = make_float2(c, s);
+      }
+      __syncthreads();
+      // blocks (i, j), i < j: rows p_i, q_i against columns p_j, q_j.  Warps take the
+      // rows back and forth (their lengths shrink), lanes the columns.
+      for (int b = warp, g = 0; g * nw < half; ++g, b = (g & 1) ? g * nw + nw - 1 - warp : g * nw + warp) {
+        if (b >= half) continue;
+        const float ci = cs[b].x, si = cs[b].y;
+        int pi = r + b, qi = r - b;
+        if (b == 0) { pi = r; qi = NP - 1; }
+        else { if (pi >= NP - 1) pi -= NP - 1; if (qi < 0) qi += NP - 1; }
+        for (int j = b + 1 + lane; j < half; j += 32) {
+          const float2 w = cs[j];
+          const float cj = w.x, sj = w.y;
+          if (si == 0.f && sj == 0.f) continue;
+          int pj = r + j, qj = r - j;
+          if (pj >= NP - 1) pj -= NP - 1;
+          if (qj < 0) qj += NP - 1;
+          float* e00 = A + min(pi, pj) * ld + max(pi, pj);
+          float* e01 = A + min(pi, qj) * ld + max(pi, qj);
+          float* e10 = A + min(qi, pj) * ld + max(qi, pj);
+          float* e11 = A + min(qi, qj) * ld + max(qi, qj);
+          const float x00 = *e00, x01 = *e01, x10 = *e10, x11 = *e11;
+          const float y00 = ci * x00 - si * x10, y01 = ci * x01 - si * x11;
+          const float y10 = si * x00 + ci * x10, y11 = si * x01 + ci * x11;
+          *e00 = cj * y00 - sj * y01;
+          *e01 = sj * y00 + cj * y01;
+          *e10 = cj * y10 - sj * y11;
+          *e11 = sj * y10 + cj * y11;
+        }
+      }
+      __syncthreads();
+    }
+    const float m = __uint_as_float(smax);
+    __syncthreads();
+    if (m <= stop) break;
+  }
+  if (tid == 0) info[0] = rounds;
+  for (int t = tid; t < n; t += blockDim.x) {
+    const int r = diag_rank(A, ld, n, t);
     lam32[r] = A[t * ld + t];
-    for (int q = 0; q < n; ++q) vec32[(long long)r * n + q] = Q[q * ld + t];
+    info[1 + t] = r;
+  }
+}
+
+// eig32, part 2: rows of Q <- I G_1 G_2 ... , one warp per row.  The row stays in
+// registers, pair i of a round in lane i % 32: players walk one seat per round
+// (round-robin), so a round is one rotation per pair and a shift of seats.  The
+// rotations come through shared memory, kJacChunk rounds at a time, the next
+// ones loading meanwhile (read per round from L2 they set the pace: 400 us for
+// n = 160).
+constexpr int kJacChunk = 32, kJacRows = 4;
+template <int G>   // pairs per lane
+__global__ void __launch_bounds__(32 * kJacRows) k_jacobi_q(int n, const float2* __restrict__ rot,
+                                                            const int* __restrict__ info, float* __restrict__ vec32) {
+  __shared__ __align__(16) float2 buf[2][kJacChunk * G * 32];
+  const int row = blockIdx.x * kJacRows + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int NP = (n + 1) & ~1, half = NP / 2;
+  const int rounds = info[0];
+  // seat i holds players (top) i and (bottom) NP - 1 - i, seat 0: 0 and NP - 1
+  float top[G], bot[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int i = g * 32 + lane;
+    top[g] = i < half && i == row ? 1.f : 0.f;
+    bot[g] = i < half && NP - 1 - i == row ? 1.f : 0.f;
+  }
+  const int last = half - 1;
+  auto load = [&](int r0, int b) {   // rotations of rounds r0 .. r0 + kJacChunk - 1
+    const int nr = min(kJacChunk, rounds - r0);
+    for (int e = threadIdx.x; e < nr * half; e += 32 * kJacRows) {
+      const int r = e / half, i = e - r * half;
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(&buf[b][r * (G * 32) + i]);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(rot + (size_t)(r0 + r) * kJacHalf + i)
+                   : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (rounds > 0) load(0, 0);
+  for (int r0 = 0, b = 0; r0 < rounds; r0 += kJacChunk, b ^= 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();   // the chunk is here, and the other buffer has been read
+    if (r0 + kJacChunk < rounds) load(r0 + kJacChunk, b ^ 1);
+    const int nr = min(kJacChunk, rounds - r0);
+    for (int r = 0; r < nr; ++r) {
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const float2 w = buf[b][r * (G * 32) + g * 32 + lane];   // (seats beyond half hold anything: not used)
+        const float x = top[g], z = bot[g];
+        if (g * 32 + lane < half) {
+          top[g] = w.x * x - w.y * z;
+          bot[g] = w.y * x + w.x * z;
+        }
+      }
+      // next round: top_i <- top_(i+1), top_last <- bot_last, bot_1 <- top_0,
+      // bot_i <- bot_(i-1) (i >= 2), bot_0 stays
+      float nt[G], nbo[G];
+      const float t0 = __shfl_sync(0xffffffffu, top[0], 0);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const float dn = __shfl_sync(0xffffffffu, top[g], (lane + 1) & 31);
+        const float first = g + 1 < G ? __shfl_sync(0xffffffffu, top[g + 1 < G ? g + 1 : g], 0) : 0.f;
+        nt[g] = lane == 31 ? first : dn;
+        const float up = __shfl_sync(0xffffffffu, bot[g], (lane + 31) & 31);
+        const float prev = g > 0 ? __shfl_sync(0xffffffffu, bot[g > 0 ? g - 1 : 0], 31) : 0.f;
+        nbo[g] = lane == 0 ? prev : up;
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const int i = g * 32 + lane;
+        if (half > 1) {
+          top[g] = i == last ? bot[g] : nt[g];
+          if (i == 1) bot[g] = t0;
+          else if (i > 1) bot[g] = nbo[g];
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (row >= n) return;
+  // whole sweeps: every player is back in its seat
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int i = g * 32 + lane;
+    if (i < half) {
+      if (i < n) vec32[(long long)info[1 + i] * n + row] = top[g];
+      if (NP - 1 - i < n) vec32[(long long)info[1 + NP - 1 - i] * n + row] = bot[g];
+    }
   }
 }
 
@@ -412,64 +604,88 @@ __global__ void __launch_bounds__(1024) k_cholesky(S* __restrict__ H, int ldh, i
 
 // Bordered Cholesky: rows < n0 of L already hold the factor of the leading
 // block; rows n0..n-1 hold the new rows of the matrix (all n columns).  Each new
-// row is first solved against the old factor by its own warp (forward
-// substitution, no block barriers), then the new diagonal block is factored
-// column by column.  Entries above the diagonal in the first n columns are zeroed.
+// row z solves L z = a against the old factor in its own warp (blocks of 32
+// unknowns in registers, a shuffle per unknown), then the new diagonal block less
+// z z^T is factored column by column.  Entries above the diagonal in the first n
+// columns are zeroed.  (A shuffle reduction and a division per element before: 19.5
+// -> 10.5 us in FP32 inner solves, n up to 160 with 20 new rows.)
 template <typename S>
 __global__ void __launch_bounds__(1024) k_chol_border(S* __restrict__ Lg, int ld, int n0, int n,
                                                       int* __restrict__ info) {
   extern __shared__ __align__(16) unsigned char cb_raw[];
-  S* L = reinterpret_cast<S*>(cb_raw);   // [n][n] working copy (row stride n)
+  S* L = reinterpret_cast<S*>(cb_raw);   // [n][ls] working copy (odd stride)
+  const int ls = n | 1;
+  __shared__ S dinv[kSmallMax];          // 1 / L[j][j]
   __shared__ int bad;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
     const int r = idx / n, c = idx - r * n;
-    L[idx] = Lg[(long long)r * ld + c];
+    L[r * ls + c] = Lg[(long long)r * ld + c];
   }
   if (threadIdx.x == 0) bad = 0;
   __syncthreads();
+  if (threadIdx.x < n0) dinv[threadIdx.x] = fast_rcp(L[threadIdx.x * ls + threadIdx.x]);
+  __syncthreads();
   // phase 1: L[i][j], j < n0, for every new row i
   for (int i = n0 + warp; i < n; i += nw) {
-    S* Li = L + i * n;
-    for (int j = 0; j < n0; ++j) {
-      const S* Lj = L + j * n;
-      S acc = S(0);
-      for (int q = lane; q < j; q += 32) acc += Li[q] * Lj[q];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      const S v = (Li[j] - acc) / Lj[j];
-      __syncwarp();
-      if (lane == 0) Li[j] = v;
+    S* Li = L + i * ls;
+    for (int j0 = 0; j0 < n0; j0 += 32) {
+      const int j = j0 + lane, jn = min(32, n0 - j0);
+      const S* Lj = L + min(j, n0 - 1) * ls;
+      S v = S(0), v1 = S(0);
+      int q = 0;
+      for (; q + 1 < j0; q += 2) {
+        v -= Lj[q] * Li[q];
+        v1 -= Lj[q + 1] * Li[q + 1];
+      }
+      if (q < j0) v -= Lj[q] * Li[q];
+      v = (lane < jn ? Li[j] : S(0)) + (v + v1);
+      const S di = lane < jn ? dinv[j] : S(0);
+      for (int t = 0; t < jn; ++t) {
+        const S x = __shfl_sync(0xffffffffu, v * di, t);
+        if (lane == t) v = x;
+        else if (lane > t) v -= Lj[j0 + t] * x;
+      }
+      if (lane < jn) Li[j] = v;
       __syncwarp();
     }
   }
   __syncthreads();
-  // phase 2: the new diagonal block, column by column
-  for (int j = n0; j < n; ++j) {
-    S* Lj = L + j * n;
-    if (warp == 0) {
-      S acc = S(0);
-      for (int q = lane; q < j; q += 32) acc += Lj[q] * Lj[q];
+  // the new diagonal block less the products of the new rows, one warp per element
+  const int m = n - n0;
+  for (int e = warp; e < m * (m + 1) / 2; e += nw) {
+    int a = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);   // e = a (a + 1) / 2 + b, b <= a
+    while (a * (a + 1) / 2 > e) --a;
+    while ((a + 1) * (a + 2) / 2 <= e) ++a;
+    const int b = e - a * (a + 1) / 2;
+    const S *La = L + (n0 + a) * ls, *Lb = L + (n0 + b) * ls;
+    S acc = S(0);
+    for (int q = lane; q < n0; q += 32) acc += La[q] * Lb[q];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      const S d = Lj[j] - acc;
-      __syncwarp();
-      if (lane == 0) {
-        if (!(d > S(0)) || !isfinite(d)) bad = j + 1;
-        else Lj[j] = sqrt(d);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) L[(n0 + a) * ls + n0 + b] -= acc;
+  }
+  __syncthreads();
+  // phase 2: its factor, column by column
+  for (int j = n0; j < n; ++j) {
+    if (threadIdx.x == 0) {
+      const S d = L[j * ls + j];
+      if (!(d > S(0)) || !isfinite(d)) {
+        bad = j + 1;
+      } else {
+        const S r = sqrt(d);
+        L[j * ls + j] = r;
+        dinv[j] = fast_rcp(r);
       }
     }
     __syncthreads();
     if (bad) break;
-    for (int i = j + 1 + warp; i < n; i += nw) {
-      S* Li = L + i * n;
-      S acc = S(0);
-      for (int q = lane; q < j; q += 32) acc += Li[q] * Lj[q];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      const S v = (Li[j] - acc) / Lj[j];
-      __syncwarp();
-      if (lane == 0) Li[j] = v;
+    const int w = n - j - 1;
+    for (int t = threadIdx.x; t < w; t += blockDim.x) L[(j + 1 + t) * ls + j] *= dinv[j];
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < w * w; idx += blockDim.x) {
+      const int r = j + 1 + idx / w, c = j + 1 + idx % w;
+      if (c <= r) L[r * ls + c] -= L[r * ls + j] * L[c * ls + j];
     }
     __syncthreads();
   }
@@ -478,7 +694,7 @@ __global__ void __launch_bounds__(1024) k_chol_border(S* __restrict__ Lg, int ld
   // write back, zero above the diagonal
   for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
     const int r = idx / n, c = idx - r * n;
-    Lg[(long long)r * ld + c] = c <= r ? L[idx] : S(0);
+    Lg[(long long)r * ld + c] = c <= r ? L[r * ls + c] : S(0);
   }
 }
 
@@ -527,40 +743,43 @@ __device__ void chol_drop_cta(const double* __restrict__ G, int nc, const double
   __syncthreads();
   // right-looking: after step j the trailing block holds the Gram matrix of the
   // candidates with the kept ones among 0..j projected out
+  // (the diagonal ends up holding 1 / R[j][j], zero for a dropped candidate)
   for (int j = 0; j < nc; ++j) {
     if (tid == 0) {
       double d = R[j * ld + j];
       const double n0 = norm0sq ? norm0sq[j] : 1.0;
       kj = (isfinite(d) && d > drop2 * n0 && d > 0.0) ? 1 : 0;
-      dj = kj ? sqrt(d) : 0.0;
+      dj = kj ? fast_rsqrt(d) : 0.0;
       keep[j] = kj;
     }
     __syncthreads();
+    for (int m = j + tid; m < nc; m += blockDim.x) R[j * ld + m] = (m == j) ? dj : (kj ? R[j * ld + m] * dj : 0.0);
+    __syncthreads();
     if (kj) {
-      for (int m = j + tid; m < nc; m += blockDim.x) R[j * ld + m] = (m == j) ? dj : R[j * ld + m] / dj;
-      __syncthreads();
       const int m = nc - j - 1;
       for (int idx = tid; idx < m * m; idx += blockDim.x) {
         int a = j + 1 + idx / m, b = j + 1 + idx % m;
-        R[a * ld + b] -= R[j * ld + a] * R[j * ld + b];
-      }
-    } else {
-      for (int m = j + tid; m < nc; m += blockDim.x) R[j * ld + m] = 0.0;
-    }
-    __syncthreads();
-  }
-  // T = R^-T restricted to kept rows: T[j] = (e_j - sum_{l<j} R[l][j] T[l]) / R[j][j]
-  for (int j = 0; j < nc; ++j) {
-    if (keep[j]) {
-      double inv = 1.0 / R[j * ld + j];
-      for (int c = tid; c <= j; c += blockDim.x) {
-        double acc = (c == j) ? 1.0 : 0.0;
-        for (int l = c; l < j; ++l) acc -= R[l * ld + j] * Ti[l * ld + c];
-        Ti[j * ld + c] = acc * inv;
+        if (b >= a) R[a * ld + b] -= R[j * ld + a] * R[j * ld + b];
       }
     }
     __syncthreads();
   }
+  // T = R^-T restricted to kept rows: T[j] = (e_j - sum_{l<j} R[l][j] T[l]) / R[j][j];
+  // a column depends on itself only
+  for (int c = tid; c < nc; c += blockDim.x)
+    for (int j = c; j < nc; ++j) {
+      const double inv = R[j * ld + j];
+      if (inv == 0.0) continue;   // dropped: its row of T stays zero
+      double a0 = (c == j) ? 1.0 : 0.0, a1 = 0.0;
+      int l = c;
+      for (; l + 1 < j; l += 2) {
+        a0 = fma(-R[l * ld + j], Ti[l * ld + c], a0);
+        a1 = fma(-R[(l + 1) * ld + j], Ti[(l + 1) * ld + c], a1);
+      }
+      if (l < j) a0 = fma(-R[l * ld + j], Ti[l * ld + c], a0);
+      Ti[j * ld + c] = (a0 + a1) * inv;
+    }
+  __syncthreads();
   for (int idx = tid; idx < nc * nc; idx += blockDim.x) {
     int a = idx / nc, b = idx - a * nc;
     T[idx] = Ti[a * ld + b];
@@ -576,68 +795,120 @@ __global__ void __launch_bounds__(1024) k_chol_drop(const double* __restrict__ G
   chol_drop_cta(G, nc, norm0sq, drop2, T, keep, smd, kj, dj);
 }
 
+// |v| as an ordered integer without its low byte, row i (< 256) there instead: the
+// maximum over rows is a pivot within 2^-12 of the largest element.
+__device__ __forceinline__ unsigned pivot_key(float v, int i) {
+  return (__float_as_uint(fabsf(v)) & ~255u) | (unsigned)(255 - i);
+}
+__device__ __forceinline__ unsigned pivot_key(double v, int i) {
+  return ((unsigned)__double2hiint(fabs(v)) & ~255u) | (unsigned)(255 - i);
+}
+
 // Gaussian elimination with partial pivoting on the augmented matrix [M | b]
 // held in shared memory (n rows, row stride ld >= n + 1, compute type T), then
 // back substitution; the solution replaces column n (in the original row order).
-// Rows are not moved: perm[] (shared, >= n ints) records the pivot order, so an
-// elimination step is one pivot search (warp 0) and one update pass.  Called by
-// all threads of the CTA.
+// Rows are not moved: ord[] (shared, >= n ints) records the pivot rows; the
+// update of a step collects the next pivot as a maximum of keys, so that a step
+// is one barrier and one pass over the trailing rows.  Called by all threads of
+// the CTA.  (With a pivot search by one warp and a second barrier a step took 1300
+// cycles for n = 100 in FP32, with a division per warp 2600 in FP64; mean launch of
+// the FP64 inner solves, n up to 60: 120 -> 68 us.)
 template <typename T>
-__device__ void lu_solve_smem(T* A, int ld, int n, int* perm, T* y) {
+__device__ void lu_solve_smem(T* A, int ld, int n, int* ord, T* y) {
+  __shared__ T pinv[kSmallMax];          // reciprocal pivots
+  __shared__ unsigned key[3];            // pivot keys of steps k, k + 1, k + 2
+  __shared__ int act[kSmallMax];         // FP64: rows not yet pivots
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  for (int i = tid; i < n; i += blockDim.x) perm[i] = i;
+  if (tid < 3) key[tid] = 0u;
+  for (int i = tid; i < n; i += blockDim.x) act[i] = i;
   __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    if (warp == 0) {   // pivot: argmax |A[perm[i]][k]|, i >= k
-      T best = T(-1);
-      int bi = k;
-      for (int i = k + lane; i < n; i += 32) {
-        T v = A[perm[i] * ld + k];
-        v = v < T(0) ? -v : v;
-        if (v > best) { best = v; bi = i; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        T ob = __shfl_xor_sync(0xffffffffu, best, o);
-        int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (lane == 0 && bi != k) {
-        const int t = perm[k];
-        perm[k] = perm[bi];
-        perm[bi] = t;
-      }
-    }
-    __syncthreads();
-    const int pk = perm[k];
-    const T* prow = A + pk * ld;
-    T piv = prow[k];
-    if (piv == T(0)) piv = T(1e-30);
-    const T inv = T(1) / piv;
-    for (int i = k + 1 + warp; i < n; i += nw) {
-      T* row = A + perm[i] * ld;
-      const T l = row[k] * inv;
-      for (int j = k + 1 + lane; j <= n; j += 32) row[j] -= l * prow[j];
-    }
-    __syncthreads();
-  }
-  // back substitution by one warp: y_k = (b_k - sum_{j>k} U_kj y_j) / U_kk
-  if (warp == 0) {
-    for (int k = n - 1; k >= 0; --k) {
-      const T* row = A + perm[k] * ld;
-      T piv = row[k];
+  if (tid < n) atomicMax(&key[0], pivot_key(A[tid * ld], tid));
+  if constexpr (sizeof(T) == 4) {
+    unsigned used = 0u;                  // bit t: row warp + t nw has been a pivot
+    for (int k = 0; k < n; ++k) {
+      __syncthreads();
+      const int bi = 255 - (int)(key[k % 3] & 255u);
+      const T* prow = A + bi * ld;
+      T piv = prow[k];
       if (piv == T(0)) piv = T(1e-30);
-      const T yk = row[n] / piv;
-      __syncwarp();
-      for (int i = lane; i < k; i += 32) {
-        T* ri = A + perm[i] * ld;
-        ri[n] -= ri[k] * yk;
+      const T inv = fast_rcp(piv);
+      if (tid == 0) {
+        key[(k + 2) % 3] = 0u;
+        ord[k] = bi;
+        pinv[k] = inv;
       }
-      if (lane == 0) y[k] = yk;
-      __syncwarp();
+#pragma unroll 2
+      for (int t = 0; warp + t * nw < n; ++t) {
+        const int i = warp + t * nw;
+        if (i == bi) used |= 1u << t;
+        if ((used >> t) & 1u) continue;
+        T* row = A + i * ld;
+        const T l = row[k] * inv;
+        for (int j = k + 1 + lane; j <= n; j += 32) {
+          const T v = row[j] - l * prow[j];
+          row[j] = v;
+          if (j == k + 1 && j < n) atomicMax(&key[(k + 1) % 3], pivot_key(v, i));
+        }
+      }
+    }
+  } else {
+    // the FP64 unit takes as long for one lane as for 32: multipliers first, then
+    // the trailing elements dealt to the lanes row after row
+    for (int k = 0; k < n; ++k) {
+      __syncthreads();
+      const int bi = 255 - (int)(key[k % 3] & 255u);
+      const T* prow = A + bi * ld;
+      const int m = n - k - 1, w = m + 1;
+      if (warp == 0) {
+        T piv = prow[k];
+        if (piv == T(0)) piv = T(1e-30);
+        const T inv = fast_rcp(piv);
+        // remove the pivot row from the list (the last one takes its place)
+        for (int t = lane; t <= m; t += 32)
+          if (act[t] == bi) act[t] = act[m];
+        if (lane == 0) {
+          key[(k + 2) % 3] = 0u;
+          ord[k] = bi;
+          pinv[k] = inv;
+        }
+        __syncwarp();
+        for (int t = lane; t < m; t += 32) A[act[t] * ld + k] *= inv;
+      }
+      __syncthreads();
+      for (int idx = tid; idx < m * w; idx += blockDim.x) {
+        const int t = idx / w, j = k + 1 + idx - t * w, i = act[t];
+        T* row = A + i * ld;
+        const T v = row[j] - row[k] * prow[j];
+        row[j] = v;
+        if (j == k + 1 && j < n) atomicMax(&key[(k + 1) % 3], pivot_key(v, i));
+      }
     }
   }
   __syncthreads();
+  // back substitution in blocks of 32 unknowns (see cta_trsv)
+  for (int j0 = (n - 1) / 32 * 32; j0 >= 0; j0 -= 32) {
+    const int jn = min(32, n - j0);
+    if (warp == 0) {
+      const T* row = A + (lane < jn ? ord[j0 + lane] : 0) * ld;
+      T v = lane < jn ? row[n] : T(0);
+      const T di = lane < jn ? pinv[j0 + lane] : T(0);
+      for (int j = jn - 1; j >= 0; --j) {
+        const T x = __shfl_sync(0xffffffffu, v * di, j);
+        if (lane == j) v = x;
+        else if (lane < j) v -= row[j0 + j] * x;
+      }
+      if (lane < jn) y[j0 + lane] = v;
+    }
+    __syncthreads();
+    for (int r = tid; r < j0; r += blockDim.x) {
+      T* row = A + ord[r] * ld;
+      T acc = row[n];
+#pragma unroll 4
+      for (int j = 0; j < jn; ++j) acc -= row[j0 + j] * y[j0 + j];
+      row[n] = acc;
+    }
+    __syncthreads();
+  }
   for (int i = tid; i < n; i += blockDim.x) A[i * ld + n] = y[i];
   __syncthreads();
 }
@@ -645,7 +916,7 @@ __device__ void lu_solve_smem(T* A, int ld, int n, int* perm, T* y) {
 // One CTA per right-hand side r: Gaussian elimination with partial pivoting on
 // [(H - sigma_r I) | b_r] in shared memory (compute type T), then back substitution.
 template <typename T>
-__global__ void __launch_bounds__(512) k_lu_shift(const T* __restrict__ H, int ldh, int n,
+__global__ void __launch_bounds__(1024) k_lu_shift(const T* __restrict__ H, int ldh, int n,
                                                   const double* __restrict__ sig,
                                                   const T* __restrict__ B, T* __restrict__ Y) {
   extern __shared__ __align__(16) unsigned char lu_raw[];
@@ -668,27 +939,38 @@ __global__ void __launch_bounds__(512) k_lu_shift(const T* __restrict__ H, int l
   for (int i = tid; i < n; i += nth) Y[(long long)r * n + i] = A[i * ld + n];
 }
 
-// Triangular solve by one warp on a vector b[n] in shared memory with the lower
-// factor L (global, row stride ldl): trans = 0: L x = b; 1: L^T x = b.
+// Triangular solve by the CTA on a vector b[n] in shared memory with the lower
+// factor L (row stride ldl): trans = 0: L x = b; 1: L^T x = b; dinv: 1 / L[j][j].
+// Blocks of 32 unknowns: warp 0 solves one in registers (a shuffle per unknown),
+// then all threads subtract its columns from the rest.
 template <typename T>
-__device__ void warp_trsv(const T* __restrict__ L, int ldl, int n, T* b, int trans) {
-  const int lane = threadIdx.x & 31;
-  if (!trans) {
-    for (int j = 0; j < n; ++j) {
-      const T xj = b[j] / L[(long long)j * ldl + j];
-      __syncwarp();
-      if (lane == 0) b[j] = xj;
-      for (int r = j + 1 + lane; r < n; r += 32) b[r] -= L[(long long)r * ldl + j] * xj;
-      __syncwarp();
+__device__ void cta_trsv(const T* __restrict__ L, int ldl, int n, const T* dinv, T* b, int trans) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int nb = (n + 31) / 32;
+  for (int q = 0; q < nb; ++q) {
+    const int j0 = (trans ? nb - 1 - q : q) * 32, jn = min(32, n - j0);
+    if (tid < 32) {
+      T v = lane < jn ? b[j0 + lane] : T(0);
+      const T di = lane < jn ? dinv[j0 + lane] : T(0);
+      for (int t = 0; t < jn; ++t) {
+        const int j = trans ? jn - 1 - t : t;
+        const T x = __shfl_sync(0xffffffffu, v * di, j);
+        if (lane == j) v = x;
+        else if (lane < jn && (trans ? lane < j : lane > j))
+          v -= (trans ? L[(long long)(j0 + j) * ldl + j0 + lane] : L[(long long)(j0 + lane) * ldl + j0 + j]) * x;
+      }
+      if (lane < jn) b[j0 + lane] = v;
     }
-  } else {
-    for (int j = n - 1; j >= 0; --j) {
-      const T xj = b[j] / L[(long long)j * ldl + j];
-      __syncwarp();
-      if (lane == 0) b[j] = xj;
-      for (int r = lane; r < j; r += 32) b[r] -= L[(long long)j * ldl + r] * xj;
-      __syncwarp();
+    __syncthreads();
+    const int r0 = trans ? 0 : j0 + jn, r1 = trans ? j0 : n;
+    for (int r = r0 + tid; r < r1; r += blockDim.x) {
+      T acc = b[r];
+#pragma unroll 4
+      for (int j = 0; j < jn; ++j)
+        acc -= (trans ? L[(long long)(j0 + j) * ldl + r] : L[(long long)r * ldl + j0 + j]) * b[j0 + j];
+      b[r] = acc;
     }
+    __syncthreads();
   }
 }
 
@@ -697,7 +979,7 @@ __device__ void warp_trsv(const T* __restrict__ L, int ldl, int n, T* b, int tra
 //   z = L^-1 h-,  rhs = L^T h+ + s z,  (H - s^2) u~ = rhs,  u = L u~,
 //   w = L^-T (z + s u~)          (h- absent: z = 0)
 template <typename T>
-__global__ void __launch_bounds__(512) k_paired_small(const T* __restrict__ Lg, const T* __restrict__ H,
+__global__ void __launch_bounds__(1024) k_paired_small(const T* __restrict__ Lg, const T* __restrict__ H,
                                                       int ld, int n, const T* __restrict__ hp,
                                                       const T* __restrict__ hm, const double* __restrict__ sh,
                                                       T* __restrict__ uc, T* __restrict__ wc) {
@@ -719,7 +1001,7 @@ __global__ void __launch_bounds__(512) k_paired_small(const T* __restrict__ Lg, 
   const T* L = kLs ? hv + n : Lg;
   const int ll = kLs ? n + 1 : ld;
   __shared__ int perm[kSmallMax];
-  __shared__ T yv[kSmallMax];
+  __shared__ T yv[kSmallMax], dinv[kSmallMax];
   const int r = blockIdx.x;
   const T s = (T)sh[r];
   const T s2 = (T)(sh[r] * sh[r]);
@@ -733,8 +1015,9 @@ __global__ void __launch_bounds__(512) k_paired_small(const T* __restrict__ Lg, 
     A[i * la + j] = T(0.5) * (H[(long long)i * ld + j] + H[(long long)j * ld + i]) - (i == j ? s2 : T(0));
   }
   __syncthreads();
-  if (hm && tid < 32) warp_trsv<T>(L, ll, n, z, 0);
+  for (int i = tid; i < n; i += nth) dinv[i] = fast_rcp(L[(long long)i * ll + i]);
   __syncthreads();
+  if (hm) cta_trsv<T>(L, ll, n, dinv, z, 0);
   for (int i = tid; i < n; i += nth) {   // rhs_i = sum_q h+_q L[q][i] + s z_i
     T acc = s * z[i];
     for (int q = i; q < n; ++q) acc += hv[q] * L[(long long)q * ll + i];
@@ -750,8 +1033,7 @@ __global__ void __launch_bounds__(512) k_paired_small(const T* __restrict__ Lg, 
     hv[i] = z[i] + s * A[i * la + n];
   }
   __syncthreads();
-  if (tid < 32) warp_trsv<T>(L, ll, n, hv, 1);
-  __syncthreads();
+  cta_trsv<T>(L, ll, n, dinv, hv, 1);
   for (int i = tid; i < n; i += nth) wc[(long long)r * n + i] = hv[i];
 }
 
@@ -831,11 +1113,18 @@ void set_smem(const void* f, size_t bytes) {
 
 void eig32(const double* H, int ldh, int n, float* lam32, float* vec32, cudaStream_t s) {
   TD_REQUIRE(n >= 1 && n <= kSmallMax, TDDFT_ERR_ARG, "eig32: size out of range");
-  const int NP = (n + 1) & ~1;
-  size_t smem = (size_t)2 * NP * (NP + 1) * sizeof(float);
-  set_smem((const void*)k_eig32, smem);
-  k_eig32<<<1, 1024, smem, s>>>(H, ldh, n, lam32, vec32);
-  count_launch();
+  const int NP = (n + 1) & ~1, half = NP / 2;
+  const size_t smem = (size_t)NP * (NP + 1) * sizeof(float);
+  set_smem((const void*)k_jacobi_a, smem);
+  DevBuf work(kJacBytes, s);
+  float2* rot = work.as<float2>();
+  int* info = reinterpret_cast<int*>(rot + kJacRounds * kJacHalf);
+  k_jacobi_a<<<1, 1024, smem, s>>>(H, ldh, n, lam32, rot, info);
+  const int grid = (n + kJacRows - 1) / kJacRows;
+  if (half <= 32) k_jacobi_q<1><<<grid, 32 * kJacRows, 0, s>>>(n, rot, info, vec32);
+  else if (half <= 64) k_jacobi_q<2><<<grid, 32 * kJacRows, 0, s>>>(n, rot, info, vec32);
+  else k_jacobi_q<3><<<grid, 32 * kJacRows, 0, s>>>(n, rot, info, vec32);
+  count_launch(2);
   TD_LAUNCH_CHECK();
 }
 
@@ -871,7 +1160,7 @@ void lu_shift_solve(const S* H, int ldh, int n, const double* sigma, int nr, con
   TD_REQUIRE(n >= 1 && n <= kSmallMax, TDDFT_ERR_ARG, "lu_shift_solve: size out of range");
   size_t smem = (size_t)n * (n + 2) * sizeof(S);
   set_smem((const void*)k_lu_shift<S>, smem);
-  k_lu_shift<S><<<nr, 512, smem, s>>>(H, ldh, n, sigma, B, Y);
+  k_lu_shift<S><<<nr, sizeof(S) == 4 ? 1024 : 512, smem, s>>>(H, ldh, n, sigma, B, Y);
   count_launch();
   TD_LAUNCH_CHECK();
 }
@@ -887,7 +1176,7 @@ void paired_small_solve(const S* L, const S* H, int ld, int n, const S* hp, cons
   TD_REQUIRE(n >= 1 && n <= kSmallMax, TDDFT_ERR_ARG, "paired_small_solve: size out of range");
   size_t smem = ((size_t)n * (n + 2) + 2 * (size_t)n + (sizeof(S) == 4 ? (size_t)n * (n + 1) : 0)) * sizeof(S);
   set_smem((const void*)k_paired_small<S>, smem);
-  k_paired_small<S><<<nr, 512, smem, s>>>(L, H, ld, n, hp, hm, sh, uc, wc);
+  k_paired_small<S><<<nr, sizeof(S) == 4 ? 1024 : 512, smem, s>>>(L, H, ld, n, hp, hm, sh, uc, wc);
   count_launch();
   TD_LAUNCH_CHECK();
 }
@@ -910,7 +1199,7 @@ template void cholesky<float>(float*, int, int, int*, cudaStream_t);
 template <typename S>
 void cholesky_border(S* L, int ld, int n0, int n, int* info, cudaStream_t s) {
   TD_REQUIRE(n >= 1 && n <= kSmallMax && n0 >= 0 && n0 <= n, TDDFT_ERR_ARG, "cholesky_border: bad sizes");
-  const size_t smem = (size_t)n * n * sizeof(S);
+  const size_t smem = (size_t)n * (n | 1) * sizeof(S);
   ensure_smem((const void*)k_chol_border<S>, smem);
   k_chol_border<S><<<1, 1024, smem, s>>>(L, ld, n0, n, info);
   count_launch();
