@@ -265,7 +265,7 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       // streaming the FP16 hi+lo copy of s_ov L_ov transposed once, with t as
       // FP16 parts of s_t t
       DevBuf t((size_t)f.nJ * m * 4, s), sct(2 * 4, s), scr(8, s), fac(4, s);
-      sk_gram(f.Jov, f.dt, ov, f.nJ, Xw, tw, ov, m, ov, t.p, tw, m, 1.0, 0.0, s);
+      tall_gram(f.Jov, f.dt, f.nJ, static_cast<const float*>(Xw), m, ov, t.as<float>(), s);
       tc_f16_tensor_scale(t.as<float>(), f.nJ, m, sct.as<float>(), scr.as<unsigned>(), s);
       const int nJp = tc_pad(f.nJ);
       DevBuf th((size_t)m * nJp * 2, s), tl((size_t)m * nJp * 2, s);
@@ -275,8 +275,13 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
                   fac.as<float>(), d.tc_err, s, nullptr, 0.0, 0.0, kCoulombKb);
     } else {
       DevBuf t((size_t)f.nJ * m * ew, s);
-      sk_gram(f.Jov, f.dt, ov, f.nJ, Xw, tw, ov, m, ov, t.p, tw, m, 1.0, 0.0, s);
-      sk_combo(t.p, tw, 1, m, m, f.nJ, f.Jov, f.dt, ov, ov, Jb.p, tw, ov, 1.0, 0.0, s);
+      if (f64) {
+        sk_gram(f.Jov, f.dt, ov, f.nJ, Xw, tw, ov, m, ov, t.p, tw, m, 1.0, 0.0, s);
+        sk_combo(t.p, tw, 1, m, m, f.nJ, f.Jov, f.dt, ov, ov, Jb.p, tw, ov, 1.0, 0.0, s);
+      } else {
+        tall_gram(f.Jov, f.dt, f.nJ, static_cast<const float*>(Xw), m, ov, t.as<float>(), s);
+        tall_combo(t.as<float>(), m, f.nJ, f.Jov, f.dt, ov, Jb.as<float>(), s);
+      }
     }
     have_J = true;
   }

@@ -391,6 +391,265 @@ void combo_typed(const void* coef, long long scm, long long sck, int M, int K, c
   TD_LAUNCH_CHECK();
 }
 
+// ---------------------------------------------------------------------------
+// Coulomb contractions of the operator: factor rows (hundreds to thousands, FP32
+// or BF16, row length K in the tens of thousands) against a few trial vectors.
+
+// Two FP32 fused multiply-adds at once.
+__device__ __forceinline__ void fma2(float2& c, float2 a, float2 b) {
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 z, {%0, %1};\n"
+      " fma.rn.f32x2 z, x, y, z;\n mov.b64 {%0, %1}, z;\n}\n"
+      : "+f"(c.x), "+f"(c.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+}
+
+// PB bytes (4, 8 or 16) to shared memory, zero beyond `bytes`
+template <int PB>
+__device__ __forceinline__ void cp_piece(void* dst, const void* src, int bytes) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if constexpr (PB == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(d), "l"(src), "r"(bytes), "n"(PB) : "memory");
+}
+
+// part[chunk][m][n] = sum over the chunk of A[m][k] B[n][k].  Bound by the FP32
+// units for about 16 vectors and more, by reading A below that.  CTA = 128 rows
+// x 4 RN vectors; 16 row groups x 4 vector groups x 4 groups of k, a thread 8
+// rows x RN vectors: 13 16-byte shared-memory loads feed 160 FMAs (RN = 5),
+// accumulated for even and odd k apart (packed FMAs), so a sum runs over at most
+// 1/8 of the chunk (<= 256 terms) before the chunk's eight are added in order.
+// cp.async keeps three stages of 64 k in flight.  n_ov 202,500, 1350 BF16 rows, 20
+// vectors: 992 -> 434 us (25 TFLOP/s); n_ov 24,000, 2000 rows, 20 vectors: 149 -> 83.
+constexpr int kTallRows = 128, kTallK = 64, kTallStages = 3, kTallChunk = 2048;
+template <typename TA> struct TallCfg {
+  static constexpr int LDA = kTallK + (sizeof(TA) == 4 ? 4 : 8);   // elements: rows skewed over the banks
+  static constexpr int LDB = kTallK + 4;
+  static constexpr int A_BYTES = kTallRows * LDA * (int)sizeof(TA);
+  static int stage_bytes(int rn) { return A_BYTES + 4 * rn * LDB * 4; }
+};
+
+__device__ __forceinline__ void quad(const float* p, float2& a, float2& b) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  a = make_float2(q.x, q.y);
+  b = make_float2(q.z, q.w);
+}
+__device__ __forceinline__ void quad(const __nv_bfloat16* p, float2& a, float2& b) {
+  const uint2 q = *reinterpret_cast<const uint2*>(p);
+  a = make_float2(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u));
+  b = make_float2(__uint_as_float(q.y << 16), __uint_as_float(q.y & 0xffff0000u));
+}
+
+// PA, PX: bytes that the rows of A and of the vectors are aligned to.
+template <typename TA, int RN, int PA, int PX>
+__global__ void __launch_bounds__(256)
+k_tall_gram(const TA* __restrict__ A, int M, const float* __restrict__ B, int N, int K, int chunk,
+            float* __restrict__ part) {
+  using C = TallCfg<TA>;
+  constexpr int NT = 4 * RN, EA = PA / (int)sizeof(TA), EX = PX / 4;   // elements per piece
+  constexpr int STAGE = C::A_BYTES + NT * C::LDB * 4;
+  extern __shared__ __align__(16) unsigned char tall_raw[];
+  const int tid = threadIdx.x;
+  const int m0 = blockIdx.x * kTallRows, n0 = blockIdx.z * NT;
+  const int k0 = blockIdx.y * chunk, k1 = min(K, k0 + chunk);
+  const int nst = (k1 - k0 + kTallK - 1) / kTallK;
+  auto load = [&](int st) {
+    if (st < nst) {
+      unsigned char* base = tall_raw + (st % kTallStages) * STAGE;
+      TA* As = reinterpret_cast<TA*>(base);
+      float* Bs = reinterpret_cast<float*>(base + C::A_BYTES);
+      const int kb = k0 + st * kTallK;
+      constexpr int CA = kTallK / EA;                       // pieces per row of A
+      for (int e = tid; e < kTallRows * CA; e += 256) {
+        const int r = e / CA, c = (e % CA) * EA;
+        const int left = min(k1 - kb - c, EA);
+        const bool in = m0 + r < M && left > 0;
+        cp_piece<PA>(As + r * C::LDA + c, in ? A + (long long)(m0 + r) * K + kb + c : A,
+                     in ? left * (int)sizeof(TA) : 0);
+      }
+      for (int e = tid; e < NT * (kTallK / EX); e += 256) {
+        const int r = e / (kTallK / EX), c = (e % (kTallK / EX)) * EX;
+        const int left = min(k1 - kb - c, EX);
+        const bool in = n0 + r < N && left > 0;
+        cp_piece<PX>(Bs + r * C::LDB + c, in ? B + (long long)(n0 + r) * K + kb + c : B, in ? left * 4 : 0);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int kg = tid >> 6, rg = tid & 15, cg = (tid >> 4) & 3;
+  float2 acc[8][RN];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < RN; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  for (int st = 0; st < kTallStages - 1; ++st) load(st);
+  for (int st = 0; st < nst; ++st) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kTallStages - 2) : "memory");
+    __syncthreads();
+    load(st + kTallStages - 1);
+    const unsigned char* base = tall_raw + (st % kTallStages) * STAGE;
+    const TA* As = reinterpret_cast<const TA*>(base) + rg * C::LDA;
+    const float* Bs = reinterpret_cast<const float*>(base + C::A_BYTES) + cg * C::LDB;
+#pragma unroll 2
+    for (int q = kg; q < kTallK / 4; q += 4) {
+      float2 b0[RN], b1[RN];
+#pragma unroll
+      for (int j = 0; j < RN; ++j) quad(Bs + 4 * j * C::LDB + 4 * q, b0[j], b1[j]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float2 a0, a1;
+        quad(As + 16 * i * C::LDA + 4 * q, a0, a1);
+#pragma unroll
+        for (int j = 0; j < RN; ++j) {
+          fma2(acc[i][j], a0, b0[j]);
+          fma2(acc[i][j], a1, b1[j]);
+        }
+      }
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // the four groups of k, added in order through shared memory
+  float* red = reinterpret_cast<float*>(tall_raw);   // [4][128][NT]
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < RN; ++j)
+      red[(kg * kTallRows + rg + 16 * i) * NT + cg + 4 * j] = acc[i][j].x + acc[i][j].y;
+  __syncthreads();
+  float* P = part + (long long)blockIdx.y * M * N;
+  for (int e = tid; e < kTallRows * NT; e += 256) {
+    const int r = e / NT, c = e - r * NT;
+    if (m0 + r >= M || n0 + c >= N) continue;
+    float v = 0.f;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) v += red[g * kTallRows * NT + e];
+    P[(long long)(m0 + r) * N + n0 + c] = v;
+  }
+}
+
+// out[n][c] = sum_P t[P][n] V[P][c] for up to RN vectors in one pass over V: a lane
+// owns four columns, the CTA's eight warps every eighth P (the next eight loads
+// in flight while eight are used), and their sums are added in order.  t is
+// staged as pairs (t, t) for packed FMAs.
+constexpr int kTallKc = 256;
+template <typename TV, int RN>
+__global__ void __launch_bounds__(256)
+k_tall_combo(const float* __restrict__ t, int N, int K, const TV* __restrict__ V, int ncols, float* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char tallc_raw[];
+  float2* cs = reinterpret_cast<float2*>(tallc_raw);      // [kTallKc][RN]
+  float* red = reinterpret_cast<float*>(tallc_raw);       // later: [4][RN][132]
+  const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
+  const int n0 = blockIdx.y * RN;
+  const int c0 = blockIdx.x * 128 + lane * 4;
+  const bool live = c0 < ncols;
+  float2 a0[RN], a1[RN];
+#pragma unroll
+  for (int j = 0; j < RN; ++j) a0[j] = a1[j] = make_float2(0.f, 0.f);
+  constexpr int U = 8;
+  float2 v0[U], v1[U], w0[U], w1[U];
+  auto load = [&](int k0, float2 (&x0)[U], float2 (&x1)[U]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = k0 + g + 8 * u;
+      if (live && k < K) quad(V + (long long)k * ncols + c0, x0[u], x1[u]);
+      else x0[u] = x1[u] = make_float2(0.f, 0.f);
+    }
+  };
+  auto use = [&](int k, const float2 (&x0)[U], const float2 (&x1)[U]) {   // k: row within the staged block
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float2* c = cs + (k + g + 8 * u) * RN;
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {
+        const float2 w = c[j];
+        fma2(a0[j], w, x0[u]);
+        fma2(a1[j], w, x1[u]);
+      }
+    }
+  };
+  load(0, v0, v1);
+  for (int k0 = 0; k0 < K; k0 += kTallKc) {
+    __syncthreads();
+    for (int e = tid; e < kTallKc * RN; e += 256) {
+      const int k = e / RN, j = e - k * RN;
+      const float v = k0 + k < K && n0 + j < N ? t[(long long)(k0 + k) * N + n0 + j] : 0.f;
+      cs[e] = make_float2(v, v);
+    }
+    __syncthreads();
+    for (int k = 0; k < kTallKc && k0 + k < K; k += 128) {
+      load(k0 + k + 64, w0, w1);
+      use(k, v0, v1);
+      load(k0 + k + 128, v0, v1);
+      use(k + 64, w0, w1);
+    }
+  }
+  // sums of the warps g and g + 4 first, then the four in order
+  __syncthreads();
+#pragma unroll
+  for (int pass = 1; pass >= 0; --pass) {
+    if ((g >> 2) == pass) {
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {
+        float* r = red + ((g & 3) * RN + j) * 132 + lane * 4;
+        float4 v = make_float4(a0[j].x, a0[j].y, a1[j].x, a1[j].y);
+        if (pass == 0) {
+          const float4 o = *reinterpret_cast<const float4*>(r);
+          v = make_float4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
+        }
+        *reinterpret_cast<float4*>(r) = v;
+      }
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < RN * 128; e += 256) {
+    const int j = e >> 7, l = e & 127, col = blockIdx.x * 128 + l;
+    if (n0 + j >= N || col >= ncols) continue;
+    float v = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v += red[(q * RN + j) * 132 + l];
+    out[(long long)(n0 + j) * ncols + col] = v;
+  }
+}
+
+template <typename TA, int RN, int PA, int PX>
+void tall_gram_launch(const TA* A, int M, const float* B, int N, int K, int chunk, int S, float* part, cudaStream_t s) {
+  const int nb = (N + 4 * RN - 1) / (4 * RN);
+  const size_t smem = std::max((size_t)kTallStages * TallCfg<TA>::stage_bytes(RN), (size_t)4 * kTallRows * 4 * RN * 4);
+  set_smem_attr((const void*)k_tall_gram<TA, RN, PA, PX>, smem);
+  k_tall_gram<TA, RN, PA, PX><<<dim3((M + kTallRows - 1) / kTallRows, S, nb), 256, smem, s>>>(A, M, B, N, K, chunk, part);
+}
+
+template <typename TA, int PA, int PX>
+void tall_gram_typed(const TA* A, int M, const float* B, int N, int K, float* part, int chunk, int S, cudaStream_t s) {
+  const int rn = N > 32 && N <= 40 ? 5 : (std::min(N, 32) + 3) / 4;
+  if (rn <= 2) tall_gram_launch<TA, 2, PA, PX>(A, M, B, N, K, chunk, S, part, s);
+  else if (rn <= 4) tall_gram_launch<TA, 4, PA, PX>(A, M, B, N, K, chunk, S, part, s);
+  else if (rn == 5) tall_gram_launch<TA, 5, PA, PX>(A, M, B, N, K, chunk, S, part, s);
+  else tall_gram_launch<TA, 8, PA, PX>(A, M, B, N, K, chunk, S, part, s);
+}
+
+template <typename TV, int RN>
+void tall_combo_launch(const float* t, int N, int K, const TV* V, int ncols, float* out, cudaStream_t s) {
+  const size_t smem = std::max((size_t)kTallKc * RN * 8, (size_t)4 * RN * 132 * 4);
+  set_smem_attr((const void*)k_tall_combo<TV, RN>, smem);
+  k_tall_combo<TV, RN><<<dim3((ncols + 127) / 128, (N + RN - 1) / RN), 256, smem, s>>>(t, N, K, V, ncols, out);
+}
+
+template <typename TV>
+void tall_combo_typed(const float* t, int N, int K, const TV* V, int ncols, float* out, cudaStream_t s) {
+  // as few passes over V as 20 vectors each allow, equally filled; more, smaller ones
+  // where that leaves less than two CTAs per SM (V then comes from L2)
+  int passes = (N + 19) / 20;
+  const int cb = (ncols + 127) / 128;
+  while (cb * passes < 304 && N > 8 * passes) ++passes;
+  const int per = (N + passes - 1) / passes;
+  if (per <= 8) tall_combo_launch<TV, 8>(t, N, K, V, ncols, out, s);
+  else if (per <= 12) tall_combo_launch<TV, 12>(t, N, K, V, ncols, out, s);
+  else if (per <= 16) tall_combo_launch<TV, 16>(t, N, K, V, ncols, out, s);
+  else tall_combo_launch<TV, 20>(t, N, K, V, ncols, out, s);
+}
+
 }  // namespace
 
 void sk_gram(const void* A, DType ta, long long lda, int M, const void* B, DType tb, long long ldb, int N,
@@ -426,6 +685,67 @@ void sk_combo(const void* coef, DType tcoef, long long scm, long long sck, int M
   } else {
     throw Error(TDDFT_ERR_ARG, "sk_combo: unsupported operand types");
   }
+}
+
+// The largest of 16, 8, 4, 2 bytes that every row of K elements begins at a multiple of
+static int row_alignment(const void* p, DType t, int K) {
+  const unsigned long long v = reinterpret_cast<uintptr_t>(p) | (unsigned long long)K * dtype_size(t) | 16ull;
+  return (int)(v & ~(v - 1));
+}
+
+void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, float* t, cudaStream_t s) {
+  if (M <= 0 || N <= 0) return;
+  // from 128 rows on, a full tile and a long K; other shapes and BF16 rows of an odd
+  // length take the skinny Gram product (n_ov 24,000, 2000 FP32 rows, 20 vectors: 186
+  // us there, 110 here; n_ov 202,500, 1350 BF16 rows: 1090
+  // and 472).  The K chunks number at most 65,535 (grid).
+  const int pa = row_alignment(A, ta, K), px = row_alignment(X, DType::F32, K);
+  if (!(M >= kTallRows && K >= 1024 && K <= 65535 * kTallChunk && pa >= 4 && (ta == DType::F32 || ta == DType::BF16))) {
+    sk_gram(A, ta, K, M, X, DType::F32, K, N, K, t, DType::F32, N, 1.0, 0.0, s);
+    return;
+  }
+  // K chunks: three waves of one CTA per SM, at most 2048 terms
+  const int mt = (M + kTallRows - 1) / kTallRows;
+  int S = std::max((3 * 152 + mt - 1) / mt, (K + kTallChunk - 1) / kTallChunk);
+  int chunk = ((K + S - 1) / S + kTallK - 1) / kTallK * kTallK;
+  chunk = std::max(chunk, 4 * kTallK);
+  S = (K + chunk - 1) / chunk;
+  DevBuf part((size_t)S * M * N * 4, s);
+  float* pt = part.as<float>();
+  if (ta == DType::F32) {
+    const float* a = static_cast<const float*>(A);
+    if (pa == 16 && px == 16) tall_gram_typed<float, 16, 16>(a, M, X, N, K, pt, chunk, S, s);
+    else tall_gram_typed<float, 4, 4>(a, M, X, N, K, pt, chunk, S, s);
+  } else {
+    const __nv_bfloat16* a = static_cast<const __nv_bfloat16*>(A);
+    if (pa == 16 && px == 16) tall_gram_typed<__nv_bfloat16, 16, 16>(a, M, X, N, K, pt, chunk, S, s);
+    else if (pa >= 8 && px == 16) tall_gram_typed<__nv_bfloat16, 8, 16>(a, M, X, N, K, pt, chunk, S, s);
+    else tall_gram_typed<__nv_bfloat16, 4, 4>(a, M, X, N, K, pt, chunk, S, s);
+  }
+  count_launch();
+  TD_LAUNCH_CHECK();
+  const long long MN = (long long)M * N;
+  const unsigned rb = (unsigned)std::min<long long>((MN + 7) / 8, 16 * 152);
+  k_sk_gram_reduce<float, float><<<rb, 256, 0, s>>>(part.as<float>(), S, M, N, t, N, 1.0, 0.0);
+  count_launch();
+  TD_LAUNCH_CHECK();
+}
+
+void tall_combo(const float* t, int N, int K, const void* V, DType tv, int ncols, float* out, cudaStream_t s) {
+  if (N <= 0 || ncols <= 0) return;
+  // four columns are one load of 16 (FP32) or 8 (BF16) bytes (n_ov 202,500, 1350 BF16
+  // rows, 20 vectors: 824 us by the skinny combination, 580 here; n_ov 24,000, 2000
+  // FP32 rows: 128 and 103)
+  if (!(K >= 64 && ncols >= 128 && ncols % 4 == 0 &&
+        ((tv == DType::F32 && row_alignment(V, tv, ncols) == 16) ||
+         (tv == DType::BF16 && row_alignment(V, tv, ncols) >= 8)))) {
+    sk_combo(t, DType::F32, 1, N, N, K, V, tv, ncols, ncols, out, DType::F32, ncols, 1.0, 0.0, s);
+    return;
+  }
+  if (tv == DType::F32) tall_combo_typed<float>(t, N, K, static_cast<const float*>(V), ncols, out, s);
+  else tall_combo_typed<__nv_bfloat16>(t, N, K, static_cast<const __nv_bfloat16*>(V), ncols, out, s);
+  count_launch();
+  TD_LAUNCH_CHECK();
 }
 
 }  // namespace tddft

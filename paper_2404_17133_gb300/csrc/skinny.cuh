@@ -26,6 +26,12 @@ void sk_combo(const void* coef, DType tcoef, long long scm, long long sck, int M
               DType tv, long long ldv, int ncols, void* out, DType tout, long long ldo, double alpha,
               double beta, cudaStream_t s);
 
+// The operator's Coulomb pair over factor rows A [M][K] (F32 or BF16) and FP32
+// vectors: t[m][n] = sum_k A[m][k] X[n][k] (X [N][K]), FP32 accumulation in runs of
+// at most 256 terms; out[n][c] = sum_k t[k][n] V[k][c] (t [K][N], V [K][ncols]).
+void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, float* t, cudaStream_t s);
+void tall_combo(const float* t, int N, int K, const void* V, DType tv, int ncols, float* out, cudaStream_t s);
+
 // Typed conveniences for same-type vectors (T = float or double).
 template <typename T> constexpr DType dtype_of();
 template <> constexpr DType dtype_of<double>() { return DType::F64; }
