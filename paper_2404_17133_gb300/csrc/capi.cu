@@ -581,8 +581,7 @@ tddft_status tddft_apply(tddft_ctx* ctx, int kind, int precision, int tensor_cor
       TD_CUDA(cudaMemcpyAsync(out0, d0, n * 8, cudaMemcpyDeviceToHost, s));
       if (paired) TD_CUDA(cudaMemcpyAsync(out1, d1, n * 8, cudaMemcpyDeviceToHost, s));
     }
-    TD_CUDA(cudaStreamSynchronize(s));
-    check_tc_error(*c);
+    check_tc_error(*c);   // waits for the stream
     return TDDFT_OK;
   })
 }

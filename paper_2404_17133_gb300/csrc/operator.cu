@@ -231,6 +231,61 @@ static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw,
   }
 }
 
+// A term of the final combination: the partial sums that its contraction left (one
+// P-chunk covers the factor set), else the summed term b, if there is one.
+static SumTerm term_of(const TcSum& k, const DevBuf& b) {
+  SumTerm t;
+  if (k.splits) {
+    t.part = k.part.as<float>();
+    t.splits = k.splits;
+    t.scale = k.scale;
+  } else if (b.p) {
+    t.part = b.as<float>();
+    t.splits = 1;
+  }
+  return t;
+}
+
+// Operand forms of the trial vectors for the tensor-core exchange contractions,
+// with their scales, in one allocation.
+struct XParts {
+  DevBuf buf;
+  void *th = nullptr, *tl = nullptr, *sh = nullptr, *sl = nullptr;   // X^T per vector, X: hi + lo
+  const float* sc = nullptr;   // tc_f16_product_scales or tc_fp8_scales block
+};
+static bool tc_exchange(const FactorSet& f, bool f64, bool tensor_cores) {
+  return tensor_cores && !f64 && f.Kvv_hi && f.Kvo_hi && f.Koo_hi && f.Kovp_hi;
+}
+// scratch: five zeroed device words; xw: FP32 copy of X to write, or NULL
+static XParts make_x_parts(const OpDims& d, const FactorSet& f, const void* X, DType xt, int m, bool paired,
+                           unsigned* scratch, float* xw, cudaStream_t s) {
+  const int no = d.no, nv = d.nv;
+  const bool f16 = f.tc_elt == TcElt::F16;
+  TD_REQUIRE(!f.fp8 || (f.Kvv8 && f.Kvo8 && f.s_vv), TDDFT_ERR_ARG, "FP8 ris copies missing");
+  TD_REQUIRE(!f16 || (f.Kvv_lo && f.Kvo_lo && f.Koo_lo && f.Kovp_lo && f.tc_scale), TDDFT_ERR_ARG,
+             "FP16 factor parts missing");
+  auto pad = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t bt = pad((size_t)m * nv * tc_pad(no) * 2), bs = paired ? pad((size_t)m * no * tc_pad(nv) * 2) : 0;
+  XParts x;
+  x.buf = DevBuf(2 * bt + 2 * bs + (f.fp8 ? (size_t)(2 + 2 * f.nK) * 4 : 32), s);
+  char* b = x.buf.as<char>();
+  x.th = b;
+  x.tl = b + bt;
+  if (paired) {
+    x.sh = b + 2 * bt;
+    x.sl = b + 2 * bt + bs;
+  }
+  float* sc = reinterpret_cast<float*>(b + 2 * bt + 2 * bs);
+  x.sc = sc;
+  const bool scaled = f.fp8 || f16;
+  if (f.fp8)
+    tc_fp8_scales(X, xt, m, no, nv, f.s_vv, f.rho_oo, f.s_vo, f.rho_ov, f.nK, sc, scratch, xw, s);
+  else if (f16)
+    tc_f16_product_scales(X, xt, m, no, nv, f.tc_scale, sc, scratch, xw, s);
+  tc_x_split(X, xt, m, no, nv, f.tc_elt, f16 ? sc : nullptr, x.th, x.tl, x.sh, x.sl, scaled ? nullptr : xw, s);
+  return x;
+}
+
 template <typename TX>
 static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, int m, OpMode mode,
                              TX* out0, TX* out1, int tc, cudaStream_t s) {
@@ -245,35 +300,54 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
   TD_REQUIRE(!(x32 && f64), TDDFT_ERR_ARG, "FP32 vectors need FP32/BF16 factors");
 
   const void* Xw = X;
-  DevBuf xbuf;
-  if (!f64 && !x32) {
+  const DType xt = x32 ? DType::F32 : DType::F64;
+  const bool need_k2 = (mode == OpMode::PAIRED);
+  const bool main_x = f.nK > 0 && d.a_x != 0.0;
+  const bool lr_x = f.lr && f.b_x != 0.0 && f.lr->nK > 0;
+  DevBuf xbuf, words;
+  XParts xp;
+  if (tensor_cores && !f64) {
+    words = DevBuf(5 * 4, s);   // [4]: max |t|
+    TD_CUDA(cudaMemsetAsync(words.p, 0, 5 * 4, s));
+  }
+  const bool cast = !f64 && !x32;
+  if (cast) {
     xbuf = DevBuf(mov * 4, s);
-    cast_f64_to_f32(reinterpret_cast<const double*>(X), xbuf.as<float>(), mov, s);
     Xw = xbuf.p;
   }
+  // the pass that prepares the exchange operands writes the FP32 copy too
+  if (main_x && tc_exchange(f, f64, tensor_cores))
+    xp = make_x_parts(d, f, X, xt, m, need_k2, words.as<unsigned>(), cast ? xbuf.as<float>() : nullptr, s);
+  else if (cast)
+    cast_f64_to_f32(reinterpret_cast<const double*>(X), xbuf.as<float>(), mov, s);
 
   // ---- Coulomb (and the low-rank kernel term, which enters with the same prefactor)
   DevBuf Jb;
+  TcSum Js;
   bool have_J = false;
+  const bool kernel_rows = d.c_J != 0.0 && (f.nFpos > 0 || f.nFneg > 0);
   if (f.nJ > 0 && d.c_J != 0.0) {
     // t[P][n] = sum_ia L_ov[P][ia] X[n][ia];  J[n][ia] = sum_P t[P][n] L_ov[P][ia]
-    Jb = DevBuf(mov * ew, s);
     if (tensor_cores && f.tc_elt == TcElt::F16 && f.JovT_hi && !f64) {
       // t = L_ov X^T on the SIMT path (K = ov: its FP32 reduction tree keeps t
       // at ~1e-7; one tensor-core accumulation run per 4096 terms left the
       // Coulomb products at ~2e-6), then J = t^T L_ov on the tensor cores,
       // streaming the FP16 hi+lo copy of s_ov L_ov transposed once, with t as
       // FP16 parts of s_t t
-      DevBuf t((size_t)f.nJ * m * 4, s), sct(2 * 4, s), scr(8, s), fac(4, s);
-      tall_gram(f.Jov, f.dt, f.nJ, static_cast<const float*>(Xw), m, ov, t.as<float>(), s);
-      tc_f16_tensor_scale(t.as<float>(), f.nJ, m, sct.as<float>(), scr.as<unsigned>(), s);
-      const int nJp = tc_pad(f.nJ);
-      DevBuf th((size_t)m * nJp * 2, s), tl((size_t)m * nJp * 2, s);
-      tc_transpose_split(t.p, DType::F32, 1, f.nJ, m, th.p, tl.p, TcElt::F16, sct.as<float>(), s);
-      tc_inv_prod(sct.as<float>(), f.tc_scale + 4, fac.as<float>(), s);      // 1 / (s_t s_ov)
-      tc_contract(th.p, tl.p, nJp, m, 1, f.nJ, f.JovT_hi, f.JovT_lo, ov, Jb.as<float>(), false, TcElt::F16,
-                  fac.as<float>(), d.tc_err, s, nullptr, 0.0, 0.0, kCoulombKb);
+      const size_t tb = ((size_t)f.nJ * m * 4 + 255) & ~(size_t)255;
+      const size_t hb = ((size_t)m * tc_pad(f.nJ) * 2 + 255) & ~(size_t)255;
+      DevBuf t(tb + 2 * hb, s);
+      Js.factor = DevBuf(4, s);
+      char* th = t.as<char>() + tb;
+      unsigned* tmax = words.as<unsigned>() + 4;
+      tall_gram(f.Jov, f.dt, f.nJ, static_cast<const float*>(Xw), m, ov, t.as<float>(), s, tmax);
+      tc_t_split(t.as<float>(), f.nJ, m, tmax, f.tc_scale + 4, th, th + hb, Js.factor.as<float>(), s);
+      const bool keep = !kernel_rows;
+      if (!keep) Jb = DevBuf(mov * ew, s);
+      tc_contract(th, th + hb, tc_pad(f.nJ), m, 1, f.nJ, f.JovT_hi, f.JovT_lo, ov, Jb.as<float>(), false, TcElt::F16,
+                  Js.factor.as<float>(), d.tc_err, s, nullptr, 0.0, 0.0, kCoulombKb, keep ? &Js : nullptr);
     } else {
+      Jb = DevBuf(mov * ew, s);
       DevBuf t((size_t)f.nJ * m * ew, s);
       if (f64) {
         sk_gram(f.Jov, f.dt, ov, f.nJ, Xw, tw, ov, m, ov, t.p, tw, m, 1.0, 0.0, s);
@@ -301,15 +375,18 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
   }
 
   // ---- exchange: K1 (and K2 for the paired products) of one factor set
-  const bool need_k2 = (mode == OpMode::PAIRED);
-  auto exchange = [&](const FactorSet& f, DevBuf& K1b, DevBuf& K2b) {
-    K1b = DevBuf(mov * ew, s);
-    if (need_k2) K2b = DevBuf(mov * ew, s);
-    const bool use_tc = tensor_cores && !f64 && f.Kvv_hi && f.Kvo_hi && f.Koo_hi && f.Kovp_hi;
+  // K1s / K2s, when given, may take the partial sums instead (term_of)
+  auto exchange = [&](const FactorSet& f, const XParts& xp, DevBuf& K1b, DevBuf& K2b, TcSum* K1s, TcSum* K2s) {
+    const bool use_tc = tc_exchange(f, f64, tensor_cores);
     TD_REQUIRE(!tensor_cores || f64 || use_tc, TDDFT_ERR_ARG, "tensor-core factor copies missing");
     const int pc = use_tc ? chunk_rows(f.nK, (long long)m * no * tc_zpad(nv, 2) * 4, m, kChunkBytesTC)
                           : chunk_rows(f.nK, (long long)m * ov * (long long)ew, m, kChunkBytes);
     const size_t es = dtype_size(f.dt);
+    if (!use_tc || pc < f.nK) K1s = K2s = nullptr;
+    if (!K1s) {
+      K1b = DevBuf(mov * ew, s);
+      if (need_k2) K2b = DevBuf(mov * ew, s);
+    }
     // 16-bit tensor-core operand pointer at element offset o
     auto at16 = [](const void* b, size_t o) { return static_cast<const void*>(static_cast<const uint16_t*>(b) + o); };
     if (use_tc && f.fp8) {
@@ -319,23 +396,12 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       // hi + lo, multiplied by mu_P; the second contractions run as
       // kind::f8f6f4 (two products: hi and lo against the e4m3 rows) and the
       // sums are multiplied back by 1/g (tc_fp8_scales).
-      TD_REQUIRE(f.Kvv8 && f.Kvo8 && f.s_vv, TDDFT_ERR_ARG, "FP8 ris copies missing");
       const int nvp = tc_pad(nv), nop = tc_pad(no), nv16 = tc_pad16(nv), no16 = tc_pad16(no);
       const int nvz = tc_zpad(nv, 1), noz = tc_zpad(no, 1);
-      const DType xt = x32 ? DType::F32 : DType::F64;
-      DevBuf sc((size_t)(2 + 2 * f.nK) * 4, s), kap(16, s);
-      tc_fp8_scales(X, xt, m, no, nv, f.s_vv, f.rho_oo, f.s_vo, f.rho_ov, f.nK, sc.as<float>(), kap.as<unsigned>(), s);
-      const float* inv1 = sc.as<float>();
+      const float* inv1 = xp.sc;
       const float* inv2 = inv1 + 1;
       const float* mu1 = inv1 + 2;
       const float* mu2 = mu1 + f.nK;
-      DevBuf Xt_hi((size_t)m * nv * nop * 2, s), Xt_lo((size_t)m * nv * nop * 2, s), Xs_hi, Xs_lo;
-      tc_transpose_split(X, xt, m, no, nv, Xt_hi.p, Xt_lo.p, TcElt::BF16, nullptr, s);
-      if (need_k2) {
-        Xs_hi = DevBuf((size_t)m * no * nvp * 2, s);
-        Xs_lo = DevBuf((size_t)m * no * nvp * 2, s);
-        tc_pad_split(X, xt, (long long)m * no, nv, Xs_hi.p, Xs_lo.p, TcElt::BF16, nullptr, s);
-      }
       DevBuf Zhi((size_t)m * no * pc * nvz, s), Zlo((size_t)m * no * pc * nvz, s), Qhi, Qlo;
       if (need_k2) {
         Qhi = DevBuf((size_t)m * no * pc * noz, s);
@@ -344,17 +410,17 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       const int Mz = m * no;
       for (int p0 = 0; p0 < f.nK; p0 += pc) {
         const int pn = (f.nK - p0 < pc) ? f.nK - p0 : pc;
-        tc_stage1_fp8(Xt_hi.as<__nv_bfloat16>(), Xt_lo.as<__nv_bfloat16>(), m, nv, no,
+        tc_stage1_fp8(static_cast<const __nv_bfloat16*>(xp.th), static_cast<const __nv_bfloat16*>(xp.tl), m, nv, no,
                       static_cast<const __nv_bfloat16*>(f.Koo_hi) + (size_t)p0 * no * nop, no, pn, mu1 + p0,
                       Zhi.as<unsigned char>(), Zlo.as<unsigned char>(), d.tc_err, s);
         tc_contract8(Zhi.as<unsigned char>(), Zlo.as<unsigned char>(), Mz, pn, nv,
-                     f.Kvv8 + (size_t)p0 * nv * nv16, nv, K1b.as<float>(), p0 > 0, inv1, d.tc_err, s);
+                     f.Kvv8 + (size_t)p0 * nv * nv16, nv, K1b.as<float>(), p0 > 0, inv1, d.tc_err, s, K1s);
         if (need_k2) {
-          tc_stage1_fp8(Xs_hi.as<__nv_bfloat16>(), Xs_lo.as<__nv_bfloat16>(), m, no, nv,
+          tc_stage1_fp8(static_cast<const __nv_bfloat16*>(xp.sh), static_cast<const __nv_bfloat16*>(xp.sl), m, no, nv,
                         static_cast<const __nv_bfloat16*>(f.Kovp_hi) + (size_t)p0 * no * nvp, no, pn, mu2 + p0,
                         Qhi.as<unsigned char>(), Qlo.as<unsigned char>(), d.tc_err, s);
           tc_contract8(Qhi.as<unsigned char>(), Qlo.as<unsigned char>(), Mz, pn, no,
-                       f.Kvo8 + (size_t)p0 * nv * no16, nv, K2b.as<float>(), p0 > 0, inv2, d.tc_err, s);
+                       f.Kvo8 + (size_t)p0 * nv * no16, nv, K2b.as<float>(), p0 > 0, inv2, d.tc_err, s, K2s);
         }
       }
     } else if (use_tc) {
@@ -366,27 +432,11 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       // that the contractions' sums remove.  ris factor sets (BF16): the
       // factors are used as they are (two products, exact with respect to them).
       const bool f16 = f.tc_elt == TcElt::F16;
-      TD_REQUIRE(!f16 || (f.Kvv_lo && f.Kvo_lo && f.Koo_lo && f.Kovp_lo && f.tc_scale), TDDFT_ERR_ARG,
-                 "FP16 factor parts missing");
       const TcElt et = f.tc_elt;
       const int nvp = tc_pad(nv), nop = tc_pad(no);
-      const DType xt = x32 ? DType::F32 : DType::F64;
-      DevBuf sc, kap;
-      const float* sx = nullptr;
       const float *mz = nullptr, *mq = nullptr, *f1 = nullptr, *f2 = nullptr;
       if (f16) {
-        sc = DevBuf(8 * 4, s);
-        kap = DevBuf(16, s);
-        tc_f16_product_scales(X, xt, m, no, nv, f.tc_scale, sc.as<float>(), kap.as<unsigned>(), s);
-        sx = sc.as<float>();
-        mz = sx + 1; mq = sx + 2; f1 = sx + 3; f2 = sx + 4;
-      }
-      DevBuf Xt_hi((size_t)m * nv * nop * 2, s), Xt_lo((size_t)m * nv * nop * 2, s), Xs_hi, Xs_lo;
-      tc_transpose_split(X, xt, m, no, nv, Xt_hi.p, Xt_lo.p, et, sx, s);
-      if (need_k2) {
-        Xs_hi = DevBuf((size_t)m * no * nvp * 2, s);
-        Xs_lo = DevBuf((size_t)m * no * nvp * 2, s);
-        tc_pad_split(X, xt, (long long)m * no, nv, Xs_hi.p, Xs_lo.p, et, sx, s);
+        mz = xp.sc + 1; mq = xp.sc + 2; f1 = xp.sc + 3; f2 = xp.sc + 4;
       }
       const int nvz = tc_zpad(nv, 2), noz = tc_zpad(no, 2);
       DevBuf Zhi((size_t)m * no * pc * nvz * 2, s), Zlo((size_t)m * no * pc * nvz * 2, s), Qhi, Qlo;
@@ -397,7 +447,7 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       const int Mz = m * no;
       for (int p0 = 0; p0 < f.nK; p0 += pc) {
         const int pn = (f.nK - p0 < pc) ? f.nK - p0 : pc;
-        tc_stage1(Xt_hi.p, Xt_lo.p, m, nv, no, at16(f.Koo_hi, (size_t)p0 * no * nop),
+        tc_stage1(xp.th, xp.tl, m, nv, no, at16(f.Koo_hi, (size_t)p0 * no * nop),
                   f16 ? at16(f.Koo_lo, (size_t)p0 * no * nop) : nullptr, no, pn, et, mz, Zhi.p, Zlo.p, d.tc_err, s);
         const bool timed = d.prof && d.prof->on && f16;
         tc_contract(Zhi.p, Zlo.p, nvz, Mz, pn, nv, at16(f.Kvv_hi, (size_t)p0 * nv * nvp),
@@ -407,13 +457,13 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
                     // written (and read back when accumulating)
                     4.0 * Mz * (double)pn * nv + (f16 ? 4.0 : 2.0) * (double)pn * nv * nv +
                         4.0 * Mz * (double)nv * (p0 > 0 ? 2.0 : 1.0),
-                    f16 ? kExchangeKb : 0);
+                    f16 ? kExchangeKb : 0, K1s);
         if (need_k2) {
-          tc_stage1(Xs_hi.p, Xs_lo.p, m, no, nv, at16(f.Kovp_hi, (size_t)p0 * no * nvp),
+          tc_stage1(xp.sh, xp.sl, m, no, nv, at16(f.Kovp_hi, (size_t)p0 * no * nvp),
                     f16 ? at16(f.Kovp_lo, (size_t)p0 * no * nvp) : nullptr, no, pn, et, mq, Qhi.p, Qlo.p, d.tc_err, s);
           tc_contract(Qhi.p, Qlo.p, noz, Mz, pn, no, at16(f.Kvo_hi, (size_t)p0 * nv * nop),
                       f16 ? at16(f.Kvo_lo, (size_t)p0 * nv * nop) : nullptr, nv, K2b.as<float>(), p0 > 0, et, f2,
-                      d.tc_err, s, nullptr, 0.0, 0.0, f16 ? kExchangeKb : 0);
+                      d.tc_err, s, nullptr, 0.0, 0.0, f16 ? kExchangeKb : 0, K2s);
         }
       }
     } else if (f.dt != DType::BF16) {
@@ -471,41 +521,35 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
     }
   };
   DevBuf K1b, K2b;
+  TcSum K1s, K2s;
   double kx = d.a_x;   // weight of the exchange parts in the final combination
-  if (f.nK > 0 && d.a_x != 0.0) exchange(f, K1b, K2b);
-  if (f.lr && f.b_x != 0.0 && f.lr->nK > 0) {
+  if (main_x) exchange(f, xp, K1b, K2b, lr_x ? nullptr : &K1s, lr_x ? nullptr : &K2s);
+  if (lr_x) {
     // second exchange set: K = a_x K[L] + b_x K[M], combined with weight 1
+    XParts xl;
+    if (tc_exchange(*f.lr, f64, tensor_cores))
+      xl = make_x_parts(d, *f.lr, X, xt, m, need_k2, words.as<unsigned>(), nullptr, s);
     DevBuf L1, L2;
-    exchange(*f.lr, L1, L2);
-    const bool have = K1b.p != nullptr;
-    if (!have) {
+    exchange(*f.lr, xl, L1, L2, nullptr, nullptr);
+    if (!main_x) {
       K1b = DevBuf(mov * ew, s);
       if (need_k2) K2b = DevBuf(mov * ew, s);
     }
-    axpby(K1b.p, L1.p, tw, have ? d.a_x : 0.0, f.b_x, mov, s);
-    if (need_k2) axpby(K2b.p, L2.p, tw, have ? d.a_x : 0.0, f.b_x, mov, s);
+    axpby(K1b.p, L1.p, tw, main_x ? d.a_x : 0.0, f.b_x, mov, s);
+    if (need_k2) axpby(K2b.p, L2.p, tw, main_x ? d.a_x : 0.0, f.b_x, mov, s);
     kx = 1.0;
   }
 
-  const void* J = Jb.p;
-  const void* K1 = K1b.p;
-  const void* K2 = K2b.p;
-  if constexpr (x32) {
-    const float* Jf = static_cast<const float*>(J);
-    const float* K1f = static_cast<const float*>(K1);
-    const float* K2f = static_cast<const float*>(K2);
+  const double cj = mode == OpMode::TDA ? d.c_J : 2.0 * d.c_J;
+  if (!f64) {
+    combine_sums<TX>(X, d.delta, term_of(Js, Jb), term_of(K1s, K1b), term_of(K2s, K2b), cj, -kx, -kx, m, ov, out0,
+                     mode == OpMode::TDA ? nullptr : out1, s);
+  } else if constexpr (!x32) {
     if (mode == OpMode::TDA) {
-      combine_f32(X, d.delta, Jf, K1f, nullptr, d.c_J, -kx, 0.0, m, ov, out0, s);
+      combine(X, d.delta, Jb.p, K1b.p, nullptr, tw, cj, -kx, 0.0, m, ov, out0, s);
     } else {
-      combine_f32(X, d.delta, Jf, K1f, K2f, 2.0 * d.c_J, -kx, -kx, m, ov, out0, s);
-      combine_f32(X, d.delta, nullptr, K1f, K2f, 0.0, -kx, kx, m, ov, out1, s);
-    }
-  } else {
-    if (mode == OpMode::TDA) {
-      combine(X, d.delta, J, K1, nullptr, tw, d.c_J, -kx, 0.0, m, ov, out0, s);
-    } else {
-      combine(X, d.delta, J, K1, K2, tw, 2.0 * d.c_J, -kx, -kx, m, ov, out0, s);
-      combine(X, d.delta, nullptr, K1, K2, tw, 0.0, -kx, kx, m, ov, out1, s);
+      combine(X, d.delta, Jb.p, K1b.p, K2b.p, tw, cj, -kx, -kx, m, ov, out0, s);
+      combine(X, d.delta, nullptr, K1b.p, K2b.p, tw, 0.0, -kx, kx, m, ov, out1, s);
     }
   }
 }

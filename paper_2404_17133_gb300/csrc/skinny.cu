@@ -146,10 +146,11 @@ k_sk_gram64(const double* __restrict__ A, long long lda, int M, const double* __
 // then a fixed butterfly adds the lanes (deterministic).
 template <typename ACC, typename TC>
 __global__ void k_sk_gram_reduce(const ACC* __restrict__ part, int S, int M, int N, TC* __restrict__ C,
-                                 long long ldc, double alpha, double beta) {
+                                 long long ldc, double alpha, double beta, unsigned* cmax = nullptr) {
   const long long MN = (long long)M * N;
   const int lane = threadIdx.x & 31;
   const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+  float big = 0.f;   // lane 0: max |C| of this warp's elements
   for (long long i = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); i < MN; i += warps) {
     double acc = 0.0;
     for (int c = lane; c < S; c += 32) acc += (double)part[(long long)c * MN + i];
@@ -161,8 +162,10 @@ __global__ void k_sk_gram_reduce(const ACC* __restrict__ part, int S, int M, int
       double v = alpha * acc;
       if (beta != 0.0) v += beta * (double)*p;
       *p = (TC)v;
+      if (cmax) big = fmaxf(big, fabsf((float)v));
     }
   }
+  if (cmax && lane == 0) atomicMax(cmax, __float_as_uint(big));
 }
 
 // Combination: CTA = 32 columns x kComboGroups warps; warp g sums k = g, g+8, ...
@@ -225,7 +228,7 @@ void set_smem_attr(const void* f, size_t bytes) {
 
 template <typename TA, typename TB, typename ACC>
 void gram_typed(const void* A, long long lda, int M, const void* B, long long ldb, int N, int K, void* C,
-                DType tc, long long ldc, double alpha, double beta, cudaStream_t s) {
+                DType tc, long long ldc, double alpha, double beta, cudaStream_t s, unsigned* cmax = nullptr) {
   TD_REQUIRE((M + kTile - 1) / kTile <= 65535 && (N + kTile - 1) / kTile <= 65535, TDDFT_ERR_ARG,
              "sk_gram: too many rows");
   // fixed K chunks: 256 columns (FP32 staging); FP64 16 to 128, so that K up to
@@ -263,9 +266,9 @@ void gram_typed(const void* A, long long lda, int M, const void* B, long long ld
   const long long MN = (long long)M * N;
   const unsigned rb = (unsigned)std::min<long long>((MN + 7) / 8, 16 * 152);   // 8 warps per block
   if (tc == DType::F64)
-    k_sk_gram_reduce<ACC, double><<<rb, 256, 0, s>>>(part.as<ACC>(), S, M, N, (double*)C, ldc, alpha, beta);
+    k_sk_gram_reduce<ACC, double><<<rb, 256, 0, s>>>(part.as<ACC>(), S, M, N, (double*)C, ldc, alpha, beta, cmax);
   else
-    k_sk_gram_reduce<ACC, float><<<rb, 256, 0, s>>>(part.as<ACC>(), S, M, N, (float*)C, ldc, alpha, beta);
+    k_sk_gram_reduce<ACC, float><<<rb, 256, 0, s>>>(part.as<ACC>(), S, M, N, (float*)C, ldc, alpha, beta, cmax);
   count_launch();
   TD_LAUNCH_CHECK();
 }
@@ -653,15 +656,15 @@ void tall_combo_typed(const float* t, int N, int K, const TV* V, int ncols, floa
 }  // namespace
 
 void sk_gram(const void* A, DType ta, long long lda, int M, const void* B, DType tb, long long ldb, int N,
-             int K, void* C, DType tc, long long ldc, double alpha, double beta, cudaStream_t s) {
+             int K, void* C, DType tc, long long ldc, double alpha, double beta, cudaStream_t s, unsigned* cmax) {
   if (M <= 0 || N <= 0) return;
   TD_REQUIRE(tc == DType::F32 || tc == DType::F64, TDDFT_ERR_ARG, "sk_gram: output type");
   if (ta == DType::F64 && tb == DType::F64)
-    gram_typed<double, double, double>(A, lda, M, B, ldb, N, K, C, tc, ldc, alpha, beta, s);
+    gram_typed<double, double, double>(A, lda, M, B, ldb, N, K, C, tc, ldc, alpha, beta, s, cmax);
   else if (ta == DType::F32 && tb == DType::F32)
-    gram_typed<float, float, float>(A, lda, M, B, ldb, N, K, C, tc, ldc, alpha, beta, s);
+    gram_typed<float, float, float>(A, lda, M, B, ldb, N, K, C, tc, ldc, alpha, beta, s, cmax);
   else if (ta == DType::BF16 && tb == DType::F32)
-    gram_typed<__nv_bfloat16, float, float>(A, lda, M, B, ldb, N, K, C, tc, ldc, alpha, beta, s);
+    gram_typed<__nv_bfloat16, float, float>(A, lda, M, B, ldb, N, K, C, tc, ldc, alpha, beta, s, cmax);
   else
     throw Error(TDDFT_ERR_ARG, "sk_gram: unsupported operand types");
 }
@@ -693,7 +696,7 @@ static int row_alignment(const void* p, DType t, int K) {
   return (int)(v & ~(v - 1));
 }
 
-void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, float* t, cudaStream_t s) {
+void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, float* t, cudaStream_t s, unsigned* tmax) {
   if (M <= 0 || N <= 0) return;
   // from 128 rows on, a full tile and a long K; other shapes and BF16 rows of an odd
   // length take the skinny Gram product (n_ov 24,000, 2000 FP32 rows, 20 vectors: 186
@@ -701,7 +704,7 @@ void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, flo
   // and 472).  The K chunks number at most 65,535 (grid).
   const int pa = row_alignment(A, ta, K), px = row_alignment(X, DType::F32, K);
   if (!(M >= kTallRows && K >= 1024 && K <= 65535 * kTallChunk && pa >= 4 && (ta == DType::F32 || ta == DType::BF16))) {
-    sk_gram(A, ta, K, M, X, DType::F32, K, N, K, t, DType::F32, N, 1.0, 0.0, s);
+    sk_gram(A, ta, K, M, X, DType::F32, K, N, K, t, DType::F32, N, 1.0, 0.0, s, tmax);
     return;
   }
   // K chunks: three waves of one CTA per SM, at most 2048 terms
@@ -726,7 +729,7 @@ void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, flo
   TD_LAUNCH_CHECK();
   const long long MN = (long long)M * N;
   const unsigned rb = (unsigned)std::min<long long>((MN + 7) / 8, 16 * 152);
-  k_sk_gram_reduce<float, float><<<rb, 256, 0, s>>>(part.as<float>(), S, M, N, t, N, 1.0, 0.0);
+  k_sk_gram_reduce<float, float><<<rb, 256, 0, s>>>(part.as<float>(), S, M, N, t, N, 1.0, 0.0, tmax);
   count_launch();
   TD_LAUNCH_CHECK();
 }

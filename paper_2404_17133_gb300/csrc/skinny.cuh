@@ -13,8 +13,10 @@ namespace tddft {
 // A, B: rows of length K with strides lda, ldb.  K is cut into chunks (one CTA
 // per chunk and 32x32 output tile); chunk sums are added in FP64 in a fixed
 // order, so results are deterministic.  C (type tc: F32 or F64) has row stride ldc.
+// *cmax, when given, is raised to the float bits of max |C|.
 void sk_gram(const void* A, DType ta, long long lda, int M, const void* B, DType tb, long long ldb, int N,
-             int K, void* C, DType tc, long long ldc, double alpha, double beta, cudaStream_t s);
+             int K, void* C, DType tc, long long ldc, double alpha, double beta, cudaStream_t s,
+             unsigned* cmax = nullptr);
 
 // out[m][c] = alpha * sum_k coef(m, k) V[k][c] + beta * out[m][c]
 // (m < M, k < K, c < ncols); coef(m, k) = coef[m*scm + k*sck] of type tcoef (F32
@@ -29,7 +31,9 @@ void sk_combo(const void* coef, DType tcoef, long long scm, long long sck, int M
 // The operator's Coulomb pair over factor rows A [M][K] (F32 or BF16) and FP32
 // vectors: t[m][n] = sum_k A[m][k] X[n][k] (X [N][K]), FP32 accumulation in runs of
 // at most 256 terms; out[n][c] = sum_k t[k][n] V[k][c] (t [K][N], V [K][ncols]).
-void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, float* t, cudaStream_t s);
+// *tmax, when given, is raised to the float bits of max |t|.
+void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, float* t, cudaStream_t s,
+               unsigned* tmax = nullptr);
 void tall_combo(const float* t, int N, int K, const void* V, DType tv, int ncols, float* out, cudaStream_t s);
 
 // Typed conveniences for same-type vectors (T = float or double).

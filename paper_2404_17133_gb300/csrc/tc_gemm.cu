@@ -34,6 +34,7 @@
 // code in `err` and leaves the loop; the host turns it into TDDFT_ERR_CUDA.
 #include <algorithm>
 #include <cstdlib>
+#include <type_traits>
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -1281,11 +1282,29 @@ void sum_splits(const Contraction& c, float* out, bool accumulate, const float* 
   count_launch();
   TD_LAUNCH_CHECK();
 }
+
+void finish_sums(const Contraction& c, DevBuf& part, float* out, bool accumulate, const float* scale, TcSum* keep) {
+  if (!keep) {
+    sum_splits(c, out, accumulate, scale);
+    return;
+  }
+  const size_t mn = (size_t)c.M * c.N * 4;
+  if (c.splits * mn <= kKeepBytes) {
+    keep->part = std::move(part);
+    keep->splits = c.splits;
+    keep->scale = scale;
+  } else {   // too much to hold on to
+    keep->part = DevBuf(mn, c.s);
+    sum_splits(c, keep->part.as<float>(), false, scale);
+    keep->splits = 1;
+    keep->scale = nullptr;
+  }
+}
 }  // namespace
 
 void tc_contract(const void* Ahi, const void* Alo, int lda, int M, int pn, int Kin, const void* Bhi, const void* Blo,
                  int N, float* out, bool accumulate, TcElt elt, const float* scale, int* err, cudaStream_t s,
-                 KernelProfile* prof, double prof_flops, double prof_bytes, int max_kb) {
+                 KernelProfile* prof, double prof_flops, double prof_bytes, int max_kb, TcSum* keep) {
   if (M <= 0 || pn <= 0 || N <= 0) return;
   const int mode = Blo ? BOTH : ASPLIT;
   TD_REQUIRE(Alo != nullptr && mode == (elt == TcElt::F16 ? BOTH : ASPLIT), TDDFT_ERR_ARG,
@@ -1310,12 +1329,12 @@ void tc_contract(const void* Ahi, const void* Alo, int lda, int M, int pn, int K
                       part.as<float>(), err, s, prof, prof_flops, prof_bytes};
   if (mode == BOTH) launch_contraction<BOTH, ET_F16, 64>(c);
   else launch_contraction<ASPLIT, ET_BF16, 128>(c);
-  sum_splits(c, out, accumulate, scale);
+  finish_sums(c, part, out, accumulate, scale, keep);
 }
 
 void tc_contract8(const unsigned char* Ahi, const unsigned char* Alo, int M, int pn, int Kin,
                   const unsigned char* B, int N, float* out, bool accumulate, const float* scale, int* err,
-                  cudaStream_t s) {
+                  cudaStream_t s, TcSum* keep) {
   if (M <= 0 || pn <= 0 || N <= 0) return;
   TD_REQUIRE(Ahi && Alo && B && scale, TDDFT_ERR_ARG, "tc_contract8: operands missing");
   constexpr int BKE = Elem<ET_E4M3>::BKE;
@@ -1329,7 +1348,7 @@ void tc_contract8(const unsigned char* Ahi, const unsigned char* Alo, int M, int
   const Contraction c{Ahi, Alo, M, pn, Kin, B, nullptr, N, tc_zpad(Kin, 1), tc_pad16(Kin), 1, total, per, splits, nab,
                       part.as<float>(), err, s, nullptr, 0.0, 0.0};
   launch_contraction<ASPLIT, ET_E4M3, 128>(c);
-  sum_splits(c, out, accumulate, scale);
+  finish_sums(c, part, out, accumulate, scale, keep);
 }
 
 namespace {
@@ -1532,45 +1551,6 @@ __global__ void k_row_norm_max(const __nv_bfloat16* __restrict__ src, int nr, in
   }
 }
 
-// kappa[0] = max_(n,a) ||X[n][:][a]||, kappa[1] = max_(n,j) ||X[n][j][:]||,
-// kappa[2] = max |X| (as float bits; non-negative floats order like their bit
-// patterns)
-template <typename T>
-__global__ void k_x_norms(const T* __restrict__ X, int no, int nv, unsigned* __restrict__ kappa) {
-  const T* x = X + (long long)blockIdx.x * no * nv;
-  __shared__ float red[3][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  float mc = 0.f, mr = 0.f, ma = 0.f;
-  for (int a = threadIdx.x; a < nv; a += blockDim.x) {
-    float acc = 0.f;
-    for (int j = 0; j < no; ++j) {
-      const float v = (float)x[(long long)j * nv + a];
-      acc += v * v;
-      ma = fmaxf(ma, fabsf(v));
-    }
-    mc = fmaxf(mc, sqrtf(acc));
-  }
-  for (int j = warp; j < no; j += nw) {
-    float acc = 0.f;
-    for (int b = lane; b < nv; b += 32) { const float v = (float)x[(long long)j * nv + b]; acc += v * v; }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    mr = fmaxf(mr, sqrtf(acc));
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, o));
-    ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
-  }
-  if (lane == 0) { red[0][warp] = mc; red[1][warp] = mr; red[2][warp] = ma; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float c = 0.f, r = 0.f, m = 0.f;
-    for (int w = 0; w < nw; ++w) { c = fmaxf(c, red[0][w]); r = fmaxf(r, red[1][w]); m = fmaxf(m, red[2][w]); }
-    atomicMax(&kappa[0], __float_as_uint(c));
-    atomicMax(&kappa[1], __float_as_uint(r));
-    atomicMax(&kappa[2], __float_as_uint(m));
-  }
-}
-
 // 2^(top - e) for b = f 2^e, f in [0.5, 1): the largest power of two s with
 // s b < 2^top (1 for b = 0).
 __device__ __forceinline__ float pow2_scale(float b, int top) {
@@ -1612,52 +1592,162 @@ __global__ void k_f16_sigma(const unsigned* __restrict__ st, float* __restrict__
   sc[1] = sg * __uint_as_float(st[1]);
 }
 
-// Per-product scales of the FP16 exact contractions (layout in tc_gemm.cuh).
-__global__ void k_f16_product_scales(const unsigned* __restrict__ kappa, const float* __restrict__ fsc,
-                                     float* __restrict__ out) {
-  const float kc = __uint_as_float(kappa[0]), kr = __uint_as_float(kappa[1]);
-  const float sx = pow2_scale(__uint_as_float(kappa[2]), 14);
-  // |Z'| <= rho_oo' ||X'[n][:][a]||, |Q'| <= ||X'[n][i][:]|| rho_ov' (Cauchy-Schwarz)
-  const float mz = pow2_scale(fsc[1] * sx * kc, 15);
-  const float mq = pow2_scale(fsc[5] * sx * kr, 15);
-  out[0] = sx;
-  out[1] = mz;
-  out[2] = mq;
-  out[3] = 1.f / (mz * fsc[0] * sx * fsc[2]);
-  out[4] = 1.f / (mq * sx * fsc[4] * fsc[4]);
+// Bounds of the trial vectors and the scales that follow from them, in one launch:
+//   kappa[0] = max_(n,a) ||X[n][:][a]||, kappa[1] = max_(n,j) ||X[n][j][:]||,
+//   kappa[2] = max |X|  (float bits: non-negative floats order like them),
+// by blocks of 32 rows (which also write the FP32 copy Xw) and of 256 columns; the
+// last block to finish turns them into the scales and leaves the scratch words
+// ready for the next call.  Bound by launch latency up to a few MB of X, then by
+// reading X twice (the second time from L2).  20 vectors of 150 x 1350: 31 us
+// (171 us with one block per vector and the scales in a second launch).
+struct XPrep {
+  int m, no, nv, rb, cb;       // row and column blocks per vector
+  unsigned* scratch;           // [0..2] kappa, [3] finished blocks, [4] max |t| (tc_t_split): zero on entry
+  float* xw;                   // FP32 copy or NULL
+  float* out;
+  const float* fsc;            // FP16: factor-set scale block
+  const float *s1, *r1, *s2, *r2;   // FP8: scales and row norms of the rows
+  int nK;
+};
+
+__device__ __forceinline__ float block_max(float v, float* red) {   // 256 threads; every thread gets it
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = red[0];
+#pragma unroll
+  for (int w = 1; w < 8; ++w) v = fmaxf(v, red[w]);
+  return v;
 }
 
-// out[0] = 1/g1, out[1] = 1/g2, out[2 + P] = s1_P g1, out[2 + nK + P] = s2_P g2
-__global__ void k_fp8_mu(const unsigned* __restrict__ kappa, const float* __restrict__ s1,
-                         const float* __restrict__ r1, const float* __restrict__ s2,
-                         const float* __restrict__ r2, int nK, float* __restrict__ out) {
-  __shared__ float red[2][32];
-  const float kc = __uint_as_float(kappa[0]), kr = __uint_as_float(kappa[1]);
-  float b1 = 0.f, b2 = 0.f;
-  for (int P = threadIdx.x; P < nK; P += blockDim.x) {
-    b1 = fmaxf(b1, s1[P] * r1[P] * kc);
-    b2 = fmaxf(b2, s2[P] * r2[P] * kr);
+template <typename T, bool FP8>
+__global__ void __launch_bounds__(256) k_x_prep(const T* __restrict__ X, const XPrep p) {
+  __shared__ float red[8];
+  __shared__ bool last;
+  const int n = blockIdx.x / (p.rb + p.cb), q = blockIdx.x - n * (p.rb + p.cb);
+  const T* x = X + (long long)n * p.no * p.nv;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (q < p.rb) {
+    float mr = 0.f, ma = 0.f;
+    for (int j = q * 32 + warp; j < min(p.no, q * 32 + 32); j += 8) {
+      float acc = 0.f;
+#pragma unroll 4
+      for (int b = lane; b < p.nv; b += 32) {
+        const float v = (float)x[(long long)j * p.nv + b];
+        acc += v * v;
+        ma = fmaxf(ma, fabsf(v));
+        if (p.xw) p.xw[((long long)n * p.no + j) * p.nv + b] = v;
+      }
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      mr = fmaxf(mr, sqrtf(acc));
+    }
+    mr = block_max(mr, red);
+    ma = block_max(ma, red);
+    if (threadIdx.x == 0) {
+      atomicMax(&p.scratch[1], __float_as_uint(mr));
+      atomicMax(&p.scratch[2], __float_as_uint(ma));
+    }
+  } else {
+    const int a = (q - p.rb) * 256 + threadIdx.x;
+    float acc = 0.f;
+    if (a < p.nv) {
+#pragma unroll 4
+      for (int j = 0; j < p.no; ++j) {
+        const float v = (float)x[(long long)j * p.nv + a];
+        acc += v * v;
+      }
+    }
+    const float mc = block_max(sqrtf(acc), red);
+    if (threadIdx.x == 0) atomicMax(&p.scratch[0], __float_as_uint(mc));
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    b1 = fmaxf(b1, __shfl_xor_sync(0xffffffffu, b1, o));
-    b2 = fmaxf(b2, __shfl_xor_sync(0xffffffffu, b2, o));
-  }
-  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if ((threadIdx.x & 31) == 0) { red[0][warp] = b1; red[1][warp] = b2; }
-  __syncthreads();
   if (threadIdx.x == 0) {
-    float x1 = 0.f, x2 = 0.f;
-    for (int w = 0; w < nw; ++w) { x1 = fmaxf(x1, red[0][w]); x2 = fmaxf(x2, red[1][w]); }
-    red[0][0] = x1 > 0.f ? 224.f / x1 : 1.f;
-    red[1][0] = x2 > 0.f ? 224.f / x2 : 1.f;
-    out[0] = 1.f / red[0][0];
-    out[1] = 1.f / red[1][0];
+    __threadfence();
+    last = atomicAdd(&p.scratch[3], 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  const float g1 = red[0][0], g2 = red[1][0];
-  for (int P = threadIdx.x; P < nK; P += blockDim.x) {
-    out[2 + P] = s1[P] * g1;
-    out[2 + nK + P] = s2[P] * g2;
+  if (!last) return;
+  __threadfence();
+  const float kc = __uint_as_float(__ldcg(&p.scratch[0])), kr = __uint_as_float(__ldcg(&p.scratch[1]));
+  const float kx = __uint_as_float(__ldcg(&p.scratch[2]));
+  if constexpr (!FP8) {
+    if (threadIdx.x == 0) {   // layout in tc_gemm.cuh
+      const float* fsc = p.fsc;
+      const float sx = pow2_scale(kx, 14);
+      // |Z'| <= rho_oo' ||X'[n][:][a]||, |Q'| <= ||X'[n][i][:]|| rho_ov' (Cauchy-Schwarz)
+      const float mz = pow2_scale(fsc[1] * sx * kc, 15);
+      const float mq = pow2_scale(fsc[5] * sx * kr, 15);
+      p.out[0] = sx;
+      p.out[1] = mz;
+      p.out[2] = mq;
+      p.out[3] = 1.f / (mz * fsc[0] * sx * fsc[2]);
+      p.out[4] = 1.f / (mq * sx * fsc[4] * fsc[4]);
+    }
+  } else {
+    // out[0] = 1/g1, out[1] = 1/g2, out[2 + P] = s1_P g1, out[2 + nK + P] = s2_P g2
+    float b1 = 0.f, b2 = 0.f;
+    for (int P = threadIdx.x; P < p.nK; P += 256) {
+      b1 = fmaxf(b1, p.s1[P] * p.r1[P] * kc);
+      b2 = fmaxf(b2, p.s2[P] * p.r2[P] * kr);
+    }
+    b1 = block_max(b1, red);
+    b2 = block_max(b2, red);
+    const float g1 = b1 > 0.f ? 224.f / b1 : 1.f, g2 = b2 > 0.f ? 224.f / b2 : 1.f;
+    if (threadIdx.x == 0) {
+      p.out[0] = 1.f / g1;
+      p.out[1] = 1.f / g2;
+    }
+    for (int P = threadIdx.x; P < p.nK; P += 256) {
+      p.out[2 + P] = p.s1[P] * g1;
+      p.out[2 + p.nK + P] = p.s2[P] * g2;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 5) p.scratch[threadIdx.x] = 0u;
+}
+
+// Both operand forms of the trial vectors from one read: X^T per vector
+// ([n][a][pad8(j)]) and, when sh is given, X ([n][j][pad8(b)]), as hi + lo parts of
+// X times *scale; the FP32 copy xw when given.
+template <typename T, typename E>
+__global__ void __launch_bounds__(256) k_x_split(const T* __restrict__ X, int no, int nv, int nop, int nvp,
+                                                 const float* __restrict__ scale, E* th, E* tl, E* sh, E* sl,
+                                                 float* xw) {
+  __shared__ float tile[32][33];
+  const int n = blockIdx.z, a0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const float sc = scale ? *scale : 1.f;
+#pragma unroll
+  for (int r = ty; r < 32; r += 8) {
+    const int j = j0 + r, a = a0 + tx;
+    float v = 0.f;
+    if (j < no && a < nv) {
+      v = (float)X[((long long)n * no + j) * nv + a];
+      if (xw) xw[((long long)n * no + j) * nv + a] = v;
+    }
+    v *= sc;
+    tile[r][tx] = v;
+    if (sh && j < no && a < nvp) split_store<E>(v, ((long long)n * no + j) * nvp + a, sh, sl);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = ty; r < 32; r += 8) {
+    const int a = a0 + r, j = j0 + tx;
+    if (a < nv && j < nop) split_store<E>(tile[tx][r], ((long long)n * nv + a) * nop + j, th, tl);
+  }
+}
+
+// t [K][m] -> FP16 hi + lo of s_t t^T [m][ldk], s_t the power of two with
+// max |s_t t| < 2^14 (tmax: float bits of max |t|); fac = 1 / (s_t s_ov).
+__global__ void __launch_bounds__(256) k_t_split(const float* __restrict__ t, int K, int m, int ldk,
+                                                 const unsigned* __restrict__ tmax, const float* __restrict__ s_ov,
+                                                 __half* hi, __half* lo, float* fac) {
+  const float st = pow2_scale(__uint_as_float(*tmax), 14);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *fac = 1.f / (st * *s_ov);
+  const long long tot = (long long)m * ldk;
+  for (long long e = blockIdx.x * 256ll + threadIdx.x; e < tot; e += (long long)gridDim.x * 256) {
+    const int n = (int)(e / ldk), k = (int)(e - (long long)n * ldk);
+    split_store<__half>(k < K ? t[(long long)k * m + n] * st : 0.f, e, hi, lo);
   }
 }
 
@@ -1678,15 +1768,54 @@ void tc_row_norm_max(const __nv_bfloat16* src, int rows, int nr, int nc, float* 
   TD_LAUNCH_CHECK();
 }
 
-void tc_fp8_scales(const void* X, DType xt, int m, int no, int nv, const float* s_vv, const float* rho_oo,
-                   const float* s_vo, const float* rho_ov, int nK, float* out, unsigned* kappa,
-                   cudaStream_t s) {
-  TD_CUDA(cudaMemsetAsync(kappa, 0, 3 * sizeof(unsigned), s));
-  if (xt == DType::F32) k_x_norms<float><<<m, 256, 0, s>>>(static_cast<const float*>(X), no, nv, kappa);
-  else k_x_norms<double><<<m, 256, 0, s>>>(static_cast<const double*>(X), no, nv, kappa);
+namespace {
+template <bool FP8>
+void x_prep(const void* X, DType xt, XPrep p, cudaStream_t s) {
+  p.rb = (p.no + 31) / 32;
+  p.cb = (p.nv + 255) / 256;
+  TD_REQUIRE((long long)p.m * (p.rb + p.cb) < (1ll << 31), TDDFT_ERR_ARG, "trial vectors: too many");
+  const unsigned grid = (unsigned)(p.m * (p.rb + p.cb));
+  if (xt == DType::F32) k_x_prep<float, FP8><<<grid, 256, 0, s>>>(static_cast<const float*>(X), p);
+  else k_x_prep<double, FP8><<<grid, 256, 0, s>>>(static_cast<const double*>(X), p);
   count_launch();
   TD_LAUNCH_CHECK();
-  k_fp8_mu<<<1, 256, 0, s>>>(kappa, s_vv, rho_oo, s_vo, rho_ov, nK, out);
+}
+}  // namespace
+
+void tc_fp8_scales(const void* X, DType xt, int m, int no, int nv, const float* s_vv, const float* rho_oo,
+                   const float* s_vo, const float* rho_ov, int nK, float* out, unsigned* scratch, float* xw,
+                   cudaStream_t s) {
+  x_prep<true>(X, xt, XPrep{m, no, nv, 0, 0, scratch, xw, out, nullptr, s_vv, rho_oo, s_vo, rho_ov, nK}, s);
+}
+
+void tc_x_split(const void* X, DType xt, int m, int no, int nv, TcElt et, const float* scale, void* th, void* tl,
+                void* sh, void* sl, float* xw, cudaStream_t s) {
+  const int nop = tc_pad(no), nvp = tc_pad(nv);
+  TD_REQUIRE(m <= 65535 && (nop + 31) / 32 <= 65535, TDDFT_ERR_ARG, "trial vectors: too many");
+  const dim3 grid((nvp + 31) / 32, (nop + 31) / 32, m);
+  auto go = [&](auto* x, auto* e) {
+    using E = std::remove_pointer_t<decltype(e)>;
+    k_x_split<<<grid, 256, 0, s>>>(x, no, nv, nop, nvp, scale, static_cast<E*>(th), static_cast<E*>(tl),
+                                   static_cast<E*>(sh), static_cast<E*>(sl), xw);
+  };
+  const bool f32 = xt == DType::F32;
+  if (et == TcElt::F16) {
+    if (f32) go(static_cast<const float*>(X), (__half*)nullptr);
+    else go(static_cast<const double*>(X), (__half*)nullptr);
+  } else {
+    if (f32) go(static_cast<const float*>(X), (__nv_bfloat16*)nullptr);
+    else go(static_cast<const double*>(X), (__nv_bfloat16*)nullptr);
+  }
+  count_launch();
+  TD_LAUNCH_CHECK();
+}
+
+void tc_t_split(const float* t, int K, int m, const unsigned* tmax, const float* s_ov, void* hi, void* lo, float* fac,
+                cudaStream_t s) {
+  const int ldk = tc_pad(K);
+  const long long g = std::min<long long>(((long long)m * ldk + 255) / 256, 152 * 8);
+  k_t_split<<<(unsigned)g, 256, 0, s>>>(t, K, m, ldk, tmax, s_ov, static_cast<__half*>(hi), static_cast<__half*>(lo),
+                                        fac);
   count_launch();
   TD_LAUNCH_CHECK();
 }
@@ -1705,28 +1834,9 @@ void tc_f16_tensor_scale(const float* src, long long rows, int n, float* sc, uns
   TD_LAUNCH_CHECK();
 }
 
-namespace {
-__global__ void k_inv_prod(const float* __restrict__ a, const float* __restrict__ b, float* __restrict__ out) {
-  out[0] = 1.f / (a[0] * b[0]);
-}
-}  // namespace
-
-void tc_inv_prod(const float* a, const float* b, float* out, cudaStream_t s) {
-  k_inv_prod<<<1, 1, 0, s>>>(a, b, out);
-  count_launch();
-  TD_LAUNCH_CHECK();
-}
-
 void tc_f16_product_scales(const void* X, DType xt, int m, int no, int nv, const float* fsc, float* out,
-                           unsigned* kappa, cudaStream_t s) {
-  TD_CUDA(cudaMemsetAsync(kappa, 0, 3 * sizeof(unsigned), s));
-  if (xt == DType::F32) k_x_norms<float><<<m, 256, 0, s>>>(static_cast<const float*>(X), no, nv, kappa);
-  else k_x_norms<double><<<m, 256, 0, s>>>(static_cast<const double*>(X), no, nv, kappa);
-  count_launch();
-  TD_LAUNCH_CHECK();
-  k_f16_product_scales<<<1, 1, 0, s>>>(kappa, fsc, out);
-  count_launch();
-  TD_LAUNCH_CHECK();
+                           unsigned* scratch, float* xw, cudaStream_t s) {
+  x_prep<false>(X, xt, XPrep{m, no, nv, 0, 0, scratch, xw, out, fsc, nullptr, nullptr, nullptr, nullptr, 0}, s);
 }
 
 }  // namespace tddft

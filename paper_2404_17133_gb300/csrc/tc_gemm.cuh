@@ -53,10 +53,21 @@ void tc_pad_split(const void* src, DType ts, long long rows, int n, void* hi, vo
 // K extent one CTA accumulates in FP32 to max_kb blocks of 64 elements (more
 // split-K partials, summed in a fixed order), for contractions whose K is long enough that the length of
 // the accumulation run sets the rounding error.
+// With `keep` the result stays there instead of in out, as the partial sums of the
+// K splits where these take no more than kKeepBytes:
+// result = (*scale or 1) * sum_(s < splits) part[s].
+constexpr size_t kKeepBytes = 256ull << 20;
+struct TcSum {
+  DevBuf factor;               // room for a scale of the caller's
+  DevBuf part;                 // [splits][M][N]
+  int splits = 0;
+  const float* scale = nullptr;
+};
 struct KernelProfile;
 void tc_contract(const void* Ahi, const void* Alo, int lda, int M, int pn, int Kin, const void* Bhi, const void* Blo,
                  int N, float* out, bool accumulate, TcElt et, const float* scale, int* err, cudaStream_t s,
-                 KernelProfile* prof = nullptr, double prof_flops = 0.0, double prof_bytes = 0.0, int max_kb = 0);
+                 KernelProfile* prof = nullptr, double prof_flops = 0.0, double prof_bytes = 0.0, int max_kb = 0,
+                 TcSum* keep = nullptr);
 
 // Stage-1 exchange contraction on the tensor cores, for every P and trial vector:
 //   C_P[n][i][r] = sum_(k<K) L_P[i][k] X[n][r][k],  X: [m][R][tc_pad(K)] as hi + lo,
@@ -80,11 +91,19 @@ void tc_f16_tensor_scale(const float* src, long long rows, int n, float* sc, uns
 //   stage-1 accumulators (Z' = s_oo s_x Z, Q' = s_x s_ov Q) before their FP16
 //   split, powers of two with |m Z'| < 2^15 by Cauchy-Schwarz;
 //   [3] 1 / (m_z s_oo s_x s_vv), [4] 1 / (m_q s_x s_ov^2): the factors of the
-//   K1 and K2 sums.  kappa: three device words.  No host synchronisation.
+//   K1 and K2 sums.  scratch: five device words, zero on entry and on return; xw:
+// the FP32 copy of X to write, or NULL.  No host synchronisation.
 void tc_f16_product_scales(const void* X, DType xt, int m, int no, int nv, const float* fsc, float* out,
-                           unsigned* kappa, cudaStream_t s);
-// out[0] = 1 / (a[0] * b[0]) (device scalars): the factor that removes two scales.
-void tc_inv_prod(const float* a, const float* b, float* out, cudaStream_t s);
+                           unsigned* scratch, float* xw, cudaStream_t s);
+// Operand parts of the trial vectors X [m][no][nv] (F64 or F32), times *scale (FP16;
+// NULL for BF16): th, tl [m][nv][tc_pad(no)] of X^T per vector and, unless sh is
+// NULL, sh, sl [m][no][tc_pad(nv)] of X; xw: the FP32 copy of X, or NULL.
+void tc_x_split(const void* X, DType xt, int m, int no, int nv, TcElt et, const float* scale, void* th, void* tl,
+                void* sh, void* sl, float* xw, cudaStream_t s);
+// FP16 hi + lo [m][tc_pad(K)] of s_t t^T for t [K][m], s_t the power of two with
+// max |s_t t| < 2^14, from *tmax = float bits of max |t|; *fac = 1 / (s_t *s_ov).
+void tc_t_split(const float* t, int K, int m, const unsigned* tmax, const float* s_ov, void* hi, void* lo, float* fac,
+                cudaStream_t s);
 
 // ---- FP8 (e4m3) ris exchange operands with one scale per auxiliary row P.
 // Factor rows src [rows][n1][n2] (BF16) -> dst [rows][n2][tc_pad16(n1)] e4m3
@@ -99,10 +118,10 @@ void tc_row_norm_max(const __nv_bfloat16* src, int rows, int nr, int nc, float* 
 // K1 and K2; out[2 + P] = s_vv[P] g1 and out[2 + nK + P] = s_vo[P] g2, the
 // multipliers of the stage-1 results (mu_P).  g1 = 224 / max_P(s_vv[P]
 // rho_oo[P] kappa_col), g2 likewise with s_vo, rho_ov and kappa_row, where
-// kappa_col = max ||X[n][:][a]|| and kappa_row = max ||X[n][j][:]||.  kappa:
-// device scratch of three words.  No host synchronisation.
+// kappa_col = max ||X[n][:][a]|| and kappa_row = max ||X[n][j][:]||.  scratch and xw
+// as for tc_f16_product_scales.
 void tc_fp8_scales(const void* X, DType xt, int m, int no, int nv, const float* s_vv, const float* rho_oo,
-                   const float* s_vo, const float* rho_ov, int nK, float* out, unsigned* kappa,
+                   const float* s_vo, const float* rho_ov, int nK, float* out, unsigned* scratch, float* xw,
                    cudaStream_t s);
 // Stage 1 with e4m3 hi + lo output (row pitch tc_zpad(R, 1) bytes): split of
 // mu[P] * C_P; X as BF16 hi + lo, L BF16.
@@ -114,6 +133,6 @@ void tc_stage1_fp8(const __nv_bfloat16* Xhi, const __nv_bfloat16* Xlo, int m, in
 // [pn][M][tc_zpad(Kin, 1)], B e4m3 [pn][N][tc_pad16(Kin)]; scale a device scalar.
 void tc_contract8(const unsigned char* Ahi, const unsigned char* Alo, int M, int pn, int Kin,
                   const unsigned char* B, int N, float* out, bool accumulate, const float* scale, int* err,
-                  cudaStream_t s);
+                  cudaStream_t s, TcSum* keep = nullptr);
 
 }  // namespace tddft

@@ -52,6 +52,19 @@ void scale_rows(T* X, const double* scale, int k, int n, cudaStream_t s);
 // y = a y + b x over n elements of type t (F64 or F32); y is not read when a == 0.
 void axpby(void* y, const void* x, DType t, double a, double b, long long n, cudaStream_t s);
 
+// One term of a product: (*scale or 1) * sum_(s < splits) part[s], part [splits][m*n]
+// FP32; splits = 0: absent.
+struct SumTerm {
+  const float* part = nullptr;
+  int splits = 0;
+  const float* scale = nullptr;
+};
+// out0 = d X + cj J + c1 K1 + c2 K2 and, when given, out1 = d X + c1 K1 - c2 K2
+// (FP64 arithmetic; TX = double or float).
+template <typename TX>
+void combine_sums(const TX* X, const double* d, const SumTerm& J, const SumTerm& K1, const SumTerm& K2, double cj,
+                  double c1, double c2, long long m, int n, TX* out0, TX* out1, cudaStream_t s);
+
 void cast_f64_to_f32(const double* in, float* out, long long n, cudaStream_t s);
 void cast_f32_to_f64(const float* in, double* out, long long n, cudaStream_t s);
 void cast_to_bf16(const void* in, DType tin, __nv_bfloat16* out, long long n, cudaStream_t s);
@@ -65,9 +78,6 @@ void mask_block(void* L, DType t, int rows, int n1, int n2, const unsigned char*
 void combine(const double* X, const double* delta, const void* J, const void* K1, const void* K2,
              DType tw, double c_j, double c_1, double c_2, long long m, int n, double* out,
              cudaStream_t s);
-// FP32 variant (FP32 vectors in and out, FP32 parts).
-void combine_f32(const float* X, const double* delta, const float* J, const float* K1, const float* K2,
-                 double c_j, double c_1, double c_2, long long m, int n, float* out, cudaStream_t s);
 // Sum `parts` partial buffers of n elements (type t) into the first.
 void reduce_parts(void* buf, DType t, int parts, long long n, cudaStream_t s);
 // Non-finite check: flag[0] |= 1 if any entry of X is NaN/Inf.
