@@ -16,14 +16,24 @@
 // before the final scaling.  The error of a product is 2^-56 (2^-32) of
 // max|A row| max|B row| per term, below what FP64 (FP32) accumulation leaves.
 //
-// Why: FP64 runs at 1.2 TFLOP/s on this GPU's vector units and FP32 at 75; S (S
-// + 1) / 2 FP16 products per term (28 or 10) leave up to 69 and 190 TFLOP/s.
+// Why: FP64 runs at 1.2 TFLOP/s on this GPU's vector units and FP32 at 75; 34
+// or 10 FP16 products per term leave up to 57 and 190 TFLOP/s.
 //
-// CTA = 128 x NT output tile (NT = 64 or 128: S levels of NT FP32 columns fill
-// the tensor memory), persistent over (tile, K split) items; warp 0 issues TMA
-// loads of all slices of a 32-element k-block (64-byte rows, SWIZZLE_64B), warp
-// 1 one tcgen05.mma per slice pair, warps 2-9 the run epilogue.  A slice of A
-// stays in the tensor core's operand collector while it meets all slices of B.
+// CTA = 128 x W output tile (W up to 64 or 128: LV levels of W FP32 columns fill the
+// tensor memory), persistent over (tile, K split) items; warp 0 issues TMA loads of
+// all slices of a 32-element k-block (64-byte rows, SWIZZLE_64B), warp 1 the
+// products, warps 2-9 the run epilogue, in which the tensor core waits (no tensor
+// memory is left for a second set of levels).  The slices of B follow one another
+// in shared memory and their levels in tensor memory, so one tcgen05.mma multiplies a
+// slice of A with several slices of B: N up to 256, 128 clocks, bound by the tensor
+// core; one product per pair of slices (N = 64) took 48 clocks instead of 32 to
+// fetch its operands.
+//
+// Measured, 60 x 400 orbitals, contraction of 118 rows P with 10 vectors (FP64): 787 ->
+// 610 us (MMAs alone 528), its first stage 375 -> 233; 212 rows, 13 vectors (FP32): 550
+// -> 458 and 290 -> 126.  Not faster: CTA pairs (N = 64 in a pair takes twice the
+// clocks), two half tiles whose runs end half a run apart (711 and 701: the shorter
+// products cost more than the overlap of the epilogue gains).
 //
 // Every wait on an mbarrier is bounded as in tc_gemm.cu.
 #include <algorithm>
@@ -46,14 +56,17 @@ constexpr int RUN = 8;            // k-blocks per exact accumulation run
 constexpr int EPI_WARPS = 8;
 constexpr int SL_THREADS = 64 + 32 * EPI_WARPS;
 
-template <int S> struct SCfg {
-  static constexpr int NT = S == 7 ? 64 : 128;
+// Tiles of NT columns (a multiple of 16): LV levels of NT FP32 columns are at most
+// the tensor memory.
+template <int S> constexpr int max_cols() { return S == 7 ? 64 : 128; }
+template <int S, int W> struct SCfg {
+  static constexpr int NT = W;
   // levels i + j kept: FP64 needs one beyond the slices (the six products of level 7
   // are 2^-58 of max max, 1e-15 of a result whose rows decay; without them the error
   // was 1.3e-15 against 1.2e-15 of FP64 arithmetic, with them 3.5e-16; 34 products
   // instead of 28)
   static constexpr int LV = S == 7 ? 8 : 4;
-  static constexpr int A_SLICE = SBM * SBK * 2, B_SLICE = NT * SBK * 2;
+  static constexpr int A_SLICE = SBM * SBK * 2, B_SLICE = W * SBK * 2;
   static constexpr int STAGE_BYTES = S * (A_SLICE + B_SLICE);
   static constexpr int STAGES = S == 7 ? 2 : 3;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
@@ -64,7 +77,7 @@ struct SParams {
   int M, N;             // output rows / columns
   int Kin, nab;         // k extent per P, k-blocks per P
   int total, per;       // k-blocks in all, per split (a multiple of RUN)
-  int tiles_n, tiles, items;
+  int w, tiles_n, tiles, items;   // columns per tile, tiles along N and in all, items
   const int* ea;        // exponent words of the rows of A and of B
   const int* eb;
   void* out;
@@ -89,26 +102,10 @@ __device__ __forceinline__ uint64_t sdesc64(const void* p) {
   return ((addr & 0x3FFFFull) >> 4) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
 }
 
-// Use of the A operand collector: the products of one A slice share its fetch.
-enum Collect { C_FILL, C_USE, C_LAST, C_NONE };
-template <int CO>
 __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t accum, uint32_t idesc) {
-  if constexpr (CO == C_FILL)
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n}\n" ::"r"(d), "l"(a),
-                 "l"(b), "r"(idesc), "r"(accum));
-  else if constexpr (CO == C_USE)
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n}\n" ::"r"(d), "l"(a),
-                 "l"(b), "r"(idesc), "r"(accum));
-  else if constexpr (CO == C_LAST)
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n}\n" ::"r"(d), "l"(a),
-                 "l"(b), "r"(idesc), "r"(accum));
-  else
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d), "l"(a), "l"(b), "r"(idesc),
-                 "r"(accum));
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+               " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d), "l"(a), "l"(b), "r"(idesc),
+               "r"(accum));
 }
 
 __device__ __forceinline__ void tmem_ld4(float (&v)[4], uint32_t taddr) {
@@ -122,50 +119,119 @@ __device__ __forceinline__ void tmem_ld4(float (&v)[4], uint32_t taddr) {
   v[3] = __uint_as_float(r3);
 }
 
-// Running sum of one output over the exact runs.  v[l]: the run's level sums.
+constexpr int kNotFinite = 1 << 20;   // exponent of a row that holds a non-finite value
+
+// Two FP32 operations at once.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n"
+      " mov.b64 {%0, %1}, z;\n}\n" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n sub.rn.f32x2 z, x, y;\n"
+      " mov.b64 {%0, %1}, z;\n}\n" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float b, float2 c) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %4};\n mov.b64 z, {%5, %6};\n"
+      " fma.rn.f32x2 z, x, y, z;\n mov.b64 {%0, %1}, z;\n}\n"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b), "f"(c.x), "f"(c.y));
+  return r;
+}
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+
+// Running sum of one output over the exact runs.
 template <int S> struct Acc;
 template <> struct Acc<7> {
-  long long hi, lo;   // units 2^-40 (levels 0-3) and 2^-72 (levels 4-7) of the scaled product
-  __device__ __forceinline__ void clear() { hi = 0; lo = 0; }
-  __device__ __forceinline__ void add(const float* v) {
-    hi += (long long)__float2int_rn(v[0]) * 16777216 + (long long)__float2int_rn(v[1]) * 65536 +
-          (long long)__float2int_rn(v[2]) * 256 + __float2int_rn(v[3]);
-    lo += (long long)__float2int_rn(v[4]) * 16777216 + (long long)__float2int_rn(v[5]) * 65536 +
-          (long long)__float2int_rn(v[6]) * 256 + __float2int_rn(v[7]);
+  // units 2^-40 (levels 0-3) and 2^-72 (levels 4-7) of the scaled product, less what
+  // the runs still to come will add as bias
+  long long hi, lo;
+  static constexpr long long BIAS = 0x4b400000;   // bits of 1.5 2^23
+  __device__ __forceinline__ void clear(int runs) {
+    hi = -(runs * ((BIAS << 24) + BIAS));
+    lo = -(runs * (BIAS << 8));
   }
-  // times 2^40 (each row's scale carries 2^-20)
-  __device__ __forceinline__ double value() const { return fma((double)lo, 0x1p-32, (double)hi); }
+  // The level sums v of a run for two neighbours.  Conversions to integers run at 16
+  // per clock and SM (eight per output bounded this step), so only levels 1, 2 and
+  // 4 are converted: x + 1.5 2^23 holds an integer |x| <= 2^22 in its low bits, and
+  // level 3 passes its multiples of 256 on to level 2, levels 6 and 5 theirs to 5
+  // and 4, all exactly (level 7 joins level 6 rounded at half a unit of level 6, 2^-65
+  // of max max; the products not formed weigh 2^-60).
+  static __device__ __forceinline__ void add(Acc& a, Acc& b, const float2 (&v)[8]) {
+    const float2 M = both(0x1.8p31f), m = both(0x1.8p23f);
+    const float2 h3 = sub2(add2(v[3], M), M), r3 = add2(sub2(v[3], h3), m);
+    const float2 x2 = fma2(h3, 0x1p-8f, v[2]);
+    const float2 x6 = fma2(v[7], 0x1p-8f, v[6]);
+    const float2 h6 = sub2(add2(x6, M), M), r6 = add2(sub2(x6, h6), m);
+    const float2 x5 = fma2(h6, 0x1p-8f, v[5]);
+    const float2 h5 = sub2(add2(x5, M), M), r56 = fma2(sub2(x5, h5), 256.f, r6);
+    const float2 x4 = fma2(h5, 0x1p-8f, v[4]), x0 = add2(v[0], m);
+    a.add1(x0.x, v[1].x, x2.x, r3.x, x4.x, r56.x);
+    b.add1(x0.y, v[1].y, x2.y, r3.y, x4.y, r56.y);
+  }
+  __device__ __forceinline__ void add1(float x0, float x1, float x2, float r3, float x4, float r56) {
+    hi += (long long)__float_as_int(x0) * 16777216 + (long long)__float2int_rn(x1) * 65536 +
+          (long long)__float2int_rn(x2) * 256 + (long long)__float_as_int(r3);
+    lo += (long long)__float2int_rn(x4) * 16777216 + (long long)__float_as_int(r56) * 256;
+  }
+  // The sum, times 2^40, times 2^e (scale exponents of the row and the column) by
+  // integer arithmetic with one rounding: conversions and products on the FP64 units
+  // (two per clock and SM) took 20,000 clocks per 128 x 64 tile.
+  __device__ __forceinline__ double value(int e) const {
+    if (e >= kNotFinite / 2) return __longlong_as_double(0x7ff8000000000000ll);
+    // 96 bits in three words, sign and magnitude
+    const long long h = hi + (lo >> 32);
+    uint32_t w0 = (uint32_t)lo, w1 = (uint32_t)h, w2 = (uint32_t)(h >> 32);
+    const uint32_t neg = w2 & 0x80000000u, m = (uint32_t)((int)w2 >> 31);
+    asm("add.cc.u32 %0, %3, %6;\n addc.cc.u32 %1, %4, 0;\n addc.u32 %2, %5, 0;"
+        : "=r"(w0), "=r"(w1), "=r"(w2)
+        : "r"(w0 ^ m), "r"(w1 ^ m), "r"(w2 ^ m), "r"(neg >> 31));
+    e += 63;                                   // exponent of the highest bit of w2
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      if (w2 == 0) { w2 = w1; w1 = w0; w0 = 0; e -= 32; }
+    if (w2 == 0) return 0.0;
+    const int lz = __clz(w2);
+    e -= lz;
+    const unsigned long long u =
+        (unsigned long long)__funnelshift_l(w1, w2, lz) << 32 | __funnelshift_l(w0, w1, lz);
+    const unsigned long long f = (u >> 11) + ((u >> 10) & 1);   // 53 bits, rounded
+    if (e < -1021 || e > 1022) return ldexp(neg ? -(double)f : (double)f, e - 52);
+    // the leading bit of f adds one to the exponent field
+    return __longlong_as_double((long long)(((unsigned long long)(e + 1022) << 52) + f | (unsigned long long)neg << 32));
+  }
 };
 template <> struct Acc<4> {
   float hi, lo;       // compensated sum in units 2^-16 (level 0)
-  __device__ __forceinline__ void clear() { hi = 0.f; lo = 0.f; }
-  __device__ __forceinline__ void add(const float* v) {
-    const float x = fmaf(fmaf(fmaf(v[3], 0x1p-8f, v[2]), 0x1p-8f, v[1]), 0x1p-8f, v[0]);
-    const float s = hi + x, bb = s - hi;
-    lo += (hi - (s - bb)) + (x - bb);
-    hi = s;
+  __device__ __forceinline__ void clear(int) { hi = 0.f; lo = 0.f; }
+  static __device__ __forceinline__ void add(Acc& a, Acc& b, const float2 (&v)[4]) {
+    const float2 x = fma2(fma2(fma2(v[3], 0x1p-8f, v[2]), 0x1p-8f, v[1]), 0x1p-8f, v[0]);
+    const float2 h = make_float2(a.hi, b.hi), s = add2(h, x), bb = sub2(s, h);
+    const float2 l = add2(make_float2(a.lo, b.lo), add2(sub2(h, sub2(s, bb)), sub2(x, bb)));
+    a.hi = s.x; b.hi = s.y;
+    a.lo = l.x; b.lo = l.y;
   }
   __device__ __forceinline__ float value() const { return hi + lo; }
 };
 
-// Power-of-two scale of a row from its exponent word (the largest biased
-// exponent field, or the all-ones field where the row holds a non-finite value).
+// Power-of-two scale of a row from its exponent word (the largest biased exponent
+// field, or the all-ones field where the row holds a non-finite value): FP64 as its
+// exponent, FP32 as its value.
 template <int S> __device__ __forceinline__ auto row_scale(int w);
-template <> __device__ __forceinline__ auto row_scale<7>(int w) {
-  const int E = max(w, 1);
-  if (E >= 2047) return __longlong_as_double(0x7ff8000000000000ll);
-  return E > 18 ? __longlong_as_double((long long)(E - 18) << 52) : ldexp(1.0, E - 1041);
-}
+template <> __device__ __forceinline__ auto row_scale<7>(int w) { return w >= 2047 ? kNotFinite : max(w, 1) - 1041; }
 template <> __device__ __forceinline__ auto row_scale<4>(int w) {
   const int E = max(w, 1);
   if (E >= 255) return __int_as_float(0x7fc00000);
   return E > 6 ? __int_as_float((E - 6) << 23) : ldexpf(1.f, E - 133);
 }
 
-template <int S>
+template <int S, int W>
 __global__ void __launch_bounds__(SL_THREADS, 1)
 k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, const SParams p) {
-  using C = SCfg<S>;
+  using C = SCfg<S, W>;
   using T = typename std::conditional<S == 7, double, float>::type;
   constexpr int NT = C::NT;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -221,71 +287,83 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
     for (long long j = i > C::STAGES ? i - C::STAGES : 0; j < i; ++j)
       if (!mbar_wait(&full[j % C::STAGES], (uint32_t)(j / C::STAGES) & 1u)) { atomicOr(p.err, 512); break; }
   } else if (warp == 1 && lane == 0) {
-    long long i = 0, run = 0;
+    // The instructions between the products of this one thread hold the tensor core
+    // up (with offsets computed in loops it ran at half its rate): offsets are
+    // constants, positions are counted up, nothing is divided in the loop.
+    //
+    // kind::f16 with FP16 operands, FP32 accumulator, both K-major, M = 128.  One
+    // product of slice ia of A with g consecutive slices of B (N = g W up to 256)
+    // reaches the g levels from ia + ib on: single slices (N = 64) are bound by
+    // fetching A and B from shared memory, 48 clocks instead of 32.
+    constexpr uint32_t IDESC = (1u << 4) | ((uint32_t)(SBM >> 4) << 24), NB = (uint32_t)(W >> 3) << 17;
+    constexpr int G = 256 / W < S ? 256 / W : S;   // slices of B per product; two products meet all of them
+    static_assert(2 * G >= S && C::LV <= S + 1, "slice_gemm: slices per product");
+    const uint64_t da0 = sdesc64(smem);
+    const int tail = p.Kin - (p.nab - 1) * SBK > 16 ? 2 : 1;   // 16-element K steps of a P's last k-block
+    uint32_t s = 0, ph = 0, run = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x) {
       int k0, nk;
       range(item, k0, nk);
-      const int n0 = ((item % p.tiles) % p.tiles_n) * NT;
-      const int nb = min(NT, (p.N - n0 + 15) & ~15);
-      // kind::f16 with FP16 operands, FP32 accumulator, both K-major, M = 128, N = nb
-      const uint32_t idesc = (1u << 4) | ((uint32_t)(nb >> 3) << 17) | ((uint32_t)(SBM >> 4) << 24);
-      for (int kb = k0; kb < k0 + nk && ok; kb += RUN, ++run) {
-        if (!mbar_wait(tempty, ((uint32_t)run & 1u) ^ 1u)) { atomicOr(p.err, 1024); ok = false; break; }
+      int pos = k0 % p.nab, left = 0;   // place among the k-blocks of a P, k-blocks left of the run
+      for (int b = 0; b < nk; ++b) {
+        const bool start = left == 0;
+        if (start) {
+          left = min(RUN, nk - b);
+          if (!mbar_wait(tempty, (run++ & 1u) ^ 1u)) { ok = false; break; }
+        }
+        if (!mbar_wait(&full[s], ph)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int kn = min(RUN, k0 + nk - kb);
-        for (int b = 0; b < kn; ++b, ++i) {
-          const int s = (int)(i % C::STAGES);
-          if (!mbar_wait(&full[s], (uint32_t)(i / C::STAGES) & 1u)) { atomicOr(p.err, 1024); ok = false; break; }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          unsigned char* st = smem + s * C::STAGE_BYTES;
-          const uint64_t da = sdesc64(st), db = sdesc64(st + S * C::A_SLICE);
-          const int rem = p.Kin - ((kb + b) % p.nab) * SBK;
-          const int nks = rem > 16 ? 2 : 1;   // 16-element K steps holding data
-          for (int kk = 0; kk < nks; ++kk) {
-            // a level of a run is opened by slice 0 of A, one past the slices by the last slice of B
-            const uint32_t acc = (b > 0 || kk > 0) ? 1u : 0u;
+        const uint64_t da = da0 + s * (C::STAGE_BYTES >> 4);
+        const int nks = pos == p.nab - 1 ? tail : 2;
+        for (int kk = 0; kk < nks; ++kk) {
+          // a run's levels are opened by slice 0 of A, one past the slices by the last slice of A
+          const bool first = start && kk == 0;
+          const uint64_t a0 = da + 2 * kk, b0 = a0 + S * C::A_SLICE / 16;
 #pragma unroll
-            for (int ia = 0; ia < S; ++ia) {
-              const uint64_t a = da + ((ia * C::A_SLICE + kk * 32) >> 4);
-              const int nbs = S < C::LV - ia ? S : C::LV - ia;   // slices of B that ia meets
-#pragma unroll
-              for (int ib = 0; ib < nbs; ++ib) {
-                const uint64_t bd = db + ((ib * C::B_SLICE + kk * 32) >> 4);
-                const uint32_t d = tmem + (uint32_t)((ia + ib) * NT);
-                const uint32_t ac = ia == 0 || ib == S - 1 ? acc : 1u;
-                if (nbs == 1) mma_f16<C_NONE>(d, a, bd, ac, idesc);
-                else if (ib == 0) mma_f16<C_FILL>(d, a, bd, ac, idesc);
-                else if (ib == nbs - 1) mma_f16<C_LAST>(d, a, bd, ac, idesc);
-                else mma_f16<C_USE>(d, a, bd, ac, idesc);
-              }
+          for (int j = 0; j < S; ++j) {
+            const int ia = j ? S - j : 0;                       // the longest products last
+            const uint64_t a = a0 + ia * (C::A_SLICE / 16);
+            const int nbs = S < C::LV - ia ? S : C::LV - ia;    // slices of B that ia meets
+            const int n0 = nbs < G ? nbs : G, n1 = nbs - n0;
+            const uint32_t d = tmem + (uint32_t)(ia * W);
+            if (C::LV > S && j == 1 && first) {
+              mma_f16(d, a, b0, 1u, IDESC + NB);
+              mma_f16(d + W, a, b0 + C::B_SLICE / 16, 0u, IDESC + NB);
+            } else {
+              const uint32_t ac = j == 0 && first ? 0u : 1u;
+              mma_f16(d, a, b0, ac, IDESC + n0 * NB);
+              if (n1 > 0) mma_f16(d + n0 * W, a, b0 + n0 * (C::B_SLICE / 16), ac, IDESC + n1 * NB);
             }
           }
-          mma_commit(&empty[s]);
         }
-        mma_commit(tfull);
+        mma_commit(&empty[s]);
+        if (--left == 0) mma_commit(tfull);
+        if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+        if (++pos == p.nab) pos = 0;
       }
     }
+    if (!ok) atomicOr(p.err, 1024);
   } else if (warp >= 2) {
-    constexpr int HC = NT / 2;               // columns per warp
+    constexpr int HC = W / 2;                // columns per warp
     constexpr int CH = 4;                    // columns per TMEM load
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * HC);
-    long long run = 0;
+    const int q = warp & 3, side = (warp - 2) >> 2;
+    const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(side * HC);
+    uint32_t run = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x) {
       int k0, nk;
       range(item, k0, nk);
       const int t = item % p.tiles;
-      const int m0 = (t / p.tiles_n) * SBM + q * 32, n0 = (t % p.tiles_n) * NT + half * HC;
+      const int m0 = (t / p.tiles_n) * SBM + q * 32, n0 = (t % p.tiles_n) * NT + side * HC;
       const int row = m0 + lane;
       const bool live = m0 < p.M;            // this warp has rows to read
       const int ncol = min(HC, p.N - n0);    // columns of this warp (may be <= 0)
       Acc<S> acc[HC];
 #pragma unroll
-      for (int c = 0; c < HC; ++c) acc[c].clear();
+      for (int c = 0; c < HC; ++c) acc[c].clear((nk + RUN - 1) / RUN);
       for (int kb = 0; kb < nk; kb += RUN, ++run) {
-        bool got = mbar_wait(tfull, (uint32_t)run & 1u);
+        bool got = mbar_wait(tfull, run & 1u);
         got = __all_sync(0xffffffffu, got);
         if (!got) { if (lane == 0) atomicOr(p.err, 2048); ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -295,14 +373,14 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
             if (c < ncol) {
               float v[C::LV][CH];
 #pragma unroll
-              for (int l = 0; l < C::LV; ++l) tmem_ld4(v[l], tb + (uint32_t)(l * NT + c));
+              for (int l = 0; l < C::LV; ++l) tmem_ld4(v[l], tb + (uint32_t)(l * W + c));
               asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-              for (int j = 0; j < CH; ++j) {
-                float w[C::LV];
+              for (int j = 0; j < CH; j += 2) {
+                float2 w[C::LV];
 #pragma unroll
-                for (int l = 0; l < C::LV; ++l) w[l] = v[l][j];
-                acc[c + j].add(w);
+                for (int l = 0; l < C::LV; ++l) w[l] = make_float2(v[l][j], v[l][j + 1]);
+                Acc<S>::add(acc[c + j], acc[c + j + 1], w);
               }
             }
           }
@@ -311,22 +389,38 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
         __syncwarp();
         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tempty)) : "memory");
       }
-      if (!ok || row >= p.M) continue;
-      const T sa = row_scale<S>(p.ea[row]);
+      if (!ok || !live || ncol <= 0) continue;
+      // the columns' scales, one or two per lane, dealt out by shuffles
+      decltype(row_scale<S>(0)) sb[(HC + 31) / 32];
+#pragma unroll
+      for (int j = 0; j < (HC + 31) / 32; ++j)
+        sb[j] = row_scale<S>(32 * j + lane < ncol ? p.eb[n0 + 32 * j + lane] : 0);
+      const bool inside = row < p.M;
+      const auto sa = row_scale<S>(inside ? p.ea[row] : 0);
       T* out = static_cast<T*>(p.out);
+      long long at, step = 1;
+      int cr = 0;
       if (p.scatter) {
-        out += (long long)(row / p.R) * p.rs1 + row % p.R;
-        int cq = n0 / p.C, cr = n0 - (n0 / p.C) * p.C;
-#pragma unroll
-        for (int c = 0; c < HC; ++c) {
-          if (c < ncol) out[cr * p.cs0 + cq * p.cs1] = acc[c].value() * sa * row_scale<S>(p.eb[n0 + c]);
-          if (++cr == p.C) { cr = 0; ++cq; }
-        }
+        cr = n0 % p.C;
+        at = (long long)(row / p.R) * p.rs1 + row % p.R + (long long)(n0 / p.C) * p.cs1 + cr * p.cs0;
+        step = p.cs0;
       } else {
-        out += ((long long)(item / p.tiles) * p.M + row) * p.N + n0;
+        at = ((long long)(item / p.tiles) * p.M + row) * p.N + n0;
+      }
+      const long long wrap = p.cs1 - (long long)(p.C - 1) * p.cs0;   // from the last of C columns to the next first
 #pragma unroll
-        for (int c = 0; c < HC; ++c)
-          if (c < ncol) out[c] = acc[c].value() * sa * row_scale<S>(p.eb[n0 + c]);
+      for (int c = 0; c < HC; ++c) {
+        const auto w = __shfl_sync(0xffffffffu, sb[c / 32], c & 31);
+        if (c < ncol && inside) {
+          if constexpr (S == 7) out[at] = acc[c].value(sa + w);
+          else out[at] = acc[c].value() * sa * w;
+        }
+        if (p.scatter && ++cr == p.C) {
+          cr = 0;
+          at += wrap;
+        } else {
+          at += step;
+        }
       }
     }
   }
@@ -477,6 +571,48 @@ __global__ void __launch_bounds__(256) k_slice_rows(const CutParams c) {
   }
 }
 
+// The same for rows of many groups, in segments: a CTA per row left the last wave
+// of a few hundred long rows nearly empty.  MAX: the exponents (zero on entry),
+// else the cut.  780 FP32 rows of 84,800 elements: 213 -> 179 us, 400 rows: 114 -> 101;
+// 600 FP64 rows of 47,200: 139 -> 144, 400 rows: 100 -> 102 (no gain, no loss to speak of).
+constexpr int SEG = 2048;   // groups of eight elements per CTA
+template <typename T, int S, bool MAX>
+__global__ void __launch_bounds__(256) k_slice_seg(const CutParams c) {
+  __shared__ int red[8];
+  const long long r = blockIdx.x;
+  const T* x = static_cast<const T*>(c.p) + (r / c.R) * c.rs1 + (r % c.R) * c.rs0;
+  const int n8 = c.ldk >> 3, g1 = min(c.np * n8, (int)(blockIdx.y + 1) * SEG);
+  if constexpr (MAX) {
+    int E = 0;
+#pragma unroll 4
+    for (int g = blockIdx.y * SEG + threadIdx.x; g < g1; g += 256) {
+      const int P = g / n8, k0 = (g - P * n8) * 8;
+      T v[8];
+      load8(x + P * c.ps + k0, c.K - k0, c.vec, v);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) E = max(E, exp_field(v[j]));
+    }
+    E = __reduce_max_sync(0xffffffffu, E);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = E;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int w = 1; w < 8; ++w) E = max(E, red[w]);
+      atomicMax(&c.exps[r], E);
+    }
+  } else {
+    const int E = c.exps[r];
+    const long long slice = (long long)c.rows * c.np * c.ldk;
+#pragma unroll 2
+    for (int g = blockIdx.y * SEG + threadIdx.x; g < g1; g += 256) {
+      const int P = g / n8, k0 = (g - P * n8) * 8;
+      T v[8];
+      load8(x + P * c.ps + k0, c.K - k0, c.vec, v);
+      store_slices<T, S>(v, E, c.dst + cut_dst(c, r, P) + k0, slice);
+    }
+  }
+}
+
 // Rows contiguous across r (transposed operands).  Exponents: one CTA per 32
 // rows and group of P, warps over k; exps must be zero on entry.
 template <typename T>
@@ -542,16 +678,32 @@ CUtensorMap slice_map(const SliceOperand& o, const void* parts, int box_rows) {
   return tc_map_f16_4d(parts, dims, strides, box, 64);
 }
 
-template <int S>
-void launch_mma(const SliceOperand& A, const void* Ap, const SliceOperand& B, const void* Bp, SParams p, int splits,
-                cudaStream_t s) {
-  using C = SCfg<S>;
-  const CUtensorMap ma = slice_map(A, Ap, SBM), mb = slice_map(B, Bp, C::NT);
-  p.items = p.tiles * splits;
-  ensure_smem((const void*)k_slice_mma<S>, C::SMEM_BYTES);
-  k_slice_mma<S><<<std::min(p.items, sm_count()), SL_THREADS, C::SMEM_BYTES, s>>>(ma, mb, p);
+template <int S, int W>
+void launch_cols(const SliceOperand& A, const void* Ap, const SliceOperand& B, const void* Bp, const SParams& p,
+                 cudaStream_t s) {
+  using C = SCfg<S, W>;
+  const CUtensorMap ma = slice_map(A, Ap, SBM), mb = slice_map(B, Bp, W);
+  ensure_smem((const void*)k_slice_mma<S, W>, C::SMEM_BYTES);
+  k_slice_mma<S, W><<<std::min(p.items, sm_count()), SL_THREADS, C::SMEM_BYTES, s>>>(ma, mb, p);
   count_launch();
   TD_LAUNCH_CHECK();
+}
+
+void launch_mma(const SliceOperand& A, const void* Ap, const SliceOperand& B, const void* Bp, SParams p, int splits,
+                cudaStream_t s) {
+  p.items = p.tiles * splits;
+  if (A.t == DType::F64) {
+    if (p.w <= 16) launch_cols<7, 16>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 32) launch_cols<7, 32>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 48) launch_cols<7, 48>(A, Ap, B, Bp, p, s);
+    else launch_cols<7, 64>(A, Ap, B, Bp, p, s);
+  } else {
+    if (p.w <= 32) launch_cols<4, 32>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 64) launch_cols<4, 64>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 96) launch_cols<4, 96>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 112) launch_cols<4, 112>(A, Ap, B, Bp, p, s);
+    else launch_cols<4, 128>(A, Ap, B, Bp, p, s);
+  }
 }
 
 template <int S>
@@ -564,7 +716,12 @@ SParams make_params(const SliceOperand& A, const int* Ae, const SliceOperand& B,
   p.nab = (A.K + SBK - 1) / SBK;
   p.total = p.nab * A.np;
   p.per = p.total;
-  p.tiles_n = (p.N + SCfg<S>::NT - 1) / SCfg<S>::NT;
+  // the fewest tiles, of equal width (rounded up to the next instance by launch_mma)
+  p.tiles_n = (p.N + max_cols<S>() - 1) / max_cols<S>();
+  p.w = (p.N + p.tiles_n - 1) / p.tiles_n;
+  constexpr int widths[2][5] = {{16, 32, 48, 64, 64}, {32, 64, 96, 112, 128}};
+  for (int w : widths[S == 7 ? 0 : 1])
+    if (w >= p.w) { p.w = w; break; }
   const long long tiles = (long long)p.tiles_n * ((p.M + SBM - 1) / SBM);
   TD_REQUIRE(tiles < (1 << 28) && (long long)p.nab * A.np < (1 << 28), TDDFT_ERR_ARG, "slice_gemm: problem too large");
   p.tiles = (int)tiles;
@@ -585,7 +742,14 @@ void cut_t(const SliceOperand& o, const CutParams& c, cudaStream_t s) {
   if (o.ks == 1) {
     // threads per row by its groups of eight elements
     const long long groups = (long long)o.np * (tc_pad(o.K) / 8);
-    if (groups > 256) k_slice_rows<T, S, 256><<<o.rows, 256, 0, s>>>(c);
+    const long long segs = (groups + SEG - 1) / SEG;
+    if (segs > 2 && segs <= 65535) {
+      TD_CUDA(cudaMemsetAsync(c.exps, 0, (size_t)o.rows * 4, s));
+      const dim3 grid(o.rows, (unsigned)segs);
+      k_slice_seg<T, S, true><<<grid, 256, 0, s>>>(c);
+      k_slice_seg<T, S, false><<<grid, 256, 0, s>>>(c);
+      count_launch();
+    } else if (groups > 256) k_slice_rows<T, S, 256><<<o.rows, 256, 0, s>>>(c);
     else if (groups > 16) k_slice_rows<T, S, 32><<<(o.rows + 7) / 8, 256, 0, s>>>(c);
     else k_slice_rows<T, S, 8><<<(o.rows + 31) / 32, 256, 0, s>>>(c);
     count_launch();
@@ -631,8 +795,7 @@ void slice_gemm_scatter(const SliceOperand& A, const void* Ap, const int* Ae, co
   p.rs1 = sc.rs1;
   p.cs0 = sc.cs0;
   p.cs1 = sc.cs1;
-  if (f64) launch_mma<7>(A, Ap, B, Bp, p, 1, s);
-  else launch_mma<4>(A, Ap, B, Bp, p, 1, s);
+  launch_mma(A, Ap, B, Bp, p, 1, s);
 }
 
 void slice_gemm(const SliceOperand& A, const void* Ap, const int* Ae, const SliceOperand& B, const void* Bp,
@@ -651,8 +814,7 @@ void slice_gemm(const SliceOperand& A, const void* Ap, const int* Ae, const Slic
   DevBuf part;
   if (!direct) part = DevBuf((size_t)splits * MN * dtype_size(A.t), s);
   p.out = direct ? C : part.p;
-  if (f64) launch_mma<7>(A, Ap, B, Bp, p, splits, s);
-  else launch_mma<4>(A, Ap, B, Bp, p, splits, s);
+  launch_mma(A, Ap, B, Bp, p, splits, s);
   if (direct) return;
   const unsigned g = (unsigned)std::min<long long>((MN + 255) / 256, 152 * 16);
   if (f64) k_slice_sum<double><<<g, 256, 0, s>>>(part.as<double>(), splits, MN, (double*)C, beta);
