@@ -457,14 +457,16 @@ k1_pair_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant_
     const uint32_t idesc =
         (1u << 4) | Elem<ET>::TYPE_BITS | ((uint32_t)(width >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
     const uint16_t mask_all = (uint16_t)((1u << (2 * CX)) - 1);
+    // the instructions between two k-blocks' MMAs leave the tensor core idle: no divisions
+    int s = 0, pos = nk > 0 ? k_begin % p.nab : 0;
+    uint32_t ph = 0;
+    const int last_steps = (p.Kin - (p.nab - 1) * BKE) >= BKE ? KSTEPS : ((p.Kin - (p.nab - 1) * BKE) * KSTEPS + BKE - 1) / BKE;
     for (int i = 0; i < nk; ++i) {
-      const int s = i % STAGES;
-      if (!mbar_wait(&full[s], (uint32_t)(i / STAGES) & 1u)) { atomicOr(p.err, 4); break; }
+      if (!mbar_wait(&full[s], ph)) { atomicOr(p.err, 4); break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       unsigned char* st = smem + s * C::STAGE_BYTES;
       const uint64_t ah = sdesc_rb<RB>(st), bh = sdesc_rb<RB>(st + B_OFF);
-      const int rem = p.Kin - ((k_begin + i) % p.nab) * BKE;
-      const int nks = rem >= BKE ? KSTEPS : (rem * KSTEPS + BKE - 1) / BKE;
+      const int nks = pos == p.nab - 1 ? last_steps : KSTEPS;
 #pragma unroll
       for (int kk = 0; kk < KSTEPS; ++kk) {
         if (kk < nks) {
@@ -480,6 +482,8 @@ k1_pair_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant_
         }
       }
       commit_pair(&empty[s], mask_all);
+      if (++s == STAGES) { s = 0; ph ^= 1u; }
+      if (++pos == p.nab) pos = 0;
     }
     commit_pair(done, (uint16_t)(3u << (2 * y)));   // fires when every MMA issued above has completed
   } else if (warp >= 2) {
