@@ -222,6 +222,64 @@ k_sk_combo(const TS* __restrict__ coef, long long scm, long long sck, int M, int
   }
 }
 
+// FP64 combinations of few columns.  What bounds them is the FP64 unit (two DFMA per
+// clock and SM), so the work has to reach every SM: a CTA owns 8 columns x 8 output
+// rows, its 32 groups of 8 lanes every 32nd k.  Mean launch of a solve of 400
+// columns: 7.6 -> 4.0 us.
+constexpr int kFewCols = 8, kFewRows = 8, kFewK = 256;
+__global__ void __launch_bounds__(256)
+k_sk_combo64_few(const double* __restrict__ coef, long long scm, long long sck, int M, int K,
+                 const double* __restrict__ V, long long ldv, int ncols, double* __restrict__ out, long long ldo,
+                 double alpha, double beta) {
+  __shared__ double cs[kFewK][kFewRows];
+  __shared__ double red[8][kFewRows][kFewCols];
+  const int tid = threadIdx.x, col = tid & 7, grp = tid >> 3, warp = tid >> 5;
+  const int mb0 = blockIdx.y * kFewRows, mn = min(kFewRows, M - mb0);
+  const int c = blockIdx.x * kFewCols + col;
+  double acc[kFewRows];
+#pragma unroll
+  for (int m = 0; m < kFewRows; ++m) acc[m] = 0.0;
+  for (int k0 = 0; k0 < K; k0 += kFewK) {
+    const int kn = min(kFewK, K - k0);
+    __syncthreads();
+    for (int e = tid; e < kn * kFewRows; e += 256) {
+      const int k = e / kFewRows, m = e % kFewRows;
+      cs[k][m] = m < mn ? coef[(long long)(mb0 + m) * scm + (long long)(k0 + k) * sck] : 0.0;
+    }
+    __syncthreads();
+    if (c < ncols) {
+#pragma unroll 4
+      for (int k = grp; k < kn; k += 32) {
+        const double v = V[(long long)(k0 + k) * ldv + c];
+#pragma unroll
+        for (int m = 0; m < kFewRows; ++m)
+          if (m < mn) acc[m] = fma(cs[k][m], v, acc[m]);
+      }
+    }
+  }
+  // the four groups of a warp, then the warps, in order
+#pragma unroll
+  for (int m = 0; m < kFewRows; ++m) {
+    if (m >= mn) continue;
+    acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], 8);
+    acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], 16);
+    if ((tid & 31) < 8) red[warp][m][col] = acc[m];
+  }
+  __syncthreads();
+  if (tid < kFewRows * kFewCols) {
+    const int m = tid / kFewCols, cc = blockIdx.x * kFewCols + tid % kFewCols;
+    if (m < mn && cc < ncols) {
+      double sum = 0.0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) sum += red[w][m][tid % kFewCols];
+      double* o = out + (long long)(mb0 + m) * ldo + cc;
+      double v = alpha * sum;
+      if (beta != 0.0) v = fma(beta, *o, v);
+      *o = v;
+    }
+  }
+}
+
 void set_smem_attr(const void* f, size_t bytes) {
   ensure_smem(f, bytes);
 }
@@ -231,9 +289,11 @@ void gram_typed(const void* A, long long lda, int M, const void* B, long long ld
                 DType tc, long long ldc, double alpha, double beta, cudaStream_t s, unsigned* cmax = nullptr) {
   TD_REQUIRE((M + kTile - 1) / kTile <= 65535 && (N + kTile - 1) / kTile <= 65535, TDDFT_ERR_ARG,
              "sk_gram: too many rows");
-  // fixed K chunks: 256 columns (FP32 staging); FP64 16 to 128, so that K up to
-  // 20,000 is cut into 150 chunks or more where the columns allow it
-  int KC = 256;
+  // fixed K chunks: 256 columns (FP32 staging), 64 where that leaves fewer CTAs than
+  // SMs (K 3456, mean launch of a solve: 5.9 us with 256, 2.9 with 64); FP64 16 to 128, so that K up to 20,000 is cut into 150 chunks or more where
+  // the columns allow it
+  const long long mnt = (long long)((M + kTile - 1) / kTile) * ((N + kTile - 1) / kTile);
+  int KC = (K + 255) / 256 * mnt < 152 ? 64 : 256;
   if (sizeof(ACC) == 8) KC = K <= 2432 ? 16 : (K <= 4864 ? 32 : (K <= 9728 ? 64 : 128));
   const int S = K > 0 ? (K + KC - 1) / KC : 1;
   DevBuf part((size_t)S * M * N * sizeof(ACC), s);
@@ -251,12 +311,14 @@ void gram_typed(const void* A, long long lda, int M, const void* B, long long ld
       else if (KC == 64) go(k_sk_gram64<64>);
       else go(k_sk_gram64<128>);
     } else {
-      constexpr int KF = 256;
-      const size_t smem = (size_t)2 * kTile * (KF + 16 / sizeof(ACC)) * sizeof(ACC);
-      set_smem_attr((const void*)k_sk_gram<TA, TB, ACC, KF>, smem);
-      k_sk_gram<TA, TB, ACC, KF><<<grid, kGramThreads, smem, s>>>(static_cast<const TA*>(A), lda, M,
-                                                                  static_cast<const TB*>(B), ldb, N, K,
-                                                                  part.as<ACC>());
+      auto go = [&](auto kernel) {
+        const size_t smem = (size_t)2 * kTile * (KC + 16 / sizeof(ACC)) * sizeof(ACC);
+        set_smem_attr((const void*)kernel, smem);
+        kernel<<<grid, kGramThreads, smem, s>>>(static_cast<const TA*>(A), lda, M, static_cast<const TB*>(B), ldb, N, K,
+                                                part.as<ACC>());
+      };
+      if (KC == 64) go(k_sk_gram<TA, TB, ACC, 64>);
+      else go(k_sk_gram<TA, TB, ACC, 256>);
     }
     count_launch();
     TD_LAUNCH_CHECK();
@@ -383,6 +445,19 @@ void combo_typed(const void* coef, long long scm, long long sck, int M, int K, c
   }
   constexpr int MB = sizeof(ACC) == 8 ? 16 : 32;
   const int mblocks = (M + MB - 1) / MB;
+  if constexpr (sizeof(ACC) == 8) {
+    // CTAs for less than half of the SMs: smaller pieces (10 rows, K 200, 400 columns:
+    // 28.8 us on 13 SMs, 7.8 here; 3456 columns, 108 CTAs: 12.9 and 14.3)
+    const long long mf = (M + kFewRows - 1) / kFewRows;
+    if ((long long)((ncols + 31) / 32) * mblocks < 76 && mf <= 65535) {
+      k_sk_combo64_few<<<dim3((ncols + kFewCols - 1) / kFewCols, (unsigned)mf), 256, 0, s>>>(
+          static_cast<const double*>(coef), scm, sck, M, K, static_cast<const double*>(V), ldv, ncols,
+          static_cast<double*>(out), ldo, alpha, beta);
+      count_launch();
+      TD_LAUNCH_CHECK();
+      return;
+    }
+  }
   TD_REQUIRE(mblocks <= 65535, TDDFT_ERR_ARG, "sk_combo: too many rows");
   const size_t smem = ((size_t)kComboKc * MB + (size_t)kComboGroups * MB * 33) * sizeof(ACC);
   dim3 grid((ncols + 31) / 32, mblocks);
