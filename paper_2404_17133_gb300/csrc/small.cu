@@ -807,80 +807,105 @@ __device__ __forceinline__ unsigned pivot_key(double v, int i) {
 // Gaussian elimination with partial pivoting on the augmented matrix [M | b]
 // held in shared memory (n rows, row stride ld >= n + 1, compute type T), then
 // back substitution; the solution replaces column n (in the original row order).
-// Rows are not moved: ord[] (shared, >= n ints) records the pivot rows; the
-// update of a step collects the next pivot as a maximum of keys, so that a step
-// is one barrier and one pass over the trailing rows.  Called by all threads of
-// the CTA.  (With a pivot search by one warp and a second barrier a step took 1300
-// cycles for n = 100 in FP32, with a division per warp 2600 in FP64; mean launch of
-// the FP64 inner solves, n up to 60: 120 -> 68 us.)
+// Rows are not moved: ord[] (shared, >= n ints) records the pivot rows.  Called by
+// all threads of the CTA (two warps or more).
+//
+// What bounds a step is its chain: update of the next column, pivot, reciprocal,
+// multipliers (700 clocks in FP64).  So warp 0 goes through it for step k + 1 while
+// the other warps form the rest of step k's update, one barrier a step.  (With the
+// chain between two barriers, FP64, or inside the update, FP32, the mean launch of
+// the FP64 inner solves, n up to 60, took 68 us, 52 now; of the paired FP32 solves,
+// n up to 120, 66 and 46.)
 template <typename T>
 __device__ void lu_solve_smem(T* A, int ld, int n, int* ord, T* y) {
-  __shared__ T pinv[kSmallMax];          // reciprocal pivots
-  __shared__ unsigned key[3];            // pivot keys of steps k, k + 1, k + 2
-  __shared__ int act[kSmallMax];         // FP64: rows not yet pivots
+  __shared__ T pinv[kSmallMax];             // reciprocal pivots
+  __shared__ T mult[2][kSmallMax];          // multipliers of steps k, k + 1
+  __shared__ int act[2][kSmallMax];         // their rows (not yet pivots)
+  __shared__ unsigned recip[kSmallMax + 2]; // ceil(2^32 / w): e / w = __umulhi(e, recip[w]) for e w < 2^32
+  constexpr int R = (kSmallMax + 31) / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  if (tid < 3) key[tid] = 0u;
-  for (int i = tid; i < n; i += blockDim.x) act[i] = i;
-  __syncthreads();
-  if (tid < n) atomicMax(&key[0], pivot_key(A[tid * ld], tid));
-  if constexpr (sizeof(T) == 4) {
-    unsigned used = 0u;                  // bit t: row warp + t nw has been a pivot
-    for (int k = 0; k < n; ++k) {
-      __syncthreads();
-      const int bi = 255 - (int)(key[k % 3] & 255u);
-      const T* prow = A + bi * ld;
-      T piv = prow[k];
-      if (piv == T(0)) piv = T(1e-30);
-      const T inv = fast_rcp(piv);
-      if (tid == 0) {
-        key[(k + 2) % 3] = 0u;
-        ord[k] = bi;
-        pinv[k] = inv;
-      }
-#pragma unroll 2
-      for (int t = 0; warp + t * nw < n; ++t) {
-        const int i = warp + t * nw;
-        if (i == bi) used |= 1u << t;
-        if ((used >> t) & 1u) continue;
-        T* row = A + i * ld;
-        const T l = row[k] * inv;
-        for (int j = k + 1 + lane; j <= n; j += 32) {
-          const T v = row[j] - l * prow[j];
-          row[j] = v;
-          if (j == k + 1 && j < n) atomicMax(&key[(k + 1) % 3], pivot_key(v, i));
+  if constexpr (sizeof(T) == 8)
+    for (int w = 2 + tid; w <= n; w += blockDim.x) recip[w] = 0xffffffffu / (unsigned)w + 1u;
+  // warp 0: column k of the rows in list `from` (m of them; subtract: step k - 1's
+  // update first), its pivot and multipliers, the rows left in list `to`
+  auto pivot = [&](int k, int m, const int* from, int* to, const T* l, T* lnext, bool subtract) {
+    T v[R];
+    int row[R];
+    unsigned best = 0u;
+    const T pk = subtract ? A[ord[k - 1] * ld + k] : T(0);
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const int e = t * 32 + lane;
+      if (e < m) {
+        row[t] = from ? from[e] : e;
+        T* q = A + row[t] * ld + k;
+        v[t] = *q;
+        if (subtract) {
+          v[t] -= l[e] * pk;
+          *q = v[t];
         }
+        best = max(best, pivot_key(v[t], row[t]));
       }
     }
-  } else {
-    // the FP64 unit takes as long for one lane as for 32: multipliers first, then
-    // the trailing elements dealt to the lanes row after row
-    for (int k = 0; k < n; ++k) {
-      __syncthreads();
-      const int bi = 255 - (int)(key[k % 3] & 255u);
-      const T* prow = A + bi * ld;
-      const int m = n - k - 1, w = m + 1;
-      if (warp == 0) {
-        T piv = prow[k];
-        if (piv == T(0)) piv = T(1e-30);
-        const T inv = fast_rcp(piv);
-        // remove the pivot row from the list (the last one takes its place)
-        for (int t = lane; t <= m; t += 32)
-          if (act[t] == bi) act[t] = act[m];
-        if (lane == 0) {
-          key[(k + 2) % 3] = 0u;
-          ord[k] = bi;
-          pinv[k] = inv;
-        }
-        __syncwarp();
-        for (int t = lane; t < m; t += 32) A[act[t] * ld + k] *= inv;
+    best = __reduce_max_sync(0xffffffffu, best);
+    const int bi = 255 - (int)(best & 255u);
+    // the pivot's place in the list and its value
+    int at = -1;
+    T piv = T(0);
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const bool hit = t * 32 + lane < m && row[t] == bi;
+      const unsigned who = __ballot_sync(0xffffffffu, hit);
+      if (who) {
+        const int src = __ffs(who) - 1;
+        at = t * 32 + src;
+        piv = __shfl_sync(0xffffffffu, v[t], src);
       }
-      __syncthreads();
-      for (int idx = tid; idx < m * w; idx += blockDim.x) {
-        const int t = idx / w, j = k + 1 + idx - t * w, i = act[t];
-        T* row = A + i * ld;
-        const T v = row[j] - row[k] * prow[j];
-        row[j] = v;
-        if (j == k + 1 && j < n) atomicMax(&key[(k + 1) % 3], pivot_key(v, i));
+    }
+    if (piv == T(0)) piv = T(1e-30);
+    const T inv = fast_rcp(piv);
+    if (lane == 0) {
+      ord[k] = bi;
+      pinv[k] = inv;
+    }
+    // the last row of the list takes the pivot's place
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const int e = t * 32 + lane;
+      if (e < m && e != at) {
+        const int o = e == m - 1 ? at : e;
+        lnext[o] = v[t] * inv;
+        to[o] = row[t];
+      }
+    }
+  };
+  __syncthreads();
+  if (warp == 0) pivot(0, n, nullptr, act[0], nullptr, mult[0], false);
+  for (int k = 0; k + 1 < n; ++k) {
+    __syncthreads();
+    const int m = n - k - 1;
+    const int* rows = act[k & 1];
+    const T* l = mult[k & 1];
+    if (warp == 0) {
+      pivot(k + 1, m, rows, act[(k + 1) & 1], l, mult[(k + 1) & 1], true);
+    } else {
+      const T* prow = A + ord[k] * ld;
+      const int j0 = k + 2, w = n + 1 - j0;          // columns j0 .. n
+      if constexpr (sizeof(T) == 4) {
+        for (int t = warp - 1; t < m; t += nw - 1) {
+          T* row = A + rows[t] * ld;
+          const T lt = l[t];
+          for (int j = j0 + lane; j <= n; j += 32) row[j] -= lt * prow[j];
+        }
+      } else {
+        // the FP64 unit takes as long for one lane as for 32: the elements are dealt to
+        // the lanes row after row
+        const unsigned rw = recip[max(w, 2)];
+        for (int e = tid - 32; e < m * w; e += blockDim.x - 32) {
+          const int t = w > 1 ? (int)__umulhi((unsigned)e, rw) : e, j = j0 + e - t * w;
+          T* row = A + rows[t] * ld;
+          row[j] -= l[t] * prow[j];
+        }
       }
     }
   }
