@@ -497,12 +497,14 @@ __device__ __forceinline__ void cp_piece(void* dst, const void* src, int bytes) 
 // rows x RN vectors: 13 16-byte shared-memory loads feed 160 FMAs (RN = 5),
 // accumulated for even and odd k apart (packed FMAs), so a sum runs over at most
 // 1/8 of the chunk (<= 256 terms) before the chunk's eight are added in order.
-// cp.async keeps three stages of 64 k in flight.  n_ov 202,500, 1350 BF16 rows, 20
-// vectors: 992 -> 434 us (25 TFLOP/s); n_ov 24,000, 2000 rows, 20 vectors: 149 -> 83.
-constexpr int kTallRows = 128, kTallK = 64, kTallStages = 3, kTallChunk = 2048;
+// cp.async keeps two (FP32) or three stages of 64 k in flight, and two CTAs share an
+// SM up to 20 vectors.  n_ov 202,500, 1350 BF16 rows, 20 vectors: 365 us (992 by the
+// skinny product, 433 with one CTA per SM); n_ov 24,000, 2000 FP32 rows: 71 (149, 83).
+constexpr int kTallRows = 128, kTallK = 64, kTallChunk = 2048;
 template <typename TA> struct TallCfg {
   static constexpr int LDA = kTallK + (sizeof(TA) == 4 ? 4 : 8);   // elements: rows skewed over the banks
-  static constexpr int LDB = kTallK + 4;
+  static constexpr int LDB = kTallK + 8;
+  static constexpr int STAGES = sizeof(TA) == 4 ? 2 : 3;          // two CTAs per SM for up to 20 vectors
   static constexpr int A_BYTES = kTallRows * LDA * (int)sizeof(TA);
   static int stage_bytes(int rn) { return A_BYTES + 4 * rn * LDB * 4; }
 };
@@ -520,12 +522,12 @@ __device__ __forceinline__ void quad(const __nv_bfloat16* p, float2& a, float2& 
 
 // PA, PX: bytes that the rows of A and of the vectors are aligned to.
 template <typename TA, int RN, int PA, int PX>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, RN <= 5 ? 2 : 1)
 k_tall_gram(const TA* __restrict__ A, int M, const float* __restrict__ B, int N, int K, int chunk,
             float* __restrict__ part) {
   using C = TallCfg<TA>;
   constexpr int NT = 4 * RN, EA = PA / (int)sizeof(TA), EX = PX / 4;   // elements per piece
-  constexpr int STAGE = C::A_BYTES + NT * C::LDB * 4;
+  constexpr int STAGE = C::A_BYTES + NT * C::LDB * 4, kTallStages = C::STAGES;
   extern __shared__ __align__(16) unsigned char tall_raw[];
   const int tid = threadIdx.x;
   const int m0 = blockIdx.x * kTallRows, n0 = blockIdx.z * NT;
@@ -568,8 +570,9 @@ k_tall_gram(const TA* __restrict__ A, int M, const float* __restrict__ B, int N,
     const unsigned char* base = tall_raw + (st % kTallStages) * STAGE;
     const TA* As = reinterpret_cast<const TA*>(base) + rg * C::LDA;
     const float* Bs = reinterpret_cast<const float*>(base + C::A_BYTES) + cg * C::LDB;
+    // BF16: rows 8 apart share banks, so every second eight take the neighbouring k
 #pragma unroll 2
-    for (int q = kg; q < kTallK / 4; q += 4) {
+    for (int q = sizeof(TA) == 2 ? kg ^ (rg >> 3) : kg; q < kTallK / 4; q += 4) {
       float2 b0[RN], b1[RN];
 #pragma unroll
       for (int j = 0; j < RN; ++j) quad(Bs + 4 * j * C::LDB + 4 * q, b0[j], b1[j]);
@@ -608,58 +611,78 @@ k_tall_gram(const TA* __restrict__ A, int M, const float* __restrict__ B, int N,
 
 // out[n][c] = sum_P t[P][n] V[P][c] for up to RN vectors in one pass over V: a lane
 // owns four columns, the CTA's eight warps every eighth P (the next eight loads
-// in flight while eight are used), and their sums are added in order.  t is
-// staged as pairs (t, t) for packed FMAs.
+// in flight while eight are used), and their sums are added in order.  The packed
+// FMAs hold two vectors: (t_n, t_n+1) comes from shared memory as it is, four at a
+// load, and only the four elements of V are doubled; the loads in flight stay as
+// stored, so that two CTAs fit an SM (one CTA, pairs of columns and doubled t: 580 us
+// for 1350 BF16 rows of 202,500 and 20 vectors, 321 now).
 constexpr int kTallKc = 256;
+template <typename TV> struct Quad;
+template <> struct Quad<float> { using raw = float4; };
+template <> struct Quad<__nv_bfloat16> { using raw = uint2; };
 template <typename TV, int RN>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 k_tall_combo(const float* __restrict__ t, int N, int K, const TV* __restrict__ V, int ncols, float* __restrict__ out) {
+  static_assert(RN % 4 == 0, "vectors in fours");
   extern __shared__ __align__(16) unsigned char tallc_raw[];
-  float2* cs = reinterpret_cast<float2*>(tallc_raw);      // [kTallKc][RN]
+  float* cs = reinterpret_cast<float*>(tallc_raw);        // [kTallKc][RN]
   float* red = reinterpret_cast<float*>(tallc_raw);       // later: [4][RN][132]
   const int tid = threadIdx.x, lane = tid & 31, g = tid >> 5;
   const int n0 = blockIdx.y * RN;
   const int c0 = blockIdx.x * 128 + lane * 4;
   const bool live = c0 < ncols;
-  float2 a0[RN], a1[RN];
+  float2 acc[RN / 2][4];
 #pragma unroll
-  for (int j = 0; j < RN; ++j) a0[j] = a1[j] = make_float2(0.f, 0.f);
-  constexpr int U = 8;
-  float2 v0[U], v1[U], w0[U], w1[U];
-  auto load = [&](int k0, float2 (&x0)[U], float2 (&x1)[U]) {
+  for (int j = 0; j < RN / 2; ++j)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[j][c] = make_float2(0.f, 0.f);
+  using Raw = typename Quad<TV>::raw;
+  constexpr int U = sizeof(TV) == 2 ? 8 : 4;
+  Raw v[U], w[U];
+  auto load = [&](int k0, Raw (&x)[U]) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int k = k0 + g + 8 * u;
-      if (live && k < K) quad(V + (long long)k * ncols + c0, x0[u], x1[u]);
-      else x0[u] = x1[u] = make_float2(0.f, 0.f);
+      x[u] = Raw{};
+      if (live && k < K) x[u] = *reinterpret_cast<const Raw*>(V + (long long)k * ncols + c0);
     }
   };
-  auto use = [&](int k, const float2 (&x0)[U], const float2 (&x1)[U]) {   // k: row within the staged block
+  auto use = [&](int k, const Raw (&x)[U]) {   // k: row within the staged block
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float2* c = cs + (k + g + 8 * u) * RN;
+      const float4* c = reinterpret_cast<const float4*>(cs + (k + g + 8 * u) * RN);
+      float2 x0, x1;
+      quad(reinterpret_cast<const TV*>(&x[u]), x0, x1);
+      const float2 e0 = make_float2(x0.x, x0.x), e1 = make_float2(x0.y, x0.y);
+      const float2 e2 = make_float2(x1.x, x1.x), e3 = make_float2(x1.y, x1.y);
 #pragma unroll
-      for (int j = 0; j < RN; ++j) {
-        const float2 w = c[j];
-        fma2(a0[j], w, x0[u]);
-        fma2(a1[j], w, x1[u]);
+      for (int j = 0; j < RN / 4; ++j) {
+        const float4 q = c[j];
+        const float2 qa = make_float2(q.x, q.y), qb = make_float2(q.z, q.w);
+        fma2(acc[2 * j][0], qa, e0);
+        fma2(acc[2 * j][1], qa, e1);
+        fma2(acc[2 * j][2], qa, e2);
+        fma2(acc[2 * j][3], qa, e3);
+        fma2(acc[2 * j + 1][0], qb, e0);
+        fma2(acc[2 * j + 1][1], qb, e1);
+        fma2(acc[2 * j + 1][2], qb, e2);
+        fma2(acc[2 * j + 1][3], qb, e3);
       }
     }
   };
-  load(0, v0, v1);
+  load(0, v);
   for (int k0 = 0; k0 < K; k0 += kTallKc) {
     __syncthreads();
     for (int e = tid; e < kTallKc * RN; e += 256) {
       const int k = e / RN, j = e - k * RN;
-      const float v = k0 + k < K && n0 + j < N ? t[(long long)(k0 + k) * N + n0 + j] : 0.f;
-      cs[e] = make_float2(v, v);
+      cs[e] = k0 + k < K && n0 + j < N ? t[(long long)(k0 + k) * N + n0 + j] : 0.f;
     }
     __syncthreads();
-    for (int k = 0; k < kTallKc && k0 + k < K; k += 128) {
-      load(k0 + k + 64, w0, w1);
-      use(k, v0, v1);
-      load(k0 + k + 128, v0, v1);
-      use(k + 64, w0, w1);
+    for (int k = 0; k < kTallKc && k0 + k < K; k += 16 * U) {
+      load(k0 + k + 8 * U, w);
+      use(k, v);
+      load(k0 + k + 16 * U, v);
+      use(k + 8 * U, w);
     }
   }
   // sums of the warps g and g + 4 first, then the four in order
@@ -670,7 +693,8 @@ k_tall_combo(const float* __restrict__ t, int N, int K, const TV* __restrict__ V
 #pragma unroll
       for (int j = 0; j < RN; ++j) {
         float* r = red + ((g & 3) * RN + j) * 132 + lane * 4;
-        float4 v = make_float4(a0[j].x, a0[j].y, a1[j].x, a1[j].y);
+        float4 v = j & 1 ? make_float4(acc[j / 2][0].y, acc[j / 2][1].y, acc[j / 2][2].y, acc[j / 2][3].y)
+                         : make_float4(acc[j / 2][0].x, acc[j / 2][1].x, acc[j / 2][2].x, acc[j / 2][3].x);
         if (pass == 0) {
           const float4 o = *reinterpret_cast<const float4*>(r);
           v = make_float4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
@@ -693,7 +717,7 @@ k_tall_combo(const float* __restrict__ t, int N, int K, const TV* __restrict__ V
 template <typename TA, int RN, int PA, int PX>
 void tall_gram_launch(const TA* A, int M, const float* B, int N, int K, int chunk, int S, float* part, cudaStream_t s) {
   const int nb = (N + 4 * RN - 1) / (4 * RN);
-  const size_t smem = std::max((size_t)kTallStages * TallCfg<TA>::stage_bytes(RN), (size_t)4 * kTallRows * 4 * RN * 4);
+  const size_t smem = std::max((size_t)TallCfg<TA>::STAGES * TallCfg<TA>::stage_bytes(RN), (size_t)4 * kTallRows * 4 * RN * 4);
   set_smem_attr((const void*)k_tall_gram<TA, RN, PA, PX>, smem);
   k_tall_gram<TA, RN, PA, PX><<<dim3((M + kTallRows - 1) / kTallRows, S, nb), 256, smem, s>>>(A, M, B, N, K, chunk, part);
 }
@@ -709,7 +733,7 @@ void tall_gram_typed(const TA* A, int M, const float* B, int N, int K, float* pa
 
 template <typename TV, int RN>
 void tall_combo_launch(const float* t, int N, int K, const TV* V, int ncols, float* out, cudaStream_t s) {
-  const size_t smem = std::max((size_t)kTallKc * RN * 8, (size_t)4 * RN * 132 * 4);
+  const size_t smem = std::max((size_t)kTallKc * RN * 4, (size_t)4 * RN * 132 * 4);
   set_smem_attr((const void*)k_tall_combo<TV, RN>, smem);
   k_tall_combo<TV, RN><<<dim3((ncols + 127) / 128, (N + RN - 1) / RN), 256, smem, s>>>(t, N, K, V, ncols, out);
 }
@@ -774,9 +798,9 @@ static int row_alignment(const void* p, DType t, int K) {
 void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, float* t, cudaStream_t s, unsigned* tmax) {
   if (M <= 0 || N <= 0) return;
   // from 128 rows on, a full tile and a long K; other shapes and BF16 rows of an odd
-  // length take the skinny Gram product (n_ov 24,000, 2000 FP32 rows, 20 vectors: 186
-  // us there, 110 here; n_ov 202,500, 1350 BF16 rows: 1090
-  // and 472).  The K chunks number at most 65,535 (grid).
+  // length take the skinny Gram product (with its reduction, 20 vectors: n_ov 24,000,
+  // 2000 FP32 rows 186 us there, 98 here; n_ov 202,500, 1350 BF16 rows 1090 and 403).
+  // The K chunks number at most 65,535 (grid).
   const int pa = row_alignment(A, ta, K), px = row_alignment(X, DType::F32, K);
   if (!(M >= kTallRows && K >= 1024 && K <= 65535 * kTallChunk && pa >= 4 && (ta == DType::F32 || ta == DType::BF16))) {
     sk_gram(A, ta, K, M, X, DType::F32, K, N, K, t, DType::F32, N, 1.0, 0.0, s, tmax);
@@ -812,8 +836,8 @@ void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, flo
 void tall_combo(const float* t, int N, int K, const void* V, DType tv, int ncols, float* out, cudaStream_t s) {
   if (N <= 0 || ncols <= 0) return;
   // four columns are one load of 16 (FP32) or 8 (BF16) bytes (n_ov 202,500, 1350 BF16
-  // rows, 20 vectors: 824 us by the skinny combination, 580 here; n_ov 24,000, 2000
-  // FP32 rows: 128 and 103)
+  // rows, 20 vectors: 824 us by the skinny combination, 321 here; n_ov 24,000, 2000
+  // FP32 rows, 13 vectors: 128 and 76)
   if (!(K >= 64 && ncols >= 128 && ncols % 4 == 0 &&
         ((tv == DType::F32 && row_alignment(V, tv, ncols) == 16) ||
          (tv == DType::BF16 && row_alignment(V, tv, ncols) >= 8)))) {
