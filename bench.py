@@ -727,7 +727,7 @@ def serving(args, api, torch):
 def batched(args, api, torch, tc=0):
     """Many small independent TDA solves submitted together: n_occ ~ U{8..64},
     n_vir = n_occ x U{4..8}, n_aux = 5 n_mo, ris n_aux = 9 ceil(n_occ/2), 5-10
-    states, MIXED (FP32 outer products on the SIMT path, or with tc the FP16
+    states, MIXED (FP32 outer products by exact slices, or with tc the FP16
     hi+lo tcgen05 products; BF16 ris), rid; all queued at time 0 on a server
     with --batch-slots slots (concurrent streams, not one persistent kernel).
     Throughput = solves / (first submit to last finish)."""
@@ -757,7 +757,7 @@ def batched(args, api, torch, tc=0):
     out.update({"slots": args.batch_slots, "distinct_problems": n_pool,
                 "note": "TDA solves queued at once, each creating its context from FP32 device arrays; "
                         "MIXED, %s outer products, BF16 ris, rid"
-                        % ("FP16 hi+lo tcgen05" if tc else "FP32 SIMT")})
+                        % ("FP16 hi+lo tcgen05" if tc else "FP32")})
     return out
 
 

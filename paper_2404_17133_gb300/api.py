@@ -340,7 +340,8 @@ class Solver:
         self._check(_lib.tddft_profile(self.h, int(bool(enable))), allow_noconv=False)
 
     def profile_read(self, which=0):
-        """which 0: the tcgen05 K1 contraction; 1: the SIMT one."""
+        """which 0: the tcgen05 K1 contraction; 1: the one without the
+        tensor-core option (exact slices)."""
         n, ms, fl = C.c_longlong(), C.c_double(), C.c_double()
         self._check(_lib.tddft_profile_read(self.h, which, C.byref(n), C.byref(ms), C.byref(fl)),
                     allow_noconv=False)
@@ -392,7 +393,7 @@ class Solver:
 
     def apply(self, kind, X, precision=PLAIN, tensor_cores=False):
         """kind 0: A X, 1: ((A+B)X, (A-B)X), 2: T X (ris), 3: ris pair.
-        tensor_cores: 0/False SIMT, 1/True tcgen05, 2 tcgen05 with the FP8 ris rows."""
+        tensor_cores: 0/False off (FP64 / FP32 products by exact slices), 1/True tcgen05, 2 tcgen05 with the FP8 ris rows."""
         if _is_cuda(X):
             import torch
             out0 = torch.empty_like(X)

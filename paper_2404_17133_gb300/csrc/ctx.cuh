@@ -72,7 +72,7 @@ struct FactorSet {
 struct ExactCopies {
   int n = 0;
   DevBuf f64_oo, f64_ov, f64_vv;  // PLAIN
-  DevBuf f32_oo, f32_ov, f32_vv;  // MIXED: SIMT operands
+  DevBuf f32_oo, f32_ov, f32_vv;  // MIXED: FP32 operands
   DevBuf vv_hi, vv_lo;            // [n][nv][tc_pad(nv)] FP16 split of s_vv L_vv
   DevBuf vo_hi, vo_lo;            // [n][nv][tc_pad(no)] FP16 split of s_ov L_ov transposed
   DevBuf oo_hi, oo_lo;            // [n][no][tc_pad(no)] (s_oo L_oo)
@@ -109,14 +109,15 @@ struct OpDims {
   double a_x = 0.0, c_J = 2.0;
   const double* delta = nullptr;  // device [ov]
   KernelProfile* prof = nullptr;       // optional timing of the K1 contraction (tcgen05)
-  KernelProfile* prof_simt = nullptr;  // the same for the SIMT contraction
+  KernelProfile* prof_simt = nullptr;  // the same for the contraction without tc
   int* tc_err = nullptr;          // device flag set by the tensor-core kernel
 };
 
 enum class OpMode { TDA, PAIRED };
 
 // out0 = A X (TDA) or (A+B) X and out1 = (A-B) X (PAIRED); X, out FP64 [m][ov].
-// tc: 0 SIMT contractions; nonzero the exchange contractions on tcgen05
+// tc: 0 exchange contractions by exact slices of the FP64 or FP32 operands (BF16 rows:
+// on the FP32 units); nonzero the exchange contractions on tcgen05
 // (exact factor sets: FP16 hi+lo operands with power-of-two scales, three
 // products, FP32-accurate; ris factor sets: trial vectors as BF16 hi+lo
 // against the plain BF16 rows, or the FP8 rows when the set has them).

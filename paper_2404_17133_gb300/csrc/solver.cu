@@ -1079,7 +1079,7 @@ tddft_status run_tda(Ctx& c, const tddft_opts& o, double* omega, double* X, doub
   }
   // MIXED certification: the converged residuals recomputed from fresh
   // products of the Ritz vectors with the solve's FP32-accurate operator (FP16
-  // hi+lo tensor-core or FP32 SIMT contractions), FP64 norms; the solve
+  // hi+lo or sliced FP32 contractions), FP64 norms; the solve
   // converges only when they are below tol too
   TdaCert certify = [&](const double* Xc, const std::vector<double>& omv, int k) {
     auto tc0 = Clock::now();

@@ -23,11 +23,12 @@
 //   K loop: for each P in the CTA's split range, k-blocks of 128 bytes (one
 //          128B-swizzle atom per row) or, for the hi+lo x hi+lo products, of
 //          64 bytes (64B swizzle); TMA zero-fills k >= Kin, n >= N and rows >= M.
-// CTA = 128 x 256 output tile, 6 warps: warp 0 issues TMA loads, warp 1 owns the
-// tensor memory and one elected lane issues tcgen05.mma, warps 2-5 drain the
+// Tiles of 256 x 256 by CTA pairs (k1_pair_kernel), of 128 x 256 by single CTAs where
+// there is one M tile (k1_tc_kernel).  6 warps: warp 0 issues TMA loads, warp 1 owns
+// the tensor memory and one elected lane issues tcgen05.mma, warps 2-5 drain the
 // FP32 accumulator from TMEM.  A 3- or 4-stage mbarrier ring (~192 KB) connects
 // producer and MMA; tcgen05.commit releases a stage when its MMAs have read it.
-// Split-K: blockIdx.z takes a contiguous range of (P, a-block) steps and writes
+// Split-K: a CTA or cluster takes a contiguous range of (P, a-block) steps and writes
 // its own FP32 partial tile; a fixed-order reduction sums the partials.
 //
 // Every wait on an mbarrier is bounded: on timeout the thread records an error
@@ -1714,30 +1715,33 @@ __global__ void __launch_bounds__(256) k_x_prep(const T* __restrict__ X, const X
 // ([n][a][pad8(j)]) and, when sh is given, X ([n][j][pad8(b)]), as hi + lo parts of
 // X times *scale; the FP32 copy xw when given.
 template <typename T, typename E>
-__global__ void __launch_bounds__(256) k_x_split(const T* __restrict__ X, int no, int nv, int nop, int nvp,
+__global__ void __launch_bounds__(256) k_x_split(const T* __restrict__ X, int m, int no, int nv, int nop, int nvp,
                                                  const float* __restrict__ scale, E* th, E* tl, E* sh, E* sl,
                                                  float* xw) {
   __shared__ float tile[32][33];
-  const int n = blockIdx.z, a0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+  const int a0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const float sc = scale ? *scale : 1.f;
+  for (int n = blockIdx.z; n < m; n += gridDim.z) {
 #pragma unroll
-  for (int r = ty; r < 32; r += 8) {
-    const int j = j0 + r, a = a0 + tx;
-    float v = 0.f;
-    if (j < no && a < nv) {
-      v = (float)X[((long long)n * no + j) * nv + a];
-      if (xw) xw[((long long)n * no + j) * nv + a] = v;
+    for (int r = ty; r < 32; r += 8) {
+      const int j = j0 + r, a = a0 + tx;
+      float v = 0.f;
+      if (j < no && a < nv) {
+        v = (float)X[((long long)n * no + j) * nv + a];
+        if (xw) xw[((long long)n * no + j) * nv + a] = v;
+      }
+      v *= sc;
+      tile[r][tx] = v;
+      if (sh && j < no && a < nvp) split_store<E>(v, ((long long)n * no + j) * nvp + a, sh, sl);
     }
-    v *= sc;
-    tile[r][tx] = v;
-    if (sh && j < no && a < nvp) split_store<E>(v, ((long long)n * no + j) * nvp + a, sh, sl);
-  }
-  __syncthreads();
+    __syncthreads();
 #pragma unroll
-  for (int r = ty; r < 32; r += 8) {
-    const int a = a0 + r, j = j0 + tx;
-    if (a < nv && j < nop) split_store<E>(tile[tx][r], ((long long)n * nv + a) * nop + j, th, tl);
+    for (int r = ty; r < 32; r += 8) {
+      const int a = a0 + r, j = j0 + tx;
+      if (a < nv && j < nop) split_store<E>(tile[tx][r], ((long long)n * nv + a) * nop + j, th, tl);
+    }
+    __syncthreads();
   }
 }
 
@@ -1795,11 +1799,11 @@ void tc_fp8_scales(const void* X, DType xt, int m, int no, int nv, const float* 
 void tc_x_split(const void* X, DType xt, int m, int no, int nv, TcElt et, const float* scale, void* th, void* tl,
                 void* sh, void* sl, float* xw, cudaStream_t s) {
   const int nop = tc_pad(no), nvp = tc_pad(nv);
-  TD_REQUIRE(m <= 65535 && (nop + 31) / 32 <= 65535, TDDFT_ERR_ARG, "trial vectors: too many");
-  const dim3 grid((nvp + 31) / 32, (nop + 31) / 32, m);
+  TD_REQUIRE((nop + 31) / 32 <= 65535, TDDFT_ERR_ARG, "tc_x_split: n_occ");
+  const dim3 grid((nvp + 31) / 32, (nop + 31) / 32, std::min(m, 65535));
   auto go = [&](auto* x, auto* e) {
     using E = std::remove_pointer_t<decltype(e)>;
-    k_x_split<<<grid, 256, 0, s>>>(x, no, nv, nop, nvp, scale, static_cast<E*>(th), static_cast<E*>(tl),
+    k_x_split<<<grid, 256, 0, s>>>(x, m, no, nv, nop, nvp, scale, static_cast<E*>(th), static_cast<E*>(tl),
                                    static_cast<E*>(sh), static_cast<E*>(sl), xw);
   };
   const bool f32 = xt == DType::F32;
