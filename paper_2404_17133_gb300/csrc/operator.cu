@@ -17,6 +17,8 @@
 // tc_gemm.cuh), else as exact slices of the FP64 or FP32 operands
 // (slice_gemm.cuh).  Only BF16 ris rows against FP32 vectors without
 // tensor_cores run on the FP32 units.
+#include <algorithm>
+
 #include "ctx.cuh"
 #include "skinny.cuh"
 #include "slice_gemm.cuh"
@@ -102,6 +104,10 @@ constexpr size_t kChunkBytesTC = 4ull << 30;
 // The sliced contractions (slice_gemm.cuh) keep Z and Q, their slices and the
 // factors' slices of a chunk: 1 GB in all.
 constexpr size_t kChunkBytesSliced = 1ull << 30;
+// Multiply-adds per FP64 Coulomb contraction from which it is sliced, too; below, the
+// launches and the cutting of L_ov cost what the FP64 units do (whole product, units
+// and slices: 2^25.2 1340 and 1310 us, 2^26.8 3456 and 3102, 2^28.8 21.0 and 19.8 ms).
+constexpr double kCoulombSliced = 1 << 25;
 // k-blocks one CTA accumulates in FP32 before its split-K partial is summed
 // (fixed order) with the others: the rounding of an FP32 run grows with its
 // length, and runs over a whole P-chunk of the exchange contraction (~1e4 MMA
@@ -131,6 +137,67 @@ void check_tc_error(Ctx& c) {
   }
 }
 
+// An operand of the sliced contractions with room for its slices.
+struct SliceCut {
+  SliceOperand o;
+  DevBuf parts, exps;
+  void alloc(cudaStream_t st) {
+    parts = DevBuf(slice_bytes(o), st);
+    exps = DevBuf((size_t)o.rows * 4, st);
+  }
+  void cut(cudaStream_t st) { slice_cut(o, parts.p, exps.as<int>(), st); }
+  int* e() const { return exps.as<int>(); }
+};
+static SliceCut slice_operand(const void* p, DType t, int rows, int np, int K) {
+  SliceCut c;
+  c.o.p = p;
+  c.o.t = t;
+  c.o.rows = rows;
+  c.o.np = np;
+  c.o.K = K;
+  return c;
+}
+
+// J = (t^T L_ov) with t = L_ov X^T of an FP64 factor set by exact slicing.  Both are
+// chunked over the rows of the first operand (P; ia), so nothing is accumulated.
+static void coulomb_sliced(const OpDims& d, const FactorSet& f, const double* X, int m, double* J, cudaStream_t s) {
+  const int ov = d.ov;
+  const double* L = static_cast<const double*>(f.Jov);
+  const long long sb = 2 * slice_count(DType::F64);
+  DevBuf t((size_t)f.nJ * m * 8, s);
+  {
+    SliceCut x = slice_operand(X, DType::F64, m, 1, ov);
+    x.o.rs0 = ov; x.o.p_outer = true;
+    x.alloc(s);
+    x.cut(s);
+    const int pc = chunk_rows(f.nJ, tc_pad(ov) * sb, 1, kChunkBytesSliced);
+    SliceCut l = slice_operand(L, DType::F64, pc, 1, ov);
+    l.o.rs0 = ov;
+    l.alloc(s);
+    for (int p0 = 0; p0 < f.nJ; p0 += pc) {
+      l.o.p = L + (long long)p0 * ov;
+      l.o.rows = std::min(pc, f.nJ - p0);
+      l.cut(s);
+      slice_gemm(l.o, l.parts.p, l.e(), x.o, x.parts.p, x.e(), t.as<double>() + (long long)p0 * m, 0.0, d.tc_err, s);
+    }
+  }
+  SliceCut tt = slice_operand(t.p, DType::F64, m, 1, f.nJ);
+  tt.o.rs0 = 1; tt.o.ks = m; tt.o.p_outer = true;
+  tt.alloc(s);
+  tt.cut(s);
+  const int cc = chunk_rows(ov, tc_pad(f.nJ) * sb, 1, kChunkBytesSliced);
+  SliceCut l = slice_operand(L, DType::F64, cc, 1, f.nJ);
+  l.o.rs0 = 1; l.o.ks = ov;
+  l.alloc(s);
+  for (int c0 = 0; c0 < ov; c0 += cc) {
+    l.o.p = L + c0;
+    l.o.rows = std::min(cc, ov - c0);
+    l.cut(s);
+    slice_gemm_scatter(l.o, l.parts.p, l.e(), tt.o, tt.parts.p, tt.e(), J + c0, SliceScatter{1 << 30, 1 << 30, 0, ov, 0},
+                       d.tc_err, s);
+  }
+}
+
 // K1 (and K2) of an FP64 or FP32 factor set, every contraction on the tensor cores
 // by exact slicing (slice_gemm.cuh): no FP64 or FP32 vector arithmetic beyond
 // the cuts.  Xw: trial vectors in the factors' type.
@@ -143,27 +210,9 @@ static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw,
   const size_t per_row = (size_t)m * no * (nv * es + nvp * sb) + (no * nop + nv * nvp) * sb +
                          (need_k2 ? (size_t)m * no * (no * es + nop * sb) + (no * nvp + nv * nop) * sb : 0);
   const int pc = chunk_rows(f.nK, (long long)per_row, 1, kChunkBytesSliced);
-  struct Cut {
-    SliceOperand o;
-    DevBuf parts, exps;
-    void alloc(cudaStream_t st) {
-      parts = DevBuf(slice_bytes(o), st);
-      exps = DevBuf((size_t)o.rows * 4, st);
-    }
-    void cut(cudaStream_t st) { slice_cut(o, parts.p, exps.as<int>(), st); }
-    int* e() const { return exps.as<int>(); }
-  };
-  auto operand = [&](const void* p, int rows, int np, int K) {
-    Cut c;
-    c.o.p = p;
-    c.o.t = t;
-    c.o.rows = rows;
-    c.o.np = np;
-    c.o.K = K;
-    return c;
-  };
+  auto operand = [&](const void* p, int rows, int np, int K) { return slice_operand(p, t, rows, np, K); };
   // X^T per vector: rows (n, a), k = j; X: rows (n, j), k = b
-  Cut xt = operand(Xw, m * nv, 1, no), xs = operand(Xw, m * no, 1, nv);
+  SliceCut xt = operand(Xw, m * nv, 1, no), xs = operand(Xw, m * no, 1, nv);
   xt.o.R = nv; xt.o.rs1 = ov; xt.o.rs0 = 1; xt.o.ks = nv;
   xt.alloc(s);
   xt.cut(s);
@@ -175,8 +224,8 @@ static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw,
   DevBuf Zb((size_t)m * no * pc * nv * es, s), Qb;
   if (need_k2) Qb = DevBuf((size_t)m * no * pc * no * es, s);
   // chunk operands, allocated for the first (largest) chunk
-  Cut oo = operand(nullptr, pc * no, 1, no), vv = operand(nullptr, nv, pc, nv), z = operand(Zb.p, m * no, pc, nv);
-  Cut ov_ = operand(nullptr, pc * no, 1, nv), vo = operand(nullptr, nv, pc, no), q = operand(Qb.p, m * no, pc, no);
+  SliceCut oo = operand(nullptr, pc * no, 1, no), vv = operand(nullptr, nv, pc, nv), z = operand(Zb.p, m * no, pc, nv);
+  SliceCut ov_ = operand(nullptr, pc * no, 1, nv), vo = operand(nullptr, nv, pc, no), q = operand(Qb.p, m * no, pc, no);
   oo.o.rs0 = no; oo.o.p_outer = true;
   vv.o.rs0 = nv; vv.o.ps = (long long)nv * nv; vv.o.p_outer = true;
   z.o.ps = nv;
@@ -348,8 +397,12 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
                   Js.factor.as<float>(), d.tc_err, s, nullptr, 0.0, 0.0, kCoulombKb, keep ? &Js : nullptr);
     } else {
       Jb = DevBuf(mov * ew, s);
-      DevBuf t((size_t)f.nJ * m * ew, s);
-      if (f64) {
+      DevBuf t;
+      const bool sliced = f64 && (double)f.nJ * ov * m >= kCoulombSliced;
+      if (!sliced) t = DevBuf((size_t)f.nJ * m * ew, s);
+      if (sliced) {
+        coulomb_sliced(d, f, static_cast<const double*>(Xw), m, Jb.as<double>(), s);
+      } else if (f64) {
         sk_gram(f.Jov, f.dt, ov, f.nJ, Xw, tw, ov, m, ov, t.p, tw, m, 1.0, 0.0, s);
         sk_combo(t.p, tw, 1, m, m, f.nJ, f.Jov, f.dt, ov, ov, Jb.p, tw, ov, 1.0, 0.0, s);
       } else {

@@ -23,7 +23,8 @@ pytestmark = pytest.mark.gpu
 TOL = {0: 3e-14, 1: 4e-6}
 
 SHAPES = [(1, 1, 1, 9, 1), (3, 7, 5, 9, 2), (16, 64, 20, 9, 4), (17, 65, 20, 18, 5), (8, 32, 30, 9, 17),
-          (33, 257, 12, 27, 3), (24, 144, 400, 27, 4), (10, 40, 300, 9, 10)]
+          (33, 257, 12, 27, 3), (24, 144, 400, 27, 4), (10, 40, 300, 9, 10),
+          (24, 144, 400, 27, 100), (19, 131, 1031, 27, 53)]
 
 
 @pytest.fixture(scope="module")
