@@ -894,7 +894,7 @@ struct Batch {
   double* hst(Prob& p) { return h_status + p.st_off; }
   void pull() {
     TD_CUDA(cudaMemcpyAsync(h_status, status.p, (size_t)stride * P.size() * 8, cudaMemcpyDeviceToHost, s));
-    TD_CUDA(cudaStreamSynchronize(s));
+    check_batch_tc(s);   // waits for the stream; ends the batch when its products are wrong
   }
 };
 

@@ -191,8 +191,11 @@ struct Ctx {
   FactorSet ris(int precision, bool fp8 = false) const;  // PLAIN -> FP64, MIXED -> BF16 (+ FP8)
 };
 
-// Throw if the tensor-core kernel reported a timeout since the last check.
+// Throw if a tensor-core kernel reported a timeout since the last check (waits for
+// the stream).
 void check_tc_error(Ctx& c);
+// The same for a code already read from the word, which is cleared.
+void raise_tc_error(int code, int* word, cudaStream_t s);
 
 tddft_status run_tda(Ctx& c, const tddft_opts& o, double* omega, double* X, double* resid,
                      tddft_stats* st);

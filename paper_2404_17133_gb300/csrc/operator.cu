@@ -127,14 +127,17 @@ int chunk_rows(int nrows, long long per_row_bytes, int m, size_t budget = kChunk
 }
 }  // namespace
 
+void raise_tc_error(int code, int* word, cudaStream_t s) {
+  if (code == 0) return;
+  TD_CUDA(cudaMemsetAsync(word, 0, 4, s));
+  throw Error(TDDFT_ERR_CUDA, "tensor-core kernel wait timed out (code " + std::to_string(code) + ")");
+}
+
 void check_tc_error(Ctx& c) {
   int h = 0;
   TD_CUDA(cudaMemcpyAsync(&h, c.tc_err.p, 4, cudaMemcpyDeviceToHost, c.s));
   TD_CUDA(cudaStreamSynchronize(c.s));
-  if (h != 0) {
-    TD_CUDA(cudaMemsetAsync(c.tc_err.p, 0, 4, c.s));
-    throw Error(TDDFT_ERR_CUDA, "tensor-core kernel wait timed out (code " + std::to_string(h) + ")");
-  }
+  raise_tc_error(h, c.tc_err.as<int>(), c.s);
 }
 
 // An operand of the sliced contractions with room for its slices.

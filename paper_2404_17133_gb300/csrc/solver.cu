@@ -110,6 +110,20 @@ std::vector<T> d2h(const T* p, size_t n, cudaStream_t s) {
   return h;
 }
 
+// d2h that reads the tensor-core kernels' error word in the same wait and throws when
+// it is set.  The iterations read their norms with it, so that a solve whose
+// products are wrong ends there and does not go on for its remaining iterations.
+template <typename T>
+std::vector<T> d2h_checked(const T* p, size_t n, int* tc_err, cudaStream_t s) {
+  int code = 0;
+  TD_CUDA(cudaMemcpyAsync(&code, tc_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+  std::vector<T> h(n);
+  TD_CUDA(cudaMemcpyAsync(h.data(), p, n * sizeof(T), cudaMemcpyDeviceToHost, s));
+  TD_CUDA(cudaStreamSynchronize(s));
+  raise_tc_error(code, tc_err, s);
+  return h;
+}
+
 template <typename T>
 void h2d(T* p, const std::vector<T>& h, cudaStream_t s) {
   if (!h.empty()) TD_CUDA(cudaMemcpyAsync(p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, s));
@@ -120,6 +134,8 @@ struct Counters {
   long long ris_mv = 0;  // ris operator vectors
   double t_mv = 0.0, t_pre = 0.0, t_guess = 0.0, t_cert = 0.0;
   int restarts = 0;
+  int* tc_err;           // the context's error word (OpDims::tc_err)
+  explicit Counters(const Ctx& c) : tc_err(c.tc_err.as<int>()) {}
 };
 
 template <typename T> constexpr DType dt_of();
@@ -346,7 +362,7 @@ TdaOut davidson_tda(int ov, const TdaOp& A, const TdaPre& pre, double* guess, in
     combo<double, double>(x.as<double>(), kk, N, Wp, ov, AX.as<double>(), 1.0, 0.0, s);
     resid_tda(X.as<double>(), AX.as<double>(), lam.as<double>(), kk, ov, R.as<double>(), s);  // Eq. residual
     row_sumsq(R.as<double>(), ov, kk, ov, rn.as<double>(), s);
-    om = d2h(lam.as<double>(), kk, s);
+    om = d2h_checked(lam.as<double>(), kk, cnt.tc_err, s);
     rr = sqrt_all(d2h(rn.as<double>(), kk, s));
     ph_vec.stop();
     check_finite_host(om, "Ritz values");
@@ -478,8 +494,8 @@ struct PairedSpace {
     n_old = N;
     n_new = 0;
   }
-  void check_definite() {
-    int inf = d2h(info.as<int>(), 1, s)[0];
+  void check_definite(int* tc_err) {
+    int inf = d2h_checked(info.as<int>(), 1, tc_err, s)[0];
     if (inf != 0)
       throw Error(TDDFT_ERR_INDEFINITE, "projected A-B is not positive definite (pivot " +
                                             std::to_string(inf - 1) + ")");
@@ -583,7 +599,7 @@ PairedLinOut paired_linear(int ov, const PairOpT<T>& op, const PairPreT<T>& pre,
   for (int it = 1; it <= max_iter; ++it) {
     o.n_iter = it;
     sp.update(false);
-    if (!dev_select) sp.check_definite();
+    if (!dev_select) sp.check_definite(cnt.tc_err);
     const int N = sp.N;
     S* Lp = sp.L.template as<S>();
     ScopedPhase ph_small(PH_SMALL, s);
@@ -627,7 +643,7 @@ PairedLinOut paired_linear(int ov, const PairOpT<T>& op, const PairPreT<T>& pre,
       zero_converged<T>(cand.as<T>(), 2 * nr, nr, ov, rn1p, rn2p, gdev.as<double>(), tol, s);
       orth_append_async<T>(sp.v(), N, cand.as<T>(), 2 * nr, ov, keep.as<int>(), st_count, s);
       TD_CUDA(cudaMemcpyAsync(st_info, sp.info.p, sizeof(int), cudaMemcpyDeviceToDevice, s));
-      std::vector<double> blk = d2h(stat.as<double>(), (size_t)2 * nr + 1, s);
+      std::vector<double> blk = d2h_checked(stat.as<double>(), (size_t)2 * nr + 1, cnt.tc_err, s);
       int ints[2];
       std::memcpy(ints, &blk[2 * nr], sizeof(ints));
       if (ints[0] != 0)
@@ -768,7 +784,7 @@ RpaOut davidson_rpa(int ov, const PairOp& op, const PairPre& pre, double* guess,
   for (int it = 1; it <= max_iter; ++it) {
     o.n_iter = it;
     sp.update(true);
-    sp.check_definite();
+    sp.check_definite(cnt.tc_err);
     const int N = sp.N;
     kk = std::min(k, N);
     double* Lp = sp.L.template as<double>();
@@ -929,7 +945,7 @@ void inner_tda(int ov, const TdaOpT<T>& Top, const double* delta, const T* R, co
       zero_converged<T>(cand.as<T>(), nu, nu, ov, rn, nullptr, r0.as<double>(), tol, s);
       orth_append_async<T>(Sb.as<T>(), N, cand.as<T>(), nu, ov, keep.as<int>(), st_count, s);
     }
-    std::vector<double> blk = d2h(stat.as<double>(), (size_t)nu + 1, s);
+    std::vector<double> blk = d2h_checked(stat.as<double>(), (size_t)nu + 1, cnt.tc_err, s);
     int m = 0;
     for (int j = 0; j < nu; ++j)
       if (!(std::sqrt(blk[j]) / r0h[j] <= tol)) ++m;
@@ -1029,7 +1045,7 @@ tddft_status run_tda(Ctx& c, const tddft_opts& o, double* omega, double* X, doub
   const Plan p = make_plan(c, o);
   const int ov = c.ov;
   cudaStream_t s = c.s;
-  Counters cnt;
+  Counters cnt(c);
   const OpDims dims = c.dims();
   const FactorSet Fx = c.exact(o.precision);
   const FactorSet Fr = c.ris(o.precision, p.fp8);
@@ -1161,7 +1177,7 @@ tddft_status run_rpa(Ctx& c, const tddft_opts& o, double* omega, double* X, doub
   const Plan p = make_plan(c, o);
   const int ov = c.ov;
   cudaStream_t s = c.s;
-  Counters cnt;
+  Counters cnt(c);
   const OpDims dims = c.dims();
   PairOp A = make_pair_op(dims, c.exact(o.precision), p.tc, s);
   PairOp T = make_pair_op(dims, c.ris(o.precision, p.fp8), p.tc, s);
@@ -1259,7 +1275,7 @@ tddft_status run_polar(Ctx& c, const tddft_opts& o, const double* mu, int n_dip,
   TD_REQUIRE(4 * nr <= p.cap, TDDFT_ERR_ARG, "polar: max_subspace must be at least 4*n_dip*n_freq");
   const int ov = c.ov;
   cudaStream_t s = c.s;
-  Counters cnt;
+  Counters cnt(c);
   const OpDims dims = c.dims();
   PairOp A = make_pair_op(dims, c.exact(o.precision), p.tc, s);
   PairOp T = make_pair_op(dims, c.ris(o.precision, p.fp8), p.tc, s);

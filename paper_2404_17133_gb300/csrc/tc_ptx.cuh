@@ -7,9 +7,14 @@
 namespace tddft {
 namespace {
 
-// Polls of an mbarrier before a wait gives up (the kernel then records an
-// error code and leaves its loop; the host reports TDDFT_ERR_CUDA).
-constexpr long long WAIT_LIMIT = 1ll << 23;
+// A wait on an mbarrier gives up after WAIT_NS (the kernel then records an error
+// code and leaves its loop; the host reports TDDFT_ERR_CUDA).  The limit is a time:
+// a number of polls is none, since a poll may suspend its thread for as long as the
+// hardware chooses.  POLL_NS bounds one suspension; the clock is read only
+// after a poll that found the phase open.  The longest wait of a kernel that works
+// is for its CTA's whole K range, some milliseconds.
+constexpr unsigned long long WAIT_NS = 2000000000ull;
+constexpr uint32_t POLL_NS = 1000000u;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -25,19 +30,31 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
                : "memory");
 }
 
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(POLL_NS)
+      : "memory");
+  return ok != 0;
+}
+
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
 // Bounded wait for the completion of phase `parity`; false on timeout.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   const uint32_t a = smem_u32(bar);
-  for (long long i = 0; i < WAIT_LIMIT; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
+  if (mbar_poll(a, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  do {
+    if (mbar_poll(a, parity)) return true;
+  } while (global_ns() - t0 < WAIT_NS);
   return false;
 }
 
