@@ -1,5 +1,5 @@
 #!/usr/bin/env python
-"""Benchmark: excitation states converged per second on one GB300 (or N replicas).
+"""Benchmark: excitation states converged per second on one GB300.
 
 One step is the whole hot path on the large mixed workload (n_occ=150,
 n_vir=1350, ov=202,500, exact n_aux=6000, ris n_aux=1350): a TDA solve and a
@@ -29,8 +29,9 @@ serving: an open-loop Poisson stream of TDA / Casida / polarizability requests
 batched: 256 small independent TDA solves queued at once on the server
        (solves/s; --batch*).
 
-Multi-GPU: one independent replica per GPU (the path does not shard on one
-box), launched under torch.distributed.run; rank 0 prints one JSON line.
+One GPU: the library's contraction kernel shares operand tiles between the CTAs of
+a cluster by TMA multicast, which is for calls on one GPU only, so --gpus above 1
+(or a launch with several ranks) is refused.
 
 --impl reference times the CPU oracle (FP64, NumPy) on a bounded sample of the
 same workload (the exact and ris products of a few vectors over a few
@@ -897,6 +898,11 @@ def main():
     rank, world, local = dist_env()
     if args.impl == "reference":
         reference_arm(args, rank, world)
+        return
+    if world > 1 or args.gpus > 1:
+        if rank == 0:
+            print(json.dumps({"metric": METRIC, "n_gpus": max(world, args.gpus), "unavailable":
+                              "the library is for calls on one GPU (TMA multicast in its contraction kernel)"}), flush=True)
         return
     our_arm(args, rank, world, local)
 
