@@ -33,6 +33,11 @@ One GPU: the library's contraction kernel shares operand tiles between the CTAs 
 a cluster by TMA multicast, which is for calls on one GPU only, so --gpus above 1
 (or a launch with several ranks) is refused.
 
+Every section's result goes to stderr when it ends.  Sections after the timed steps
+have a time limit (--section-limit): where one does not end within it, the line is
+printed with what was measured up to there, "unfinished" names the section, and
+the process leaves.
+
 --impl reference times the CPU oracle (FP64, NumPy) on a bounded sample of the
 same workload (the exact and ris products of a few vectors over a few
 auxiliary rows, scaled to all rows and to the products one step makes) and
@@ -47,6 +52,7 @@ import statistics
 import subprocess
 import sys
 import tempfile
+import threading
 import time
 
 import numpy as np
@@ -94,6 +100,8 @@ def parse():
     ap.add_argument("--batch", type=int, default=256, help="independent small TDA solves queued at once (0: none)")
     ap.add_argument("--batch-slots", type=int, default=16)
     ap.add_argument("--serve-budget-gb", type=float, default=150.0)
+    ap.add_argument("--section-limit", type=float, default=300.0,
+                    help="seconds that each section after the timed steps may take")
     ap.add_argument("--apply-only", type=int, default=0, metavar="K",
                     help="time K exact pair products ((A+B)X, (A-B)X) of 2*n_states device vectors "
                          "and exit (a short program for kernel profiling)")
@@ -326,13 +334,47 @@ def make_solver(api, meta, src, stream_ptr):
                       dtype=api.F32, stream=stream_ptr)
 
 
-def our_arm(args, rank, world, local):
+class Sections:
+    """Progress of the bench on stderr and a time limit for each section: past it
+    the line is printed with what there is, and the process leaves (a call into the
+    library cannot be interrupted from Python)."""
+
+    def __init__(self, limit):
+        self.limit = limit
+        self.line = {}
+        self.t0 = time.time()
+
+    def note(self, name, result=None):
+        text = "" if result is None else " " + json.dumps(result, default=str)
+        print("[bench %7.1f s] %s%s" % (time.time() - self.t0, name, text), file=sys.stderr, flush=True)
+
+    def _expired(self, name):
+        self.note(name + ": time limit")
+        print(json.dumps(dict(self.line, unfinished=name)), flush=True)
+        os._exit(0 if "value" in self.line else 1)
+
+    def run(self, name, fn, limit=None, required=False):
+        """fn() within the limit; an error is the section's result, unless it is required."""
+        self.note(name + " ...")
+        timer = threading.Timer(limit or self.limit, self._expired, (name,))
+        timer.daemon = True
+        timer.start()
+        try:
+            r = fn()
+        except Exception as e:
+            if required:
+                raise
+            r = {"error": "%s: %s" % (type(e).__name__, e)}
+        finally:
+            timer.cancel()
+        self.note(name, r)
+        return r
+
+
+def our_arm(args):
     import torch
 
-    torch.cuda.set_device(local)
-    if world > 1:
-        import torch.distributed as dist
-        dist.init_process_group("nccl", device_id=torch.device("cuda", local))
+    torch.cuda.set_device(0)
     import __graft_entry__ as ge
     ge.build()
     from paper_2404_17133_gb300 import api
@@ -347,7 +389,9 @@ def our_arm(args, rank, world, local):
             kernel_breakdown(args, api, solver, tc)
         solver.close()
         return
-    want_e2e = not args.no_e2e and rank == 0
+    sec = Sections(args.section_limit)
+    sec.note("loading")
+    want_e2e = not args.no_e2e
     solver, meta, host, t_load = load_large(api, torch, stream.cuda_stream, pinned_copy=want_e2e)
     h2d_bytes = sum(v.numel() * v.element_size() for v in host.values()) if host else 0
     d2h_bytes = 8 * (2 * N_STATES + 2 * N_STATES)     # energies and residual norms of both solves
@@ -359,56 +403,72 @@ def our_arm(args, rank, world, local):
         b = s.solve_rpa(o, want_vectors=False)
         return a, b
 
-    for _ in range(max(args.warmup, 0)):
-        step(solver)
-    if world > 1:
-        torch.distributed.barrier()
-    torch.cuda.synchronize()
-    clocks = ClockSampler(torch.cuda.current_device()) if rank == 0 else None
-    solver.profile(True)
-    ev = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps + 1)]
-    ev[0].record(stream)
-    launches = 0
-    results = []
-    for i in range(args.steps):
-        a, b = step(solver)
-        ev[i + 1].record(stream)
-        launches += a["stats"]["gpu_launches"] + b["stats"]["gpu_launches"]
-        results.append((a, b))
-    torch.cuda.synchronize()
-    if world > 1:
-        torch.distributed.barrier()
-    prof = solver.profile_read(0 if tc else 1)
-    rec_ms, rec_fl, rec_by = solver.profile_records(0 if tc else 1)
-    solver.profile(False)
-    clk = clocks.stop() if clocks else None
-    per_step = [ev[i].elapsed_time(ev[i + 1]) for i in range(args.steps)]
-    total_ms = ev[0].elapsed_time(ev[-1])
-    total_ms = max_over_ranks(total_ms, world)
-    value = replica_throughput(STATES_PER_STEP * args.steps, world, total_ms)
-    a, b = results[-1]
-    conv = all(r["status"] == api.OK for pair in results for r in pair)
+    def timed_steps():
+        for i in range(max(args.warmup, 0)):
+            step(solver)
+            sec.note("warm-up step %d" % i)
+        torch.cuda.synchronize()
+        clocks = ClockSampler(torch.cuda.current_device())
+        solver.profile(True)
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps + 1)]
+        ev[0].record(stream)
+        launches = 0
+        results = []
+        for i in range(args.steps):
+            a, b = step(solver)
+            ev[i + 1].record(stream)
+            launches += a["stats"]["gpu_launches"] + b["stats"]["gpu_launches"]
+            results.append((a, b))
+        torch.cuda.synchronize()
+        prof = solver.profile_read(0 if tc else 1)
+        records = solver.profile_records(0 if tc else 1)
+        solver.profile(False)
+        clk = clocks.stop()
+        per_step = [ev[i].elapsed_time(ev[i + 1]) for i in range(args.steps)]
+        total_ms = ev[0].elapsed_time(ev[-1])
+        a, b = results[-1]
+        peaks, src = load_peaks()
+        solved = lambda r: {"omega0": float(r["omega"][0]), "n_iter": r["stats"]["n_iter"],
+                            "n_matvec": r["stats"]["n_matvec"], "n_ris_matvec": r["stats"]["n_ris_matvec"],
+                            "max_resid_certified": r["stats"]["max_resid_certified"], "s": r["stats"]["t_total_s"],
+                            "exact_product_s": r["stats"]["t_matvec_s"], "precond_s": r["stats"]["t_precond_s"]}
+        sec.last = (a, b)
+        return {"metric": METRIC, "value": replica_throughput(STATES_PER_STEP * args.steps, 1, total_ms), "unit": UNIT,
+                "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": total_ms / args.steps,
+                "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+                "dtype": "f32 (tensor: fp16 hi+lo x3) + fp64 subspace", "data": "synthetic",
+                "config": {"workload": WORKLOAD, "n_occ": meta["n_occ"], "n_vir": meta["n_vir"],
+                           "n_aux": meta["n_aux"], "n_aux_ris": meta["n_ris"], "n_states": N_STATES,
+                           "solves_per_step": ["tda", "casida"], "precond": args.precond,
+                           "tensor_cores": bool(tc), "parallelism": "single",
+                           "l2": "inputs larger than L2 (~100 GB resident factor copies), no flush"},
+                "p50_ms": statistics.median(per_step),
+                "p99_ms": sorted(per_step)[min(len(per_step) - 1, int(0.99 * len(per_step)))],
+                "converged": all(r["status"] == api.OK for pair in results for r in pair), "load_s": t_load,
+                "tda": solved(a), "rpa": solved(b),
+                "roofline": roofline(prof, *records, peaks, src, tc, clk, total_ms),
+                "gpu_launches": launches, "clocks": clk,
+                "e2e": {"value": None, "unit": UNIT, "ms_per_step": None}}
+
+    line = sec.run("timed steps", timed_steps, limit=max(600.0, 40.0 * (args.steps + max(args.warmup, 0))),
+                   required=True)
+    sec.line = line
+    a, b = sec.last
     counts = {"tda_mv": a["stats"]["n_matvec"], "tda_ris_mv": a["stats"]["n_ris_matvec"],
               "rpa_mv": b["stats"]["n_matvec"], "rpa_ris_mv": b["stats"]["n_ris_matvec"]}
 
-    diag = None
-    if not args.no_diag and rank == 0:
+    def diag():
         od = api.default_opts(n_states=N_STATES, precond=api.DIAG, precision=api.MIXED, tensor_cores=tc)
         da, db = solver.solve_tda(od, want_vectors=False), solver.solve_rpa(od, want_vectors=False)
-        diag = {"tda_n_iter": da["stats"]["n_iter"], "rpa_n_iter": db["stats"]["n_iter"],
+        return {"tda_n_iter": da["stats"]["n_iter"], "rpa_n_iter": db["stats"]["n_iter"],
                 "tda_s": da["stats"]["t_total_s"], "rpa_s": db["stats"]["t_total_s"],
                 "converged": da["status"] == api.OK and db["status"] == api.OK,
                 "max_abs_omega_diff_vs_rid": float(max(np.max(np.abs(da["omega"] - a["omega"])),
                                                        np.max(np.abs(db["omega"] - b["omega"]))))}
-    peaks, src = load_peaks()
-    roof = roofline(prof, rec_ms, rec_fl, rec_by, peaks, src, tc, clk, total_ms)
 
-    # ---- end to end through the C ABI with pinned host inputs and host outputs
-    e2e_ms = []
-    if want_e2e:
-        solver.close()
-        solver = None
-        torch.cuda.empty_cache()
+    # end to end through the C ABI with pinned host inputs and host outputs
+    def end_to_end():
+        ms = []
         for _ in range(max(args.e2e_steps, 1)):
             torch.cuda.synchronize()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -418,78 +478,39 @@ def our_arm(args, rank, world, local):
             s2.close()
             e1.record(stream)
             torch.cuda.synchronize()
-            e2e_ms.append(e0.elapsed_time(e1))
-        host = None
-    e2e_t = statistics.mean(e2e_ms) if e2e_ms else float("nan")
-    e2e_t = max_over_ranks(e2e_t, world)
-    if solver is not None:
-        solver.close()
-        solver = None
+            ms.append(e0.elapsed_time(e1))
+        t = statistics.mean(ms)
+        return {"value": STATES_PER_STEP / (t / 1e3), "unit": UNIT, "ms_per_step": t,
+                "h2d_bytes_per_step": int(h2d_bytes), "d2h_bytes_per_step": int(d2h_bytes)}
+
+    line["diag"] = None if args.no_diag else sec.run("diag", diag)
+    solver.close()
+    solver = None
     torch.cuda.empty_cache()
-    if rank != 0:
-        if world > 1:
-            torch.distributed.destroy_process_group()
-        return
-    line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
-            "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "f32 (tensor: fp16 hi+lo x3) + fp64 subspace",
-            "data": "synthetic",
-            "config": {"workload": WORKLOAD, "n_occ": meta["n_occ"], "n_vir": meta["n_vir"],
-                       "n_aux": meta["n_aux"], "n_aux_ris": meta["n_ris"], "n_states": N_STATES,
-                       "solves_per_step": ["tda", "casida"], "precond": args.precond,
-                       "tensor_cores": bool(tc), "parallelism": "replicas" if world > 1 else "single",
-                       "l2": "inputs larger than L2 (~100 GB resident factor copies), no flush"},
-            "p50_ms": statistics.median(per_step),
-            "p99_ms": sorted(per_step)[min(len(per_step) - 1, int(0.99 * len(per_step)))],
-            "converged": conv, "load_s": t_load,
-            "tda": {"omega0": float(a["omega"][0]), "n_iter": a["stats"]["n_iter"],
-                    "n_matvec": a["stats"]["n_matvec"], "n_ris_matvec": a["stats"]["n_ris_matvec"],
-                    "max_resid_certified": a["stats"]["max_resid_certified"], "s": a["stats"]["t_total_s"],
-                    "exact_product_s": a["stats"]["t_matvec_s"], "precond_s": a["stats"]["t_precond_s"]},
-            "rpa": {"omega0": float(b["omega"][0]), "n_iter": b["stats"]["n_iter"],
-                    "n_matvec": b["stats"]["n_matvec"], "n_ris_matvec": b["stats"]["n_ris_matvec"],
-                    "max_resid_certified": b["stats"]["max_resid_certified"], "s": b["stats"]["t_total_s"],
-                    "exact_product_s": b["stats"]["t_matvec_s"], "precond_s": b["stats"]["t_precond_s"]},
-            "diag": diag,
-            "roofline": roof,
-            "gpu_launches": launches,
-            "clocks": clk,
-            "e2e": {"value": STATES_PER_STEP * world / (e2e_t / 1e3) if e2e_ms else None, "unit": UNIT,
-                    "ms_per_step": e2e_t if e2e_ms else None,
-                    "h2d_bytes_per_step": int(h2d_bytes), "d2h_bytes_per_step": int(d2h_bytes)}}
-    if args.medium_steps > 0 and world == 1:
-        try:
-            line["medium"] = medium(args, api, torch, stream, tc)
-        except Exception as e:
-            line["medium"] = {"error": "%s: %s" % (type(e).__name__, e)}
-    if args.serve_seconds > 0 and world == 1:
-        try:
-            line["serving"] = serving(args, api, torch)
-        except Exception as e:   # the served stream is reported, not required for the line
-            line["serving"] = {"error": "%s: %s" % (type(e).__name__, e)}
-    if args.batch > 0 and world == 1:
-        try:
-            line["batched_lockstep"] = batched_lockstep(args, api, torch)
-        except Exception as e:
-            line["batched_lockstep"] = {"error": "%s: %s" % (type(e).__name__, e)}
+    if want_e2e:
+        line["e2e"] = sec.run("e2e", end_to_end)
+    host = None
+    torch.cuda.empty_cache()
+    if args.medium_steps > 0:
+        line["medium"] = sec.run("medium", lambda: medium(args, api, torch, stream, tc))
+    if args.serve_seconds > 0:
+        line["serving"] = sec.run("serving", lambda: serving(args, api, torch))
+    if args.batch > 0:
+        line["batched_lockstep"] = sec.run("batched_lockstep", lambda: batched_lockstep(args, api, torch))
         for key, t in (("batched", 0), ("batched_tc", 1)):
-            try:
-                line[key] = batched(args, api, torch, tc=t)
-            except Exception as e:
-                line[key] = {"error": "%s: %s" % (type(e).__name__, e)}
-    if not args.no_cpu_baseline and world == 1:
-        try:
-            tm = oracle_sample()
-            t1 = oracle_sample(threads=1)
-            step_s = oracle_step_seconds(tm, counts)
-            line["cpu_baseline"] = {"value": STATES_PER_STEP / step_s, "unit": UNIT, "cores": os.cpu_count(),
-                                    "kind": "oracle", "sample": sample_note(tm, counts),
-                                    "single_thread_value": STATES_PER_STEP / oracle_step_seconds(t1, counts)}
-        except Exception as e:
-            line["cpu_baseline"] = {"error": "%s: %s" % (type(e).__name__, e)}
+            line[key] = sec.run(key, lambda: batched(args, api, torch, tc=t))
+
+    def cpu_baseline():
+        tm = oracle_sample()
+        t1 = oracle_sample(threads=1)
+        step_s = oracle_step_seconds(tm, counts)
+        return {"value": STATES_PER_STEP / step_s, "unit": UNIT, "cores": os.cpu_count(), "kind": "oracle",
+                "sample": sample_note(tm, counts),
+                "single_thread_value": STATES_PER_STEP / oracle_step_seconds(t1, counts)}
+
+    if not args.no_cpu_baseline:
+        line["cpu_baseline"] = sec.run("cpu baseline", cpu_baseline)
     print(json.dumps(line), flush=True)
-    if world > 1:
-        torch.distributed.destroy_process_group()
 
 
 # DRAM traffic of the K1 contraction from one ncu capture of full-size launches
@@ -895,7 +916,7 @@ def kernel_breakdown(args, api, solver, tc):
 
 def main():
     args = parse()
-    rank, world, local = dist_env()
+    rank, world, _ = dist_env()
     if args.impl == "reference":
         reference_arm(args, rank, world)
         return
@@ -904,7 +925,7 @@ def main():
             print(json.dumps({"metric": METRIC, "n_gpus": max(world, args.gpus), "unavailable":
                               "the library is for calls on one GPU (TMA multicast in its contraction kernel)"}), flush=True)
         return
-    our_arm(args, rank, world, local)
+    our_arm(args)
 
 
 if __name__ == "__main__":
