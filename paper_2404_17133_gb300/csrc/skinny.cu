@@ -481,6 +481,13 @@ __device__ __forceinline__ void fma2(float2& c, float2 a, float2 b) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
 }
 
+// a + b as its FP32 sum and the rounding of it (Knuth); none where the sum is not finite
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  const float r = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  return make_float2(s, isfinite(s) ? r : 0.f);
+}
+
 // PB bytes (4, 8 or 16) to shared memory, zero beyond `bytes`
 template <int PB>
 __device__ __forceinline__ void cp_piece(void* dst, const void* src, int bytes) {
@@ -491,12 +498,13 @@ __device__ __forceinline__ void cp_piece(void* dst, const void* src, int bytes) 
     asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(d), "l"(src), "r"(bytes), "n"(PB) : "memory");
 }
 
-// part[chunk][m][n] = sum over the chunk of A[m][k] B[n][k].  Bound by the FP32
+// part[2 chunk][m][n] + part[2 chunk + 1][m][n] = sum over the chunk of A[m][k] B[n][k].  Bound by the FP32
 // units for about 16 vectors and more, by reading A below that.  CTA = 128 rows
 // x 4 RN vectors; 16 row groups x 4 vector groups x 4 groups of k, a thread 8
 // rows x RN vectors: 13 16-byte shared-memory loads feed 160 FMAs (RN = 5),
 // accumulated for even and odd k apart (packed FMAs), so a sum runs over at most
-// 1/8 of the chunk (<= 256 terms) before the chunk's eight are added in order.
+// 1/8 of the chunk (<= 256 terms).  The chunk's eight are added with the roundings
+// kept, so that beyond those runs everything is added in FP64, as by the skinny product.
 // cp.async keeps two (FP32) or three stages of 64 k in flight, and two CTAs share an
 // SM up to 20 vectors.  n_ov 202,500, 1350 BF16 rows, 20 vectors: 365 us (992 by the
 // skinny product, 433 with one CTA per SM); n_ov 24,000, 2000 FP32 rows: 71 (149, 83).
@@ -590,22 +598,29 @@ k_tall_gram(const TA* __restrict__ A, int M, const float* __restrict__ B, int N,
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  // the four groups of k, added in order through shared memory
-  float* red = reinterpret_cast<float*>(tall_raw);   // [4][128][NT]
+  // the eight sums (even and odd k of four groups), added in order without loss: the
+  // rounding of every addition is kept, and the chunk leaves a sum and its remainder
+  float2* red = reinterpret_cast<float2*>(tall_raw);   // [4][128][NT]
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = 0; j < RN; ++j)
-      red[(kg * kTallRows + rg + 16 * i) * NT + cg + 4 * j] = acc[i][j].x + acc[i][j].y;
+      red[(kg * kTallRows + rg + 16 * i) * NT + cg + 4 * j] = two_sum(acc[i][j].x, acc[i][j].y);
   __syncthreads();
-  float* P = part + (long long)blockIdx.y * M * N;
+  const long long MN = (long long)M * N;
+  float* P = part + 2 * blockIdx.y * MN;
   for (int e = tid; e < kTallRows * NT; e += 256) {
     const int r = e / NT, c = e - r * NT;
     if (m0 + r >= M || n0 + c >= N) continue;
-    float v = 0.f;
+    float2 v = red[e];
 #pragma unroll
-    for (int g = 0; g < 4; ++g) v += red[g * kTallRows * NT + e];
-    P[(long long)(m0 + r) * N + n0 + c] = v;
+    for (int g = 1; g < 4; ++g) {
+      const float2 w = red[g * kTallRows * NT + e], t = two_sum(v.x, w.x);
+      v = make_float2(t.x, t.y + v.y + w.y);
+    }
+    const long long at = (long long)(m0 + r) * N + n0 + c;
+    P[at] = v.x;
+    P[MN + at] = v.y;
   }
 }
 
@@ -717,7 +732,7 @@ k_tall_combo(const float* __restrict__ t, int N, int K, const TV* __restrict__ V
 template <typename TA, int RN, int PA, int PX>
 void tall_gram_launch(const TA* A, int M, const float* B, int N, int K, int chunk, int S, float* part, cudaStream_t s) {
   const int nb = (N + 4 * RN - 1) / (4 * RN);
-  const size_t smem = std::max((size_t)TallCfg<TA>::STAGES * TallCfg<TA>::stage_bytes(RN), (size_t)4 * kTallRows * 4 * RN * 4);
+  const size_t smem = std::max((size_t)TallCfg<TA>::STAGES * TallCfg<TA>::stage_bytes(RN), (size_t)4 * kTallRows * 4 * RN * 8);
   set_smem_attr((const void*)k_tall_gram<TA, RN, PA, PX>, smem);
   k_tall_gram<TA, RN, PA, PX><<<dim3((M + kTallRows - 1) / kTallRows, S, nb), 256, smem, s>>>(A, M, B, N, K, chunk, part);
 }
@@ -812,7 +827,7 @@ void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, flo
   int chunk = ((K + S - 1) / S + kTallK - 1) / kTallK * kTallK;
   chunk = std::max(chunk, 4 * kTallK);
   S = (K + chunk - 1) / chunk;
-  DevBuf part((size_t)S * M * N * 4, s);
+  DevBuf part((size_t)2 * S * M * N * 4, s);
   float* pt = part.as<float>();
   if (ta == DType::F32) {
     const float* a = static_cast<const float*>(A);
@@ -828,7 +843,7 @@ void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, flo
   TD_LAUNCH_CHECK();
   const long long MN = (long long)M * N;
   const unsigned rb = (unsigned)std::min<long long>((MN + 7) / 8, 16 * 152);
-  k_sk_gram_reduce<float, float><<<rb, 256, 0, s>>>(part.as<float>(), S, M, N, t, N, 1.0, 0.0, tmax);
+  k_sk_gram_reduce<float, float><<<rb, 256, 0, s>>>(part.as<float>(), 2 * S, M, N, t, N, 1.0, 0.0, tmax);
   count_launch();
   TD_LAUNCH_CHECK();
 }

@@ -30,7 +30,7 @@ void sk_combo(const void* coef, DType tcoef, long long scm, long long sck, int M
 
 // The operator's Coulomb pair over factor rows A [M][K] (F32 or BF16) and FP32
 // vectors: t[m][n] = sum_k A[m][k] X[n][k] (X [N][K]), FP32 accumulation in runs of
-// at most 256 terms; out[n][c] = sum_k t[k][n] V[k][c] (t [K][N], V [K][ncols]).
+// at most 256 terms, whose sums are added in FP64; out[n][c] = sum_k t[k][n] V[k][c] (t [K][N], V [K][ncols]).
 // *tmax, when given, is raised to the float bits of max |t|.
 void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, float* t, cudaStream_t s,
                unsigned* tmax = nullptr);
