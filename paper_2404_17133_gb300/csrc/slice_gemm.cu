@@ -148,11 +148,12 @@ template <int S> struct Acc;
 template <> struct Acc<7> {
   // units 2^-40 (levels 0-3) and 2^-72 (levels 4-7) of the scaled product, less what
   // the runs still to come will add as bias
-  long long hi, lo;
-  static constexpr long long BIAS = 0x4b400000;   // bits of 1.5 2^23
+  // (unsigned: the biases pass 2^63 on the way, what is left in the end does not)
+  unsigned long long hi, lo;
+  static constexpr unsigned long long BIAS = 0x4b400000;   // bits of 1.5 2^23
   __device__ __forceinline__ void clear(int runs) {
-    hi = -(runs * ((BIAS << 24) + BIAS));
-    lo = -(runs * (BIAS << 8));
+    hi = 0ull - (unsigned long long)runs * ((BIAS << 24) + BIAS);
+    lo = 0ull - (unsigned long long)runs * (BIAS << 8);
   }
   // The level sums v of a run for two neighbours.  Conversions to integers run at 16
   // per clock and SM (eight per output bounded this step), so only levels 1, 2 and
@@ -173,9 +174,9 @@ template <> struct Acc<7> {
     b.add1(x0.y, v[1].y, x2.y, r3.y, x4.y, r56.y);
   }
   __device__ __forceinline__ void add1(float x0, float x1, float x2, float r3, float x4, float r56) {
-    hi += (long long)__float_as_int(x0) * 16777216 + (long long)__float2int_rn(x1) * 65536 +
-          (long long)__float2int_rn(x2) * 256 + (long long)__float_as_int(r3);
-    lo += (long long)__float2int_rn(x4) * 16777216 + (long long)__float_as_int(r56) * 256;
+    hi += (unsigned long long)((long long)__float_as_int(x0) * 16777216 + (long long)__float2int_rn(x1) * 65536 +
+                               (long long)__float2int_rn(x2) * 256 + (long long)__float_as_int(r3));
+    lo += (unsigned long long)((long long)__float2int_rn(x4) * 16777216 + (long long)__float_as_int(r56) * 256);
   }
   // The sum, times 2^40, times 2^e (scale exponents of the row and the column) by
   // integer arithmetic with one rounding: conversions and products on the FP64 units
@@ -183,7 +184,7 @@ template <> struct Acc<7> {
   __device__ __forceinline__ double value(int e) const {
     if (e >= kNotFinite / 2) return __longlong_as_double(0x7ff8000000000000ll);
     // 96 bits in three words, sign and magnitude
-    const long long h = hi + (lo >> 32);
+    const unsigned long long h = hi + (unsigned long long)((long long)lo >> 32);
     uint32_t w0 = (uint32_t)lo, w1 = (uint32_t)h, w2 = (uint32_t)(h >> 32);
     const uint32_t neg = w2 & 0x80000000u, m = (uint32_t)((int)w2 >> 31);
     asm("add.cc.u32 %0, %3, %6;\n addc.cc.u32 %1, %4, 0;\n addc.u32 %2, %5, 0;"
