@@ -143,13 +143,12 @@ void check_tc_error(Ctx& c) {
 // An operand of the sliced contractions with room for its slices.
 struct SliceCut {
   SliceOperand o;
-  DevBuf parts, exps;
+  DevBuf parts, info;
   void alloc(cudaStream_t st) {
     parts = DevBuf(slice_bytes(o), st);
-    exps = DevBuf((size_t)o.rows * 4, st);
+    info = DevBuf(slice_info_bytes(o), st);
   }
-  void cut(cudaStream_t st) { slice_cut(o, parts.p, exps.as<int>(), st); }
-  int* e() const { return exps.as<int>(); }
+  void cut(cudaStream_t st) { slice_cut(o, parts.p, info.p, st); }
 };
 static SliceCut slice_operand(const void* p, DType t, int rows, int np, int K) {
   SliceCut c;
@@ -166,7 +165,7 @@ static SliceCut slice_operand(const void* p, DType t, int rows, int np, int K) {
 static void coulomb_sliced(const OpDims& d, const FactorSet& f, const double* X, int m, double* J, cudaStream_t s) {
   const int ov = d.ov;
   const double* L = static_cast<const double*>(f.Jov);
-  const long long sb = 2 * slice_count(DType::F64);
+  const long long sb = slice_element_bytes(DType::F64);
   DevBuf t((size_t)f.nJ * m * 8, s);
   {
     SliceCut x = slice_operand(X, DType::F64, m, 1, ov);
@@ -181,7 +180,7 @@ static void coulomb_sliced(const OpDims& d, const FactorSet& f, const double* X,
       l.o.p = L + (long long)p0 * ov;
       l.o.rows = std::min(pc, f.nJ - p0);
       l.cut(s);
-      slice_gemm(l.o, l.parts.p, l.e(), x.o, x.parts.p, x.e(), t.as<double>() + (long long)p0 * m, 0.0, d.tc_err, s);
+      slice_gemm(l.o, l.parts.p, l.info.p, x.o, x.parts.p, x.info.p, t.as<double>() + (long long)p0 * m, 0.0, d.tc_err, s);
     }
   }
   SliceCut tt = slice_operand(t.p, DType::F64, m, 1, f.nJ);
@@ -196,7 +195,7 @@ static void coulomb_sliced(const OpDims& d, const FactorSet& f, const double* X,
     l.o.p = L + c0;
     l.o.rows = std::min(cc, ov - c0);
     l.cut(s);
-    slice_gemm_scatter(l.o, l.parts.p, l.e(), tt.o, tt.parts.p, tt.e(), J + c0, SliceScatter{1 << 30, 1 << 30, 0, ov, 0},
+    slice_gemm_scatter(l.o, l.parts.p, l.info.p, tt.o, tt.parts.p, tt.info.p, J + c0, SliceScatter{1 << 30, 1 << 30, 0, ov, 0},
                        d.tc_err, s);
   }
 }
@@ -208,7 +207,7 @@ static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw,
                             void* K2, cudaStream_t s) {
   const int no = d.no, nv = d.nv, ov = d.ov;
   const DType t = f.dt;
-  const size_t es = dtype_size(t), sb = 2 * (size_t)slice_count(t);
+  const size_t es = dtype_size(t), sb = (size_t)slice_element_bytes(t);
   const size_t nop = tc_pad(no), nvp = tc_pad(nv);
   const size_t per_row = (size_t)m * no * (nv * es + nvp * sb) + (no * nop + nv * nvp) * sb +
                          (need_k2 ? (size_t)m * no * (no * es + nop * sb) + (no * nvp + nv * nop) * sb : 0);
@@ -250,7 +249,7 @@ static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw,
     oo.o.p = (const char*)f.Koo + (size_t)p0 * no * no * es;
     oo.o.rows = pn * no;
     oo.cut(s);
-    slice_gemm_scatter(xt.o, xt.parts.p, xt.e(), oo.o, oo.parts.p, oo.e(), Zb.p,
+    slice_gemm_scatter(xt.o, xt.parts.p, xt.info.p, oo.o, oo.parts.p, oo.info.p, Zb.p,
                        SliceScatter{nv, no, (long long)no * pn * nv, (long long)pn * nv, nv}, d.tc_err, s);
     z.o.rs0 = (long long)pn * nv;
     z.o.np = pn;
@@ -260,7 +259,7 @@ static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw,
     vv.cut(s);
     const bool timed = d.prof_simt && d.prof_simt->on;
     if (timed) d.prof_simt->begin(s);
-    slice_gemm(z.o, z.parts.p, z.e(), vv.o, vv.parts.p, vv.e(), K1, beta, d.tc_err, s);
+    slice_gemm(z.o, z.parts.p, z.info.p, vv.o, vv.parts.p, vv.info.p, K1, beta, d.tc_err, s);
     if (timed)
       d.prof_simt->end(s, 2.0 * m * no * (double)nv * (double)pn * nv,
                        (double)es * ((double)m * no * pn * nv + (double)pn * nv * nv +
@@ -270,7 +269,7 @@ static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw,
       ov_.o.p = (const char*)f.Kov + (size_t)p0 * ov * es;
       ov_.o.rows = pn * no;
       ov_.cut(s);
-      slice_gemm_scatter(xs.o, xs.parts.p, xs.e(), ov_.o, ov_.parts.p, ov_.e(), Qb.p,
+      slice_gemm_scatter(xs.o, xs.parts.p, xs.info.p, ov_.o, ov_.parts.p, ov_.info.p, Qb.p,
                          SliceScatter{no, no, (long long)no * pn * no, (long long)pn * no, no}, d.tc_err, s);
       q.o.rs0 = (long long)pn * no;
       q.o.np = pn;
@@ -278,7 +277,7 @@ static void exchange_sliced(const OpDims& d, const FactorSet& f, const void* Xw,
       vo.o.p = ov_.o.p;
       vo.o.np = pn;
       vo.cut(s);
-      slice_gemm(q.o, q.parts.p, q.e(), vo.o, vo.parts.p, vo.e(), K2, beta, d.tc_err, s);
+      slice_gemm(q.o, q.parts.p, q.info.p, vo.o, vo.parts.p, vo.info.p, K2, beta, d.tc_err, s);
     }
   }
 }

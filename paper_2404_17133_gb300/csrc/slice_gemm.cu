@@ -13,8 +13,13 @@
 // 2^-32.)  Levels l < S are kept, each in its own TMEM columns; after each run
 // the epilogue warps move them to 64-bit integers (FP64) or a compensated FP32
 // pair (FP32), so nothing but the digits below the last slice is ever rounded
-// before the final scaling.  The error of a product is 2^-56 (2^-32) of
-// max|A row| max|B row| per term, below what FP64 (FP32) accumulation leaves.
+// before the final scaling.  An element is rounded to 2^-55 (2^-31) of its row's
+// largest at most, so the error of a product is 2^-55 (2^-31) of (max|A row| |b| +
+// |a| max|B row|) per term, and FP32 leaves out three products of up to 2^-28.4 max max
+// together.  Where an output's terms are as large as its rows' elements that is below
+// what FP64 (FP32) accumulation leaves; where they are not, the output is formed
+// again on the FP64 (FP32) units (the guard, below), so that none has fewer bits than
+// FP64 (FP32) arithmetic gives it.
 //
 // Why: FP64 runs at 1.2 TFLOP/s on this GPU's vector units and FP32 at 75; 34
 // or 10 FP16 products per term leave up to 57 and 190 TFLOP/s.
@@ -31,7 +36,8 @@
 //
 // Measured, 60 x 400 orbitals, contraction of 118 rows P with 10 vectors (FP64): 787 ->
 // 610 us (MMAs alone 528), its first stage 375 -> 233; 212 rows, 13 vectors (FP32): 550
-// -> 458 and 290 -> 126.  Not faster: CTA pairs (N = 64 in a pair takes twice the
+// -> 458 and 290 -> 126.  The guard takes 65 and 43 us per 103 rows (FP64), 85 and 63 per
+// 180 (FP32), and a sixth (fourth) more to store per element cut.  Not faster: CTA pairs (N = 64 in a pair takes twice the
 // clocks), two half tiles whose runs end half a run apart (711 and 701: the shorter
 // products cost more than the overlap of the epilogue gains).
 //
@@ -59,18 +65,42 @@ constexpr int SL_THREADS = 64 + 32 * EPI_WARPS;
 // Tiles of NT columns (a multiple of 16): LV levels of NT FP32 columns are at most
 // the tensor memory.
 template <int S> constexpr int max_cols() { return S == 7 ? 64 : 128; }
+// Tile width of a guard that writes its sums of a K split to out: twice the others', since it
+// is bound by fetching the magnitudes of long rows (780 x 400 outputs, K 73,000: 132 -> 85 us).
+constexpr int GUARD_SUMS = 256;
+template <int S> constexpr int run_length() { return S == 1 ? 1 << 24 : RUN; }   // the guard accumulates in one run
 template <int S, int W> struct SCfg {
   static constexpr int NT = W;
   // levels i + j kept: FP64 needs one beyond the slices (the six products of level 7
   // are 2^-58 of max max, 1e-15 of a result whose rows decay; without them the error
   // was 1.3e-15 against 1.2e-15 of FP64 arithmetic, with them 3.5e-16; 34 products
   // instead of 28)
-  static constexpr int LV = S == 7 ? 8 : 4;
+  static constexpr int LV = S == 7 ? 8 : S;
   static constexpr int A_SLICE = SBM * SBK * 2, B_SLICE = W * SBK * 2;
   static constexpr int STAGE_BYTES = S * (A_SLICE + B_SLICE);
-  static constexpr int STAGES = S == 7 ? 2 : 3;
+  static constexpr int STAGES = S == 7 ? 2 : (S == 4 ? 3 : (W == 256 ? 6 : 10));
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
-  static constexpr int TMEM_COLS = 512;
+  static constexpr int NBUF = S == 1 ? 2 : 1;   // sets of levels in tensor memory
+  static constexpr int TMEM_COLS = S == 1 ? 2 * W : 512;
+};
+
+// What the guard knows of an operand's rows: sum of the squared magnitudes (units
+// 2^-8), largest biased exponent field, nonzero elements; and where its elements are.
+struct RowInfo {
+  const unsigned long long* ss;
+  const int* e;
+  const unsigned* nnz;
+};
+struct View {
+  const void* p;
+  int R;
+  long long rs1, rs0, ps, ks;
+};
+struct Guard {
+  RowInfo ra, rb;
+  View a, b;
+  int np, K;
+  float wn, wc;   // weights of the row norms and of the element counts (guard_weights)
 };
 
 struct SParams {
@@ -85,6 +115,7 @@ struct SParams {
   int R, C;
   long long rs1, cs0, cs1;
   int* err;
+  Guard g;              // the guard's launches
 };
 
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2,
@@ -117,6 +148,17 @@ __device__ __forceinline__ void tmem_ld4(float (&v)[4], uint32_t taddr) {
   v[1] = __uint_as_float(r1);
   v[2] = __uint_as_float(r2);
   v[3] = __uint_as_float(r3);
+}
+
+__device__ __forceinline__ void tmem_ld16(float (&v)[16], uint32_t taddr) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 constexpr int kNotFinite = 1 << 20;   // exponent of a row that holds a non-finite value
@@ -215,40 +257,108 @@ template <> struct Acc<4> {
     a.hi = s.x; b.hi = s.y;
     a.lo = l.x; b.lo = l.y;
   }
-  __device__ __forceinline__ float value() const { return hi + lo; }
+  // times the scales r of the row and c of the column
+  __device__ __forceinline__ float value(float r, float c) const { return (hi + lo) * r * c; }
+  // Takes in the factor 2^e, where a product with one of the scales alone could leave FP32's
+  // range (of a special row or column: any number, the guard puts the result).
+  __device__ __forceinline__ void scale_any(int e) {
+    const int e1 = min(max(e, -126), 127), e2 = min(max(e - e1, -126), 127);
+    hi = (hi + lo) * __int_as_float((e1 + 127) << 23) * __int_as_float((e2 + 127) << 23);
+    lo = 0.f;
+  }
 };
 
-// Power-of-two scale of a row from its exponent word (the largest biased exponent
-// field, or the all-ones field where the row holds a non-finite value): FP64 as its
-// exponent, FP32 as its value.
-template <int S> __device__ __forceinline__ auto row_scale(int w);
-template <> __device__ __forceinline__ auto row_scale<7>(int w) { return w >= 2047 ? kNotFinite : max(w, 1) - 1041; }
-template <> __device__ __forceinline__ auto row_scale<4>(int w) {
-  const int E = max(w, 1);
-  if (E >= 255) return __int_as_float(0x7fc00000);
-  return E > 6 ? __int_as_float((E - 6) << 23) : ldexpf(1.f, E - 133);
+// Exponent of a row's power-of-two scale from its exponent word (the largest biased
+// exponent field, or the all-ones field where the row holds a non-finite value).
+template <int S> __device__ __forceinline__ int row_scale(int w);
+template <> __device__ __forceinline__ int row_scale<7>(int w) { return w >= 2047 ? kNotFinite : max(w, 1) - 1041; }
+template <> __device__ __forceinline__ int row_scale<4>(int w) { return w >= 255 ? kNotFinite : max(w, 1) - 133; }
+
+// ---------------------------------------------------------------------------
+// The guard.  Slices are fixed point against the largest element of a row, so an
+// output whose terms are all small beside max|A row| max|B row| (a row that spans
+// decades where the other operand has zeros) would have fewer bits than FP64 (FP32)
+// arithmetic gives it.  With the magnitudes a', b' = |x| 2^(14 - e) < 2^14 of a row
+// (2^e the power of two above its largest element), the error of a sliced output is
+// (root mean square over the roundings)
+//   FP64: 2^-42.8 (|a'| + |b'|),   FP32: 2^-18.8 (|a'| + |b'|) + 2^-4.8 sqrt(n)
+// (|.| 2-norms over the terms, n the nonzero elements of A's row: the three products of
+// FP32's dropped level 4), and that of a run of FP64 (FP32) additions is
+// 2^-54.3 N (2^-25.3 N) with N = sum_k a'_k b'_k.  N comes from one more FP16 product
+// of the magnitudes, and an output where it is too small for the slices to be as good
+// is formed again from the operands themselves on the FP64 (FP32) units: so is every
+// output of a row with a non-finite element, which then reaches what it meets and
+// no more.
+constexpr int kThreadTerms = 256;   // terms up to which a thread forms an output alone (else its warp)
+template <typename T> struct GuardWeights;   // of |.| and of sqrt(n)
+template <> struct GuardWeights<double> { static constexpr float NORM = 2896.f, COUNT = 0.f; };        // 2^(54.3 - 42.8)
+template <> struct GuardWeights<float> { static constexpr float NORM = 91.f, COUNT = 1482910.f; };     // 2^6.5, 2^20.5
+template <typename T> constexpr int kExpSpecial = sizeof(T) == 8 ? 2047 : 255;
+
+// A row's part of the bound on N; an output is formed again unless N - (the column's)
+// > (the row's).  A zero row is exact, a special one never (in both places: not exact).
+template <typename T>
+__device__ __forceinline__ float row_bound(const RowInfo& r, long long i, float wn, float wc) {
+  const int e = r.e[i];
+  const unsigned n = r.nnz[i];
+  const float ss = (float)r.ss[i];
+  if (e >= kExpSpecial<T>) return __int_as_float(0x7f800000);
+  return n == 0 ? __int_as_float(0xff800000) : fmaf(wn * 0.0625f, sqrtf(ss), wc * sqrtf((float)n));
 }
 
-template <int S, int W>
+template <typename T>
+__device__ __forceinline__ const T* row_of(const View& v, int r) {
+  const int q = r / v.R;
+  return static_cast<const T*>(v.p) + q * v.rs1 + (r - q * v.R) * v.rs0;
+}
+// The output (r, c) on the FP64 or FP32 units, by one thread.
+template <typename T>
+__device__ T dot_thread(const Guard& g, int r, int c) {
+  const T *a = row_of<T>(g.a, r), *b = row_of<T>(g.b, c);
+  T acc = T(0);
+  for (int P = 0; P < g.np; ++P) {
+    const T *x = a + P * g.a.ps, *y = b + P * g.b.ps;
+#pragma unroll 8
+    for (int k = 0; k < g.K; ++k) acc = fma(x[k * g.a.ks], y[k * g.b.ks], acc);
+  }
+  return acc;
+}
+// The same by a warp, the terms dealt to its lanes; every lane gets it.
+template <typename T>
+__device__ T dot_warp(const Guard& g, int r, int c) {
+  const T *a = row_of<T>(g.a, r), *b = row_of<T>(g.b, c);
+  T acc = T(0);
+  int k = threadIdx.x & 31, P = 0;
+  while (k >= g.K && P < g.np) { k -= g.K; ++P; }
+  while (P < g.np) {
+    acc = fma(a[P * g.a.ps + k * g.a.ks], b[P * g.b.ps + k * g.b.ks], acc);
+    k += 32;
+    while (k >= g.K && P < g.np) { k -= g.K; ++P; }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
+
+// S = 1: the guard over the magnitudes, of operands of type T.
+template <int S, int W, typename T>
 __global__ void __launch_bounds__(SL_THREADS, 1)
 k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, const SParams p) {
   using C = SCfg<S, W>;
-  using T = typename std::conditional<S == 7, double, float>::type;
-  constexpr int NT = C::NT;
+  constexpr int NT = C::NT, RUNL = run_length<S>();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::STAGES * C::STAGE_BYTES);
   uint64_t* empty = full + C::STAGES;
   uint64_t* tfull = empty + C::STAGES;    // the run's levels are complete
-  uint64_t* tempty = tfull + 1;           // ... and have been read
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 1);
+  uint64_t* tempty = tfull + C::NBUF;     // ... and have been read
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + C::NBUF);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    mbar_init(tfull, 1);
-    mbar_init(tempty, EPI_WARPS);
+    for (int b = 0; b < C::NBUF; ++b) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], EPI_WARPS); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -301,7 +411,7 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
     static_assert(2 * G >= S && C::LV <= S + 1, "slice_gemm: slices per product");
     const uint64_t da0 = sdesc64(smem);
     const int tail = p.Kin - (p.nab - 1) * SBK > 16 ? 2 : 1;   // 16-element K steps of a P's last k-block
-    uint32_t s = 0, ph = 0, run = 0;
+    uint32_t s = 0, ph = 0, run = 0, buf = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x) {
       int k0, nk;
@@ -310,8 +420,9 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
       for (int b = 0; b < nk; ++b) {
         const bool start = left == 0;
         if (start) {
-          left = min(RUN, nk - b);
-          if (!mbar_wait(tempty, (run++ & 1u) ^ 1u)) { ok = false; break; }
+          left = min(RUNL, nk - b);
+          buf = run % C::NBUF;
+          if (!mbar_wait(&tempty[buf], ((run++ / C::NBUF) & 1u) ^ 1u)) { ok = false; break; }
         }
         if (!mbar_wait(&full[s], ph)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -327,7 +438,7 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
             const uint64_t a = a0 + ia * (C::A_SLICE / 16);
             const int nbs = S < C::LV - ia ? S : C::LV - ia;    // slices of B that ia meets
             const int n0 = nbs < G ? nbs : G, n1 = nbs - n0;
-            const uint32_t d = tmem + (uint32_t)(ia * W);
+            const uint32_t d = tmem + buf * W + (uint32_t)(ia * W);
             if (C::LV > S && j == 1 && first) {
               mma_f16(d, a, b0, 1u, IDESC + NB);
               mma_f16(d + W, a, b0 + C::B_SLICE / 16, 0u, IDESC + NB);
@@ -339,7 +450,7 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
           }
         }
         mma_commit(&empty[s]);
-        if (--left == 0) mma_commit(tfull);
+        if (--left == 0) mma_commit(&tfull[buf]);
         if (++s == C::STAGES) { s = 0; ph ^= 1u; }
         if (++pos == p.nab) pos = 0;
       }
@@ -360,10 +471,105 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
       const int row = m0 + lane;
       const bool live = m0 < p.M;            // this warp has rows to read
       const int ncol = min(HC, p.N - n0);    // columns of this warp (may be <= 0)
+      if constexpr (S == 1) {
+        static_assert(W == GUARD_SUMS || HC <= 64, "one bit per column");
+        constexpr bool SUMS = W == GUARD_SUMS;   // k_slice_sum judges
+        // the bounds of this warp's rows and columns, while the tile is being formed
+        __shared__ __align__(16) float colb[EPI_WARPS][HC];
+        const float ninf = __int_as_float(0xff800000);
+        const bool inside = row < p.M;
+        float ba = ninf;
+        float* cb = colb[warp - 2];
+        if (!SUMS) {
+          if (inside) ba = row_bound<T>(p.g.ra, row, p.g.wn, p.g.wc);
+          for (int c = lane; c < HC; c += 32) cb[c] = c < ncol ? row_bound<T>(p.g.rb, n0 + c, p.g.wn, 0.f) : ninf;
+          __syncwarp();
+        }
+        const uint32_t buf = run % C::NBUF;
+        bool got = mbar_wait(&tfull[buf], (run / C::NBUF) & 1u);
+        ++run;
+        got = __all_sync(0xffffffffu, got);
+        if (!got) { if (lane == 0) atomicOr(p.err, 4096); ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        unsigned long long again = 0;
+        if (live) {
+#pragma unroll 1
+          for (int c = 0; c < ncol; c += 16) {
+            float v[16];
+            tmem_ld16(v, tb + buf * W + (uint32_t)c);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (SUMS) {
+              float* o = static_cast<float*>(p.out) + ((long long)(item / p.tiles) * p.M + row) * p.N + n0 + c;
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                if (inside && c + j < ncol) o[j] = v[j];
+            } else {
+              float least = __int_as_float(0x7f800000);
+#pragma unroll
+              for (int j = 0; j < 16; j += 4) {
+                const float4 b4 = *reinterpret_cast<const float4*>(cb + c + j);
+                v[j] -= b4.x; v[j + 1] -= b4.y; v[j + 2] -= b4.z; v[j + 3] -= b4.w;
+                least = fminf(least, fminf(fminf(v[j], v[j + 1]), fminf(v[j + 2], v[j + 3])));
+              }
+              if (!(least > ba)) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  if (!(v[j] > ba)) again |= 1ull << (c + j);
+              }
+            }
+          }
+          if (!inside) again = 0;
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])) : "memory");
+        if (!SUMS && __any_sync(0xffffffffu, again != 0)) {
+          T* out = static_cast<T*>(p.out);
+          auto put = [&](int r, int col, T v) {
+            out[p.scatter ? (long long)(r / p.R) * p.rs1 + r % p.R + (long long)(col / p.C) * p.cs1 +
+                                (long long)(col % p.C) * p.cs0
+                          : (long long)r * p.N + col] = v;
+          };
+          if (p.g.np * p.g.K <= kThreadTerms) {
+            // 16 columns at a time, dealt to the lanes (one row may hold most of them)
+            __shared__ unsigned short list[EPI_WARPS][512];
+            unsigned short* mine = list[warp - 2];
+            for (int c = 0; c < ncol; c += 16) {
+              unsigned bits = (unsigned)(again >> c) & (ncol - c < 16 ? (1u << (ncol - c)) - 1u : 0xffffu);
+              const int n = __popc(bits);
+              int at = n;
+#pragma unroll
+              for (int o = 1; o < 32; o <<= 1) {
+                const int q = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += q;
+              }
+              const int total = __shfl_sync(0xffffffffu, at, 31);
+              at -= n;
+              for (; bits; bits &= bits - 1) mine[at++] = (unsigned short)(lane << 8 | (__ffs(bits) - 1));
+              __syncwarp();
+              for (int e = lane; e < total; e += 32) {
+                const int r = m0 + (mine[e] >> 8), col = n0 + c + (mine[e] & 255);
+                put(r, col, dot_thread<T>(p.g, r, col));
+              }
+              __syncwarp();
+            }
+          } else {
+            for (int c = 0; c < ncol; ++c) {
+              const bool mine = again >> c & 1;
+              for (unsigned who = __ballot_sync(0xffffffffu, mine); who; who &= who - 1) {
+                const int src = __ffs(who) - 1;
+                const T v = dot_warp<T>(p.g, m0 + src, n0 + c);
+                if (lane == src) put(row, n0 + c, v);
+              }
+            }
+          }
+          __syncwarp();
+        }
+      } else {
       Acc<S> acc[HC];
 #pragma unroll
-      for (int c = 0; c < HC; ++c) acc[c].clear((nk + RUN - 1) / RUN);
-      for (int kb = 0; kb < nk; kb += RUN, ++run) {
+      for (int c = 0; c < HC; ++c) acc[c].clear((nk + RUNL - 1) / RUNL);
+      for (int kb = 0; kb < nk; kb += RUNL, ++run) {
         bool got = mbar_wait(tfull, run & 1u);
         got = __all_sync(0xffffffffu, got);
         if (!got) { if (lane == 0) atomicOr(p.err, 2048); ok = false; break; }
@@ -392,12 +598,12 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
       }
       if (!ok || !live || ncol <= 0) continue;
       // the columns' scales, one or two per lane, dealt out by shuffles
-      decltype(row_scale<S>(0)) sb[(HC + 31) / 32];
+      int sb[(HC + 31) / 32];
 #pragma unroll
       for (int j = 0; j < (HC + 31) / 32; ++j)
         sb[j] = row_scale<S>(32 * j + lane < ncol ? p.eb[n0 + 32 * j + lane] : 0);
       const bool inside = row < p.M;
-      const auto sa = row_scale<S>(inside ? p.ea[row] : 0);
+      const int sa = row_scale<S>(inside ? p.ea[row] : 0);
       T* out = static_cast<T*>(p.out);
       long long at, step = 1;
       int cr = 0;
@@ -408,13 +614,34 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
       } else {
         at = ((long long)(item / p.tiles) * p.M + row) * p.N + n0;
       }
+      // FP32: scales near enough to 1 are multiplied one after the other
+      bool near = true;
+      float fa = 1.f, fb[(HC + 31) / 32];
+      if constexpr (S == 4) {
+        near = !inside || (sa >= -60 && sa <= 60);
+        fa = __int_as_float((max(-60, min(sa, 60)) + 127) << 23);
+#pragma unroll
+        for (int j = 0; j < (HC + 31) / 32; ++j) {
+          near = near && (32 * j + lane >= ncol || (sb[j] >= -60 && sb[j] <= 60));
+          fb[j] = __int_as_float((max(-60, min(sb[j], 60)) + 127) << 23);
+        }
+        if (!__all_sync(0xffffffffu, near)) {
+#pragma unroll
+          for (int c = 0; c < HC; ++c) acc[c].scale_any(sa + __shfl_sync(0xffffffffu, sb[c / 32], c & 31));
+          fa = 1.f;
+#pragma unroll
+          for (int j = 0; j < (HC + 31) / 32; ++j) fb[j] = 1.f;
+        }
+      }
       const long long wrap = p.cs1 - (long long)(p.C - 1) * p.cs0;   // from the last of C columns to the next first
 #pragma unroll
       for (int c = 0; c < HC; ++c) {
-        const auto w = __shfl_sync(0xffffffffu, sb[c / 32], c & 31);
-        if (c < ncol && inside) {
-          if constexpr (S == 7) out[at] = acc[c].value(sa + w);
-          else out[at] = acc[c].value() * sa * w;
+        if constexpr (S == 4) {
+          const float w = __shfl_sync(0xffffffffu, fb[c / 32], c & 31);
+          if (c < ncol && inside) out[at] = acc[c].value(fa, w);
+        } else {
+          const int w = __shfl_sync(0xffffffffu, sb[c / 32], c & 31);
+          if (c < ncol && inside) out[at] = acc[c].value(sa + w);
         }
         if (p.scatter && ++cr == p.C) {
           cr = 0;
@@ -422,6 +649,7 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
         } else {
           at += step;
         }
+      }
       }
     }
   }
@@ -478,12 +706,37 @@ __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned lo
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// The guard's magnitude of x against the row exponent E: |x| scaled to less than 2^14
+// (zero 2^-40 below the largest, where FP16 ends).
+__device__ __forceinline__ float magnitude(double x, int E) {
+  const long long bits = __double_as_longlong(x);
+  const int ef = (int)((bits >> 52) & 0x7ff), r = E - ef;
+  return ef == 0 || r > 40 ? 0.f : __uint_as_float((unsigned)(140 - r) << 23 | ((unsigned)(bits >> 29) & 0x7fffffu));
+}
+__device__ __forceinline__ float magnitude(float x, int E) {
+  const unsigned bits = __float_as_uint(x);
+  const int ef = (int)((bits >> 23) & 0xff), r = E - ef;
+  return ef == 0 || r > 40 ? 0.f : __uint_as_float((unsigned)(140 - r) << 23 | (bits & 0x7fffffu));
+}
+
+// Eight elements' slices and magnitudes; their squared magnitudes and number of
+// nonzeros are added to ss and nnz.
 template <typename T, int S>
-__device__ __forceinline__ void store_slices(const T (&x)[8], int E, __half* dst, long long slice) {
+__device__ __forceinline__ void store_slices(const T (&x)[8], int E, __half* dst, long long slice, float& ss, int& nnz) {
   unsigned long long d[8];
-  const bool special = E >= (S == 7 ? 2047 : 255);
+  const bool special = E >= kExpSpecial<T>;
+  __half2 mag[4];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) d[j] = digits(special ? T(0) : x[j], E);
+  for (int j = 0; j < 8; j += 2) {
+    const T x0 = special ? T(0) : x[j], x1 = special ? T(0) : x[j + 1];
+    d[j] = digits(x0, E);
+    d[j + 1] = digits(x1, E);
+    const float m0 = magnitude(x0, E), m1 = magnitude(x1, E);
+    mag[j / 2] = __floats2half2_rn(m0, m1);
+    ss = fmaf(m0, m0, fmaf(m1, m1, ss));
+    nnz += (x0 != T(0)) + (x1 != T(0));
+  }
+  *reinterpret_cast<uint4*>(dst + S * slice) = *reinterpret_cast<const uint4*>(mag);
 #pragma unroll
   for (int s = 0; s < S; ++s) {
     uint4 w;
@@ -500,8 +753,11 @@ struct CutParams {
   int rows, np, K, ldk, R, p_outer, vec;
   long long rs1, rs0, ps, ks;
   __half* dst;
+  unsigned long long* ss;   // per row, see RowInfo
   int* exps;
+  unsigned* nnz;
 };
+__device__ __forceinline__ unsigned long long fixed_ss(float ss) { return __float2ull_ru(ss * 256.f); }
 
 __device__ __forceinline__ long long cut_dst(const CutParams& c, long long r, int P) {
   return (c.p_outer ? (long long)P * c.rows + r : r * c.np + P) * c.ldk;
@@ -530,6 +786,31 @@ __device__ __forceinline__ void load8(const float* p, int n, bool vec, float (&v
   } else {
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = j < n ? p[j] : 0.f;
+  }
+}
+
+// Sums over groups of TPR neighbouring threads (256: the CTA) in a fixed order, for the
+// group's first thread.
+template <int TPR>
+__device__ __forceinline__ void sum_group(float& ss, int& nnz) {
+  __shared__ float rs[8];
+  __shared__ int rn[8];
+#pragma unroll
+  for (int o = (TPR < 32 ? TPR : 32) / 2; o > 0; o >>= 1) {
+    ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    nnz += __shfl_xor_sync(0xffffffffu, nnz, o);
+  }
+  if (TPR > 32) {
+    if ((threadIdx.x & 31) == 0) {
+      rs[threadIdx.x >> 5] = ss;
+      rn[threadIdx.x >> 5] = nnz;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int w = 1; w < 8; ++w) {
+        ss += rs[w];
+        nnz += rn[w];
+      }
   }
 }
 
@@ -562,13 +843,20 @@ __global__ void __launch_bounds__(256) k_slice_rows(const CutParams c) {
 #pragma unroll
     for (int w = 0; w < 8; ++w) E = max(E, red[w]);
   }
-  if (have && sub == 0) c.exps[r] = E;
   const long long slice = (long long)c.rows * c.np * c.ldk;
+  float ss = 0.f;
+  int nnz = 0;
   for (int g = sub; g < ng; g += TPR) {
     const int P = g / n8, k0 = (g - P * n8) * 8;
     T v[8];
     load8(x + P * c.ps + k0, c.K - k0, c.vec, v);
-    store_slices<T, S>(v, E, c.dst + cut_dst(c, r, P) + k0, slice);
+    store_slices<T, S>(v, E, c.dst + cut_dst(c, r, P) + k0, slice, ss, nnz);
+  }
+  sum_group<TPR>(ss, nnz);
+  if (have && sub == 0) {
+    c.exps[r] = E;
+    c.ss[r] = fixed_ss(ss);
+    c.nnz[r] = (unsigned)nnz;
   }
 }
 
@@ -604,12 +892,19 @@ __global__ void __launch_bounds__(256) k_slice_seg(const CutParams c) {
   } else {
     const int E = c.exps[r];
     const long long slice = (long long)c.rows * c.np * c.ldk;
+    float ss = 0.f;
+    int nnz = 0;
 #pragma unroll 2
     for (int g = blockIdx.y * SEG + threadIdx.x; g < g1; g += 256) {
       const int P = g / n8, k0 = (g - P * n8) * 8;
       T v[8];
       load8(x + P * c.ps + k0, c.K - k0, c.vec, v);
-      store_slices<T, S>(v, E, c.dst + cut_dst(c, r, P) + k0, slice);
+      store_slices<T, S>(v, E, c.dst + cut_dst(c, r, P) + k0, slice, ss, nnz);
+    }
+    sum_group<256>(ss, nnz);
+    if (threadIdx.x == 0) {   // whole numbers: the same sum in any order
+      atomicAdd(&c.ss[r], fixed_ss(ss));
+      atomicAdd(&c.nnz[r], (unsigned)nnz);
     }
   }
 }
@@ -641,6 +936,8 @@ __global__ void __launch_bounds__(256) k_slice_cut_t(const CutParams c) {
   const T* x = static_cast<const T*>(c.p) + (rl < c.rows ? (rl / c.R) * c.rs1 + (rl % c.R) : 0);
   const int rr = w * 4 + (lane >> 3), kg = (lane & 7) * 8;   // the row and 8-element group this thread cuts
   const int E = r0 + rr < c.rows ? c.exps[r0 + rr] : 0;
+  float ss = 0.f;
+  int nnz = 0;
   for (int P = blockIdx.y; P < c.np; P += gridDim.y)
     for (int k0 = 0; k0 < c.K; k0 += 64) {
       __syncthreads();
@@ -652,25 +949,64 @@ __global__ void __launch_bounds__(256) k_slice_cut_t(const CutParams c) {
         T v[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = tile[kg + j][rr];
-        store_slices<T, S>(v, E, c.dst + cut_dst(c, r0 + rr, P) + k0 + kg, slice);
+        store_slices<T, S>(v, E, c.dst + cut_dst(c, r0 + rr, P) + k0 + kg, slice, ss, nnz);
       }
     }
-}
-
-// Sum of the K-split partials in a fixed order (FP64), C = sum + beta C.
-template <typename T>
-__global__ void k_slice_sum(const T* __restrict__ part, int S, long long MN, T* C, double beta) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < MN; t += (long long)gridDim.x * blockDim.x) {
-    double v = 0.0;
-    for (int s = 0; s < S; ++s) v += (double)part[s * MN + t];
-    if (beta != 0.0) v += beta * (double)C[t];
-    C[t] = (T)v;
+  sum_group<8>(ss, nnz);
+  if ((lane & 7) == 0 && r0 + rr < c.rows) {
+    atomicAdd(&c.ss[r0 + rr], fixed_ss(ss));
+    atomicAdd(&c.nnz[r0 + rr], (unsigned)nnz);
   }
 }
 
-CUtensorMap slice_map(const SliceOperand& o, const void* parts, int box_rows) {
-  const int S = slice_count(o.t);
+// Sum of the K-split partials in a fixed order (FP64), C = sum + beta C; N: the
+// guard's partials, whose verdict falls here: the outputs to be formed again are
+// dealt to the CTA's warps.  A CTA takes OPB outputs.
+template <typename T, int OPB>
+__global__ void __launch_bounds__(256) k_slice_sum(const T* __restrict__ part, int S, const float* __restrict__ N, int SN,
+                                                   long long M, int ncol, T* C, double beta, const Guard g) {
+  __shared__ T again[OPB];      // values formed again
+  __shared__ int list[OPB];
+  __shared__ int count;
+  const long long MN = M * ncol;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (long long t0 = (long long)blockIdx.x * OPB; t0 < MN; t0 += (long long)gridDim.x * OPB) {
+    const long long t = t0 + tid;
+    const bool in = tid < OPB && t < MN;
+    double v = 0.0;
+    bool bad = false;
+    if (tid == 0) count = 0;
+    __syncthreads();
+    if (in) {
+      for (int s = 0; s < S; ++s) v += (double)part[s * MN + t];
+      float n = 0.f;
+      for (int s = 0; s < SN; ++s) n += N[s * MN + t];
+      const long long r = t / ncol;
+      bad = !(n - row_bound<T>(g.rb, t - r * ncol, g.wn, 0.f) > row_bound<T>(g.ra, r, g.wn, g.wc));
+      if (bad) list[atomicAdd(&count, 1)] = tid;
+    }
+    if (__syncthreads_or(bad)) {
+      for (int q = warp; q < count; q += 8) {
+        const long long u = t0 + list[q], r = u / ncol;
+        const T w = dot_warp<T>(g, (int)r, (int)(u - r * ncol));
+        if (lane == 0) again[list[q]] = w;
+      }
+      __syncthreads();
+      if (bad) v = (double)again[tid];
+    }
+    if (in) {
+      if (beta != 0.0) v += beta * (double)C[t];
+      C[t] = (T)v;
+    }
+    __syncthreads();
+  }
+}
+
+// guard: the magnitudes, which follow the slices
+CUtensorMap slice_map(const SliceOperand& o, const void* parts, int box_rows, bool guard) {
+  const int S = guard ? 1 : slice_count(o.t);
   const long long ldk = tc_pad(o.K);
+  if (guard) parts = static_cast<const __half*>(parts) + slice_count(o.t) * (long long)o.rows * o.np * ldk;
   // (k, P, row, slice) or, p_outer, (k, row, P, slice)
   const uint64_t n1 = o.p_outer ? o.rows : o.np, n2 = o.p_outer ? o.np : o.rows;
   const uint64_t dims[4] = {(uint64_t)o.K, n1, n2, (uint64_t)S};
@@ -679,13 +1015,13 @@ CUtensorMap slice_map(const SliceOperand& o, const void* parts, int box_rows) {
   return tc_map_f16_4d(parts, dims, strides, box, 64);
 }
 
-template <int S, int W>
+template <int S, int W, typename T>
 void launch_cols(const SliceOperand& A, const void* Ap, const SliceOperand& B, const void* Bp, const SParams& p,
                  cudaStream_t s) {
   using C = SCfg<S, W>;
-  const CUtensorMap ma = slice_map(A, Ap, SBM), mb = slice_map(B, Bp, W);
-  ensure_smem((const void*)k_slice_mma<S, W>, C::SMEM_BYTES);
-  k_slice_mma<S, W><<<std::min(p.items, sm_count()), SL_THREADS, C::SMEM_BYTES, s>>>(ma, mb, p);
+  const CUtensorMap ma = slice_map(A, Ap, SBM, S == 1), mb = slice_map(B, Bp, W, S == 1);
+  ensure_smem((const void*)k_slice_mma<S, W, T>, C::SMEM_BYTES);
+  k_slice_mma<S, W, T><<<std::min(p.items, sm_count()), SL_THREADS, C::SMEM_BYTES, s>>>(ma, mb, p);
   count_launch();
   TD_LAUNCH_CHECK();
 }
@@ -694,21 +1030,47 @@ void launch_mma(const SliceOperand& A, const void* Ap, const SliceOperand& B, co
                 cudaStream_t s) {
   p.items = p.tiles * splits;
   if (A.t == DType::F64) {
-    if (p.w <= 16) launch_cols<7, 16>(A, Ap, B, Bp, p, s);
-    else if (p.w <= 32) launch_cols<7, 32>(A, Ap, B, Bp, p, s);
-    else if (p.w <= 48) launch_cols<7, 48>(A, Ap, B, Bp, p, s);
-    else launch_cols<7, 64>(A, Ap, B, Bp, p, s);
+    if (p.w <= 16) launch_cols<7, 16, double>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 32) launch_cols<7, 32, double>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 48) launch_cols<7, 48, double>(A, Ap, B, Bp, p, s);
+    else launch_cols<7, 64, double>(A, Ap, B, Bp, p, s);
   } else {
-    if (p.w <= 32) launch_cols<4, 32>(A, Ap, B, Bp, p, s);
-    else if (p.w <= 64) launch_cols<4, 64>(A, Ap, B, Bp, p, s);
-    else if (p.w <= 96) launch_cols<4, 96>(A, Ap, B, Bp, p, s);
-    else if (p.w <= 112) launch_cols<4, 112>(A, Ap, B, Bp, p, s);
-    else launch_cols<4, 128>(A, Ap, B, Bp, p, s);
+    if (p.w <= 32) launch_cols<4, 32, float>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 64) launch_cols<4, 64, float>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 96) launch_cols<4, 96, float>(A, Ap, B, Bp, p, s);
+    else if (p.w <= 112) launch_cols<4, 112, float>(A, Ap, B, Bp, p, s);
+    else launch_cols<4, 128, float>(A, Ap, B, Bp, p, s);
   }
 }
 
+// The guard's launch: p as for the product, in tiles of its own.
+void launch_guard(const SliceOperand& A, const void* Ap, const SliceOperand& B, const void* Bp, SParams p, int splits,
+                  cudaStream_t s) {
+  p.items = p.tiles * splits;
+  if (p.w == GUARD_SUMS) launch_cols<1, GUARD_SUMS, float>(A, Ap, B, Bp, p, s);   // (of either type)
+  else if (A.t == DType::F64) {
+    if (p.w <= 32) launch_cols<1, 32, double>(A, Ap, B, Bp, p, s);
+    else launch_cols<1, 128, double>(A, Ap, B, Bp, p, s);
+  } else {
+    if (p.w <= 32) launch_cols<1, 32, float>(A, Ap, B, Bp, p, s);
+    else launch_cols<1, 128, float>(A, Ap, B, Bp, p, s);
+  }
+}
+
+// Row information of an operand behind `info` (info_bytes).
+RowInfo row_info(const SliceOperand& o, const void* info) {
+  RowInfo r;
+  r.ss = static_cast<const unsigned long long*>(info);
+  r.e = reinterpret_cast<const int*>(r.ss + o.rows);
+  r.nnz = reinterpret_cast<const unsigned*>(r.e + o.rows);
+  return r;
+}
+View view_of(const SliceOperand& o) { return View{o.p, o.R, o.rs1, o.rs0, o.ps, o.ks}; }
+
+// Parameters of a product of S slices (1: its guard).
 template <int S>
-SParams make_params(const SliceOperand& A, const int* Ae, const SliceOperand& B, const int* Be, int* err) {
+SParams make_params(const SliceOperand& A, const void* Ai, const SliceOperand& B, const void* Bi, int* err,
+                    bool sums = false) {
   SParams p;
   std::memset(&p, 0, sizeof(p));
   p.M = A.rows;
@@ -717,20 +1079,41 @@ SParams make_params(const SliceOperand& A, const int* Ae, const SliceOperand& B,
   p.nab = (A.K + SBK - 1) / SBK;
   p.total = p.nab * A.np;
   p.per = p.total;
-  // the fewest tiles, of equal width (rounded up to the next instance by launch_mma)
-  p.tiles_n = (p.N + max_cols<S>() - 1) / max_cols<S>();
-  p.w = (p.N + p.tiles_n - 1) / p.tiles_n;
-  constexpr int widths[2][5] = {{16, 32, 48, 64, 64}, {32, 64, 96, 112, 128}};
-  for (int w : widths[S == 7 ? 0 : 1])
-    if (w >= p.w) { p.w = w; break; }
+  if constexpr (S == 1) {
+    p.w = sums ? GUARD_SUMS : (p.N <= 32 ? 32 : 128);
+    p.tiles_n = (p.N + p.w - 1) / p.w;
+  } else {
+    // the fewest tiles, of equal width, rounded up to an instance (at most 16 columns of a
+    // narrower tile are idle in FP64; in FP32 the widths between 64 and 128 are those at
+    // which 256 columns per MMA are best filled: 2 x 96, 2 x 112, 2 x 128)
+    p.tiles_n = (p.N + max_cols<S>() - 1) / max_cols<S>();
+    p.w = (p.N + p.tiles_n - 1) / p.tiles_n;
+    constexpr int widths[2][5] = {{16, 32, 48, 64, 64}, {32, 64, 96, 112, 128}};
+    for (int w : widths[S == 7 ? 0 : 1])
+      if (w >= p.w) { p.w = w; break; }
+  }
   const long long tiles = (long long)p.tiles_n * ((p.M + SBM - 1) / SBM);
   TD_REQUIRE(tiles < (1 << 28) && (long long)p.nab * A.np < (1 << 28), TDDFT_ERR_ARG, "slice_gemm: problem too large");
   p.tiles = (int)tiles;
-  p.ea = Ae;
-  p.eb = Be;
+  const RowInfo ra = row_info(A, Ai), rb = row_info(B, Bi);
+  p.ea = ra.e;
+  p.eb = rb.e;
   p.err = err;
   p.R = p.C = 1;
+  const bool f64 = A.t == DType::F64;
+  using GD = GuardWeights<double>;
+  using GF = GuardWeights<float>;
+  p.g = Guard{ra, rb, view_of(A), view_of(B), A.np, A.K, f64 ? GD::NORM : GF::NORM, f64 ? GD::COUNT : GF::COUNT};
   return p;
+}
+
+// K splits in whole runs; a CTA's fixed cost (pipeline fill, output) is about half a run
+int choose_splits(SParams& p) {
+  const int runs = (p.total + RUN - 1) / RUN;
+  int splits = wave_splits(p.tiles, runs, 1);
+  const int per = (runs + splits - 1) / splits;
+  p.per = per * RUN;
+  return (runs + per - 1) / per;
 }
 
 void check_pair(const SliceOperand& A, const SliceOperand& B) {
@@ -745,7 +1128,7 @@ void cut_t(const SliceOperand& o, const CutParams& c, cudaStream_t s) {
     const long long groups = (long long)o.np * (tc_pad(o.K) / 8);
     const long long segs = (groups + SEG - 1) / SEG;
     if (segs > 2 && segs <= 65535) {
-      TD_CUDA(cudaMemsetAsync(c.exps, 0, (size_t)o.rows * 4, s));
+      TD_CUDA(cudaMemsetAsync(c.ss, 0, slice_info_bytes(o), s));
       const dim3 grid(o.rows, (unsigned)segs);
       k_slice_seg<T, S, true><<<grid, 256, 0, s>>>(c);
       k_slice_seg<T, S, false><<<grid, 256, 0, s>>>(c);
@@ -755,7 +1138,7 @@ void cut_t(const SliceOperand& o, const CutParams& c, cudaStream_t s) {
     else k_slice_rows<T, S, 8><<<(o.rows + 31) / 32, 256, 0, s>>>(c);
     count_launch();
   } else {
-    TD_CUDA(cudaMemsetAsync(c.exps, 0, (size_t)o.rows * 4, s));
+    TD_CUDA(cudaMemsetAsync(c.ss, 0, slice_info_bytes(o), s));
     const int rt = (o.rows + 31) / 32;
     const dim3 grid(rt, std::min(o.np, std::max(1, 16 * 152 / rt)));
     k_slice_exp_t<T><<<grid, 256, 0, s>>>(c);
@@ -768,58 +1151,74 @@ void cut_t(const SliceOperand& o, const CutParams& c, cudaStream_t s) {
 }  // namespace
 
 size_t slice_bytes(const SliceOperand& o) {
-  return (size_t)slice_count(o.t) * o.rows * o.np * tc_pad(o.K) * 2;
+  return (size_t)slice_element_bytes(o.t) * o.rows * o.np * tc_pad(o.K);
 }
 
-void slice_cut(const SliceOperand& o, void* parts, int* exps, cudaStream_t s) {
+void slice_cut(const SliceOperand& o, void* parts, void* info, cudaStream_t s) {
   TD_REQUIRE((o.t == DType::F64 || o.t == DType::F32) && (o.ks == 1 || o.rs0 == 1) && o.rows >= 1 && o.K >= 1,
              TDDFT_ERR_ARG, "slice_cut: unsupported operand");
   const long long es = (long long)dtype_size(o.t);
   const bool vec = o.ks == 1 && reinterpret_cast<uintptr_t>(o.p) % 16 == 0 && o.rs0 * es % 16 == 0 &&
                    o.rs1 * es % 16 == 0 && o.ps * es % 16 == 0;
+  const RowInfo ri = row_info(o, info);
   const CutParams c{o.p, o.rows, o.np, o.K, tc_pad(o.K), o.R, o.p_outer ? 1 : 0, vec ? 1 : 0, o.rs1, o.rs0, o.ps,
-                    o.ks, static_cast<__half*>(parts), exps};
+                    o.ks, static_cast<__half*>(parts), const_cast<unsigned long long*>(ri.ss), const_cast<int*>(ri.e),
+                    const_cast<unsigned*>(ri.nnz)};
   TD_REQUIRE((long long)o.np * (tc_pad(o.K) / 8) < (1ll << 31), TDDFT_ERR_ARG, "slice_cut: row too long");
   if (o.t == DType::F64) cut_t<double, 7>(o, c, s);
   else cut_t<float, 4>(o, c, s);
 }
 
-void slice_gemm_scatter(const SliceOperand& A, const void* Ap, const int* Ae, const SliceOperand& B, const void* Bp,
-                        const int* Be, void* out, const SliceScatter& sc, int* err, cudaStream_t s) {
+void slice_gemm_scatter(const SliceOperand& A, const void* Ap, const void* Ai, const SliceOperand& B, const void* Bp,
+                        const void* Bi, void* out, const SliceScatter& sc, int* err, cudaStream_t s) {
   check_pair(A, B);
   const bool f64 = A.t == DType::F64;
-  SParams p = f64 ? make_params<7>(A, Ae, B, Be, err) : make_params<4>(A, Ae, B, Be, err);
-  p.out = out;
-  p.scatter = 1;
-  p.R = sc.R;
-  p.C = sc.C;
-  p.rs1 = sc.rs1;
-  p.cs0 = sc.cs0;
-  p.cs1 = sc.cs1;
+  SParams p = f64 ? make_params<7>(A, Ai, B, Bi, err) : make_params<4>(A, Ai, B, Bi, err);
+  SParams q = make_params<1>(A, Ai, B, Bi, err);
+  for (SParams* x : {&p, &q}) {
+    x->out = out;
+    x->scatter = 1;
+    x->R = sc.R;
+    x->C = sc.C;
+    x->rs1 = sc.rs1;
+    x->cs0 = sc.cs0;
+    x->cs1 = sc.cs1;
+  }
   launch_mma(A, Ap, B, Bp, p, 1, s);
+  launch_guard(A, Ap, B, Bp, q, 1, s);
 }
 
-void slice_gemm(const SliceOperand& A, const void* Ap, const int* Ae, const SliceOperand& B, const void* Bp,
-                const int* Be, void* C, double beta, int* err, cudaStream_t s) {
+void slice_gemm(const SliceOperand& A, const void* Ap, const void* Ai, const SliceOperand& B, const void* Bp,
+                const void* Bi, void* C, double beta, int* err, cudaStream_t s) {
   check_pair(A, B);
   const bool f64 = A.t == DType::F64;
-  SParams p = f64 ? make_params<7>(A, Ae, B, Be, err) : make_params<4>(A, Ae, B, Be, err);
-  // splits in whole runs; a CTA's fixed cost (pipeline fill, output) is about half a run
-  const int runs = (p.total + RUN - 1) / RUN;
-  int splits = wave_splits(p.tiles, runs, 1);
-  const int per = (runs + splits - 1) / splits;
-  splits = (runs + per - 1) / per;
-  p.per = per * RUN;
+  SParams p = f64 ? make_params<7>(A, Ai, B, Bi, err) : make_params<4>(A, Ai, B, Bi, err);
+  const int splits = choose_splits(p);
   const long long MN = (long long)p.M * p.N;
-  const bool direct = splits == 1 && beta == 0.0;
-  DevBuf part;
-  if (!direct) part = DevBuf((size_t)splits * MN * dtype_size(A.t), s);
-  p.out = direct ? C : part.p;
+  const bool direct = splits == 1 && beta == 0.0;   // no partials: the guard forms outputs again in place
+  SParams q = make_params<1>(A, Ai, B, Bi, err, !direct);
+  if (direct) {
+    p.out = q.out = C;
+    launch_mma(A, Ap, B, Bp, p, 1, s);
+    launch_guard(A, Ap, B, Bp, q, 1, s);
+    return;
+  }
+  const int gs = choose_splits(q);
+  const size_t pb = ((size_t)splits * MN * dtype_size(A.t) + 255) & ~(size_t)255;
+  DevBuf part(pb + (size_t)gs * MN * 4, s);
+  p.out = part.p;
+  q.out = part.as<char>() + pb;
   launch_mma(A, Ap, B, Bp, p, splits, s);
-  if (direct) return;
-  const unsigned g = (unsigned)std::min<long long>((MN + 255) / 256, 152 * 16);
-  if (f64) k_slice_sum<double><<<g, 256, 0, s>>>(part.as<double>(), splits, MN, (double*)C, beta);
-  else k_slice_sum<float><<<g, 256, 0, s>>>(part.as<float>(), splits, MN, (float*)C, beta);
+  launch_guard(A, Ap, B, Bp, q, gs, s);
+  const float* N = static_cast<const float*>(q.out);
+  // 32 outputs per CTA where 256 leave most SMs without any
+  auto sum = [&](auto* pt, auto* out, auto kernel, int opb) {
+    const unsigned g = (unsigned)std::min<long long>((MN + opb - 1) / opb, 152 * 16);
+    kernel<<<g, 256, 0, s>>>(pt, splits, N, gs, (long long)p.M, p.N, out, beta, q.g);
+  };
+  const bool few = MN < 152 * 256;
+  if (f64) sum(part.as<double>(), (double*)C, few ? k_slice_sum<double, 32> : k_slice_sum<double, 256>, few ? 32 : 256);
+  else sum(part.as<float>(), (float*)C, few ? k_slice_sum<float, 32> : k_slice_sum<float, 256>, few ? 32 : 256);
   count_launch();
   TD_LAUNCH_CHECK();
 }
