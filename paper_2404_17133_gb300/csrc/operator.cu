@@ -15,8 +15,8 @@
 // workspace; the contractions of K1 and K2 (most of the flops) run on the tcgen05
 // tensor cores: as FP16 hi + lo operands when asked (MIXED with tensor_cores,
 // tc_gemm.cuh), else as exact slices of the FP64 or FP32 operands
-// (slice_gemm.cuh).  Only BF16 ris rows against FP32 vectors without
-// tensor_cores run on the FP32 units.
+// (slice_gemm.cuh).  Without tensor_cores, BF16 ris rows against FP32 vectors and
+// small products run on the FP32 or FP64 units.
 #include <algorithm>
 
 #include "ctx.cuh"
@@ -108,6 +108,12 @@ constexpr size_t kChunkBytesSliced = 1ull << 30;
 // launches and the cutting of L_ov cost what the FP64 units do (whole product, units
 // and slices: 2^25.2 1340 and 1310 us, 2^26.8 3456 and 3102, 2^28.8 21.0 and 19.8 ms).
 constexpr double kCoulombSliced = 1 << 25;
+// Multiply-adds of the exchange contractions from which these are sliced; below, the
+// FP64 (FP32) units need fewer launches.  Products of A, units and slices, us: FP64 6 x 30
+// with 180 rows, 4 vectors (2^22.1) 143 and 174, 20 vectors (2^24.5) 743 and 189; 5 x 20,
+// 20 vectors (2^22.6) 206 and 187; FP32 12 x 60 with 360 rows, 8 vectors (2^27.1) 209 and
+// 210, 20 vectors (2^28.5) 267 and 248; 16 x 90 with 500 rows, 4 vectors (2^28.2) 235 and 264.
+constexpr double kExchangeSliced64 = 1 << 22, kExchangeSliced32 = 1 << 28;
 // k-blocks one CTA accumulates in FP32 before its split-K partial is summed
 // (fixed order) with the others: the rounding of an FP32 run grows with its
 // length, and runs over a whole P-chunk of the exchange contraction (~1e4 MMA
@@ -521,10 +527,11 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
                       d.tc_err, s, nullptr, 0.0, 0.0, f16 ? kExchangeKb : 0, K2s);
         }
       }
-    } else if (f.dt != DType::BF16) {
+    } else if (f.dt != DType::BF16 && (double)m * f.nK * no * nv * (no + nv + (need_k2 ? 2.0 * no : 0.0)) >=
+                                          (f64 ? kExchangeSliced64 : kExchangeSliced32)) {
       exchange_sliced(d, f, Xw, m, need_k2, K1b.p, K2b.p, s);
     } else {
-      // ris rows (BF16) against FP32 trial vectors on the FP32 units
+      // ris rows (BF16) against FP32 trial vectors, and small products, on the FP32 or FP64 units
       DevBuf Zb((size_t)m * no * pc * nv * ew, s);
       DevBuf Qb;
       if (need_k2) Qb = DevBuf((size_t)m * no * pc * no * ew, s);
@@ -550,7 +557,13 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
         k.B = (const char*)f.Kvv + (size_t)p0 * nv * nv * es; k.tb = f.dt; k.sbk = nv; k.sbn = 1;
         k.C = K1b.p; k.tc = tw; k.scm = nv; k.scn = 1;
         k.beta = (p0 > 0) ? 1.0 : 0.0;
+        const bool timed = d.prof_simt && d.prof_simt->on && f.dt != DType::BF16;
+        if (timed) d.prof_simt->begin(s);
         gemm_splitk(k, auto_splits(k.M, k.N, k.K), s);
+        if (timed)
+          d.prof_simt->end(s, 2.0 * Mz * (double)nv * (double)Kz,
+                           (double)es * ((double)Mz * (double)Kz + (double)Kz * nv +
+                                         (double)Mz * nv * (p0 > 0 ? 2.0 : 1.0)));
         if (need_k2) {
           // Q[n][i][P][j] = sum_b Kov[P][i][b] X[n][j][b]
           GemmDesc q;
