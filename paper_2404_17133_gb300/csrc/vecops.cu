@@ -297,9 +297,10 @@ void unit_rows(double* out, int k, int n, const int* idx, cudaStream_t s) {
 template <typename T>
 void row_sumsq(const T* X, long long ldx, int k, int n, double* out, cudaStream_t s) {
   if (k <= 0) return;
-  // about 16 elements per thread: the FP64 butterflies of 32 warps are what short rows
-  // wait for (rows of 3456: 4.8 us with 1024 threads, 3.7 with 256)
-  int threads = 64;
+  // FP64: about 16 elements per thread, since short rows wait for the butterflies of 32
+  // warps (rows of 3456: 4.8 us with 1024 threads, 3.7 with 256).  FP32 rows keep 1024, so
+  // that as few squares as can be are added in FP32.
+  int threads = sizeof(T) == 8 ? 64 : 1024;
   while (threads < 1024 && threads * 16 < n) threads *= 2;
   k_row_sumsq<T><<<k, threads, 0, s>>>(X, ldx, n, out);
   count_launch(); TD_LAUNCH_CHECK();
