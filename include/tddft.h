@@ -295,9 +295,11 @@ typedef struct {
 /* Device-memory charge of one request: the factor copies tddft_create makes
  * for desc (factor_bytes, may be NULL) and a bound on the solve's work
  * buffers (work_bytes, may be NULL): the outer subspace and its work vectors,
- * the rid inner space, the operator's P-chunk intermediates (at most three
- * of 512 MiB) and 64 MiB for the small algebra.  n_dip / n_freq are used for
- * kind 2 only.  TDDFT_ERR_ARG on bad sizes or kind.                        */
+ * the rid inner space, the intermediates of one operator product (tensor
+ * cores: P-chunks of 4 GB and up to 256 MB of partial sums per term; sliced
+ * products: chunks of 1 GB; fewer for small problems), half of all that (at
+ * most 4 GB) for freed blocks kept for reuse, and 64 MiB for the small algebra.
+ * n_dip / n_freq are used for kind 2 only.  TDDFT_ERR_ARG on bad sizes or kind.                        */
 tddft_status tddft_estimate_bytes(const tddft_desc* desc, int kind, const tddft_opts* opts, int n_dip,
                                   int n_freq, unsigned long long* factor_bytes,
                                   unsigned long long* work_bytes);

@@ -127,6 +127,11 @@ void apply_operator(const OpDims& d, const FactorSet& f, const double* X, int m,
 void apply_operator(const OpDims& d, const FactorSet& f, const float* X, int m, OpMode mode,
                     float* out0, float* out1, int tc, cudaStream_t s);
 
+// Device bytes that apply_operator takes at most for m vectors beside its operands and
+// results (a second exchange set's sums included), for a factor set of type t with nJ
+// Coulomb and nK exchange rows.
+double product_work_bytes(int no, int nv, int nJ, int nK, int m, DType t, bool tensor_cores, bool paired);
+
 struct Request {
   int kind = 0;
   tddft_request* req = nullptr;

@@ -18,6 +18,7 @@
 // (slice_gemm.cuh).  Without tensor_cores, BF16 ris rows against FP32 vectors and
 // small products run on the FP32 or FP64 units.
 #include <algorithm>
+#include <cmath>
 
 #include "ctx.cuh"
 #include "skinny.cuh"
@@ -620,6 +621,46 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       combine(X, d.delta, nullptr, K1b.p, K2b.p, tw, 0.0, -kx, kx, m, ov, out1, s);
     }
   }
+}
+
+double product_work_bytes(int no, int nv, int nJ, int nK, int m, DType t, bool tensor_cores, bool paired) {
+  const double ov = (double)no * nv, mov = m * ov, es = (double)dtype_size(t);
+  const bool f64 = t == DType::F64;
+  const double nop = tc_pad(no), nvp = tc_pad(nv);
+  auto rows = [&](double per_row, size_t budget) {   // rows of a chunk, as chunk_rows has them
+    return std::max(1.0, std::min((double)nK, std::floor((double)budget / per_row)));
+  };
+  // K-split partials of a product of M x N outputs: whole waves of tiles, or runs of at
+  // most `run` terms
+  auto partials = [&](double M, double N, double K, double run, double tile_bytes) {
+    return std::max(4.0 * 152 * tile_bytes, M * N * 4.0 * (std::floor(K / run) + 2.0));
+  };
+  // terms' sums (two exchange sets), t, and what the Coulomb Gram products of FP32 rows leave per chunk
+  double b = 5.0 * mov * (f64 ? 8 : 4) + (f64 ? 0.0 : mov * 4.0) + 2.0 * nJ * m * 8.0;
+  const double gram = 8.0 * m * std::max(584.0 * 128.0, (double)nJ * (ov / 2048.0 + 1.0));
+  if (tensor_cores) {
+    const double nvz = tc_zpad(nv, 2), noz = tc_zpad(no, 2);
+    const double pc = rows(m * no * nvz * 4.0, kChunkBytesTC);
+    const double tile = 128.0 * 256 * 4;
+    const double k1 = partials(m * no, nv, pc * nvp, 64.0 * kExchangeKb, tile);
+    const double j = partials(m, ov, nJ, 64.0 * kCoulombKb, tile), keep = (double)kKeepBytes;
+    return b + gram + m * no * pc * (nvz + (paired ? noz : 0.0)) * 4.0 + 4.0 * m * (nv * nop + no * nvp) +
+           std::min(j, keep) + (paired ? std::min(k1, keep) : 0.0) + std::max(j, k1);
+  }
+  if (t == DType::BF16) {
+    const double pc = rows(mov * 4.0, kChunkBytes);
+    return b + gram + pc * m * no * (nv + (paired ? no : 0.0)) * 4.0 + partials(m * no, nv, pc * nv, 1e30, 2.0 * 64 * 64 * 4);
+  }
+  const double sb = slice_element_bytes(t);
+  const double row = m * no * (nv * es + nvp * sb) + (no * nop + nv * nvp) * sb +
+                     (paired ? m * no * (no * es + nop * sb) + (no * nvp + nv * nop) * sb : 0.0);
+  const double pc = rows(row, kChunkBytesSliced);
+  const double sums = 4.0 * 152 * (128 * 128 * 4 + 128 * 256 * 4) + 12.0 * std::max(mov, (double)nJ * m);
+  const double exchange = pc * row + 16.0 * (pc * 2 * no + 4.0 * m * (no + nv)) + m * (nv * nop + no * nvp) * sb;
+  const double coulomb = f64 ? std::max((double)kChunkBytesSliced, std::max(ov, (double)nJ) * sb) + m * (ov + 8) * sb +
+                                   m * (nJ + 8.0) * sb + 16.0 * (ov + nJ)
+                             : gram;
+  return b + sums + std::max(exchange, coulomb);
 }
 
 void apply_operator(const OpDims& d, const FactorSet& f, const double* X, int m, OpMode mode,

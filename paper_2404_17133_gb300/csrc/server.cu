@@ -154,12 +154,25 @@ tddft_status tddft_estimate_bytes(const tddft_desc* desc, int kind, const tddft_
     const double inner_es = opts->precision == TDDFT_MIXED ? 4.0 : 8.0;
     // Outer subspace (paired: V, U, W of cap rows in FP64) and its ~24 k-row
     // work vectors; the rid inner space (cap + 2k rows and ~24 k-row vectors in
-    // the inner precision); operator intermediates (at most three P-chunks of
-    // 512 MiB, fewer for small problems); 64 MiB for the small algebra.
+    // the inner precision); one product's intermediates (product_work_bytes), for the
+    // largest block of vectors that the solve multiplies with the exact operator (a
+    // restart's, or the guess's) and with the ris operator; for freed blocks that the
+    // stream keeps (devpool.cu), half of all that, up to the cache's cap (solves of 24 x 144
+    // and 60 x 400 orbitals in every arithmetic needed up to 0.12); 64 MiB for the small
+    // algebra.
     const double outer = 8.0 * ov * (3.0 * cap + 24.0 * k);
     const double inner = opts->precond == TDDFT_PRECOND_RID ? inner_es * ov * (4.0 * cap + 26.0 * k) : 0.0;
-    const double inter = 3.0 * std::min(512.0 * 1048576.0, (double)d.n_aux * cap * ov * 8.0);
-    *work_bytes = (unsigned long long)(outer + inner + inter + 64.0 * 1048576.0);
+    const bool mixed = opts->precision == TDDFT_MIXED, tc = mixed && opts->tensor_cores;
+    const int m = (int)std::min(ov, std::min((double)cap, kind == 0 ? k + 8.0 : std::max(4.0 * k, k + 8.0)));
+    using tddft::DType;
+    const double inter = std::max(
+        tddft::product_work_bytes(d.n_occ, d.n_vir, d.n_aux, d.n_aux, m, mixed ? DType::F32 : DType::F64, tc, kind != 0),
+        opts->precond == TDDFT_PRECOND_RID
+            ? tddft::product_work_bytes(d.n_occ, d.n_vir, d.n_aux_ris_J, std::max(d.n_aux_ris_K, 1), m,
+                                        mixed ? DType::BF16 : DType::F64, tc, kind != 0)
+            : 0.0);
+    const double live = outer + inner + inter;
+    *work_bytes = (unsigned long long)(live + std::min(0.5 * live, (double)tddft::kCachedPerStream) + 64.0 * 1048576.0);
   }
   return TDDFT_OK;
 }
