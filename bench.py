@@ -18,8 +18,7 @@ e2e:   the same through the C ABI with host (pinned) inputs: tddft_create
        solves with host outputs + tddft_destroy, every step.
 medium: the medium workload (n_occ=60, n_vir=400, n_aux=2000) as context:
        Casida (10 states) + alpha(omega) per step, MIXED, and the same step in
-       the plain FP64 form (the plain form of the large step would take most
-       of an hour on GB300's FP64 units).
+       the plain FP64 form.
 Inputs (the resident factor copies, ~100 GB) are far larger than L2, so no L2
 flush is added between steps.
 
@@ -446,7 +445,7 @@ def our_arm(args):
                 "p99_ms": sorted(per_step)[min(len(per_step) - 1, int(0.99 * len(per_step)))],
                 "converged": all(r["status"] == api.OK for pair in results for r in pair), "load_s": t_load,
                 "tda": solved(a), "rpa": solved(b),
-                "roofline": roofline(prof, *records, peaks, src, tc, clk, total_ms),
+                "roofline": roofline(prof, *records, peaks, src, tc, total_ms),
                 "gpu_launches": launches, "clocks": clk,
                 "e2e": {"value": None, "unit": UNIT, "ms_per_step": None}}
 
@@ -519,25 +518,22 @@ def our_arm(args):
 K1_TRAFFIC_PER_ALGORITHMIC_BYTE = 11.46e9 / 5.07e9
 
 
-def roofline(prof, rec_ms, rec_fl, rec_by, peaks, src, tc, clk, total_ms):
+def roofline(prof, rec_ms, rec_fl, rec_by, peaks, src, tc, total_ms):
     """Roofline object of the dominant kernel (the K1 exchange contraction)."""
     kernel_ms = prof["ms"] / max(prof["launches"], 1)
     flops_launch = prof["flops"] / max(prof["launches"], 1)
     achieved = flops_launch / (kernel_ms * 1e-3) / 1e12 if prof["launches"] else 0.0
-    if tc:
-        # FP16 and BF16 run at the same dense tensor rate (nominal ratio 1)
-        peak = peaks["bf16_tflops_sustained"]
-        roof = {"bound": "tensor", "unit": "TFLOP/s",
-                "peak_kind": "fp16 dense = bf16 sustained (nominal ratio 1), " + src,
-                "note": "algorithmic flops 2*M*N*K; the hi+lo split issues 3 FP16 products per flop, "
-                        "so frac <= 1/3 (mma_pipe_frac = 3 x frac)"}
-    else:
-        sm = (clk or {}).get("sm_max_mhz") or peaks.get("sm_max_mhz", 2070.0)
-        peak = 152 * 128 * 2 * sm * 1e6 / 1e12
-        roof = {"bound": "alu", "unit": "TFLOP/s",
-                "peak_kind": "FP32 FFMA: 152 SMs x 128 lanes x 2 flop x %.0f MHz" % sm}
+    # FP16 and BF16 run at the same dense tensor rate (nominal ratio 1).  FP16 products per
+    # flop: hi*hi + hi*lo + lo*hi; without the tensor-core option ten of base-256 digits of
+    # FP32 operands and one of the magnitudes that bound their error.
+    per_flop = 3.0 if tc else 11.0
+    peak = peaks["bf16_tflops_sustained"]
+    roof = {"bound": "tensor", "unit": "TFLOP/s",
+            "peak_kind": "fp16 dense = bf16 sustained (nominal ratio 1), " + src,
+            "note": "algorithmic flops 2*M*N*K; %s, so frac <= 1/%g (mma_pipe_frac = %g x frac)"
+                    % ("the hi+lo split issues 3 FP16 products per flop" if tc else
+                       "the sliced FP32 product issues 11 FP16 products per flop", per_flop, per_flop)}
     if rec_ms.size:
-        per_flop = 3.0 if tc else 1.0
         t_ten = rec_fl * per_flop / (peak * 1e12) * 1e3
         t_hbm = rec_by / (peaks["hbm_gbs"] * 1e9) * 1e3
         t_att = np.maximum(t_ten, t_hbm)
@@ -556,7 +552,7 @@ def roofline(prof, rec_ms, rec_fl, rec_by, peaks, src, tc, clk, total_ms):
                                 "capture (%.2f) times this run's mean algorithmic bytes per launch"
                                 % K1_TRAFFIC_PER_ALGORITHMIC_BYTE)
     roof.update({"achieved": achieved, "peak": peak, "frac": achieved / peak if peak else None,
-                 "mma_pipe_frac": 3.0 * achieved / peak if (peak and tc) else None,
+                 "mma_pipe_frac": per_flop * achieved / peak if peak else None,
                  "traffic": traffic, "kernel": "exchange K1 contraction sum_(P,a) Z L_vv",
                  "launches": prof["launches"], "ms_per_launch": kernel_ms,
                  "share_of_step": prof["ms"] / total_ms if total_ms else None})
