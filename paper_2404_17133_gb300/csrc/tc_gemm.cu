@@ -728,7 +728,7 @@ k_stage1_pair(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__
     // ---- TMA producer (both CTAs)
     const uint32_t lead_full = mapa(smem_u32(full), 0u), lead_bfull = mapa(smem_u32(bfull), 0u);
     const uint32_t bytes_a = 2u * (LSPLIT ? 2u : 1u) * C::AB, bytes_b = 4u * (uint32_t)p.b_rows * S1_RB;
-    int i = 0, w = 0;
+    int i = 0, w = 0, xw = 0;   // xw: units whose X rows have been asked for
     bool ok = true;
     for (int u = cl; u < p.units && ok; u += ncl, ++w) {
       int n0, r0, width;
@@ -742,6 +742,7 @@ k_stage1_pair(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__
           tma_load_3d_pair(bres + kb * 2 * C::HB, &mB_hi, lead_bfull, kb * BKE, rb, nb);
           tma_load_3d_pair(bres + kb * 2 * C::HB + C::HB, &mB_lo, lead_bfull, kb * BKE, rb, nb);
         }
+        ++xw;
       }
       for (int mt = mt0; mt < mt1 && ok; ++mt) {
         const int m0 = mt * 2 * BM + h * BM;
@@ -767,9 +768,9 @@ k_stage1_pair(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__
         if (!mbar_wait(&full[j % STAGES], (uint32_t)(j / STAGES) & 1u)) { atomicOr(p.err, 32); break; }
     for (int j = i; j < i + STAGES; ++j)
       if (!mbar_wait(&empty[j % STAGES], ((uint32_t)(j / STAGES) & 1u) ^ 1u)) { atomicOr(p.err, 32); break; }
-    if (RES && ok) {
-      if (h == 0 && w > 0 && !mbar_wait(bfull, (uint32_t)(w - 1) & 1u)) atomicOr(p.err, 32);
-      if (!mbar_wait(bempty, ((uint32_t)w & 1u) ^ 1u)) atomicOr(p.err, 32);
+    if (RES) {
+      if (h == 0 && xw > 0 && !mbar_wait(bfull, (uint32_t)(xw - 1) & 1u)) atomicOr(p.err, 32);
+      if (ok && !mbar_wait(bempty, ((uint32_t)w & 1u) ^ 1u)) atomicOr(p.err, 32);
     }
   } else if (warp == 1 && lane == 0 && h == 0) {
     // ---- MMA issuer (the leader)
