@@ -71,12 +71,12 @@ typedef enum { TDDFT_PRECOND_DIAG = 0, TDDFT_PRECOND_RID = 1 } tddft_precond;
  * PLAIN: every step in FP64 (factors, products, subspace algebra); large
  *        exchange and Coulomb contractions run on the tensor cores as exact
  *        integer slices of the FP64 operands (fixed point against the largest
- *        element of a row: each element to 2^-55 of it), and every output
- *        whose terms are too small beside those for the slices to be as
- *        accurate as FP64 arithmetic is formed again on the FP64 units.
+ *        element of a row: each element to 2^-55 of it); an output whose terms
+ *        are too small beside those for an error of 2^-52 of the sum of their
+ *        absolute values is formed again on the FP64 units.
  * MIXED: exact products with FP32 factors (large exchange contractions: exact
- *        integer slices in the same way, 2^-31 of a row's largest element,
- *        checked output by output; others and Coulomb: FP32 accumulation), or, when
+ *        integer slices in the same way, 2^-31 of a row's largest element and
+ *        2^-23 of an output's absolute sum; others and Coulomb: FP32 accumulation), or, when
  *        `tensor_cores` is set, on the tcgen05 tensor cores with every operand
  *        (factors, trial vectors, the first contraction's results) scaled by
  *        a power of two and split into FP16 hi + lo parts (22 significand

@@ -107,7 +107,9 @@ constexpr size_t kChunkBytesTC = 4ull << 30;
 constexpr size_t kChunkBytesSliced = 1ull << 30;
 // Multiply-adds per FP64 Coulomb contraction from which it is sliced, too; below, the
 // launches and the cutting of L_ov cost what the FP64 units do (whole product, units
-// and slices: 2^25.2 1340 and 1310 us, 2^26.8 3456 and 3102, 2^28.8 21.0 and 19.8 ms).
+// and slices: 60 x 400 with 360 rows, 2 vectors, 2^24.0 1.61 and 1.61 ms; 24 x 144 with 840
+// rows, 13 vectors, 2^25.2 1.58 and 1.59, 40 vectors, 2^26.8 3.87 and 3.54; 60 x 400 with 2000
+// rows, 1 vector, 2^25.5 6.89 and 6.43, 6 vectors, 2^28.1 15.8 and 15.0).
 constexpr double kCoulombSliced = 1 << 25;
 // Multiply-adds of the exchange contractions from which these are sliced; below, the
 // FP64 (FP32) units need fewer launches.  Products of A, units and slices, us: FP64 6 x 30

@@ -739,6 +739,8 @@ void tall_gram_launch(const TA* A, int M, const float* B, int N, int K, int chun
 
 template <typename TA, int PA, int PX>
 void tall_gram_typed(const TA* A, int M, const float* B, int N, int K, float* part, int chunk, int S, cudaStream_t s) {
+  // one pass over A up to 32 vectors; above that passes of 32, but two of 20 for 33 to 40
+  // (two CTAs share an SM up to RN 5, and two passes of 32 would leave 24 or more columns idle)
   const int rn = N > 32 && N <= 40 ? 5 : (std::min(N, 32) + 3) / 4;
   if (rn <= 2) tall_gram_launch<TA, 2, PA, PX>(A, M, B, N, K, chunk, S, part, s);
   else if (rn <= 4) tall_gram_launch<TA, 4, PA, PX>(A, M, B, N, K, chunk, S, part, s);

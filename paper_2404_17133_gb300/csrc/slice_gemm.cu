@@ -18,8 +18,8 @@
 // |a| max|B row|) per term, and FP32 leaves out three products of up to 2^-28.4 max max
 // together.  Where an output's terms are as large as its rows' elements that is below
 // what FP64 (FP32) accumulation leaves; where they are not, the output is formed
-// again on the FP64 (FP32) units (the guard, below), so that none has fewer bits than
-// FP64 (FP32) arithmetic gives it.
+// again on the FP64 (FP32) units (the guard, below), so that every output is within
+// two roundings, 2^-52 (2^-23), of the sum of its terms' absolute values.
 //
 // Why: FP64 runs at 1.2 TFLOP/s on this GPU's vector units and FP32 at 75; 34
 // or 10 FP16 products per term leave up to 57 and 190 TFLOP/s.
@@ -78,7 +78,7 @@ template <int S, int W> struct SCfg {
   static constexpr int LV = S == 7 ? 8 : S;
   static constexpr int A_SLICE = SBM * SBK * 2, B_SLICE = W * SBK * 2;
   static constexpr int STAGE_BYTES = S * (A_SLICE + B_SLICE);
-  static constexpr int STAGES = S == 7 ? 2 : (S == 4 ? 3 : (W == 256 ? 6 : 10));
+  static constexpr int STAGES = S == 7 ? 2 : (S == 4 ? 3 : (W == 256 ? 6 : (W == 32 ? 12 : 10)));
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
   static constexpr int NBUF = S == 1 ? 2 : 1;   // sets of levels in tensor memory
   static constexpr int TMEM_COLS = S == 1 ? 2 * W : 512;
@@ -100,7 +100,6 @@ struct Guard {
   RowInfo ra, rb;
   View a, b;
   int np, K;
-  float wn, wc;   // weights of the row norms and of the element counts (guard_weights)
 };
 
 struct SParams {
@@ -260,11 +259,13 @@ template <> struct Acc<4> {
   // times the scales r of the row and c of the column
   __device__ __forceinline__ float value(float r, float c) const { return (hi + lo) * r * c; }
   // Takes in the factor 2^e, where a product with one of the scales alone could leave FP32's
-  // range (of a special row or column: any number, the guard puts the result).
+  // range (of a non-finite row or column: NaN, as what it gives with a zero row; the guard
+  // puts the others).
   __device__ __forceinline__ void scale_any(int e) {
     const int e1 = min(max(e, -126), 127), e2 = min(max(e - e1, -126), 127);
     hi = (hi + lo) * __int_as_float((e1 + 127) << 23) * __int_as_float((e2 + 127) << 23);
     lo = 0.f;
+    if (e >= kNotFinite / 2) hi = __int_as_float(0x7fc00000);
   }
 };
 
@@ -282,28 +283,35 @@ template <> __device__ __forceinline__ int row_scale<4>(int w) { return w >= 255
 // (2^e the power of two above its largest element), the error of a sliced output is
 // (root mean square over the roundings)
 //   FP64: 2^-42.8 (|a'| + |b'|),   FP32: 2^-18.8 (|a'| + |b'|) + 2^-4.8 sqrt(n)
-// (|.| 2-norms over the terms, n the nonzero elements of A's row: the three products of
-// FP32's dropped level 4), and that of a run of FP64 (FP32) additions is
-// 2^-54.3 N (2^-25.3 N) with N = sum_k a'_k b'_k.  N comes from one more FP16 product
-// of the magnitudes, and an output where it is too small for the slices to be as good
-// is formed again from the operands themselves on the FP64 (FP32) units: so is every
-// output of a row with a non-finite element, which then reaches what it meets and
-// no more.
+// where |.| are 2-norms over the n terms with both factors nonzero (a zero is exact; the
+// last term is FP32's dropped level 4, three products).  Asked for are two roundings of
+// the sum of the terms' absolute values, 2^-52 N (2^-23 N) with N = sum_k a'_k b'_k, which FP64
+// (FP32) arithmetic gives for sums of two terms and only bounds by n / 2 times that for
+// more.  N comes from one more FP16 product of the magnitudes; |a'| is bounded by the
+// norm of the whole row and by 2^14 times the square root of the other row's nonzeros.  An
+// output where N is too small is formed again from the operands themselves on the FP64
+// (FP32) units: so is every output of a row with a non-finite element (whose magnitudes
+// are zero), which then reaches what it meets and no more.
 constexpr int kThreadTerms = 256;   // terms up to which a thread forms an output alone (else its warp)
-template <typename T> struct GuardWeights;   // of |.| and of sqrt(n)
-template <> struct GuardWeights<double> { static constexpr float NORM = 2896.f, COUNT = 0.f; };        // 2^(54.3 - 42.8)
-template <> struct GuardWeights<float> { static constexpr float NORM = 91.f, COUNT = 1482910.f; };     // 2^6.5, 2^20.5
+template <typename T> struct GuardWeights;
+template <> struct GuardWeights<double> { static constexpr float NORM = 588.f, COUNT = 0.f; };                // 2^(52 - 42.8)
+template <> struct GuardWeights<float> { static constexpr float NORM = 18.4f, COUNT = 301124.f / (18.4f * 16384.f); };   // 2^(23 - 18.8), 2^(23 - 4.8)
 template <typename T> constexpr int kExpSpecial = sizeof(T) == 8 ? 2047 : 255;
 
-// A row's part of the bound on N; an output is formed again unless N - (the column's)
-// > (the row's).  A zero row is exact, a special one never (in both places: not exact).
+// A row's part of the bound on N: from its norm and from its nonzeros (both zero: a zero row).
 template <typename T>
-__device__ __forceinline__ float row_bound(const RowInfo& r, long long i, float wn, float wc) {
+__device__ __forceinline__ float2 row_bound(const RowInfo& r, long long i) {
+  const float inf = __int_as_float(0x7f800000);
   const int e = r.e[i];
-  const unsigned n = r.nnz[i];
-  const float ss = (float)r.ss[i];
-  if (e >= kExpSpecial<T>) return __int_as_float(0x7f800000);
-  return n == 0 ? __int_as_float(0xff800000) : fmaf(wn * 0.0625f, sqrtf(ss), wc * sqrtf((float)n));
+  const float n = (float)r.nnz[i], ss = (float)r.ss[i];
+  if (e >= kExpSpecial<T>) return make_float2(inf, inf);
+  return make_float2(GuardWeights<T>::NORM * 0.0625f * sqrtf(ss), GuardWeights<T>::NORM * 16384.f * sqrtf(n));
+}
+// N less the bound; the output is formed again unless it is >= 0.
+template <typename T>
+__device__ __forceinline__ float margin(float N, float2 a, float2 b) {
+  N -= fminf(a.x, b.y) + fminf(b.x, a.y);
+  return sizeof(T) == 8 ? N : N - GuardWeights<T>::COUNT * fminf(a.y, b.y);
 }
 
 template <typename T>
@@ -475,14 +483,14 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
         static_assert(W == GUARD_SUMS || HC <= 64, "one bit per column");
         constexpr bool SUMS = W == GUARD_SUMS;   // k_slice_sum judges
         // the bounds of this warp's rows and columns, while the tile is being formed
-        __shared__ __align__(16) float colb[EPI_WARPS][HC];
-        const float ninf = __int_as_float(0xff800000);
+        __shared__ __align__(16) float2 colb[EPI_WARPS][SUMS ? 1 : HC];
+        const float2 none = make_float2(0.f, 0.f);
         const bool inside = row < p.M;
-        float ba = ninf;
-        float* cb = colb[warp - 2];
+        float2 ba = none;
+        float2* cb = colb[warp - 2];
         if (!SUMS) {
-          if (inside) ba = row_bound<T>(p.g.ra, row, p.g.wn, p.g.wc);
-          for (int c = lane; c < HC; c += 32) cb[c] = c < ncol ? row_bound<T>(p.g.rb, n0 + c, p.g.wn, 0.f) : ninf;
+          if (inside) ba = row_bound<T>(p.g.ra, row);
+          for (int c = lane; c < HC; c += 32) cb[c] = c < ncol ? row_bound<T>(p.g.rb, n0 + c) : none;
           __syncwarp();
         }
         const uint32_t buf = run % C::NBUF;
@@ -504,17 +512,18 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
               for (int j = 0; j < 16; ++j)
                 if (inside && c + j < ncol) o[j] = v[j];
             } else {
-              float least = __int_as_float(0x7f800000);
+              float least = 0.f;
 #pragma unroll
-              for (int j = 0; j < 16; j += 4) {
-                const float4 b4 = *reinterpret_cast<const float4*>(cb + c + j);
-                v[j] -= b4.x; v[j + 1] -= b4.y; v[j + 2] -= b4.z; v[j + 3] -= b4.w;
-                least = fminf(least, fminf(fminf(v[j], v[j + 1]), fminf(v[j + 2], v[j + 3])));
+              for (int j = 0; j < 16; j += 2) {
+                const float4 q = *reinterpret_cast<const float4*>(cb + c + j);
+                v[j] = margin<T>(v[j], ba, make_float2(q.x, q.y));
+                v[j + 1] = margin<T>(v[j + 1], ba, make_float2(q.z, q.w));
+                least = fminf(least, fminf(v[j], v[j + 1]));
               }
-              if (!(least > ba)) {
+              if (!(least >= 0.f)) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
-                  if (!(v[j] > ba)) again |= 1ull << (c + j);
+                  if (!(v[j] >= 0.f)) again |= 1ull << (c + j);
               }
             }
           }
@@ -982,7 +991,7 @@ __global__ void __launch_bounds__(256) k_slice_sum(const T* __restrict__ part, i
       float n = 0.f;
       for (int s = 0; s < SN; ++s) n += N[s * MN + t];
       const long long r = t / ncol;
-      bad = !(n - row_bound<T>(g.rb, t - r * ncol, g.wn, 0.f) > row_bound<T>(g.ra, r, g.wn, g.wc));
+      bad = !(margin<T>(n, row_bound<T>(g.ra, r), row_bound<T>(g.rb, t - r * ncol)) >= 0.f);
       if (bad) list[atomicAdd(&count, 1)] = tid;
     }
     if (__syncthreads_or(bad)) {
@@ -1083,9 +1092,8 @@ SParams make_params(const SliceOperand& A, const void* Ai, const SliceOperand& B
     p.w = sums ? GUARD_SUMS : (p.N <= 32 ? 32 : 128);
     p.tiles_n = (p.N + p.w - 1) / p.w;
   } else {
-    // the fewest tiles, of equal width, rounded up to an instance (at most 16 columns of a
-    // narrower tile are idle in FP64; in FP32 the widths between 64 and 128 are those at
-    // which 256 columns per MMA are best filled: 2 x 96, 2 x 112, 2 x 128)
+    // the fewest tiles, of equal width, rounded up to an instance: FP64 every 16 columns; FP32
+    // every 32 and one between the two widest, where most columns are idle otherwise
     p.tiles_n = (p.N + max_cols<S>() - 1) / max_cols<S>();
     p.w = (p.N + p.tiles_n - 1) / p.tiles_n;
     constexpr int widths[2][5] = {{16, 32, 48, 64, 64}, {32, 64, 96, 112, 128}};
@@ -1100,10 +1108,7 @@ SParams make_params(const SliceOperand& A, const void* Ai, const SliceOperand& B
   p.eb = rb.e;
   p.err = err;
   p.R = p.C = 1;
-  const bool f64 = A.t == DType::F64;
-  using GD = GuardWeights<double>;
-  using GF = GuardWeights<float>;
-  p.g = Guard{ra, rb, view_of(A), view_of(B), A.np, A.K, f64 ? GD::NORM : GF::NORM, f64 ? GD::COUNT : GF::COUNT};
+  p.g = Guard{ra, rb, view_of(A), view_of(B), A.np, A.K};
   return p;
 }
 

@@ -32,9 +32,10 @@ inline size_t slice_info_bytes(const SliceOperand& o) { return (size_t)o.rows * 
 // Cut an operand into slices: parts (slice_bytes), info (slice_info_bytes).
 void slice_cut(const SliceOperand& o, void* parts, void* info, cudaStream_t s);
 
-// The products below are as accurate as FP64 (FP32) arithmetic output by output:
-// one that the slices cannot give as well (its terms are small beside the largest
-// elements of its rows) is formed again from the operands on the FP64 (FP32) units.
+// Every output of the products below is within two roundings of the sum of its terms'
+// absolute values (root mean square): one that the slices cannot give so (its terms
+// are small beside the largest elements of its rows) is formed again from the operands
+// on the FP64 (FP32) units.
 
 // Batched products (np == 1 on both sides, no split):
 //   out[(r / R) * rs1 + (r % R) + (c % C) * cs0 + (c / C) * cs1] = sum_k A(r, k) B(c, k)
