@@ -498,17 +498,18 @@ __device__ __forceinline__ void cp_piece(void* dst, const void* src, int bytes) 
     asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(d), "l"(src), "r"(bytes), "n"(PB) : "memory");
 }
 
-// part[2 chunk][m][n] + part[2 chunk + 1][m][n] = sum over the chunk of A[m][k] B[n][k].  Bound by the FP32
+// part[chunk][m][n] (chunks longer than kTallRun: part[2 chunk] + part[2 chunk + 1]) = sum
+// over the chunk of A[m][k] B[n][k].  Bound by the FP32
 // units for about 16 vectors and more, by reading A below that.  CTA = 128 rows
 // x 4 RN vectors; 16 row groups x 4 vector groups x 4 groups of k, a thread 8
 // rows x RN vectors: 13 16-byte shared-memory loads feed 160 FMAs (RN = 5),
 // accumulated for even and odd k apart (packed FMAs), so a sum runs over at most
-// 1/8 of the chunk (<= 256 terms).  The chunk's eight are added with the roundings
-// kept, so that beyond those runs everything is added in FP64, as by the skinny product.
+// 1/8 of the chunk (<= 256 terms).  Beyond 256 terms everything is added in FP64, as by
+// the skinny product.
 // cp.async keeps two (FP32) or three stages of 64 k in flight, and two CTAs share an
 // SM up to 20 vectors.  n_ov 202,500, 1350 BF16 rows, 20 vectors: 365 us (992 by the
 // skinny product, 433 with one CTA per SM); n_ov 24,000, 2000 FP32 rows: 71 (149, 83).
-constexpr int kTallRows = 128, kTallK = 64, kTallChunk = 2048;
+constexpr int kTallRows = 128, kTallK = 64, kTallChunk = 2048, kTallRun = 256;
 template <typename TA> struct TallCfg {
   static constexpr int LDA = kTallK + (sizeof(TA) == 4 ? 4 : 8);   // elements: rows skewed over the banks
   static constexpr int LDB = kTallK + 8;
@@ -598,29 +599,31 @@ k_tall_gram(const TA* __restrict__ A, int M, const float* __restrict__ B, int N,
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  // the eight sums (even and odd k of four groups), added in order without loss: the
-  // rounding of every addition is kept, and the chunk leaves a sum and its remainder
+  // the eight sums (even and odd k of four groups), added in order: of a chunk of 256
+  // terms as one run of FP32; of a longer one without loss, the rounding of every
+  // addition kept, so that it leaves a sum and its remainder
   float2* red = reinterpret_cast<float2*>(tall_raw);   // [4][128][NT]
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < RN; ++j)
-      red[(kg * kTallRows + rg + 16 * i) * NT + cg + 4 * j] = two_sum(acc[i][j].x, acc[i][j].y);
+    for (int j = 0; j < RN; ++j) red[(kg * kTallRows + rg + 16 * i) * NT + cg + 4 * j] = acc[i][j];
   __syncthreads();
   const long long MN = (long long)M * N;
-  float* P = part + 2 * blockIdx.y * MN;
+  const bool lng = chunk > kTallRun;
+  float* P = part + (lng ? 2 : 1) * blockIdx.y * MN;
   for (int e = tid; e < kTallRows * NT; e += 256) {
     const int r = e / NT, c = e - r * NT;
     if (m0 + r >= M || n0 + c >= N) continue;
-    float2 v = red[e];
+    float v = 0.f, rest = 0.f;
 #pragma unroll
-    for (int g = 1; g < 4; ++g) {
-      const float2 w = red[g * kTallRows * NT + e], t = two_sum(v.x, w.x);
-      v = make_float2(t.x, t.y + v.y + w.y);
+    for (int g = 0; g < 4; ++g) {
+      const float2 q = red[g * kTallRows * NT + e], w = two_sum(q.x, q.y), t = two_sum(v, w.x);
+      v = t.x;
+      rest += t.y + w.y;
     }
     const long long at = (long long)(m0 + r) * N + n0 + c;
-    P[at] = v.x;
-    P[MN + at] = v.y;
+    P[at] = v;
+    if (lng) P[MN + at] = rest;
   }
 }
 
@@ -829,7 +832,8 @@ void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, flo
   int chunk = ((K + S - 1) / S + kTallK - 1) / kTallK * kTallK;
   chunk = std::max(chunk, 4 * kTallK);
   S = (K + chunk - 1) / chunk;
-  DevBuf part((size_t)2 * S * M * N * 4, s);
+  const int parts = chunk > kTallRun ? 2 * S : S;
+  DevBuf part((size_t)parts * M * N * 4, s);
   float* pt = part.as<float>();
   if (ta == DType::F32) {
     const float* a = static_cast<const float*>(A);
@@ -845,7 +849,7 @@ void tall_gram(const void* A, DType ta, int M, const float* X, int N, int K, flo
   TD_LAUNCH_CHECK();
   const long long MN = (long long)M * N;
   const unsigned rb = (unsigned)std::min<long long>((MN + 7) / 8, 16 * 152);
-  k_sk_gram_reduce<float, float><<<rb, 256, 0, s>>>(part.as<float>(), 2 * S, M, N, t, N, 1.0, 0.0, tmax);
+  k_sk_gram_reduce<float, float><<<rb, 256, 0, s>>>(part.as<float>(), parts, M, N, t, N, 1.0, 0.0, tmax);
   count_launch();
   TD_LAUNCH_CHECK();
 }
