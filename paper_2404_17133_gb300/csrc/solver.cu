@@ -245,11 +245,11 @@ int orth_append(T* V, int N, T* cand, int nc, int ov, cudaStream_t s) {
 // into V[N...] (V must have room for nc rows there) and their number is left in
 // count[0] on the device; the caller caps it at ov - N when it reads it.
 template <typename T>
-void orth_append_async(T* V, int N, T* cand, int nc, int ov, int* keep, int* count, cudaStream_t s) {
-  if (nc <= 0) { TD_CUDA(cudaMemsetAsync(count, 0, sizeof(int), s)); return; }
+void orth_append_async(T* V, int N, T* cand, int nc, int ov, int* keep, int* count, const int* info, const int* err,
+                       cudaStream_t s) {
   ScopedPhase ph(PH_ORTH, s);
   orth_block<T>(V, N, cand, nc, ov, keep, s);
-  compact_rows<T>(cand, keep, nc, ov, V + (size_t)N * ov, count, s);
+  compact_rows<T>(cand, keep, nc, ov, V + (size_t)N * ov, count, info, err, s);
 }
 
 // Orthonormalise `cand` against V (N rows) and each other and compact the
@@ -565,9 +565,9 @@ PairedLinOut paired_linear(int ov, const PairOpT<T>& op, const PairPreT<T>& pre,
     for (int r = 0; r < nr; ++r) gnh[r] += t[r];
   }
   for (auto& v : gnh) v = std::sqrt(v);
-  // status block read once per iteration: rn1[nr], rn2[nr] (doubles), then the
-  // Cholesky info and the number of accepted directions (ints)
-  DevBuf stat((size_t)2 * nr * 8 + 8, s), gdev(nr * 8, s), keep(2 * nr * 4, s);
+  // status block read once per iteration: rn1[nr], rn2[nr] (doubles), then the Cholesky
+  // info, the number of accepted directions and the tensor-core kernels' error word (ints)
+  DevBuf stat((size_t)2 * nr * 8 + 16, s), gdev(nr * 8, s), keep(2 * nr * 4, s);
   double* rn1p = dev_select ? stat.as<double>() : rn1.as<double>();
   double* rn2p = dev_select ? stat.as<double>() + nr : rn2.as<double>();
   int* st_info = reinterpret_cast<int*>(stat.as<double>() + 2 * nr);
@@ -641,11 +641,12 @@ PairedLinOut paired_linear(int ov, const PairOpT<T>& op, const PairPreT<T>& pre,
       ph_vec.stop();
       pre(Rp.as<T>(), Rm.as<T>(), sh.as<double>(), shifts, nr, cand.as<T>(), cand.as<T>() + (size_t)nr * ov);
       zero_converged<T>(cand.as<T>(), 2 * nr, nr, ov, rn1p, rn2p, gdev.as<double>(), tol, s);
-      orth_append_async<T>(sp.v(), N, cand.as<T>(), 2 * nr, ov, keep.as<int>(), st_count, s);
-      TD_CUDA(cudaMemcpyAsync(st_info, sp.info.p, sizeof(int), cudaMemcpyDeviceToDevice, s));
-      std::vector<double> blk = d2h_checked(stat.as<double>(), (size_t)2 * nr + 1, cnt.tc_err, s);
-      int ints[2];
+      orth_append_async<T>(sp.v(), N, cand.as<T>(), 2 * nr, ov, keep.as<int>(), st_count, sp.info.template as<int>(),
+                           cnt.tc_err, s);
+      std::vector<double> blk = d2h(stat.as<double>(), (size_t)2 * nr + 2, s);
+      int ints[3];
       std::memcpy(ints, &blk[2 * nr], sizeof(ints));
+      raise_tc_error(ints[2], cnt.tc_err, s);
       if (ints[0] != 0)
         throw Error(TDDFT_ERR_INDEFINITE, "projected A-B is not positive definite (pivot " +
                                               std::to_string(ints[0] - 1) + ")");
@@ -911,6 +912,7 @@ void inner_tda(int ov, const TdaOpT<T>& Top, const double* delta, const T* R, co
   DevBuf Sb((size_t)(cap + nu) * ov * es, s), TS((size_t)cap * ov * es, s), t((size_t)cap * cap * sizeof(S), s);
   DevBuf h((size_t)nu * cap * sizeof(S), s), y((size_t)nu * cap * sizeof(S), s);
   DevBuf Tv((size_t)nu * ov * es, s), res((size_t)nu * ov * es, s), r0(nu * 8, s);
+  // status block: residual norms, then the accepted count and the error word (ints)
   DevBuf cand((size_t)nu * ov * es, s), keep(nu * 4, s), stat((size_t)nu * 8 + 8, s);
   double* rn = stat.as<double>();
   int* st_count = reinterpret_cast<int*>(stat.as<double>() + nu);
@@ -943,17 +945,19 @@ void inner_tda(int ov, const TdaOpT<T>& Top, const double* delta, const T* R, co
     if (!last) {
       precond_tda<T>(res.as<T>(), sh, delta, nu, ov, cand.as<T>(), s);
       zero_converged<T>(cand.as<T>(), nu, nu, ov, rn, nullptr, r0.as<double>(), tol, s);
-      orth_append_async<T>(Sb.as<T>(), N, cand.as<T>(), nu, ov, keep.as<int>(), st_count, s);
+      orth_append_async<T>(Sb.as<T>(), N, cand.as<T>(), nu, ov, keep.as<int>(), st_count, nullptr, cnt.tc_err, s);
     }
-    std::vector<double> blk = d2h_checked(stat.as<double>(), (size_t)nu + 1, cnt.tc_err, s);
+    std::vector<double> blk = last ? d2h_checked(stat.as<double>(), (size_t)nu + 1, cnt.tc_err, s)
+                                   : d2h(stat.as<double>(), (size_t)nu + 1, s);
+    int ints[2];   // accepted count, error word
+    std::memcpy(ints, &blk[nu], sizeof(ints));
+    if (!last) raise_tc_error(ints[1], cnt.tc_err, s);
     int m = 0;
     for (int j = 0; j < nu; ++j)
       if (!(std::sqrt(blk[j]) / r0h[j] <= tol)) ++m;
     if (m == 0 || last) break;
     if (N + m > cap) break;
-    int dev_count;
-    std::memcpy(&dev_count, &blk[nu], sizeof(int));
-    const int nacc = std::min(dev_count, ov - N);   // already in S[N...]
+    const int nacc = std::min(ints[0], ov - N);   // already in S[N...]
     if (nacc == 0) break;
     {
       ScopedPhase ph(PH_RIS, s);

@@ -51,17 +51,36 @@ template <typename T>
 __global__ void __launch_bounds__(1024) k_row_sumsq(const T* X, long long ldx, int n, double* out) {
   __shared__ double red[32];
   const T* x = X + blockIdx.x * ldx;
+  double acc;
   // per-thread partials in the row's precision (FP32 rows: FP32 FMA rate); four
-  // independent accumulators keep four loads in flight
-  T p0 = T(0), p1 = T(0), p2 = T(0), p3 = T(0);
-  const int st = blockDim.x;
-  int e = threadIdx.x;
-  for (; e + 3 * st < n; e += 4 * st) {
-    const T v0 = x[e], v1 = x[e + st], v2 = x[e + 2 * st], v3 = x[e + 3 * st];
-    p0 = fma(v0, v0, p0); p1 = fma(v1, v1, p1); p2 = fma(v2, v2, p2); p3 = fma(v3, v3, p3);
+  // independent accumulators keep four loads in flight.  FP32 ones keep the roundings of
+  // their squares and sums, so that all else is added in FP64.
+  if constexpr (sizeof(T) == 4) {
+    float p[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int e = threadIdx.x; e < n; e += 4 * blockDim.x) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int q = e + j * blockDim.x;
+        const float v = q < n ? x[q] : 0.f, w = __fmul_rn(v, v);
+        const float t = __fadd_rn(p[j], w), b = __fsub_rn(t, p[j]);
+        c[j] += __fmaf_rn(v, v, -w) + __fadd_rn(__fsub_rn(p[j], __fsub_rn(t, b)), __fsub_rn(w, b));
+        p[j] = t;
+      }
+    }
+    acc = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc += (double)p[j] + (double)(isfinite(p[j]) ? c[j] : 0.f);
+  } else {
+    T p0 = T(0), p1 = T(0), p2 = T(0), p3 = T(0);
+    const int st = blockDim.x;
+    int e = threadIdx.x;
+    for (; e + 3 * st < n; e += 4 * st) {
+      const T v0 = x[e], v1 = x[e + st], v2 = x[e + 2 * st], v3 = x[e + 3 * st];
+      p0 = fma(v0, v0, p0); p1 = fma(v1, v1, p1); p2 = fma(v2, v2, p2); p3 = fma(v3, v3, p3);
+    }
+    for (; e < n; e += st) { const T v = x[e]; p0 = fma(v, v, p0); }
+    acc = ((double)p0 + (double)p1) + ((double)p2 + (double)p3);
   }
-  for (; e < n; e += st) { const T v = x[e]; p0 = fma(v, v, p0); }
-  double acc = ((double)p0 + (double)p1) + ((double)p2 + (double)p3);
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
@@ -130,14 +149,19 @@ __global__ void k_gather_rows(const T* src, const int* idx, int k, int n, T* dst
 // Grid: x over column blocks, y over source rows.
 template <typename T>
 __global__ void k_compact_rows(const T* __restrict__ src, const int* __restrict__ keep, int nc, int n,
-                               T* __restrict__ dst, int* __restrict__ count) {
+                               T* __restrict__ dst, int* __restrict__ count, const int* __restrict__ info,
+                               const int* __restrict__ err) {
   const int r = blockIdx.y;
   __shared__ int pos;
   if (threadIdx.x == 0) {
     int p = 0;
     for (int q = 0; q < r; ++q) p += keep[q] ? 1 : 0;
     pos = p;
-    if (r == nc - 1 && blockIdx.x == 0) *count = p + (keep[r] ? 1 : 0);
+    if (r == nc - 1 && blockIdx.x == 0) {
+      count[0] = p + (keep[r] ? 1 : 0);
+      if (info) count[-1] = *info;
+      if (err) count[1] = *err;
+    }
   }
   __syncthreads();
   if (!keep[r]) return;
@@ -297,10 +321,9 @@ void unit_rows(double* out, int k, int n, const int* idx, cudaStream_t s) {
 template <typename T>
 void row_sumsq(const T* X, long long ldx, int k, int n, double* out, cudaStream_t s) {
   if (k <= 0) return;
-  // FP64: about 16 elements per thread, since short rows wait for the butterflies of 32
-  // warps (rows of 3456: 4.8 us with 1024 threads, 3.7 with 256).  FP32 rows keep 1024, so
-  // that as few squares as can be are added in FP32.
-  int threads = sizeof(T) == 8 ? 64 : 1024;
+  // about 16 elements per thread: the FP64 butterflies of 32 warps are what short rows
+  // wait for (rows of 3456: 4.8 us with 1024 threads, 3.7 with 256)
+  int threads = 64;
   while (threads < 1024 && threads * 16 < n) threads *= 2;
   k_row_sumsq<T><<<k, threads, 0, s>>>(X, ldx, n, out);
   count_launch(); TD_LAUNCH_CHECK();
@@ -347,15 +370,16 @@ void gather_rows(const T* src, const int* idx, int k, int n, T* dst, cudaStream_
 template void gather_rows<double>(const double*, const int*, int, int, double*, cudaStream_t);
 template void gather_rows<float>(const float*, const int*, int, int, float*, cudaStream_t);
 template <typename T>
-void compact_rows(const T* src, const int* keep, int nc, int n, T* dst, int* count, cudaStream_t s) {
-  if (nc <= 0) { TD_CUDA(cudaMemsetAsync(count, 0, sizeof(int), s)); return; }
+void compact_rows(const T* src, const int* keep, int nc, int n, T* dst, int* count, const int* info, const int* err,
+                  cudaStream_t s) {
+  TD_REQUIRE(nc > 0, TDDFT_ERR_ARG, "compact_rows: no rows");
   TD_REQUIRE(nc <= 65535, TDDFT_ERR_ARG, "compact_rows: too many rows");
   dim3 grid((unsigned)std::min<long long>((n + 255) / 256, 64), nc);
-  k_compact_rows<T><<<grid, 256, 0, s>>>(src, keep, nc, n, dst, count);
+  k_compact_rows<T><<<grid, 256, 0, s>>>(src, keep, nc, n, dst, count, info, err);
   count_launch(); TD_LAUNCH_CHECK();
 }
-template void compact_rows<double>(const double*, const int*, int, int, double*, int*, cudaStream_t);
-template void compact_rows<float>(const float*, const int*, int, int, float*, int*, cudaStream_t);
+template void compact_rows<double>(const double*, const int*, int, int, double*, int*, const int*, const int*, cudaStream_t);
+template void compact_rows<float>(const float*, const int*, int, int, float*, int*, const int*, const int*, cudaStream_t);
 
 template <typename T>
 void zero_converged(T* X, int rows, int nr, int n, const double* a1, const double* a2, const double* g,

@@ -30,9 +30,11 @@ template <typename T>
 void precond_paired(const T* gp, const T* gm, const double* shift, const double* delta, int k, int n,
                     T* out_u, T* out_w, cudaStream_t s);
 // Stream compaction of rows: the rows r < nc of src with keep[r] != 0 go, in
-// order, to the leading rows of dst; count[0] = their number.
+// order, to the leading rows of dst; count[0] = their number.  For a status block that
+// the host reads in one copy: count[-1] = *info and count[1] = *err, each unless NULL.
 template <typename T>
-void compact_rows(const T* src, const int* keep, int nc, int n, T* dst, int* count, cudaStream_t s);
+void compact_rows(const T* src, const int* keep, int nc, int n, T* dst, int* count, const int* info, const int* err,
+                  cudaStream_t s);
 // Zero row r of X [rows][n] when sqrt(a1[q] + a2[q]) / g[q] <= tol, q = r % nr
 // (a2 may be NULL): masks the directions of converged systems on the device.
 template <typename T>

@@ -1,6 +1,6 @@
-"""Squared norms of FP32 rows (row_sumsq, csrc/vecops.cu): with 1024 elements or fewer
-every square is its thread's only one and everything is added in FP64, so whole
-numbers below 2^12 (exact squares, inexact FP32 sums of them) give exact norms."""
+"""Squared norms of FP32 rows (row_sumsq, csrc/vecops.cu) keep the roundings of their FP32
+squares and sums: whole numbers below 2^15 (inexact squares and sums of them) give
+exact norms."""
 import ctypes as C
 import os
 import subprocess
@@ -18,7 +18,7 @@ extern "C" void norms(const float* x, long long ld, int k, int n, double* out) {
 """
 
 
-@pytest.mark.parametrize("n", [1, 65, 500, 1023, 1024])
+@pytest.mark.parametrize("n", [1, 65, 500, 1023, 1024, 3456, 20001])
 def test_exact_squares_add_exactly(n, tmp_path):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
@@ -33,7 +33,7 @@ def test_exact_squares_add_exactly(n, tmp_path):
                    ["-I", build.CSRC, "-shared", "-cudart", "shared", src, build.LIBPATH, "-o", lib,
                     "-Xlinker", "-rpath=" + os.path.dirname(build.LIBPATH)], check=True)
     shim = C.CDLL(lib)
-    x = np.random.default_rng(n).integers(3000, 4096, (5, n)).astype(np.float64)
+    x = np.random.default_rng(n).integers(30000, 32768, (5, n)).astype(np.float64)
     xd = torch.from_numpy(x.astype(np.float32)).cuda()
     out = torch.zeros(5, dtype=torch.float64, device="cuda")
     torch.cuda.synchronize()
