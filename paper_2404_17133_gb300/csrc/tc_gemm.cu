@@ -327,6 +327,16 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
   return r;
 }
 
+// Tensor memory of a pair (cta_group::2).  Both CTAs have to be running when either
+// allocates, neither gives up the permit before both have allocated, and neither leaves before both
+// have freed: a cluster barrier stands before the allocation, after it and after the
+// freeing.  With only the one after it, where kernels of several streams share the
+// GPU and the two CTAs start at different times, the second CTA's allocation now and then
+// waited forever (once in some thousands of products, 16 streams).
+__device__ __forceinline__ void pair_relinquish() {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+}
+
 // Load into this CTA (or, with a mask, into the same offset of its CTAs), signalling
 // the mbarrier `bar` (a shared::cluster address) of the pair's leader.
 __device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
@@ -409,13 +419,15 @@ k1_pair_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant_
     mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncwarp();
+  cluster_sync_all();   // every barrier of the cluster initialised, and both CTAs of a pair running
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)), "r"(BN));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   __syncthreads();
-  cluster_sync_all();   // every barrier of the cluster initialised
+  cluster_sync_all();   // both CTAs' tensor memory allocated
+  if (warp == 1) pair_relinquish();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
@@ -531,11 +543,12 @@ k1_pair_kernel(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant_
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  cluster_sync_all();   // no CTA frees its half or leaves while the other may still use it
+  cluster_sync_all();   // no CTA frees its half while the other may still use it
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
   }
+  cluster_sync_all();   // nor leaves before both halves are free
 }
 
 // ---------------------------------------------------------------------------
@@ -700,13 +713,15 @@ k_stage1_pair(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__
     mbar_init(bempty, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncwarp();
+  cluster_sync_all();   // every barrier of the cluster initialised, and both CTAs of a pair running
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)), "r"(2 * BN));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   __syncthreads();
-  cluster_sync_all();   // every barrier of the cluster initialised
+  cluster_sync_all();   // both CTAs' tensor memory allocated
+  if (warp == 1) pair_relinquish();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
@@ -944,11 +959,12 @@ k_stage1_pair(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  cluster_sync_all();   // no CTA frees its half or leaves while the other may still use it
+  cluster_sync_all();   // no CTA frees its half while the other may still use it
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN));
   }
+  cluster_sync_all();   // nor leaves before both halves are free
 }
 
 __device__ __forceinline__ unsigned char to_e4m3(float x) {
