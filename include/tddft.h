@@ -425,7 +425,8 @@ tddft_status tddft_pool_usage(int device, unsigned long long* used_current,
  * number of launches, their summed device time (ms) and the algorithmic
  * flops (2*M*N*K per launch) since the last reset: which = 0 for the
  * tcgen05 kernel (tensor_cores on), 1 for the contraction of products without
- * tensor_cores (the sliced FP64 / FP32 kernel and the sum of its K splits).  Other values:
+ * tensor_cores (the sliced FP64 / FP32 kernel with its guard and the sum of
+ * its K splits, or the FP64 / FP32 units' in small products).  Other values:
  * TDDFT_ERR_ARG.                                                          */
 tddft_status tddft_profile(tddft_ctx* ctx, int enable);
 tddft_status tddft_profile_read(const tddft_ctx* ctx, int which, long long* launches,

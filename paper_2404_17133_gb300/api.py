@@ -393,7 +393,7 @@ class Solver:
 
     def apply(self, kind, X, precision=PLAIN, tensor_cores=False):
         """kind 0: A X, 1: ((A+B)X, (A-B)X), 2: T X (ris), 3: ris pair.
-        tensor_cores: 0/False off (FP64 / FP32 products by exact slices), 1/True tcgen05, 2 tcgen05 with the FP8 ris rows."""
+        tensor_cores: 0/False off (large FP64 / FP32 products by exact slices), 1/True tcgen05, 2 tcgen05 with the FP8 ris rows."""
         if _is_cuda(X):
             import torch
             out0 = torch.empty_like(X)

@@ -116,8 +116,8 @@ struct OpDims {
 enum class OpMode { TDA, PAIRED };
 
 // out0 = A X (TDA) or (A+B) X and out1 = (A-B) X (PAIRED); X, out FP64 [m][ov].
-// tc: 0 exchange contractions by exact slices of the FP64 or FP32 operands (BF16 rows:
-// on the FP32 units); nonzero the exchange contractions on tcgen05
+// tc: 0 exchange contractions by exact slices of the FP64 or FP32 operands (BF16 rows
+// and small products: on the FP32 or FP64 units); nonzero the exchange contractions on tcgen05
 // (exact factor sets: FP16 hi+lo operands with power-of-two scales, three
 // products, FP32-accurate; ris factor sets: trial vectors as BF16 hi+lo
 // against the plain BF16 rows, or the FP8 rows when the set has them).

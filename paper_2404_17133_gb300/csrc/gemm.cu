@@ -1,5 +1,5 @@
 // Strided, batched SIMT GEMM used for the operator's contractions in the
-// allocation-free product and over BF16 rows without tensor cores, and for the skinny products of the Davidson subspace algebra
+// allocation-free product, over BF16 rows without tensor cores and in small products, and for the skinny products of the Davidson subspace algebra
 // (projection V^T (AV), Ritz vectors V x, Gram-Schmidt coefficients).
 //
 // Tiling: a CTA computes a BM x BN tile of C from BK-deep slabs of A and B staged

@@ -36,7 +36,7 @@
 //
 // Measured, 60 x 400 orbitals, contraction of 118 rows P with 10 vectors (FP64): 787 ->
 // 610 us (MMAs alone 528), its first stage 375 -> 233; 212 rows, 13 vectors (FP32): 550
-// -> 458 and 290 -> 126.  The guard takes 65 and 43 us per 103 rows (FP64), 85 and 63 per
+// -> 458 and 290 -> 126.  The guard takes 51 and 29 us per 103 rows (FP64), 81 and 57 per
 // 180 (FP32), and a sixth (fourth) more to store per element cut.  Not faster: CTA pairs (N = 64 in a pair takes twice the
 // clocks), two half tiles whose runs end half a run apart (711 and 701: the shorter
 // products cost more than the overlap of the epilogue gains).
