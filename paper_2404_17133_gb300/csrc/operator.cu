@@ -306,6 +306,21 @@ static SumTerm term_of(const TcSum& k, const DevBuf& b) {
   return t;
 }
 
+// Hi and lo parts of Z and Q for pc rows of a chunk (elements of es bytes in rows of nvz and
+// noz; noz = 0: no Q), in one allocation: on a fresh stream each of megabytes takes 40 us.
+struct StageParts {
+  DevBuf buf;
+  unsigned char *z[2], *q[2];
+  StageParts(int m, int no, int pc, int nvz, int noz, int es, cudaStream_t s) {
+    const size_t rows = (size_t)m * no * pc, zb = rows * nvz * es, qb = rows * noz * es;   // whole 128-byte lines
+    buf = DevBuf(2 * (zb + qb), s);
+    z[0] = buf.as<unsigned char>();
+    z[1] = z[0] + zb;
+    q[0] = z[1] + zb;
+    q[1] = q[0] + qb;
+  }
+};
+
 // Operand forms of the trial vectors for the tensor-core exchange contractions,
 // with their scales, in one allocation.
 struct XParts {
@@ -466,24 +481,20 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
       const float* inv2 = inv1 + 1;
       const float* mu1 = inv1 + 2;
       const float* mu2 = mu1 + f.nK;
-      DevBuf Zhi((size_t)m * no * pc * nvz, s), Zlo((size_t)m * no * pc * nvz, s), Qhi, Qlo;
-      if (need_k2) {
-        Qhi = DevBuf((size_t)m * no * pc * noz, s);
-        Qlo = DevBuf((size_t)m * no * pc * noz, s);
-      }
+      const StageParts zq(m, no, pc, nvz, need_k2 ? noz : 0, 1, s);
       const int Mz = m * no;
       for (int p0 = 0; p0 < f.nK; p0 += pc) {
         const int pn = (f.nK - p0 < pc) ? f.nK - p0 : pc;
         tc_stage1_fp8(static_cast<const __nv_bfloat16*>(xp.th), static_cast<const __nv_bfloat16*>(xp.tl), m, nv, no,
                       static_cast<const __nv_bfloat16*>(f.Koo_hi) + (size_t)p0 * no * nop, no, pn, mu1 + p0,
-                      Zhi.as<unsigned char>(), Zlo.as<unsigned char>(), d.tc_err, s);
-        tc_contract8(Zhi.as<unsigned char>(), Zlo.as<unsigned char>(), Mz, pn, nv,
+                      zq.z[0], zq.z[1], d.tc_err, s);
+        tc_contract8(zq.z[0], zq.z[1], Mz, pn, nv,
                      f.Kvv8 + (size_t)p0 * nv * nv16, nv, K1b.as<float>(), p0 > 0, inv1, d.tc_err, s, K1s);
         if (need_k2) {
           tc_stage1_fp8(static_cast<const __nv_bfloat16*>(xp.sh), static_cast<const __nv_bfloat16*>(xp.sl), m, no, nv,
                         static_cast<const __nv_bfloat16*>(f.Kovp_hi) + (size_t)p0 * no * nvp, no, pn, mu2 + p0,
-                        Qhi.as<unsigned char>(), Qlo.as<unsigned char>(), d.tc_err, s);
-          tc_contract8(Qhi.as<unsigned char>(), Qlo.as<unsigned char>(), Mz, pn, no,
+                        zq.q[0], zq.q[1], d.tc_err, s);
+          tc_contract8(zq.q[0], zq.q[1], Mz, pn, no,
                        f.Kvo8 + (size_t)p0 * nv * no16, nv, K2b.as<float>(), p0 > 0, inv2, d.tc_err, s, K2s);
         }
       }
@@ -503,18 +514,14 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
         mz = xp.sc + 1; mq = xp.sc + 2; f1 = xp.sc + 3; f2 = xp.sc + 4;
       }
       const int nvz = tc_zpad(nv, 2), noz = tc_zpad(no, 2);
-      DevBuf Zhi((size_t)m * no * pc * nvz * 2, s), Zlo((size_t)m * no * pc * nvz * 2, s), Qhi, Qlo;
-      if (need_k2) {
-        Qhi = DevBuf((size_t)m * no * pc * noz * 2, s);
-        Qlo = DevBuf((size_t)m * no * pc * noz * 2, s);
-      }
+      const StageParts zq(m, no, pc, nvz, need_k2 ? noz : 0, 2, s);
       const int Mz = m * no;
       for (int p0 = 0; p0 < f.nK; p0 += pc) {
         const int pn = (f.nK - p0 < pc) ? f.nK - p0 : pc;
         tc_stage1(xp.th, xp.tl, m, nv, no, at16(f.Koo_hi, (size_t)p0 * no * nop),
-                  f16 ? at16(f.Koo_lo, (size_t)p0 * no * nop) : nullptr, no, pn, et, mz, Zhi.p, Zlo.p, d.tc_err, s);
+                  f16 ? at16(f.Koo_lo, (size_t)p0 * no * nop) : nullptr, no, pn, et, mz, zq.z[0], zq.z[1], d.tc_err, s);
         const bool timed = d.prof && d.prof->on && f16;
-        tc_contract(Zhi.p, Zlo.p, nvz, Mz, pn, nv, at16(f.Kvv_hi, (size_t)p0 * nv * nvp),
+        tc_contract(zq.z[0], zq.z[1], nvz, Mz, pn, nv, at16(f.Kvv_hi, (size_t)p0 * nv * nvp),
                     f16 ? at16(f.Kvv_lo, (size_t)p0 * nv * nvp) : nullptr, nv, K1b.as<float>(), p0 > 0, et, f1,
                     d.tc_err, s, timed ? d.prof : nullptr, 2.0 * Mz * (double)nv * (double)pn * nv,
                     // Z hi+lo [Mz][pn*nv], L_vv chunk [pn*nv][nv] (hi+lo for FP16), K1 FP32
@@ -524,8 +531,8 @@ static void apply_operator_t(const OpDims& d, const FactorSet& f, const TX* X, i
                     f16 ? kExchangeKb : 0, K1s);
         if (need_k2) {
           tc_stage1(xp.sh, xp.sl, m, no, nv, at16(f.Kovp_hi, (size_t)p0 * no * nvp),
-                    f16 ? at16(f.Kovp_lo, (size_t)p0 * no * nvp) : nullptr, no, pn, et, mq, Qhi.p, Qlo.p, d.tc_err, s);
-          tc_contract(Qhi.p, Qlo.p, noz, Mz, pn, no, at16(f.Kvo_hi, (size_t)p0 * nv * nop),
+                    f16 ? at16(f.Kovp_lo, (size_t)p0 * no * nvp) : nullptr, no, pn, et, mq, zq.q[0], zq.q[1], d.tc_err, s);
+          tc_contract(zq.q[0], zq.q[1], noz, Mz, pn, no, at16(f.Kvo_hi, (size_t)p0 * nv * nop),
                       f16 ? at16(f.Kvo_lo, (size_t)p0 * nv * nop) : nullptr, nv, K2b.as<float>(), p0 > 0, et, f2,
                       d.tc_err, s, nullptr, 0.0, 0.0, f16 ? kExchangeKb : 0, K2s);
         }
