@@ -49,6 +49,7 @@ inline void count_launch(int n = 1) { g_launches += n; }
 // same stream (stream order makes the reuse safe), so the many small buffers
 // of an iterative solve cost no allocator calls; larger blocks go straight to
 // cudaMallocAsync / cudaFreeAsync.  pool_trim returns a stream's cached blocks.
+constexpr size_t kCacheMax = 64ull << 20;           // larger blocks are not cached
 constexpr size_t kCachedPerStream = 4ull << 30;     // cap on idle cached bytes per stream
 void* pool_get(size_t bytes, cudaStream_t s);
 void pool_put(void* p, size_t bytes, cudaStream_t s);

@@ -12,7 +12,6 @@ namespace tddft {
 
 namespace {
 
-constexpr size_t kCacheMax = 64ull << 20;           // larger blocks are not cached
 
 // size class: 256 B minimum, powers of two up to 1 MiB, then 1 MiB multiples
 size_t size_class(size_t n) {

@@ -307,17 +307,27 @@ static SumTerm term_of(const TcSum& k, const DevBuf& b) {
 }
 
 // Hi and lo parts of Z and Q for pc rows of a chunk (elements of es bytes in rows of nvz and
-// noz; noz = 0: no Q), in one allocation: on a fresh stream each of megabytes takes 40 us.
+// noz; noz = 0: no Q), in one allocation where the stream's cache takes it: on a fresh stream
+// each of megabytes costs 40 us.
 struct StageParts {
-  DevBuf buf;
+  DevBuf buf[4];
   unsigned char *z[2], *q[2];
   StageParts(int m, int no, int pc, int nvz, int noz, int es, cudaStream_t s) {
     const size_t rows = (size_t)m * no * pc, zb = rows * nvz * es, qb = rows * noz * es;   // whole 128-byte lines
-    buf = DevBuf(2 * (zb + qb), s);
-    z[0] = buf.as<unsigned char>();
-    z[1] = z[0] + zb;
-    q[0] = z[1] + zb;
-    q[1] = q[0] + qb;
+    if (2 * (zb + qb) <= kCacheMax) {
+      buf[0] = DevBuf(2 * (zb + qb), s);
+      z[0] = buf[0].as<unsigned char>();
+      z[1] = z[0] + zb;
+      q[0] = z[1] + zb;
+      q[1] = q[0] + qb;
+      return;
+    }
+    for (int k = 0; k < 4; ++k)
+      if (k < 2 || qb) buf[k] = DevBuf(k < 2 ? zb : qb, s);
+    for (int k = 0; k < 2; ++k) {
+      z[k] = buf[k].as<unsigned char>();
+      q[k] = buf[2 + k].as<unsigned char>();
+    }
   }
 };
 
