@@ -481,7 +481,7 @@ k_slice_mma(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUte
       const int ncol = min(HC, p.N - n0);    // columns of this warp (may be <= 0)
       if constexpr (S == 1) {
         static_assert(W == GUARD_SUMS || HC <= 64, "one bit per column");
-        constexpr bool SUMS = W == GUARD_SUMS;   // k_slice_sum judges
+        constexpr bool SUMS = W == GUARD_SUMS;   // k_slice_sum decides
         // the bounds of this warp's rows and columns, while the tile is being formed
         __shared__ __align__(16) float2 colb[EPI_WARPS][SUMS ? 1 : HC];
         const float2 none = make_float2(0.f, 0.f);
@@ -969,7 +969,7 @@ __global__ void __launch_bounds__(256) k_slice_cut_t(const CutParams c) {
 }
 
 // Sum of the K-split partials in a fixed order (FP64), C = sum + beta C; N: the
-// guard's partials, whose verdict falls here: the outputs to be formed again are
+// guard's partials, decided on here: the outputs to be formed again are
 // dealt to the CTA's warps.  A CTA takes OPB outputs.
 template <typename T, int OPB>
 __global__ void __launch_bounds__(256) k_slice_sum(const T* __restrict__ part, int S, const float* __restrict__ N, int SN,
